@@ -1,6 +1,6 @@
 // force.cu -- particle-particle (EPJ) and particle-superparticle (SPJ)
 // forces from the interaction lists: one CTA per i-group (FP32-relative) or
-// one warp per i-group (FP64 variant).
+// one cluster of CTAs per i-group (FP64 variant).
 //
 // Per i-particle (Sect. 2.2, Eqs. ParticleParticleNbody and
 // ParticleSuperparticleNbody, G = 1, softening eps_i of the receiving
@@ -27,7 +27,7 @@
 // the list in plain FP32 and adds the chunk's sum to its running total with
 // Kahan compensation.  Small groups split their list over several threads
 // per i-particle ("slices"), reduced in FP64 at the end.  The FP64 kernel
-// (one warp per group) is the same walk of the list on FP64 absolute
+// (a cluster of CTAs per group) evaluates the same terms on FP64 absolute
 // coordinates with FP64 sums.
 #include "fdps_internal.cuh"
 
@@ -63,37 +63,6 @@ struct ForceArgs {
 };
 
 namespace {
-
-constexpr int kFBlock = 128;
-constexpr int kFWarps = kFBlock / 32;
-constexpr int kJCap64 = 128;  // EPJ particles per FP64 tile
-
-// Lane -> (i offset, slice) split of a group of n_i particles.
-struct Split {
-    int P, nsl;
-    __device__ __forceinline__ Split(uint32_t ni) {
-        if (ni <= 16u) {
-            P = (int)ni;
-            nsl = 32 / P;
-        } else {
-            P = 32;
-            nsl = 1;
-        }
-    }
-};
-
-// Find the entry owning expanded item `item`: largest e with scan[e] <= item.
-__device__ __forceinline__ int owner(const uint32_t* scan, uint32_t item) {
-    int lo = 0, hi = 32;
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (scan[mid] <= item)
-            lo = mid;
-        else
-            hi = mid;
-    }
-    return lo;
-}
 
 // ---------------------------------------------------------------- FP32
 // One CTA of CB threads (64, 128 or 256: the "block shape" the autotuner
@@ -615,132 +584,264 @@ __global__ void __launch_bounds__(CB, (QUAD ? 512 / CB : 1)) k_force_f32(ForceAr
     }
 }
 
+// ---------------------------------------------------------------- FP64
+// One cluster of kCl64 CTAs (128 threads each) per i-group.  Bound by the
+// FP64 pipe (two lanes per SM and clock: a warp instruction takes it for 16
+// clocks whatever its active lanes), so the split is the one that costs the
+// pipe least: thread t of a CTA owns K <= 4 i-particles (i = t % P + k P) and
+// slice t / P of the CTA's list entries, (K, P, slices) minimising the warps
+// times K per entry (plan_f64: 9 in 10 lanes busy on groups of 30 to 128
+// particles, where one warp per group kept 6 in 10 busy).  The entries of a
+// list go to the cluster's CTAs in turn (entry u to CTA u % kCl64), so every
+// CTA has the same mix of cells and opened leaves, and a group of a few
+// thousand entries takes a twelfth of the time one CTA would need: with one
+// warp or CTA per group the last groups of a 10^5-particle system left most
+// of the SMs idle.  Entries are staged in shared memory by chunk.  Slices
+// and CTAs are summed in a fixed order, through distributed shared memory.
+// Plummer N = 100,003, quadrupoles, n_grp 128: 56.4 -> 19.3 ms for the
+// whole force calculation (one warp per group before).
+constexpr int kF64Block = 128;
+constexpr int kCl64 = 8;     // CTAs per cluster
+constexpr int kCE64 = 128;   // list entries of a CTA staged per chunk (one per thread)
+constexpr int kCJ64 = 128;   // leaf particles per shared tile
+constexpr int kK64 = 4;      // most i-particles per thread
+
+struct F64Shared {
+    dvec4 spj[kCE64];            // centre of mass and -M
+    double q[kCE64][6];          // quadrupole (xx yy zz xy xz yz)
+    dvec4 j[kCJ64];
+    uint32_t ef[kCE64];
+    uint32_t es[kCE64];
+    uint32_t w[2 * (kF64Block / 32)];
+    double part[kK64 * 4][kF64Block];  // a thread's sums: row q * 4 + component
+    double row[4][kK64 * kF64Block];   // the CTA's sums of its i-rows
+    uint32_t g;
+};
+
+// (K, P, slices) of ni i-particles: least FP64 pipe time K * warps / slices
+// per list entry; more slices on ties.
+__device__ __forceinline__ GroupPlan plan_f64(uint32_t ni) {
+    GroupPlan best{kK64, kF64Block, 1};  // more than a CTA holds: rounds
+    float bc = 3.0e38f;
+#pragma unroll
+    for (int K = 1; K <= kK64; ++K) {
+        const int P = (int)((ni + K - 1) / K);
+        if (P > kF64Block) continue;
+        const int nsl = kF64Block / P;
+        const float c = (float)(K * ((P * nsl + 31) / 32)) / (float)nsl;
+        if (c < bc - 1e-6f) {
+            bc = c;
+            best = GroupPlan{K, P, nsl};
+        }
+    }
+    return best;
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// The cluster's address of this CTA's shared variable p in CTA `rank`.
+__device__ __forceinline__ uint32_t peer_smem(const void* p, uint32_t rank) {
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ double ld_peer_f64(uint32_t a) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_peer_u32(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// One round of i-particles (ib .. ib + P K - 1 of the group) with K per
+// thread, over this CTA's share of the list; called by the whole cluster.
+template <bool QUAD, int K>
+__device__ __forceinline__ void force_round_f64(const ForceArgs& A, uint32_t gf, uint32_t ni,
+                                                unsigned long long off, uint32_t len, int P, int nsl,
+                                                uint32_t ib, uint32_t rank, F64Shared& sm) {
+    const int t = threadIdx.x;
+    const int ip = t % P, sl = t / P;
+    const bool on = sl < nsl;
+    double xi[K], yi[K], zi[K], e2[K], ax[K], ay[K], az[K], pp[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+        const uint32_t i = ib + (uint32_t)(ip + q * P);
+        const bool iv = on && i < ni;
+        const uint32_t p = gf + (iv ? i : 0u);
+        const double e = iv ? A.peps[p] : 1.0;
+        xi[q] = A.px[p];
+        yi[q] = A.py[p];
+        zi[q] = A.pz[p];
+        e2[q] = e * e;
+        ax[q] = ay[q] = az[q] = pp[q] = 0.0;
+    }
+    const int kbeg = on ? sl : 0x3FFFFFFF;
+    // entries rank, rank + kCl64, ... of the list are this CTA's
+    const uint32_t mine = len > rank ? (len - rank + kCl64 - 1) / kCl64 : 0u;
+    for (uint32_t base = 0; base < mine; base += kCE64) {
+        const uint32_t u = base + t;
+        const uint32_t ent = u < mine ? A.pool[off + rank + (unsigned long long)u * kCl64] : 0xFFFFFFFFu;
+        const bool leaf = ent != 0xFFFFFFFFu && (ent & kLeafTag);
+        const bool spj = ent != 0xFFFFFFFFu && !(ent & kLeafTag);
+        const uint32_t node = ent & ~kLeafTag;
+        const uint32_t cnt = leaf ? A.nd_count[node] : 0u;
+        uint32_t rs, es, ns, total;
+        block_scan2<kF64Block>(spj ? 1u : 0u, cnt, &rs, &es, &ns, &total, sm.w);
+        if (spj) {
+            const dvec4 c = A.nd_com[node];
+            sm.spj[rs] = make_dvec4(c.x, c.y, c.z, -c.w);
+            if (QUAD)
+#pragma unroll
+                for (int k = 0; k < 6; ++k) sm.q[rs][k] = A.nd_quad[6 * (int64_t)node + k];
+        }
+        sm.ef[t] = leaf ? A.nd_first[node] : 0u;
+        sm.es[t] = es;
+        __syncthreads();
+        for (int k = kbeg; k < (int)ns; k += nsl) {
+            const dvec4 c = sm.spj[k];
+            double qxx, qyy, qzz, qxy, qxz, qyz;
+            if (QUAD) {
+                qxx = sm.q[k][0];
+                qyy = sm.q[k][1];
+                qzz = sm.q[k][2];
+                qxy = sm.q[k][3];
+                qxz = sm.q[k][4];
+                qyz = sm.q[k][5];
+            }
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                const double rx = xi[q] - c.x, ry = yi[q] - c.y, rz = zi[q] - c.z;
+                const double R2 = fma(rx, rx, fma(ry, ry, fma(rz, rz, e2[q])));
+                const double Ri = rsqrt(R2);
+                const double Ri2 = Ri * Ri;
+                if (QUAD) {  // regrouped as in the FP32 kernel: 32 operations and the root
+                    const double Ri4 = Ri2 * Ri2;
+                    const double Ri5 = Ri4 * Ri;
+                    const double Qrx = fma(qxx, rx, fma(qxy, ry, qxz * rz));
+                    const double Qry = fma(qxy, rx, fma(qyy, ry, qyz * rz));
+                    const double Qrz = fma(qxz, rx, fma(qyz, ry, qzz * rz));
+                    const double rQr = fma(rx, Qrx, fma(ry, Qry, rz * Qrz));
+                    const double w = rQr * Ri4;
+                    const double hh = fma(-2.5, w, c.w);
+                    const double hR2 = hh * R2;
+                    ax[q] = fma(Ri5, fma(hR2, rx, Qrx), ax[q]);
+                    ay[q] = fma(Ri5, fma(hR2, ry, Qry), ay[q]);
+                    az[q] = fma(Ri5, fma(hR2, rz, Qrz), az[q]);
+                    pp[q] = fma(Ri, fma(2.0, w, hh), pp[q]);
+                } else {
+                    const double nMRi = c.w * Ri;
+                    const double nMRi3 = nMRi * Ri2;
+                    ax[q] = fma(nMRi3, rx, ax[q]);
+                    ay[q] = fma(nMRi3, ry, ay[q]);
+                    az[q] = fma(nMRi3, rz, az[q]);
+                    pp[q] += nMRi;
+                }
+            }
+        }
+        for (uint32_t c0 = 0; c0 < total; c0 += kCJ64) {
+            const uint32_t m = total - c0 < (uint32_t)kCJ64 ? total - c0 : (uint32_t)kCJ64;
+            if (c0 > 0) __syncthreads();  // previous tile fully consumed
+            for (uint32_t k = t; k < m; k += kF64Block) {
+                const uint32_t item = c0 + k;
+                const int src = owner_chunk<kCE64>(sm.es, item);
+                const uint32_t p = sm.ef[src] + (item - sm.es[src]);
+                sm.j[k] = make_dvec4(A.px[p], A.py[p], A.pz[p], A.pm[p]);
+            }
+            __syncthreads();
+            for (int k = kbeg; k < (int)m; k += nsl) {
+                const dvec4 j = sm.j[k];
+#pragma unroll
+                for (int q = 0; q < K; ++q) {
+                    const double dx = j.x - xi[q], dy = j.y - yi[q], dz = j.z - zi[q];
+                    const double r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, e2[q])));
+                    const double ri = rsqrt(r2);
+                    const double mri = j.w * ri;
+                    const double mri3 = mri * (ri * ri);
+                    ax[q] = fma(mri3, dx, ax[q]);
+                    ay[q] = fma(mri3, dy, ay[q]);
+                    az[q] = fma(mri3, dz, az[q]);
+                    pp[q] -= mri;
+                }
+            }
+        }
+        __syncthreads();  // chunk buffers are rewritten next
+    }
+    // slices, then the cluster's CTAs, in order
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+        sm.part[q * 4 + 0][t] = ax[q];
+        sm.part[q * 4 + 1][t] = ay[q];
+        sm.part[q * 4 + 2][t] = az[q];
+        sm.part[q * 4 + 3][t] = pp[q];
+    }
+    __syncthreads();
+    const int rows = P * K;
+    for (int k = t; k < 4 * rows; k += kF64Block) {
+        const int c = k / rows, r = k - c * rows;
+        const int q = r / P, ipr = r - q * P;
+        double v = 0.0;
+        for (int s2 = 0; s2 < nsl; ++s2) v += sm.part[q * 4 + c][s2 * P + ipr];
+        sm.row[c][r] = v;
+    }
+    cluster_barrier();  // every CTA's rows are written
+    // each CTA finishes every kCl64-th value
+    for (int k = t * kCl64 + (int)rank; k < 4 * rows; k += kF64Block * kCl64) {
+        const int r = k >> 2, c = k & 3;
+        const uint32_t i = ib + (uint32_t)r;
+        if (i >= ni) continue;
+        double v = 0.0;
+#pragma unroll
+        for (int b = 0; b < kCl64; ++b) v += ld_peer_f64(peer_smem(&sm.row[c][r], (uint32_t)b));
+        const uint32_t p = gf + i;
+        if (c == 0)
+            A.ax[p] = v;
+        else if (c == 1)
+            A.ay[p] = v;
+        else if (c == 2)
+            A.az[p] = v;
+        else
+            A.pot[p] = v + A.pm[p] / A.peps[p];  // without the particle's own entry
+    }
+    cluster_barrier();  // the rows have been read: they may be rewritten
+}
+
 template <bool QUAD>
-__global__ void __launch_bounds__(kFBlock) k_force_f64(ForceArgs A) {
-    __shared__ dvec4 s_j[kFWarps][kJCap64];
-    __shared__ uint32_t s_ef[kFWarps][32];
-    __shared__ uint32_t s_es[kFWarps][33];
-    __shared__ double s_red[kFWarps][4][32];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+__global__ void __cluster_dims__(kCl64, 1, 1) __launch_bounds__(kF64Block, 4) k_force_f64(ForceArgs A) {
+    extern __shared__ __align__(32) unsigned char f64_smem[];
+    F64Shared& sm = *reinterpret_cast<F64Shared*>(f64_smem);
     DevState* st = A.st;
     if (st->overflow & kStepInvalid) return;  // as in the FP32 kernel
     const uint32_t ngroups = (uint32_t)st->n_groups;
+    const uint32_t rank = cluster_rank();
     for (;;) {
-        uint32_t g = 0;
-        if (lane == 0) g = atomicAdd(&st->force_counter, 1u);
-        g = __shfl_sync(0xFFFFFFFFu, g, 0);
+        if (rank == 0 && threadIdx.x == 0) sm.g = atomicAdd(&st->force_counter, 1u);
+        cluster_barrier();
+        const uint32_t g = ld_peer_u32(peer_smem(&sm.g, 0));
+        cluster_barrier();  // read by all before it is rewritten or its CTA ends
         if (g >= ngroups) break;
         const uint32_t ni = A.g_count[g], gf = A.g_first[g];
         const unsigned long long off = A.g_off[g];
         const uint32_t len = A.g_len[g];
-        const Split sp(ni);
-        const int ioff = lane % sp.P;
-        const int sl = lane / sp.P;
-        const bool lane_on = sl < sp.nsl;
-        for (uint32_t ib = 0; ib < ni; ib += (uint32_t)sp.P) {
-            const uint32_t i = ib + (uint32_t)ioff;
-            const bool iv = lane_on && i < ni;
-            double xi = 0.0, yi = 0.0, zi = 0.0, e2 = 1.0;
-            if (iv) {
-                xi = A.px[gf + i];
-                yi = A.py[gf + i];
-                zi = A.pz[gf + i];
-                e2 = A.peps[gf + i] * A.peps[gf + i];
-            }
-            const int kbeg = iv ? sl : 0x7FFFFFFF;
-            double ax = 0.0, ay = 0.0, az = 0.0, pp = 0.0;
-            for (uint32_t t = 0; t < len; t += 32) {
-                const bool ve = t + lane < len;
-                const uint32_t e = ve ? A.pool[off + t + lane] : 0u;
-                const bool isleaf = ve && (e & kLeafTag);
-                const uint32_t node = e & ~kLeafTag;
-                uint32_t cnt = 0, first = 0;
-                if (isleaf) {
-                    cnt = A.nd_count[node];
-                    first = A.nd_first[node];
-                }
-                uint32_t inc = cnt;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-                    if (lane >= o) inc += v;
-                }
-                const uint32_t total = __shfl_sync(0xFFFFFFFFu, inc, 31);
-                s_ef[w][lane] = first;
-                s_es[w][lane] = inc - cnt;
-                // superparticles: every lane of a slice reads the entry from the pool
-                const uint32_t nent = len - t < 32u ? len - t : 32u;
-                for (int k = kbeg; k < (int)nent; k += sp.nsl) {
-                    const uint32_t ek = A.pool[off + t + k];
-                    if (ek & kLeafTag) continue;
-                    const dvec4 c = A.nd_com[ek];
-                    const double rx = xi - c.x, ry = yi - c.y, rz = zi - c.z;
-                    const double R2 = rx * rx + ry * ry + rz * rz + e2;
-                    const double Ri = rsqrt(R2);
-                    const double Ri2 = Ri * Ri;
-                    const double MRi = c.w * Ri;
-                    const double MRi3 = MRi * Ri2;
-                    ax -= MRi3 * rx;
-                    ay -= MRi3 * ry;
-                    az -= MRi3 * rz;
-                    pp -= MRi;
-                    if (QUAD) {
-                        const double* Q = A.nd_quad + 6 * (int64_t)ek;
-                        const double Qrx = Q[0] * rx + Q[3] * ry + Q[4] * rz;
-                        const double Qry = Q[3] * rx + Q[1] * ry + Q[5] * rz;
-                        const double Qrz = Q[4] * rx + Q[5] * ry + Q[2] * rz;
-                        const double rQr = rx * Qrx + ry * Qry + rz * Qrz;
-                        const double Ri5 = Ri2 * Ri2 * Ri;
-                        const double c7 = 2.5 * rQr * Ri5 * Ri2;
-                        ax += Qrx * Ri5 - c7 * rx;
-                        ay += Qry * Ri5 - c7 * ry;
-                        az += Qrz * Ri5 - c7 * rz;
-                        pp -= 0.5 * rQr * Ri5;
-                    }
-                }
-                __syncwarp();
-                for (uint32_t c0 = 0; c0 < total; c0 += kJCap64) {
-                    const uint32_t m = total - c0 < (uint32_t)kJCap64 ? total - c0 : (uint32_t)kJCap64;
-                    for (uint32_t k = lane; k < m; k += 32) {
-                        const uint32_t item = c0 + k;
-                        const int src = owner(s_es[w], item);
-                        const uint32_t p = s_ef[w][src] + (item - s_es[w][src]);
-                        s_j[w][k] = make_dvec4(A.px[p], A.py[p], A.pz[p], A.pm[p]);
-                    }
-                    __syncwarp();
-                    for (int k = kbeg; k < (int)m; k += sp.nsl) {
-                        const dvec4 j = s_j[w][k];
-                        const double dx = j.x - xi, dy = j.y - yi, dz = j.z - zi;
-                        const double r2 = dx * dx + dy * dy + dz * dz + e2;
-                        const double ri = rsqrt(r2);
-                        const double mri = j.w * ri;
-                        const double mri3 = mri * ri * ri;
-                        ax += mri3 * dx;
-                        ay += mri3 * dy;
-                        az += mri3 * dz;
-                        pp -= mri;
-                    }
-                    __syncwarp();
-                }
-                __syncwarp();
-            }
-            s_red[w][0][lane] = iv ? ax : 0.0;
-            s_red[w][1][lane] = iv ? ay : 0.0;
-            s_red[w][2][lane] = iv ? az : 0.0;
-            s_red[w][3][lane] = iv ? pp : 0.0;
-            __syncwarp();
-            if (iv && sl == 0) {
-                double r[4] = {0.0, 0.0, 0.0, 0.0};
-                for (int s2 = 0; s2 < sp.nsl; ++s2)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) r[k] += s_red[w][k][s2 * sp.P + ioff];
-                const uint32_t p = gf + i;
-                A.ax[p] = r[0];
-                A.ay[p] = r[1];
-                A.az[p] = r[2];
-                A.pot[p] = r[3] + A.pm[p] / A.peps[p];
-            }
-            __syncwarp();
+        for (uint32_t ib = 0; ib < ni;) {
+            const GroupPlan pl = plan_f64(ni - ib);
+            if (pl.K == 1)
+                force_round_f64<QUAD, 1>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
+            else if (pl.K == 2)
+                force_round_f64<QUAD, 2>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
+            else if (pl.K == 3)
+                force_round_f64<QUAD, 3>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
+            else
+                force_round_f64<QUAD, 4>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
+            ib += (uint32_t)(pl.P * pl.K);
         }
     }
 }
@@ -781,12 +882,19 @@ void launch_f32_shape(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s, int cb,
     }
 }
 
-int force_blocks_f64(fdps_ctx* ctx, int quad) {
+// One resident wave of clusters of FP64 force CTAs.
+template <bool QUAD>
+int launch_f64(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s) {
+    FDPS_CUDA_TRY(ctx, cudaFuncSetAttribute(k_force_f64<QUAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)sizeof(F64Shared)));
     int per_sm = 0;
-    const cudaError_t e = quad ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_force_f64<true>, kFBlock, 0)
-                               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_force_f64<false>, kFBlock, 0);
-    if (e != cudaSuccess || per_sm < 1) per_sm = 4;
-    return per_sm * ctx->sm_count;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_force_f64<QUAD>, kF64Block, sizeof(F64Shared)) !=
+            cudaSuccess ||
+        per_sm < 1)
+        per_sm = 1;
+    const int clusters = per_sm * ctx->sm_count / kCl64;
+    k_force_f64<QUAD><<<(clusters > 0 ? clusters : 1) * kCl64, kF64Block, sizeof(F64Shared), s>>>(A);
+    return FDPS_OK;
 }
 
 ForceArgs force_args(fdps_tree* t, fdps_psys* ps) {
@@ -827,11 +935,8 @@ int compute_forces(fdps_tree* t, fdps_psys* ps, int spj_kind) {
     const bool quad = spj_kind == FDPS_GRAV_SPJ_QUAD;
     cudaStream_t s = ctx->stream;
     if (t->p.precision == FDPS_FP64) {
-        const int blocks = force_blocks_f64(ctx, quad);
-        if (quad)
-            k_force_f64<true><<<blocks, kFBlock, 0, s>>>(A);
-        else
-            k_force_f64<false><<<blocks, kFBlock, 0, s>>>(A);
+        const int rc = quad ? launch_f64<true>(A, ctx, s) : launch_f64<false>(A, ctx, s);
+        if (rc) return rc;
     } else {
         // tile depth: list entries staged per chunk (0 = default 512); block
         // shape: threads per CTA (0 = 128) and i-particles per thread (0 = 5)
