@@ -39,6 +39,7 @@ struct ForceArgs {
     const uint32_t* g_count;
     const unsigned long long* g_off;
     const uint32_t* g_len;
+    const uint32_t* g_nspj;
     const float4* g_ch;
     const float4* g_cl;
     const uint32_t* pool;
@@ -69,13 +70,17 @@ namespace {
 // picks, with the cap KMAX on i-particles per thread) per i-group.  Thread t
 // owns K <= KMAX i-particles (i = t % P + k P, k < K) and the list slice
 // j = t / P (mod nsl); (K, P, nsl) is chosen per group to keep the most
-// lanes busy.  The list is consumed in chunks of 256 or 512 entries (the
-// tile depth, EPT per thread); each chunk's superparticles and leaf
-// particles are staged in shared memory, and each thread folds its FP32
-// partial sums of the chunk into Kahan-compensated running sums once per
-// chunk.
-
-constexpr int kCJ = 224;  // leaf particles per shared tile (the shared memory of 128 x 5 fits 48 KB)
+// lanes busy.  A list holds its superparticles first and its opened leaves
+// after them: the superparticles are consumed in chunks of 256 or 512 (the
+// tile depth, EPT per thread), then the leaves' particles in tiles of up to
+// 1024, staged in shared memory; each thread folds its FP32 partial sums of a
+// chunk or tile into Kahan-compensated running sums.  With the two kinds
+// mixed in the list, every chunk needed a scan and four smaller tiles with
+// two barriers each, about 70 barriers a group instead of 21: the pass over
+// 190,000 monopole groups of 16 particles (256 clusters, n_grp 64) took 7.51
+// ms and takes 6.03, 2^20 Plummer particles with quadrupoles at n_grp 128
+// 3.94 and 3.72, 2^24 at n_grp 256 73.2 and 72.0 (FMA pipe 74 % busy: bound by
+// the FP32 pipe and its register-operand conflicts), for 4 % in the walk.
 
 struct GroupPlan {
     int K, P, nsl;
@@ -144,6 +149,33 @@ __device__ __forceinline__ void block_scan2(uint32_t a, uint32_t b, uint32_t* ea
     *eb = ob + ib - b;
     *ta = sa;
     *tb = sb;
+}
+
+// Block-wide exclusive scan (CB threads); s_w holds CB / 32 words.
+template <int CB>
+__device__ __forceinline__ uint32_t block_scan1(uint32_t a, uint32_t* total, uint32_t* s_w) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t ia = a;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, ia, o);
+        if (lane >= o) ia += v;
+    }
+    if (CB == 32) {
+        *total = __shfl_sync(0xFFFFFFFFu, ia, 31);
+        return ia - a;
+    }
+    if (lane == 31) s_w[w] = ia;
+    __syncthreads();
+    uint32_t o = 0, sum = 0;
+#pragma unroll
+    for (int k = 0; k < CB / 32; ++k) {
+        const uint32_t x = s_w[k];
+        if (k < w) o += x;
+        sum += x;
+    }
+    *total = sum;
+    return o + ia - a;
 }
 
 // EPT consecutive u32 slots of one thread written as one vector.
@@ -226,27 +258,45 @@ __device__ __forceinline__ f2 f2_rsqrt(f2 v) {
     f2_up(v, a, b);
     return f2_pk(rsqrtf(a), rsqrtf(b));
 }
-// Shared-memory layouts (coordinates relative to the group centre):
-//   superparticles: float4 (x, y, z, -M), float4 (Qxx, Qyy, Qzz, Qxy),
-//     float2 (Qxz, Qyz) in three arrays
-//   leaf particles: float4 (x, y, z, m).
-// A thread's i-particles are paired (2h, 2h+1) in the two lanes; each list
-// entry is broadcast to both lanes.
-template <bool QUAD>
-struct SpjBuf {
-    float4* s0;
-    float4* s1;
-    float2* s2;
+// Shared memory of the FP32 kernels (one CTA per group at a time;
+// coordinates relative to the group centre).  The buffer u holds a chunk of
+// superparticles, float4 (x, y, z, -M), float4 (Qxx, Qyy, Qzz, Qxy), float2
+// (Qxz, Qyz) in three arrays (the first only for monopoles), and after them
+// a tile of leaf particles, float4 (x, y, z, m), with the first particles
+// and the scanned counts of a batch of leaves behind it.  A thread's
+// i-particles are paired (2h, 2h+1) in the two lanes of a packed register;
+// each list entry is broadcast to both lanes.
+constexpr int cmax(int a, int b) { return a > b ? a : b; }
+template <bool QUAD, int EPT, int CB, int KMAX>
+struct F32Shared {
+    static constexpr int kCE = CB * EPT;  // superparticles per chunk
+    static constexpr int kCL = CB * EPT;  // leaves per batch
+    static constexpr int kCJ = 8 * CB < 1024 ? 8 * CB : 1024;  // leaf particles per tile
+    __align__(16) unsigned char u[cmax(kCE * (QUAD ? 40 : 16), kCJ * 16 + 2 * kCL * 4)];
+    uint32_t w[2 * (CB / 32)];
+    float k[KMAX * 8 * CB];  // Kahan sums and compensations
 };
 __device__ __forceinline__ f2 f2_bc(float v) { return f2_pk(v, v); }
 
 template <bool QUAD, int K, int EPT, int CB, int KMAX>
 __device__ __forceinline__ void force_round_f32(const ForceArgs& A, uint32_t gf, uint32_t ni,
-                                                unsigned long long off, uint32_t len, float4 gch,
+                                                unsigned long long off, uint32_t nspj, uint32_t len, float4 gch,
                                                 float4 gcl, int P, int nsl, uint32_t ib,
-                                                float4* s_j, SpjBuf<QUAD> sb, uint32_t* s_ef,
-                                                uint32_t* s_es, uint32_t* s_w,
-                                                float* s_k) {
+                                                F32Shared<QUAD, EPT, CB, KMAX>& sm) {
+    using SM = F32Shared<QUAD, EPT, CB, KMAX>;
+    constexpr int kCJ = SM::kCJ;
+    float4* const s_s0 = reinterpret_cast<float4*>(sm.u);
+    float4* const s_s1 = reinterpret_cast<float4*>(sm.u + (QUAD ? SM::kCE * 16 : 0));
+    float2* const s_s2 = reinterpret_cast<float2*>(sm.u + (QUAD ? SM::kCE * 32 : 0));
+    float4* const s_j = reinterpret_cast<float4*>(sm.u);
+    uint32_t* const s_ef = reinterpret_cast<uint32_t*>(sm.u + kCJ * 16);
+    uint32_t* const s_es = s_ef + SM::kCL;
+    float* const s_k = sm.k;
+    // list entries per loop turn, measured (2, 3, 5, 6 and 1 to 4): quadrupoles
+    // at 2^24 particles 73.5 ms with 2 and 2, 71.9 with 3 and 3; monopoles of
+    // 256 clusters 6.22 ms with 2 and 2, 6.03 with 6 and 2, 7.2 with 3 in the
+    // second loop (registers)
+    constexpr int kUnrollSpj = QUAD ? 5 : 6, kUnrollEpj = QUAD ? 3 : 2;
     constexpr int KP = K / 2;  // i-pairs; an odd K takes its last i-particle on the scalar path
     const int t = threadIdx.x;
     const int ip = t % P, sl = t / P;
@@ -280,65 +330,70 @@ __device__ __forceinline__ void force_round_f32(const ForceArgs& A, uint32_t gf,
 #pragma unroll
     for (int k = 0; k < 8 * K; ++k) s_k[k * CB + t] = 0.0f;
 
-    constexpr int CE = CB * EPT;
-    for (uint32_t base = 0; base < len; base += CE) {
-        // ---- this thread's EPT consecutive entries: type, node data, leaf range
-        uint32_t nspj = 0, npart = 0;
-        uint32_t ent[EPT];
-#pragma unroll
-        for (int r = 0; r < EPT; ++r) {
-            const uint32_t u = base + (uint32_t)(t * EPT + r);
-            ent[r] = u < len ? A.pool[off + u] : 0xFFFFFFFFu;
-        }
-        uint32_t lcnt[EPT], lfirst[EPT];
-#pragma unroll
-        for (int r = 0; r < EPT; ++r) {
-            const bool leaf = ent[r] != 0xFFFFFFFFu && (ent[r] & kLeafTag);
-            const bool spj = ent[r] != 0xFFFFFFFFu && !(ent[r] & kLeafTag);
-            lcnt[r] = leaf ? A.nd_count[ent[r] & ~kLeafTag] : 0u;
-            lfirst[r] = leaf ? A.nd_first[ent[r] & ~kLeafTag] : 0u;
-            nspj += spj ? 1u : 0u;
-            npart += lcnt[r];
-        }
-        uint32_t rs, es, ns, total, esc[EPT];
-        block_scan2<CB>(nspj, npart, &rs, &es, &ns, &total, s_w);
-#pragma unroll
-        for (int r = 0; r < EPT; ++r) {
-            const bool spj = ent[r] != 0xFFFFFFFFu && !(ent[r] & kLeafTag);
-            if (spj) {
-                const uint32_t node = ent[r];
-                const float4 fh = A.nd_f[2 * node], fl = A.nd_f[2 * node + 1];
-                sb.s0[rs] = make_float4((fh.x - gch.x) + (fl.x - gcl.x),
-                                        (fh.y - gch.y) + (fl.y - gcl.y),
-                                        (fh.z - gch.z) + (fl.z - gcl.z), -fh.w);
-                if (QUAD) {
-                    sb.s1[rs] = A.nd_fq0[node];
-                    sb.s2[rs] = A.nd_fq1[node];
-                }
-                ++rs;
-            }
-            esc[r] = es;
-            es += lcnt[r];
-        }
-        // each thread's EPT consecutive slots in one vector store (no bank conflicts)
-        store_entries<EPT>(s_ef + t * EPT, lfirst);
-        store_entries<EPT>(s_es + t * EPT, esc);
-        __syncthreads();
-        float sax[K], say[K], saz[K], spp[K];  // scalar path (K = 1)
-        f2 pax[KP > 0 ? KP : 1], pay[KP > 0 ? KP : 1], paz[KP > 0 ? KP : 1], pp[KP > 0 ? KP : 1];
+    float sax[K], say[K], saz[K], spp[K];  // scalar path (K = 1)
+    f2 pax[KP > 0 ? KP : 1], pay[KP > 0 ? KP : 1], paz[KP > 0 ? KP : 1], pp[KP > 0 ? KP : 1];
+    auto clear = [&]() {
 #pragma unroll
         for (int q = 0; q < K; ++q) sax[q] = say[q] = saz[q] = spp[q] = 0.f;
 #pragma unroll
         for (int h = 0; h < KP; ++h) pax[h] = pay[h] = paz[h] = pp[h] = 0ull;
-        // ---- superparticles of this chunk
-#pragma unroll 2
+    };
+    // the FP32 sums of a chunk into the Kahan sums
+    auto fold = [&]() {
+        if (K & 1) {
+            kahan_smem_add<CB>(s_k, K - 1, 0, sax[K - 1]);
+            kahan_smem_add<CB>(s_k, K - 1, 1, say[K - 1]);
+            kahan_smem_add<CB>(s_k, K - 1, 2, saz[K - 1]);
+            kahan_smem_add<CB>(s_k, K - 1, 3, spp[K - 1]);
+        }
+#pragma unroll
+        for (int h = 0; h < KP; ++h) {
+            float lo, hi;
+            f2_up(pax[h], lo, hi);
+            kahan_smem_add<CB>(s_k, 2 * h, 0, lo);
+            kahan_smem_add<CB>(s_k, 2 * h + 1, 0, hi);
+            f2_up(pay[h], lo, hi);
+            kahan_smem_add<CB>(s_k, 2 * h, 1, lo);
+            kahan_smem_add<CB>(s_k, 2 * h + 1, 1, hi);
+            f2_up(paz[h], lo, hi);
+            kahan_smem_add<CB>(s_k, 2 * h, 2, lo);
+            kahan_smem_add<CB>(s_k, 2 * h + 1, 2, hi);
+            f2_up(pp[h], lo, hi);
+            kahan_smem_add<CB>(s_k, 2 * h, 3, lo);
+            kahan_smem_add<CB>(s_k, 2 * h + 1, 3, hi);
+        }
+    };
+    // ---- the list's superparticles, in chunks
+    for (uint32_t base = 0; base < nspj; base += SM::kCE) {
+        const uint32_t ns = nspj - base < (uint32_t)SM::kCE ? nspj - base : (uint32_t)SM::kCE;
+        uint32_t node[EPT];
+#pragma unroll
+        for (int r = 0; r < EPT; ++r) {
+            const uint32_t k = (uint32_t)(r * CB + t);
+            node[r] = k < ns ? A.pool[off + base + k] : 0u;
+        }
+#pragma unroll
+        for (int r = 0; r < EPT; ++r) {
+            const int k = r * CB + t;
+            if (k >= (int)ns) continue;
+            const float4 fh = A.nd_f[2 * node[r]], fl = A.nd_f[2 * node[r] + 1];
+            s_s0[k] = make_float4((fh.x - gch.x) + (fl.x - gcl.x), (fh.y - gch.y) + (fl.y - gcl.y),
+                                  (fh.z - gch.z) + (fl.z - gcl.z), -fh.w);
+            if (QUAD) {
+                s_s1[k] = A.nd_fq0[node[r]];
+                s_s2[k] = A.nd_fq1[node[r]];
+            }
+        }
+        __syncthreads();
+        clear();
+#pragma unroll kUnrollSpj
         for (int k = kbeg; k < (int)ns; k += nsl) {
-            const float4 a = sb.s0[k];
+            const float4 a = s_s0[k];
             float4 q0;
             float2 q1;
             if (QUAD) {
-                q0 = sb.s1[k];
-                q1 = sb.s2[k];
+                q0 = s_s1[k];
+                q1 = s_s2[k];
             }
             if (K & 1) {  // the odd i-particle (index K - 1) in scalar FP32
                 const float rx = xi[K - 1] - a.x, ry = yi[K - 1] - a.y, rz = zi[K - 1] - a.z;
@@ -410,20 +465,51 @@ __device__ __forceinline__ void force_round_f32(const ForceArgs& A, uint32_t gf,
                 }
             }
         }
-        // ---- particles of the opened leaves, in shared tiles of kCJ
+        fold();
+        __syncthreads();  // the chunk is rewritten next
+    }
+    // ---- the opened leaves: their particle ranges in batches, the
+    // particles in shared tiles
+    for (uint32_t base = nspj; base < len; base += SM::kCL) {
+        // this thread's EPT consecutive leaves
+        uint32_t lcnt[EPT], lfirst[EPT], esc[EPT], npart = 0;
+#pragma unroll
+        for (int r = 0; r < EPT; ++r) {
+            const uint32_t u = base + (uint32_t)(t * EPT + r);
+            lfirst[r] = u < len ? A.pool[off + u] & ~kLeafTag : 0xFFFFFFFFu;
+        }
+#pragma unroll
+        for (int r = 0; r < EPT; ++r) {
+            const bool leaf = lfirst[r] != 0xFFFFFFFFu;
+            lcnt[r] = leaf ? A.nd_count[lfirst[r]] : 0u;
+            lfirst[r] = leaf ? A.nd_first[lfirst[r]] : 0u;
+            npart += lcnt[r];
+        }
+        uint32_t total;
+        uint32_t es = block_scan1<CB>(npart, &total, sm.w);
+#pragma unroll
+        for (int r = 0; r < EPT; ++r) {
+            esc[r] = es;
+            es += lcnt[r];
+        }
+        // each thread's EPT consecutive slots in one vector store (no bank conflicts)
+        store_entries<EPT>(s_ef + t * EPT, lfirst);
+        store_entries<EPT>(s_es + t * EPT, esc);
+        __syncthreads();
         for (uint32_t c0 = 0; c0 < total; c0 += kCJ) {
             const uint32_t m = total - c0 < (uint32_t)kCJ ? total - c0 : (uint32_t)kCJ;
             if (c0 > 0) __syncthreads();  // previous tile fully consumed
             for (uint32_t k = t; k < m; k += CB) {
                 const uint32_t item = c0 + k;
-                const int src = owner_chunk<CE>(s_es, item);
+                const int src = owner_chunk<SM::kCL>(s_es, item);
                 const uint32_t p = s_ef[src] + (item - s_es[src]);
                 const float4 h = A.pf_hi[p], l = A.pf_lo[p];
                 s_j[k] = make_float4((h.x - gch.x) + (l.x - gcl.x), (h.y - gch.y) + (l.y - gcl.y),
                                      (h.z - gch.z) + (l.z - gcl.z), h.w);
             }
             __syncthreads();
-#pragma unroll 2
+            clear();
+#pragma unroll kUnrollEpj
             for (int k = kbeg; k < (int)m; k += nsl) {
                 const float4 j = s_j[k];
                 if (K & 1) {
@@ -453,28 +539,7 @@ __device__ __forceinline__ void force_round_f32(const ForceArgs& A, uint32_t gf,
                     }
                 }
             }
-        }
-        if (K & 1) {
-            kahan_smem_add<CB>(s_k, K - 1, 0, sax[K - 1]);
-            kahan_smem_add<CB>(s_k, K - 1, 1, say[K - 1]);
-            kahan_smem_add<CB>(s_k, K - 1, 2, saz[K - 1]);
-            kahan_smem_add<CB>(s_k, K - 1, 3, spp[K - 1]);
-        }
-#pragma unroll
-        for (int h = 0; h < KP; ++h) {
-            float lo, hi;
-            f2_up(pax[h], lo, hi);
-            kahan_smem_add<CB>(s_k, 2 * h, 0, lo);
-            kahan_smem_add<CB>(s_k, 2 * h + 1, 0, hi);
-            f2_up(pay[h], lo, hi);
-            kahan_smem_add<CB>(s_k, 2 * h, 1, lo);
-            kahan_smem_add<CB>(s_k, 2 * h + 1, 1, hi);
-            f2_up(paz[h], lo, hi);
-            kahan_smem_add<CB>(s_k, 2 * h, 2, lo);
-            kahan_smem_add<CB>(s_k, 2 * h + 1, 2, hi);
-            f2_up(pp[h], lo, hi);
-            kahan_smem_add<CB>(s_k, 2 * h, 3, lo);
-            kahan_smem_add<CB>(s_k, 2 * h + 1, 3, hi);
+            fold();
         }
         __syncthreads();  // chunk buffers are rewritten next
     }
@@ -510,55 +575,28 @@ __device__ __forceinline__ void force_round_f32(const ForceArgs& A, uint32_t gf,
     __syncthreads();
 }
 
-// Shared memory of the FP32 kernels (one CTA per group at a time).
-template <bool QUAD, int EPT, int CB, int KMAX>
-struct F32Shared {
-    static constexpr int kCE = CB * EPT;
-    static constexpr int kSpjBytes = kCE * (QUAD ? 40 : 16);
-    __align__(16) unsigned char u[kSpjBytes];  // superparticles of a chunk
-    __align__(16) float4 j[kCJ];
-    __align__(16) uint32_t ef[kCE];
-    __align__(16) uint32_t es[kCE];
-    uint32_t w[2 * (CB / 32)];
-    float k[KMAX * 8 * CB];  // Kahan sums and compensations
-};
-
 // Forces on the particles of group g, with the whole CTA.
 template <bool QUAD, int EPT, int CB, int KMAX>
 __device__ __forceinline__ void force_group(const ForceArgs& A, uint32_t g, F32Shared<QUAD, EPT, CB, KMAX>& sm) {
-    constexpr int kCE = F32Shared<QUAD, EPT, CB, KMAX>::kCE;
-    SpjBuf<QUAD> sb;
-    sb.s0 = reinterpret_cast<float4*>(sm.u);
-    sb.s1 = nullptr;  // a monopole chunk holds the first array only
-    sb.s2 = nullptr;
-    if constexpr (QUAD) {
-        sb.s1 = reinterpret_cast<float4*>(sm.u + kCE * 16);
-        sb.s2 = reinterpret_cast<float2*>(sm.u + kCE * 32);
-    }
     const uint32_t ni = A.g_count[g], gf = A.g_first[g];
     const unsigned long long off = A.g_off[g];
-    const uint32_t len = A.g_len[g];
+    const uint32_t len = A.g_len[g], nspj = A.g_nspj[g];
     const float4 gch = A.g_ch[g], gcl = A.g_cl[g];
     for (uint32_t ib = 0; ib < ni;) {
         const GroupPlan pl = plan_group<CB, KMAX>(ni - ib);
         if (pl.K == 1) {
-            force_round_f32<QUAD, 1, EPT, CB, KMAX>(A, gf, ni, off, len, gch, gcl, pl.P, pl.nsl, ib, sm.j, sb,
-                                                    sm.ef, sm.es, sm.w, sm.k);
+            force_round_f32<QUAD, 1, EPT, CB, KMAX>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
         } else if (KMAX >= 5 && pl.K == 5) {
             if constexpr (KMAX >= 5)
-                force_round_f32<QUAD, 5, EPT, CB, KMAX>(A, gf, ni, off, len, gch, gcl, pl.P, pl.nsl, ib, sm.j, sb,
-                                                        sm.ef, sm.es, sm.w, sm.k);
+                force_round_f32<QUAD, 5, EPT, CB, KMAX>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
         } else if (KMAX >= 4 && pl.K == 3) {
             if constexpr (KMAX >= 4)
-                force_round_f32<QUAD, 3, EPT, CB, KMAX>(A, gf, ni, off, len, gch, gcl, pl.P, pl.nsl, ib, sm.j, sb,
-                                                        sm.ef, sm.es, sm.w, sm.k);
+                force_round_f32<QUAD, 3, EPT, CB, KMAX>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
         } else if (KMAX == 2 || pl.K == 2) {
-            force_round_f32<QUAD, 2, EPT, CB, KMAX>(A, gf, ni, off, len, gch, gcl, pl.P, pl.nsl, ib, sm.j, sb,
-                                                    sm.ef, sm.es, sm.w, sm.k);
+            force_round_f32<QUAD, 2, EPT, CB, KMAX>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
         } else {
             if constexpr (KMAX >= 4)
-                force_round_f32<QUAD, 4, EPT, CB, KMAX>(A, gf, ni, off, len, gch, gcl, pl.P, pl.nsl, ib, sm.j,
-                                                        sb, sm.ef, sm.es, sm.w, sm.k);
+                force_round_f32<QUAD, 4, EPT, CB, KMAX>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
         }
         ib += (uint32_t)(pl.P * pl.K);
     }
@@ -578,7 +616,6 @@ __global__ void __launch_bounds__(CB, (QUAD ? 512 / CB : 1)) k_force_f32(ForceAr
         if (threadIdx.x == 0) s_g = atomicAdd(&st->force_counter, 1u);
         __syncthreads();
         const uint32_t g = s_g;
-        __syncthreads();
         if (g >= ngroups) break;
         force_group<QUAD, EPT, CB, KMAX>(A, g, sm);
     }
@@ -905,6 +942,7 @@ ForceArgs force_args(fdps_tree* t, fdps_psys* ps) {
     A.g_count = t->g_count;
     A.g_off = t->g_off;
     A.g_len = t->g_len;
+    A.g_nspj = t->g_nspj;
     A.g_ch = t->g_ch;
     A.g_cl = t->g_cl;
     A.pool = t->pool;

@@ -20,8 +20,11 @@
 // ids) to the next frontier, opened leaves append one EPJ entry (node id
 // with bit 31 set: all of the leaf's particles), unopened cells one SPJ
 // entry.  A group's list is contiguous in a pool handed out in chunks of at
-// least 2^16 entries; when a chunk fills, the group's partial list moves to
-// a fresh chunk twice its length.  Overflow of the pool or of the frontier sets a flag; the
+// least 2^16 entries, its SPJ entries first and its leaves after them (they
+// collect at the chunk's end and move down once the group is done), so that
+// the force kernel stages superparticles and leaf particles without sorting
+// them apart; when a chunk fills, the group's partial list moves to a fresh
+// chunk twice its length.  Overflow of the pool or of the frontier sets a flag; the
 // host then grows the buffer and repeats the walk.
 #include "fdps_internal.cuh"
 
@@ -81,22 +84,23 @@ __device__ __forceinline__ bool open_fp64(double L, int level, double theta2, co
 }
 
 // What a warp carries from one group's walk to the next: its pool chunk
-// and its totals for the device state word.  Every field is the same in
-// all lanes.
+// and its totals for the device state word.  Every field but the total is
+// the same in all lanes; lane k holds total k (list entries, EPJ, SPJ, EPJ and
+// SPJ interactions).
 struct WalkState {
-    unsigned long long cbase;  // start of the warp's pool chunk
+    uint32_t* cptr;            // start of the warp's pool chunk
     uint32_t coff, clen;       // cursor and length within it
     bool ovf;
-    unsigned long long acc_entries, acc_epj, acc_spj, acc_iepj, acc_ispj;
+    unsigned long long total;
     uint32_t max_front;
 };
 
 __device__ __forceinline__ WalkState walk_state_init() {
     WalkState S;
-    S.cbase = 0;
+    S.cptr = nullptr;
     S.coff = S.clen = 0;
     S.ovf = false;
-    S.acc_entries = S.acc_epj = S.acc_spj = S.acc_iepj = S.acc_ispj = 0;
+    S.total = 0;
     S.max_front = 0;
     return S;
 }
@@ -163,13 +167,9 @@ __device__ __forceinline__ void walk_group(const WalkArgs& A, uint32_t g, uint32
     }
     __syncwarp();
 
-    if (S.ovf) {  // counting only: keep the in-chunk cursor small
-        S.cbase += S.coff;
-        S.coff = 0;
-    }
-    unsigned long long gstart = S.cbase + S.coff;
-    uint32_t* cptr = A.pool + S.cbase;
-    uint32_t nspj = 0, nepj_lane = 0;
+    if (S.ovf) S.coff = 0;  // counting only
+    uint32_t goff = S.coff;  // where the list starts in the chunk
+    uint32_t nleaf = 0, nepj_lane = 0;
     uint32_t fsize = 1;
     if (lane == 0) fa[0] = sysid;
     __syncwarp();
@@ -241,17 +241,19 @@ __device__ __forceinline__ void walk_group(const WalkArgs& A, uint32_t g, uint32
                     nch = rec.x >> 27;
                 }
             }
-            // ---- append SPJ / EPJ entries
-            const bool emit = action == 1 || action == 2;
-            const uint32_t emask = __ballot_sync(0xFFFFFFFFu, emit);
-            const uint32_t k = __popc(emask);
-            if (k) {
-                if (S.coff + k > S.clen) {
+            // ---- append SPJ entries upwards, EPJ entries downwards from the
+            // chunk's end
+            const uint32_t smask = __ballot_sync(0xFFFFFFFFu, action == 1);
+            const uint32_t lmask = __ballot_sync(0xFFFFFFFFu, action == 2);
+            if (smask | lmask) {
+                const uint32_t ks = __popc(smask), kl = __popc(lmask);
+                if (S.coff + nleaf + ks + kl > S.clen) {
                     // new chunk: at least kChunk entries and twice the
                     // group's list so far, so long lists move O(log) times
-                    const unsigned long long sofar = S.cbase + S.coff - gstart;
+                    const uint32_t nsp = S.coff - goff;
+                    const unsigned long long sofar = (unsigned long long)nsp + nleaf;
                     const unsigned long long want =
-                        2 * (sofar + k) > kChunk ? 2 * (sofar + k) : kChunk;
+                        2 * (sofar + ks + kl) > kChunk ? 2 * (sofar + ks + kl) : kChunk;
                     unsigned long long nb = 0;
                     if (lane == 0) nb = atomicAdd(&st->pool_cursor, want);
                     nb = shfl_u64(nb, 0);
@@ -260,25 +262,30 @@ __device__ __forceinline__ void walk_group(const WalkArgs& A, uint32_t g, uint32
                         S.ovf = true;
                     }
                     if (!S.ovf) {
-                        for (unsigned long long j = lane; j < sofar; j += 32)
-                            A.pool[nb + j] = A.pool[gstart + j];
+                        uint32_t* np = A.pool + nb;
+#pragma unroll 1
+                        for (uint32_t j = lane; j < nsp; j += 32) np[j] = S.cptr[goff + j];
+                        const uint32_t* lsrc = S.cptr + (S.clen - nleaf);
+                        uint32_t* ldst = np + (want - nleaf);
+#pragma unroll 1
+                        for (uint32_t j = lane; j < nleaf; j += 32) ldst[j] = lsrc[j];
                         __syncwarp();
-                        gstart = nb;
-                        S.cbase = nb;
-                        S.coff = (uint32_t)sofar;
+                        S.cptr = np;
                         S.clen = (uint32_t)want;
-                        cptr = A.pool + nb;
                     } else {
-                        // count only from here on
-                        S.cbase = gstart;
-                        S.coff = (uint32_t)sofar;
-                        S.clen = 0xFFFFFFFFu;
+                        S.clen = 0xFFFFFFFFu;  // count only from here on
                     }
+                    goff = 0;
+                    S.coff = nsp;
                 }
-                if (emit && !S.ovf) cptr[S.coff + __popc(emask & lt)] = action == 2 ? (node | kLeafTag) : node;
-                S.coff += k;
+                if ((action == 1 || action == 2) && !S.ovf) {
+                    const bool spj = action == 1;
+                    const uint32_t r = __popc((spj ? smask : lmask) & lt);
+                    S.cptr[spj ? S.coff + r : S.clen - 1u - nleaf - r] = spj ? node : node | kLeafTag;
+                }
+                S.coff += ks;
+                nleaf += kl;
             }
-            nspj += __popc(__ballot_sync(0xFFFFFFFFu, action == 1));
             // ---- push children of opened internal cells (deep in the
             // tree most batches open none)
             if (__ballot_sync(0xFFFFFFFFu, nch > 0u)) {
@@ -305,34 +312,53 @@ __device__ __forceinline__ void walk_group(const WalkArgs& A, uint32_t g, uint32
         fb = tmp;
         fsize = nsize;
     }
+    // the leaves behind the superparticles (towards lower addresses, 128 at a
+    // time: a batch is read before it is written, so the ranges may overlap)
+    const uint32_t nspj = S.coff - goff;
+    if (!S.ovf && S.clen - nleaf > S.coff) {
+        const uint32_t* src = S.cptr + (S.clen - nleaf);
+        uint32_t* dst = S.cptr + S.coff;
+#pragma unroll 1
+        for (uint32_t j = lane; j < ((nleaf + 31u) & ~31u); j += 128) {
+            uint32_t e[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) e[r] = j + 32 * r < nleaf ? src[j + 32 * r] : 0u;
+            __syncwarp();
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (j + 32 * r < nleaf) dst[j + 32 * r] = e[r];
+            __syncwarp();
+        }
+    }
+    S.coff += nleaf;
     const uint32_t nepj = __reduce_add_sync(0xFFFFFFFFu, nepj_lane);
-    const unsigned long long len = S.cbase + S.coff - gstart;
+    const uint32_t len = nspj + nleaf;
     if (lane == 0) {
-        A.g_off[g] = gstart;
-        A.g_len[g] = (uint32_t)len;
+        A.g_off[g] = (unsigned long long)(S.cptr + goff - A.pool);
+        A.g_len[g] = len;
         A.g_nspj[g] = nspj;
         A.g_nepj[g] = nepj;
     }
     const unsigned long long ni = A.g_count[g];
-    S.acc_entries += len;
-    S.acc_epj += nepj;
-    S.acc_spj += nspj;
-    S.acc_iepj += ni * nepj;
-    S.acc_ispj += ni * nspj;
+    const unsigned long long mul = lane < 3 ? 1ull : ni;
+    S.total += mul * (lane == 0 ? len : (lane & 1) ? nepj : nspj);
 }
 
-// The warp's totals into the device state word (lane 0).
+// The warp's totals into the device state word.
 __device__ __forceinline__ void walk_flush(const WalkArgs& A, const WalkState& S) {
     DevState* st = A.st;
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&st->pool_needed, S.acc_entries);
-        atomicAdd(&st->list_entries, S.acc_entries);
-        atomicAdd(&st->n_epj, S.acc_epj);
-        atomicAdd(&st->n_spj, S.acc_spj);
-        atomicAdd(&st->int_epj, S.acc_iepj);
-        atomicAdd(&st->int_spj, S.acc_ispj);
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) {
+        atomicAdd(&st->pool_needed, S.total);
         atomicMax(&st->max_frontier, S.max_front);
     }
+    if (lane < 5)
+        atomicAdd(lane == 0   ? &st->list_entries
+                  : lane == 1 ? &st->n_epj
+                  : lane == 2 ? &st->n_spj
+                  : lane == 3 ? &st->int_epj
+                              : &st->int_spj,
+                  S.total);
 }
 
 constexpr int kWalkBlock = 128;
