@@ -8,12 +8,14 @@
 // bits; each pair in FP32 with MUFU rsqrt; per-tile FP32 sums added into
 // Kahan-compensated totals, finished in FP64.  Particle i's own term is
 // skipped.
+#include <algorithm>
+
 #include "fdps_internal.cuh"
 
 namespace fdps {
 namespace {
 
-constexpr int kDB = 128;  // sampled i-particles per block
+constexpr int kDB = 128;  // threads per block
 constexpr int kDT = 256;  // j-particles per shared tile
 
 __global__ void __launch_bounds__(256) k_direct_prep(int64_t n, const double* __restrict__ x,
@@ -26,10 +28,12 @@ __global__ void __launch_bounds__(256) k_direct_prep(int64_t n, const double* __
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const double rx = x[i] - ox, ry = y[i] - oy, rz = z[i] - oz;
-        const float hx = __double2float_rn(rx), hy = __double2float_rn(ry), hz = __double2float_rn(rz);
-        hi[i] = make_float4(hx, hy, hz, __double2float_rn(m[i]));
-        lo[i] = make_float4(__double2float_rn(rx - (double)hx), __double2float_rn(ry - (double)hy),
-                            __double2float_rn(rz - (double)hz), __double2float_rn(eps[i] * eps[i]));
+        float hx, hy, hz, lx, ly, lz;
+        split_f32(rx, hx, lx);
+        split_f32(ry, hy, ly);
+        split_f32(rz, hz, lz);
+        hi[i] = make_float4(hx, hy, hz, to_f32(m[i]));
+        lo[i] = make_float4(lx, ly, lz, to_f32(eps[i] * eps[i]));
     }
 }
 
@@ -65,25 +69,131 @@ __device__ __forceinline__ void pair(const float4 ih, const float4 il, const flo
     pp -= mri;
 }
 
-// One system: block (x: 128 sampled particles, y: one slice of the j range),
-// j-particles staged in shared tiles; partial sums per slice in FP64.
-__global__ void __launch_bounds__(kDB) k_direct_tiled(int64_t n, int64_t ns, const uint32_t* __restrict__ inv,
+// Two FP32 lanes in one 64-bit register: one packed instruction evaluates
+// an operation of the pair law for two i-particles, each lane rounded as the
+// scalar instruction.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_pk(float lo, float hi) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void f2_up(f2 v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
+    f2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+// rsqrtf for arguments that are no subnormals: the bare MUFU operation
+__device__ __forceinline__ float rsqrt_normal(float v) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+// One tile of m j-particles, entries kbeg, kbeg + kstep, ... of it, on the
+// 2 KP i-particles of a thread.  SELF: an i-particle of the warp is in the
+// tile (at rel), and its own term gets no mass.  NORMAL: every eps^2
+// of the warp is a normal FP32 number, so every r^2 is.
+template <int KP, bool SELF, bool NORMAL>
+__device__ __forceinline__ void direct_tile(const float4* s_h, const float4* s_l, int m, int kbeg, int kstep,
+                                            const uint32_t* rel, const f2* hx, const f2* hy, const f2* hz,
+                                            const f2* lx, const f2* ly, const f2* lz, const f2* e2, f2* ax, f2* ay,
+                                            f2* az, f2* pp) {
+#pragma unroll 2
+    for (int k = kbeg; k < m; k += kstep) {
+        const float4 jh = s_h[k], jl = s_l[k];
+        const f2 jx = f2_pk(jh.x, jh.x), jy = f2_pk(jh.y, jh.y), jz = f2_pk(jh.z, jh.z);
+        const f2 kx = f2_pk(jl.x, jl.x), ky = f2_pk(jl.y, jl.y), kz = f2_pk(jl.z, jl.z);
+        const f2 jm = f2_pk(jh.w, jh.w);
+#pragma unroll
+        for (int q = 0; q < KP; ++q) {
+            const f2 dx = f2_add(f2_sub(jx, hx[q]), f2_sub(kx, lx[q]));
+            const f2 dy = f2_add(f2_sub(jy, hy[q]), f2_sub(ky, ly[q]));
+            const f2 dz = f2_add(f2_sub(jz, hz[q]), f2_sub(kz, lz[q]));
+            const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, f2_fma(dz, dz, e2[q])));
+            float ra, rb;
+            f2_up(r2, ra, rb);
+            const f2 ri = NORMAL ? f2_pk(rsqrt_normal(ra), rsqrt_normal(rb)) : f2_pk(rsqrtf(ra), rsqrtf(rb));
+            const f2 mj = SELF ? f2_pk((uint32_t)k == rel[2 * q] ? 0.0f : jh.w, (uint32_t)k == rel[2 * q + 1] ? 0.0f : jh.w) : jm;
+            const f2 mri = f2_mul(mj, ri);
+            const f2 mri3 = f2_mul(mri, f2_mul(ri, ri));
+            ax[q] = f2_fma(mri3, dx, ax[q]);
+            ay[q] = f2_fma(mri3, dy, ay[q]);
+            az[q] = f2_fma(mri3, dz, az[q]);
+            pp[q] = f2_sub(pp[q], mri);
+        }
+    }
+}
+
+// One system: a block takes P sampled rows per i-slot of a thread (thread t
+// rows (blockIdx.x * 2 KP + q) P + t % P) and the j-slices of its threads t / P
+// within slice blockIdx.y of the j range; j-particles are staged in shared
+// tiles, FP32 sums of a tile go into Kahan sums, partial sums of a slice into
+// part[slice].  Bound by the FP32 pipe: 19 operations a pair term, in packed
+// instructions for two i-particles, with each staged j-particle read once
+// for the thread's 2 KP; the own-term check runs only on the tiles that hold
+// one of the warp's i-particles.  4096 rows of 2^20 particles: 5.76 ms of
+// kernel time with one i-particle a thread and scalar instructions; the whole
+// call 6.34 -> 3.47 ms.
+template <int KP>
+__global__ void __launch_bounds__(kDB, KP == 2 ? 4 : 5) k_direct_tiled(int64_t n, int64_t ns, int P,
+                                                      const uint32_t* __restrict__ inv,
                                                       const int64_t* __restrict__ rows,
                                                       const float4* __restrict__ hi,
                                                       const float4* __restrict__ lo, int64_t jper,
                                                       double* __restrict__ part) {
     __shared__ float4 s_h[kDT], s_l[kDT];
+    constexpr int K = 2 * KP;
     const int t = threadIdx.x;
-    const int64_t s = blockIdx.x * (int64_t)kDB + t;
-    const bool valid = s < ns;
-    const int64_t p = valid ? (int64_t)inv[rows[s]] : -1;
-    const float4 ih = valid ? hi[p] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4 il = valid ? lo[p] : make_float4(0.f, 0.f, 0.f, 1.f);
+    const int ip = t % P, sl = t / P, nsl = kDB / P;
+    uint32_t p[K];  // positions of the i-particles (n < 2^31), all ones for none
+    f2 hx[KP], hy[KP], hz[KP], lx[KP], ly[KP], lz[KP], e2[KP];
+    bool normal = true;
+#pragma unroll
+    for (int q = 0; q < KP; ++q) {
+        float4 h[2], l[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int64_t s = ((int64_t)blockIdx.x * K + 2 * q + c) * P + ip;
+            p[2 * q + c] = s < ns ? inv[rows[s]] : 0xFFFFFFFFu;
+            h[c] = s < ns ? hi[p[2 * q + c]] : make_float4(0.f, 0.f, 0.f, 0.f);
+            l[c] = s < ns ? lo[p[2 * q + c]] : make_float4(0.f, 0.f, 0.f, 1.f);
+            normal = normal && l[c].w >= 1.1754944e-38f;
+        }
+        hx[q] = f2_pk(h[0].x, h[1].x);
+        hy[q] = f2_pk(h[0].y, h[1].y);
+        hz[q] = f2_pk(h[0].z, h[1].z);
+        lx[q] = f2_pk(l[0].x, l[1].x);
+        ly[q] = f2_pk(l[0].y, l[1].y);
+        lz[q] = f2_pk(l[0].z, l[1].z);
+        e2[q] = f2_pk(l[0].w, l[1].w);
+    }
+    normal = __all_sync(0xFFFFFFFFu, normal);
     const int64_t j0 = blockIdx.y * jper;
     const int64_t j1 = j0 + jper < n ? j0 + jper : n;
-    Comp4 acc;
+    Comp4 acc[K];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc.s[k] = acc.c[k] = 0.f;
+    for (int i = 0; i < K; ++i)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[i].s[k] = acc[i].c[k] = 0.f;
     for (int64_t jt = j0; jt < j1; jt += kDT) {
         const int m = j1 - jt < kDT ? (int)(j1 - jt) : kDT;
         __syncthreads();
@@ -92,20 +202,44 @@ __global__ void __launch_bounds__(kDB) k_direct_tiled(int64_t n, int64_t ns, con
             s_l[k] = lo[jt + k];
         }
         __syncthreads();
-        float ax = 0.f, ay = 0.f, az = 0.f, pp = 0.f;
-        for (int k = 0; k < m; ++k) {
-            if (jt + k == p) continue;  // no self term
-            pair(ih, il, s_h[k], s_l[k], il.w, ax, ay, az, pp);
-        }
-        acc.add(0, ax);
-        acc.add(1, ay);
-        acc.add(2, az);
-        acc.add(3, pp);
-    }
-    if (valid)
+        bool self = false;
+        uint32_t rel[K];
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            part[((int64_t)blockIdx.y * ns + s) * 4 + k] = (double)acc.s[k] - (double)acc.c[k];
+        for (int i = 0; i < K; ++i) {
+            rel[i] = p[i] - (uint32_t)jt;
+            self = self || rel[i] < (uint32_t)m;
+        }
+        self = __any_sync(0xFFFFFFFFu, self);
+        f2 ax[KP], ay[KP], az[KP], pp[KP];
+#pragma unroll
+        for (int q = 0; q < KP; ++q) ax[q] = ay[q] = az[q] = pp[q] = 0ull;
+        if (!normal)
+            direct_tile<KP, true, false>(s_h, s_l, m, sl, nsl, rel, hx, hy, hz, lx, ly, lz, e2, ax, ay, az, pp);
+        else if (self)
+            direct_tile<KP, true, true>(s_h, s_l, m, sl, nsl, rel, hx, hy, hz, lx, ly, lz, e2, ax, ay, az, pp);
+        else
+            direct_tile<KP, false, true>(s_h, s_l, m, sl, nsl, rel, hx, hy, hz, lx, ly, lz, e2, ax, ay, az, pp);
+#pragma unroll
+        for (int q = 0; q < KP; ++q) {
+            const f2 v[4] = {ax[q], ay[q], az[q], pp[q]};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float a, b;
+                f2_up(v[k], a, b);
+                acc[2 * q].add(k, a);
+                acc[2 * q + 1].add(k, b);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        const int64_t s = ((int64_t)blockIdx.x * K + i) * P + ip;
+        if (s < ns)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                part[(((int64_t)blockIdx.y * nsl + sl) * ns + s) * 4 + k] =
+                    (double)acc[i].s[k] - (double)acc[i].c[k];
+    }
 }
 
 // Several systems: each sampled particle sums over its own system's range.
@@ -140,15 +274,25 @@ __global__ void __launch_bounds__(kDB) k_direct_systems(int64_t ns, const uint32
     for (int c = 0; c < 4; ++c) part[s * 4 + c] = (double)acc.s[c] - (double)acc.c[c];
 }
 
-__global__ void k_direct_final(int64_t ns, int js, const double* __restrict__ part, double* __restrict__ out) {
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < ns;
-         s += (int64_t)gridDim.x * blockDim.x)
+// The slices' partial sums of each row: a warp per row, lanes over the
+// slices, in a fixed order.
+__global__ void __launch_bounds__(256) k_direct_final(int64_t ns, int js, const double* __restrict__ part,
+                                                      double* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; s < ns;
+         s += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int y = lane; y < js; y += 32)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            double v = 0.0;
-            for (int y = 0; y < js; ++y) v += part[((int64_t)y * ns + s) * 4 + k];
-            out[s * 4 + k] = v;
-        }
+            for (int k = 0; k < 4; ++k) v[k] += part[((int64_t)y * ns + s) * 4 + k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] += __shfl_down_sync(0xFFFFFFFFu, v[k], o);
+        if (lane == 0)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) out[s * 4 + k] = v[k];
+    }
 }
 
 // Tree results (acceleration, potential) at the sampled rows.
@@ -205,11 +349,16 @@ int direct_sample_device(fdps_psys* ps, int64_t ns, const int64_t* d_rows, doubl
     SampleScratch sc;
     int rc = invert_ids(ps, sc);
     const bool one = ps->n_sys == 1;
-    // slices of the j range: enough blocks to fill the GPU
-    const int64_t bx = (ns + kDB - 1) / kDB;
-    int js = one ? (int)((4 * ctx->sm_count + bx - 1) / bx) : 1;
-    if (js < 1) js = 1;
-    if (js > 1024) js = 1024;
+    // i-particles: 4 per thread where the rows fill a block of 128 threads
+    // with them, else 2; fewer rows than threads leave the other threads to
+    // slices of the j range.  j-slices (blocks): one resident wave.
+    const int K = ns > 2 * kDB ? 4 : 2;
+    const int P = ns > kDB || K == 4 ? kDB : ns > 64 ? 64 : ns > 32 ? 32 : 16;
+    const int per_sm = K == 4 ? 4 : 5;
+    const int64_t bx = one ? (ns + (int64_t)K * P - 1) / ((int64_t)K * P) : (ns + kDB - 1) / kDB;
+    int64_t by = one ? (int64_t)per_sm * ctx->sm_count / bx : 1;
+    by = std::max<int64_t>(1, std::min<int64_t>({by, 1024, (n + 63) / 64}));
+    const int js = one ? (int)by * (kDB / P) : 1;
     if (!rc && (cudaMalloc(&sc.hi, sizeof(float4) * (size_t)n) != cudaSuccess ||
                 cudaMalloc(&sc.lo, sizeof(float4) * (size_t)n) != cudaSuccess ||
                 cudaMalloc(&sc.part, sizeof(double) * 4 * (size_t)ns * js) != cudaSuccess)) {
@@ -229,15 +378,18 @@ int direct_sample_device(fdps_psys* ps, int64_t ns, const int64_t* d_rows, doubl
                 n, ps->x[c], ps->y[c], ps->z[c], ps->m[c], ps->eps[c], o[0], o[1], o[2], sc.hi, sc.lo);
             FDPS_LAUNCH_CHECK(ctx);
             if (one) {
-                const int64_t jper = (n + js - 1) / js;
-                k_direct_tiled<<<dim3((unsigned)bx, (unsigned)js), kDB, 0, s>>>(n, ns, sc.inv, d_rows, sc.hi,
-                                                                              sc.lo, jper, sc.part);
+                const int64_t jper = (n + by - 1) / by;
+                const dim3 grid((unsigned)bx, (unsigned)by);
+                if (K == 4)
+                    k_direct_tiled<2><<<grid, kDB, 0, s>>>(n, ns, P, sc.inv, d_rows, sc.hi, sc.lo, jper, sc.part);
+                else
+                    k_direct_tiled<1><<<grid, kDB, 0, s>>>(n, ns, P, sc.inv, d_rows, sc.hi, sc.lo, jper, sc.part);
             } else {
                 k_direct_systems<<<(unsigned)bx, kDB, 0, s>>>(ns, sc.inv, d_rows, ps->d_sys, ps->d_off, sc.hi,
                                                               sc.lo, sc.part);
             }
             FDPS_LAUNCH_CHECK(ctx);
-            k_direct_final<<<grid_for(ns, 256, 1024), 256, 0, s>>>(ns, js, sc.part, d_out4);
+            k_direct_final<<<grid_for(32 * ns, 256, 4 * ctx->sm_count), 256, 0, s>>>(ns, js, sc.part, d_out4);
             FDPS_LAUNCH_CHECK(ctx);
             if (cudaStreamSynchronize(s) != cudaSuccess) rc = set_error(ctx, FDPS_ECUDA, "direct sum failed");
         }
