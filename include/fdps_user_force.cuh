@@ -52,45 +52,58 @@ struct Epi {
     uint32_t row;
 };
 // particle of an opened leaf, relative to the group centre
-struct Epj {
+struct __align__(16) Epj {
     float x, y, z, m;
 };
 // superparticle: a cell's centre of mass relative to the group centre, its
 // mass and traceless quadrupole about the centre of mass (zero for a
-// monopole tree)
-struct Spj {
+// monopole tree).  Both list types are aligned for 16-byte loads.
+struct __align__(16) Spj {
     float x, y, z, m;
     float qxx, qyy, qzz, qxy, qxz, qyz;
 };
 
 namespace detail {
 
-constexpr int kWarps = 4;     // warps per block; a warp works on one group at a time
-constexpr int kTile = 32;     // list entries per step, one per lane
-constexpr int kEpjTile = 64;  // leaf particles per shared tile
+constexpr int kThreads = 64;  // threads of a block, and list entries per step
+constexpr int kSlots = 4;     // blocks sharing a group's i-particles (grid y)
+constexpr int kSpjCall = 32;  // most superparticles per functor call
+constexpr int kEpjCall = 64;  // most leaf particles per functor call
 
 __device__ __forceinline__ float4 ld4(const float* p, uint64_t i) {
     return reinterpret_cast<const float4*>(p)[i];
 }
 
-// The whole walk over the view's groups, for a block of kWarps warps.
+// The walk of the view's groups by a grid (any x, any y) of blocks of
+// kThreads: block (x, y) takes groups x, x + gridDim.x, ... and of each the
+// i-particles kThreads y .. + kThreads - 1 (and on by kThreads gridDim.y),
+// one per thread.  The block stages kThreads list entries at a time for all
+// its warps.  The law's own instructions bound it, so what counts is that
+// every SM has warps with i-particles until the end: one block per group and
+// 64 i-particles, started by the hardware as others finish, where a fixed
+// share of the groups for each warp of one resident wave, eight passes over
+// the list for a group of 256, left most of the SMs idle behind the warps
+// with the large groups (2^20 Hernquist particles, n_grp 256, gravity with
+// quadrupoles: 13.6 -> 10.1 ms for lists and law, 8.4 -> 8.1 ms a
+// call where the next call's lists overlap the law).
 template <class Force, class FEpj, class FSpj>
 __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const FEpj& f_epj,
                                                 const FSpj& f_spj, Force* out) {
-    __shared__ Spj s_spj[kWarps][kTile];
-    __shared__ Epj s_epj[kWarps][kEpjTile];
-    __shared__ uint32_t s_first[kWarps][kTile];
-    __shared__ uint32_t s_start[kWarps][kTile];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int kW = kThreads / 32;
+    __shared__ Spj s_spj[kThreads];
+    __shared__ Epj s_epj[kEpjCall];
+    __shared__ uint32_t s_first[kThreads];
+    __shared__ uint32_t s_start[kThreads];
+    __shared__ uint32_t s_sum[2 * kW];
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const uint32_t lt = (1u << lane) - 1u;
-    const int64_t nwarps = (int64_t)gridDim.x * kWarps;
-    for (int64_t g = (int64_t)blockIdx.x * kWarps + w; g < v.n_groups; g += nwarps) {
+    for (int64_t g = blockIdx.x; g < v.n_groups; g += gridDim.x) {
         const uint32_t gf = v.g_first[g], ni = v.g_count[g];
         const unsigned long long off = v.g_off[g];
         const uint32_t len = v.g_len[g];
         const float4 ch = ld4(v.g_ch, (uint64_t)g), cl = ld4(v.g_cl, (uint64_t)g);
-        for (uint32_t ib = 0; ib < ni; ib += 32) {
-            const uint32_t i = ib + lane;
+        for (uint32_t ib = blockIdx.y * kThreads; ib < ni; ib += kThreads * gridDim.y) {
+            const uint32_t i = ib + t;
             const bool act = i < ni;
             Epi epi{0.f, 0.f, 0.f, 1.f, 0u};
             if (act) {
@@ -103,15 +116,38 @@ __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const F
             }
             Force f;
             f.clear();
-            for (uint32_t base = 0; base < len; base += kTile) {
-                const uint32_t u = base + lane;
+            for (uint32_t base = 0; base < len; base += kThreads) {
+                const uint32_t u = base + t;
                 const bool valid = u < len;
                 const uint32_t e = valid ? v.pool[off + u] : 0u;
                 const bool leaf = valid && (e & v.leaf_tag);
                 const bool spj = valid && !leaf;
                 const uint32_t node = e & ~v.leaf_tag;
-                // superparticles of this step, compacted into the warp's tile
+                // ranks of the superparticles and of the leaves' particles
+                // in this step
                 const uint32_t smask = __ballot_sync(0xFFFFFFFFu, spj);
+                const uint32_t cnt = leaf ? v.nd_count[node] : 0u;
+                uint32_t inc = cnt;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+                    if (lane >= o) inc += x;
+                }
+                if (lane == 31) {
+                    s_sum[w] = __popc(smask);
+                    s_sum[kW + w] = inc;
+                }
+                __syncthreads();  // also: the previous step's tiles are consumed
+                uint32_t rank = __popc(smask & lt), start = inc - cnt, nspj = 0, total = 0;
+#pragma unroll
+                for (int k = 0; k < kW; ++k) {
+                    if (k < w) {
+                        rank += s_sum[k];
+                        start += s_sum[kW + k];
+                    }
+                    nspj += s_sum[k];
+                    total += s_sum[kW + k];
+                }
                 if (spj) {
                     const float4 fh = ld4(v.nd_f, 2ull * node), fl = ld4(v.nd_f, 2ull * node + 1);
                     Spj s;
@@ -130,50 +166,42 @@ __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const F
                         s.qxz = q1.x;
                         s.qyz = q1.y;
                     }
-                    s_spj[w][__popc(smask & lt)] = s;
+                    s_spj[rank] = s;
                 }
-                // opened leaves: particle counts and their offsets in this step
-                const uint32_t cnt = leaf ? v.nd_count[node] : 0u;
-                uint32_t inc = cnt;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-                    if (lane >= o) inc += t;
-                }
-                const uint32_t total = __shfl_sync(0xFFFFFFFFu, inc, 31);
-                s_first[w][lane] = leaf ? v.nd_first[node] : 0u;
-                s_start[w][lane] = inc - cnt;
-                __syncwarp();
-                const int nspj = __popc(smask);
-                if (act && nspj > 0) f_spj(epi, &s_spj[w][0], nspj, f);
-                for (uint32_t c0 = 0; c0 < total; c0 += kEpjTile) {
-                    const uint32_t m = total - c0 < (uint32_t)kEpjTile ? total - c0 : (uint32_t)kEpjTile;
-                    __syncwarp();
-                    for (uint32_t k = lane; k < m; k += 32) {
-                        // the owning lane: last lane whose start <= item (lanes
-                        // with no particles share the next lane's start)
+                s_first[t] = leaf ? v.nd_first[node] : 0u;
+                s_start[t] = start;
+                __syncthreads();
+                if (act)
+                    for (uint32_t k = 0; k < nspj; k += kSpjCall)
+                        f_spj(epi, &s_spj[k], (int)(nspj - k < (uint32_t)kSpjCall ? nspj - k : (uint32_t)kSpjCall), f);
+                for (uint32_t c0 = 0; c0 < total; c0 += kEpjCall) {
+                    const uint32_t m = total - c0 < (uint32_t)kEpjCall ? total - c0 : (uint32_t)kEpjCall;
+                    if (c0 > 0) __syncthreads();
+                    for (uint32_t k = t; k < m; k += kThreads) {
+                        // the owning entry: the last one whose start <= item
+                        // (entries with no particles share the next one's start)
                         const uint32_t item = c0 + k;
                         int src = 0;
 #pragma unroll
-                        for (int step = 16; step > 0; step >>= 1)
-                            if (s_start[w][src + step] <= item) src += step;
-                        const uint32_t p = s_first[w][src] + (item - s_start[w][src]);
+                        for (int step = kThreads / 2; step > 0; step >>= 1)
+                            if (s_start[src + step] <= item) src += step;
+                        const uint32_t p = s_first[src] + (item - s_start[src]);
                         const float4 h = ld4(v.pf_hi, p), l = ld4(v.pf_lo, p);
-                        s_epj[w][k] = Epj{(h.x - ch.x) + (l.x - cl.x), (h.y - ch.y) + (l.y - cl.y),
-                                          (h.z - ch.z) + (l.z - cl.z), h.w};
+                        s_epj[k] = Epj{(h.x - ch.x) + (l.x - cl.x), (h.y - ch.y) + (l.y - cl.y),
+                                       (h.z - ch.z) + (l.z - cl.z), h.w};
                     }
-                    __syncwarp();
-                    if (act) f_epj(epi, &s_epj[w][0], (int)m, f);
+                    __syncthreads();
+                    if (act) f_epj(epi, &s_epj[0], (int)m, f);
                 }
-                __syncwarp();  // the tiles are rewritten in the next step
             }
             if (act) out[epi.row] = f;
+            __syncthreads();  // the tiles are rewritten for the next i-particles
         }
     }
 }
 
 template <class Force, class FEpj, class FSpj>
-__global__ void __launch_bounds__(kWarps * 32)
+__global__ void __launch_bounds__(kThreads)
     calc_force_kernel(fdps_tree_view v, FEpj f_epj, FSpj f_spj, Force* out) {
     calc_force_body<Force>(v, f_epj, f_spj, out);
 }
@@ -188,18 +216,9 @@ template <class Force, class FEpj, class FSpj>
 cudaError_t calc_force(const fdps_tree_view& v, const FEpj& f_epj, const FSpj& f_spj, Force* out,
                        cudaStream_t stream) {
     if (v.n_groups <= 0) return cudaSuccess;
-    int dev = 0, sms = 1, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-             &per_sm, detail::calc_force_kernel<Force, FEpj, FSpj>, detail::kWarps * 32, 0)) != cudaSuccess)
-        return e;
-    const int64_t need = (v.n_groups + detail::kWarps - 1) / detail::kWarps;
-    const int64_t cap = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
-    const int blocks = (int)(need < cap ? need : cap);
-    detail::calc_force_kernel<Force, FEpj, FSpj>
-        <<<blocks, detail::kWarps * 32, 0, stream>>>(v, f_epj, f_spj, out);
+    const int64_t most = 0x7FFFFFFF;
+    const dim3 grid((unsigned)(v.n_groups < most ? v.n_groups : most), detail::kSlots);
+    detail::calc_force_kernel<Force, FEpj, FSpj><<<grid, detail::kThreads, 0, stream>>>(v, f_epj, f_spj, out);
     return cudaGetLastError();
 }
 #endif  // __CUDACC_RTC__

@@ -15,6 +15,7 @@
 #include <string>
 #include <vector>
 
+#include "../../include/fdps_user_force.cuh"
 #include "fdps_internal.cuh"
 #include "fdps_embedded_headers.inc"  // kHeaderGpu, kHeaderUserForce (generated)
 
@@ -23,7 +24,6 @@ struct fdps_user_law {
     cudaLibrary_t lib = nullptr;
     cudaKernel_t kern = nullptr;
     int64_t force_size = 0;
-    int per_sm = 0;
 };
 
 namespace fdps {
@@ -44,7 +44,7 @@ std::string program_text(const char* user) {
     s += "#line 1 \"user_law\"\n";
     s += user;
     s += "\n#line 1 \"fdps_user_entry\"\n";
-    s += "extern \"C\" __global__ void __launch_bounds__(fdps_user::detail::kWarps * 32)\n"
+    s += "extern \"C\" __global__ void __launch_bounds__(fdps_user::detail::kThreads)\n"
          "fdps_user_entry(fdps_tree_view v, Force* out) {\n"
          "    fdps_user::detail::calc_force_body<Force>(v, Law{}, Law{}, out);\n}\n";
     s += "extern \"C\" __device__ const long long fdps_user_force_size = (long long)sizeof(Force);\n";
@@ -112,16 +112,13 @@ int fdps_user_law_compile(fdps_ctx* ctx, const char* source, fdps_user_law** out
     size_t bytes = 0;
     long long fs = 0;
     if (cudaLibraryGetGlobal(&dsize, &bytes, law->lib, "fdps_user_force_size") != cudaSuccess ||
-        bytes != sizeof(fs) || cudaMemcpy(&fs, dsize, sizeof(fs), cudaMemcpyDeviceToHost) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&law->per_sm, (const void*)law->kern, 128, 0) !=
-            cudaSuccess) {
+        bytes != sizeof(fs) || cudaMemcpy(&fs, dsize, sizeof(fs), cudaMemcpyDeviceToHost) != cudaSuccess) {
         cudaGetLastError();
         cudaLibraryUnload(law->lib);
         delete law;
         return set_error(ctx, FDPS_ECUDA, "querying the compiled user law failed");
     }
     law->force_size = fs;
-    if (law->per_sm < 1) law->per_sm = 1;
     *out = law;
     return FDPS_OK;
 }
@@ -136,11 +133,10 @@ int fdps_user_law_run(fdps_user_law* law, const fdps_tree* tree, const fdps_psys
     const int rc = fdps_tree_get_view(tree, ps, &v);
     if (rc) return rc;
     if (v.n_groups <= 0) return FDPS_OK;
-    const int64_t need = (v.n_groups + 3) / 4;
-    const int64_t cap = (int64_t)ctx->sm_count * law->per_sm;
-    const unsigned int blocks = (unsigned int)(need < cap ? need : cap);
+    // the launch shape of the header's calc_force
+    const dim3 grid((unsigned int)v.n_groups, fdps_user::detail::kSlots);
     void* args[2] = {&v, &out};
-    if (cudaLaunchKernel((const void*)law->kern, dim3(blocks), dim3(128), args, 0, ctx->stream) != cudaSuccess) {
+    if (cudaLaunchKernel((const void*)law->kern, grid, dim3(fdps_user::detail::kThreads), args, 0, ctx->stream) != cudaSuccess) {
         cudaGetLastError();
         return set_error(ctx, FDPS_ECUDA, "user law launch failed");
     }
