@@ -454,7 +454,7 @@ int fdps_user_law_destroy(fdps_user_law* law);
    unbounded latency of a cudaMalloc / cudaFree.  It computes what
    fdps_tree_calc_force_all_and_write_back
    computes first (root box, 63-bit Morton keys, stable radix sort) for one
-   particle set and allocates nothing: its scratch (about 5.3 MB) is a
+   particle set and allocates nothing: its scratch (about 3.2 MB) is a
    file-scope device array that every GPU which loads the library holds
    until the process exits.
      x, y, z      device arrays of n FP64 positions (SoA), borrowed
