@@ -52,6 +52,8 @@ int ensure_particles(fdps_tree* t, int64_t n) {
     if (n <= t->cap_n) return FDPS_OK;
     free_particles(t);
     const int64_t tiles = (n + kSortTile - 1) / kSortTile;
+    // a smaller set on this tree has its build tiles of kBuildTileSmall
+    const int64_t small_tiles = (std::min<int64_t>(n, kBuildSmall) + kBuildTileSmall - 1) / kBuildTileSmall;
     bool ok = dev_alloc(&t->keys_in, n) == cudaSuccess && dev_alloc(&t->keys_a, n) == cudaSuccess &&
               dev_alloc(&t->keys_b, n) == cudaSuccess && dev_alloc(&t->vals_a, n) == cudaSuccess &&
               dev_alloc(&t->vals_b, n) == cudaSuccess && dev_alloc(&t->pf_hi, n) == cudaSuccess &&
@@ -59,7 +61,7 @@ int ensure_particles(fdps_tree* t, int64_t n) {
               dev_alloc(&t->pmx, n) == cudaSuccess && dev_alloc(&t->pmy, n) == cudaSuccess &&
               dev_alloc(&t->pmz, n) == cudaSuccess &&
               dev_alloc(&t->sort_hist, 2 * 256 * tiles) == cudaSuccess &&
-              dev_alloc(&t->bt_count, kMaxLevel * (kBuildWarps + 1) * (tiles + 1) + 32) == cudaSuccess &&
+              dev_alloc(&t->bt_count, kMaxLevel * (kBuildWarps + 1) * (std::max(tiles, small_tiles) + 1) + 32) == cudaSuccess &&
               dev_alloc(&t->coh_bkt, n) == cudaSuccess && dev_alloc(&t->coh_cnt, 3 * ((n + kCohT - 1) / kCohT + 1) + 8) == cudaSuccess;
     t->cap_coh = ok ? 3 * ((n + kCohT - 1) / kCohT + 1) + 8 : 0;
     if (!ok) {
@@ -279,7 +281,7 @@ int run_tree_stages(fdps_tree* t, fdps_psys* ps) {
         const uint32_t ov = t->h_st.overflow;
         if (ov & kSortStall) {
             t->coh_ok = false;
-            return set_error(ctx, FDPS_ETIMEOUT, "a radix-sort look-back wait exceeded its bound");
+            return set_error(ctx, FDPS_ETIMEOUT, "a device-side wait (sort look-back or grid barrier) exceeded its bound");
         }
         if (ov & kSortRedo) {
             if (sort_try > 0) return set_error(ctx, FDPS_ECUDA, "coherent sort asked for a second redo");
@@ -442,7 +444,6 @@ int fdps_psys_create(fdps_ctx* ctx, int64_t n, fdps_psys** out) {
     if (!ps) return FDPS_ENOMEM;
     ps->ctx = ctx;
     ps->n = n;
-    ps->max_sys_n = n;
     bool ok = true;
     for (int b = 0; b < 2; ++b)
         ok = ok && dev_alloc(&ps->x[b], n) == cudaSuccess && dev_alloc(&ps->y[b], n) == cudaSuccess &&
@@ -487,7 +488,6 @@ int fdps_psys_destroy(fdps_psys* ps) {
     dev_free(ps->inv);
     dev_free(ps->rec);
     dev_free(ps->d_off);
-    dev_free(ps->d_order);
     dev_free(ps->d_sys);
     dev_free(ps->d_sys_red);
     dev_free(ps->d_cbs);
@@ -1295,7 +1295,6 @@ int fdps_psys_set_systems(fdps_psys* ps, int32_t n_sys, const int64_t* offsets) 
             return set_error(ctx, FDPS_EINVAL, "system %d is empty or offsets decrease", (int)k);
     cudaSetDevice(ctx->device);
     dev_free(ps->d_off);
-    dev_free(ps->d_order);
     dev_free(ps->d_sys);
     dev_free(ps->d_sys_red);
     dev_free(ps->d_cbs);
@@ -1303,33 +1302,20 @@ int fdps_psys_set_systems(fdps_psys* ps, int32_t n_sys, const int64_t* offsets) 
     dev_free(ps->d_csfb);
     ps->coh_nb = 0;
     ps->n_sys = 1;
-    ps->max_sys_n = ps->n;
     ps->gen++;
     ps->has_data = false;
     ps->has_forces = false;
     if (n_sys == 1) return FDPS_OK;
     if (dev_alloc(&ps->d_off, n_sys + 1) != cudaSuccess || dev_alloc(&ps->d_sys, ps->n) != cudaSuccess ||
-        dev_alloc(&ps->d_sys_red, 2 * (int64_t)n_sys) != cudaSuccess ||
-        dev_alloc(&ps->d_order, n_sys) != cudaSuccess) {
+        dev_alloc(&ps->d_sys_red, 2 * (int64_t)n_sys) != cudaSuccess) {
         cudaGetLastError();
         dev_free(ps->d_off);
-        dev_free(ps->d_order);
         dev_free(ps->d_sys);
         dev_free(ps->d_sys_red);
         return set_error(ctx, FDPS_ENOMEM, "device allocation for %d systems failed", (int)n_sys);
     }
     ps->n_sys = n_sys;
-    ps->max_sys_n = 0;
-    for (int32_t k = 0; k < n_sys; ++k) ps->max_sys_n = std::max<int64_t>(ps->max_sys_n, offsets[k + 1] - offsets[k]);
-    // per-system work (the moments) is handed out largest system first
-    std::vector<int32_t> order(n_sys);
-    for (int32_t k = 0; k < n_sys; ++k) order[k] = k;
-    std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
-        return offsets[a + 1] - offsets[a] > offsets[b + 1] - offsets[b];
-    });
     FDPS_CUDA_TRY(ctx, cudaMemcpyAsync(ps->d_off, offsets, sizeof(int64_t) * (n_sys + 1),
-                                       cudaMemcpyHostToDevice, ctx->stream));
-    FDPS_CUDA_TRY(ctx, cudaMemcpyAsync(ps->d_order, order.data(), sizeof(int32_t) * n_sys,
                                        cudaMemcpyHostToDevice, ctx->stream));
     int rc = launch_sys_index(ps);
     if (rc) return rc;

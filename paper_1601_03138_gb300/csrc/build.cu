@@ -156,8 +156,13 @@ __device__ __forceinline__ void write_roots(const RootArgs& R) {
 constexpr int kBT = 256;                    // threads per tile
 constexpr int kBWarps = kBT / 32;
 constexpr int kBRows = 8;                   // rows of 32 positions per warp
-constexpr int kBSpan = 32 * kBRows;         // positions per warp
 constexpr int kBTile = kBT * kBRows;        // positions per tile
+// Sets of at most kBuildSmall positions take one row per warp and tiles of
+// kBT: the rows of a warp follow one another (about 3 us each in the node
+// pass), and a tile of 2048 leaves all but a few SMs idle.  Plummer 2001
+// particles: count and node pass 14 + 25 us with 8 rows; the whole build
+// of 2^14 particles 46 us with 8 rows and 23 with one.
+static_assert(kBuildTileSmall == kBT && kBuildSmall % kBT == 0, "tile shape shared with the allocation");
 constexpr int kHalo = kMaxLeaf;             // window either side of a row
 static_assert(kBTile == kBuildTile && kBWarps == kBuildWarps, "tile shape shared with the allocation");
 static_assert(kHalo == 16, "a row's window is 64 positions: 16 before, 32 own, 16 after");
@@ -189,16 +194,18 @@ __device__ __forceinline__ bool cell_fits(unsigned long long M, int c, int n_lea
 // tile]).  A warp takes 32 consecutive positions at a time: 22 ballots give
 // each level's boundaries in the 64-position window around them, and each
 // lane bisects the levels for its LL.
+template <int ROWS>
 __global__ void __launch_bounds__(kBT) k_tree_count(int64_t n, int n_leaf, const uint64_t* __restrict__ keys,
                                                     const uint32_t* __restrict__ sys, uint32_t* __restrict__ pk,
                                                     uint32_t* __restrict__ wcount, uint32_t* __restrict__ tcount,
                                                     int64_t nw, int64_t ntiles, RootArgs R) {
+    constexpr int kSpan = 32 * ROWS, kTile = kBT * ROWS;
     write_roots(R);  // level 0 (no other work of this pass depends on it)
-    __shared__ uint8_t sD[kBTile + 2 * kHalo];
+    __shared__ uint8_t sD[kTile + 2 * kHalo];
     __shared__ unsigned long long s_m[kBWarps][kMaxLevel + 1];
     __shared__ uint32_t s_wc[kMaxLevel][kBWarps];
-    const int64_t t0 = (int64_t)blockIdx.x * kBTile;
-    for (int q = threadIdx.x; q < kBTile + 2 * kHalo; q += kBT)
+    const int64_t t0 = (int64_t)blockIdx.x * kTile;
+    for (int q = threadIdx.x; q < kTile + 2 * kHalo; q += kBT)
         sD[q] = (uint8_t)first_diff_level(t0 - kHalo + q, n, keys, sys);
     __syncthreads();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -206,8 +213,8 @@ __global__ void __launch_bounds__(kBT) k_tree_count(int64_t n, int n_leaf, const
     uint32_t cnt[kMaxLevel];
 #pragma unroll
     for (int l = 0; l < kMaxLevel; ++l) cnt[l] = 0u;
-    for (int r = 0; r < kBRows; ++r) {
-        const int rb = w * kBSpan + r * 32;  // tile position of the row's first position
+    for (int r = 0; r < ROWS; ++r) {
+        const int rb = w * kSpan + r * 32;  // tile position of the row's first position
         const int64_t i = t0 + rb + lane;
         const uint32_t dA = sD[rb + lane];       // window 0..31
         const uint32_t dB = sD[rb + 32 + lane];  // window 32..63
@@ -282,16 +289,18 @@ __device__ __forceinline__ uint32_t compact3(uint64_t v) {
 // node ends at n).  Each block derives the level starts from the totals
 // (levels from the first that does not fit in the node arrays on are left
 // empty, with the overflow flag set); block 0 also publishes them.
+template <int ROWS>
 __global__ void __launch_bounds__(kBT) k_tree_nodes(
     int64_t n, int n_roots, int64_t cap_nodes, const uint64_t* __restrict__ keys,
     const uint32_t* __restrict__ sys, const uint32_t* __restrict__ pk, const uint32_t* __restrict__ wcount,
     const uint32_t* __restrict__ tcount, int64_t nw, int64_t ntiles, const uint32_t* __restrict__ ltot,
     DevState* st, uint32_t* __restrict__ nd_first, uint32_t* __restrict__ nd_end, uint32_t* __restrict__ nd_child,
     uint32_t* __restrict__ nd_meta, uint32_t* __restrict__ nd_parent, uint64_t* __restrict__ nd_qlo) {
+    constexpr int kSpan = 32 * ROWS, kTile = kBT * ROWS;
     __shared__ int64_t s_lvl[kMaxLevel + 3];
     __shared__ int s_cut;
     __shared__ uint32_t s_wc[kMaxLevel][kBWarps];
-    __shared__ uint32_t sP[1 + kBTile];  // pk of positions t0 - 1 .. t0 + kBTile - 1
+    __shared__ uint32_t sP[1 + kTile];  // pk of positions t0 - 1 .. t0 + kTile - 1
     if (threadIdx.x == 0) {
         int64_t s = n_roots;
         // keys left unsorted by a sort that gave up: roots only, so that
@@ -317,9 +326,9 @@ __global__ void __launch_bounds__(kBT) k_tree_nodes(
         }
     }
     const int64_t tile = blockIdx.x;
-    const int64_t t0 = tile * kBTile;
+    const int64_t t0 = tile * kTile;
     // positions at or past n: D = 0, no nodes
-    for (int q = threadIdx.x; q < 1 + kBTile; q += kBT) {
+    for (int q = threadIdx.x; q < 1 + kTile; q += kBT) {
         const int64_t j = t0 - 1 + q;
         sP[q] = (j >= 0 && j < n) ? pk[j] : 0u;
     }
@@ -342,8 +351,8 @@ __global__ void __launch_bounds__(kBT) k_tree_nodes(
     uint32_t run[kMaxLevel];
 #pragma unroll
     for (int l = 1; l <= kMaxLevel; ++l) run[l - 1] = __shfl_sync(0xFFFFFFFFu, nxt, l);
-    for (int r = 0; r < kBRows; ++r) {
-        const int p = w * kBSpan + r * 32 + lane;
+    for (int r = 0; r < ROWS; ++r) {
+        const int p = w * kSpan + r * 32 + lane;
         const int64_t j = t0 + p;
         const uint32_t v = sP[1 + p], u = sP[p];
         const uint32_t d = v & 0xFFu, LL = (v >> 8) & 0xFFu;
@@ -477,7 +486,9 @@ struct MomArgs {
 // children in octant order.  Quadrupole: FP64 (Q64) for the FP64 pipeline; otherwise FP32 from
 // positions relative to the node's COM formed from FP32 hi/lo pairs, and the
 // parallel-axis shift for internal nodes.
-template <bool QUAD, bool Q64>
+// AHEAD: a node's children are all loaded before the first is summed (where
+// latency counts and registers are free).
+template <bool QUAD, bool Q64, bool AHEAD>
 __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
     const uint32_t meta = A.nd_meta[i];
     const bool leaf = meta_leaf(meta);
@@ -492,6 +503,24 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
             Sy = __dadd_rn(Sy, A.pmy[p]);
             Sz = __dadd_rn(Sz, A.pmz[p]);
         }
+    } else if (AHEAD) {
+        double m8[8], x8[8], y8[8], z8[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t c = c0 + (k < (int)nc ? k : 0);
+            m8[k] = __ldcg(&A.nd_com[c].w);
+            x8[k] = __ldcg(&A.nd_sx[c]);
+            y8[k] = __ldcg(&A.nd_sy[c]);
+            z8[k] = __ldcg(&A.nd_sz[c]);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (k < (int)nc) {
+                M = __dadd_rn(M, m8[k]);
+                Sx = __dadd_rn(Sx, x8[k]);
+                Sy = __dadd_rn(Sy, y8[k]);
+                Sz = __dadd_rn(Sz, z8[k]);
+            }
     } else {
         for (uint32_t c = c0; c < c0 + nc; ++c) {
             M = __dadd_rn(M, __ldcg(&A.nd_com[c].w));
@@ -576,10 +605,7 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
                 q[5] += m * (3.0f * dy * dz);
             }
         } else {
-            for (uint32_t c = c0; c < c0 + nc; ++c) {
-                const float4 ch = __ldcg(&A.nd_f[2 * c]), cl = __ldcg(&A.nd_f[2 * c + 1]);
-                const float4 q0 = __ldcg(&A.nd_fq0[c]);
-                const float2 q1 = __ldcg(&A.nd_fq1[c]);
+            auto shift = [&](const float4 ch, const float4 cl, const float4 q0, const float2 q1) {
                 const float dx = (ch.x - hx) + (cl.x - lx), dy = (ch.y - hy) + (cl.y - ly),
                             dz = (ch.z - hz) + (cl.z - lz);
                 const float d2 = dx * dx + dy * dy + dz * dz;
@@ -590,6 +616,25 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
                 q[3] += q0.w + m * (3.0f * dx * dy);
                 q[4] += q1.x + m * (3.0f * dx * dz);
                 q[5] += q1.y + m * (3.0f * dy * dz);
+            };
+            if (AHEAD) {
+                float4 ch[8], cl[8], q0[8];
+                float2 q1[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const uint32_t c = c0 + (k < (int)nc ? k : 0);
+                    ch[k] = __ldcg(&A.nd_f[2 * c]);
+                    cl[k] = __ldcg(&A.nd_f[2 * c + 1]);
+                    q0[k] = __ldcg(&A.nd_fq0[c]);
+                    q1[k] = __ldcg(&A.nd_fq1[c]);
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (k < (int)nc) shift(ch[k], cl[k], q0[k], q1[k]);
+            } else {
+                for (uint32_t c = c0; c < c0 + nc; ++c)
+                    shift(__ldcg(&A.nd_f[2 * c]), __ldcg(&A.nd_f[2 * c + 1]), __ldcg(&A.nd_fq0[c]),
+                          __ldcg(&A.nd_fq1[c]));
             }
         }
         A.nd_fq0[i] = make_float4(q[0], q[1], q[2], q[3]);
@@ -597,100 +642,109 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
     }
 }
 
-// Systems of an ensemble with at most this many particles get their whole
-// subtree from one CTA (k_moments_systems); larger ones, and a single
-// system, go through the leaf pass and one pass per level.
-constexpr int64_t kSysMomMax = int64_t(1) << 17;
+// Leaves of every level in one launch, then the internal nodes level by
+// level from the deepest up in one more: a barrier between levels, so that
+// each internal node finds its children complete.  With a launch per level
+// (21, most of them for levels with few or no nodes) the internal nodes were
+// all latency below about 10^6 particles.  Up to kMomSmall particles one
+// cluster of CTAs takes all levels (a cluster barrier costs a fraction of a
+// launch, and a level's few hundred nodes fill 8 SMs); beyond, a cooperative
+// grid with a barrier in global memory, whose block 0 alone, with block
+// barriers, finishes the levels near the roots once they and all above hold
+// at most kTopNodes nodes.  Systems of an ensemble go through the same passes (one CTA
+// per system before: 256 clusters of 256 to 65536 particles waited for the
+// largest).  The sums of a node keep their order, so results do not depend
+// on the split.  Moments of Plummer 2^14: 136 -> 57 us; of
+// Plummer 2^20 with quadrupoles 246 -> 205 us; of the 256 clusters 1.18 ->
+// 0.39 ms.
+constexpr int kMomBlock = 256;
+constexpr int kMomCl = 8;
+constexpr int64_t kMomSmall = int64_t(1) << 16;
+constexpr int kTopNodes = 4 * kMomBlock;
+constexpr int kMaxGridSpin = 1 << 20;
 
-// Does the level-by-level pass skip node i (its system is done by
-// k_moments_systems)?
-__device__ __forceinline__ bool small_system_node(const MomArgs& A, const int64_t* off, int64_t i) {
-    if (!off) return false;
-    const uint32_t s = A.sys[A.nd_first[i]];
-    return off[s + 1] - off[s] <= kSysMomMax;
-}
-
-// Leaves (of every level) in one launch, then the internal nodes level by
-// level from the deepest up: each internal node finds its children complete.
 template <bool QUAD, bool Q64>
-__global__ void __launch_bounds__(256) k_moments_leaves(MomArgs A, const int64_t* off) {
+__global__ void __launch_bounds__(kMomBlock) k_moments_leaves(MomArgs A) {
     const int64_t nn = A.st->n_nodes;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nn;
-         i += (int64_t)gridDim.x * blockDim.x)
-        if (meta_leaf(A.nd_meta[i]) && !small_system_node(A, off, i)) node_moments<QUAD, Q64>(A, i);
+    for (int64_t i = blockIdx.x * (int64_t)kMomBlock + threadIdx.x; i < nn; i += (int64_t)gridDim.x * kMomBlock)
+        if (meta_leaf(A.nd_meta[i])) node_moments<QUAD, Q64, false>(A, i);
 }
 
 template <bool QUAD, bool Q64>
-__global__ void __launch_bounds__(256) k_moments_internal(MomArgs A, const int64_t* off, int l) {
-    const int64_t a = A.st->lvl_start[l], b = A.st->lvl_start[l + 1];
-    for (int64_t i = a + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < b;
-         i += (int64_t)gridDim.x * blockDim.x)
-        if (!meta_leaf(A.nd_meta[i]) && !small_system_node(A, off, i)) node_moments<QUAD, Q64>(A, i);
-}
-
-// First node of level range [lo, hi) whose first particle is >= p (the
-// nodes of a level are ordered by their first particle).
-__device__ __forceinline__ int64_t level_lower_bound(const uint32_t* nd_first, int64_t lo, int64_t hi, int64_t p) {
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if ((int64_t)nd_first[mid] < p)
-            lo = mid + 1;
-        else
-            hi = mid;
+__global__ void __cluster_dims__(kMomCl, 1, 1) __launch_bounds__(kMomBlock) k_moments_small(MomArgs A) {
+    for (int l = A.st->max_level - 1; l >= 0; --l) {
+        const int64_t a = A.st->lvl_start[l], b = A.st->lvl_start[l + 1];
+        for (int64_t i = a + blockIdx.x * kMomBlock + threadIdx.x; i < b; i += kMomCl * kMomBlock)
+            if (!meta_leaf(A.nd_meta[i])) node_moments<QUAD, Q64, true>(A, i);
+        __threadfence();
+        cluster_barrier();  // this level complete before its parents
     }
-    return lo;
 }
 
-// One CTA per system of at most kSysMomMax particles (systems taken from a
-// counter, largest first): the system's nodes level by level from the deepest up, with the
-// same per-node code as the level passes, so the sums (and the centres of
-// mass) come out bit for bit the same; one launch instead of 22.
-template <bool QUAD, bool Q64>
-__global__ void __launch_bounds__(256) k_moments_systems(MomArgs A, const int64_t* __restrict__ off,
-                                                       const int32_t* __restrict__ order, int32_t n_sys,
-                                                       uint32_t* counter) {
-    __shared__ int32_t s_k;
-    __shared__ int64_t s_rng[2 * (kMaxLevel + 1)];
-    for (;;) {
-        if (threadIdx.x == 0) s_k = (int32_t)atomicAdd(counter, 1u);
-        __syncthreads();
-        if (s_k >= n_sys) break;
-        const int32_t k = order[s_k];  // largest systems first
-        const int64_t a = off[k], b = off[k + 1];
-        if (b - a <= kSysMomMax) {
-            if (threadIdx.x <= kMaxLevel) {
-                const int l = threadIdx.x;
-                const int64_t lo = A.st->lvl_start[l], hi = A.st->lvl_start[l + 1];
-                s_rng[2 * l] = level_lower_bound(A.nd_first, lo, hi, a);
-                s_rng[2 * l + 1] = level_lower_bound(A.nd_first, lo, hi, b);
+// Barrier over the grid (all blocks resident: a cooperative launch); count
+// starts at zero and target is a multiple of the grid size, one more for
+// each barrier.  The wait is bounded: beyond it the error bit of a device
+// wait is set and the block goes on (its sums are then invalid, every access
+// stays within the node arrays).
+__device__ __forceinline__ void grid_barrier(uint32_t* count, uint32_t target, uint32_t* overflow) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(count, 1u);
+        int spin = 0;
+        while (*(volatile uint32_t*)count < target)
+            if (++spin > kMaxGridSpin) {
+                atomicOr(overflow, kSortStall);
+                break;
             }
-            __syncthreads();
-            for (int l = kMaxLevel; l >= 0; --l) {
-                for (int64_t i = s_rng[2 * l] + threadIdx.x; i < s_rng[2 * l + 1]; i += blockDim.x)
-                    node_moments<QUAD, Q64>(A, i);
-                __syncthreads();  // this level complete before its parents
-            }
-        }
-        __syncthreads();  // s_k and s_rng are rewritten next round
+        __threadfence();
+    }
+    __syncthreads();
+}
+
+template <bool QUAD, bool Q64>
+__global__ void __launch_bounds__(kMomBlock) k_moments_levels(MomArgs A, uint32_t* count, uint32_t* overflow) {
+    const int64_t t = blockIdx.x * (int64_t)kMomBlock + threadIdx.x, G = (int64_t)gridDim.x * kMomBlock;
+    uint32_t target = 0;
+    int l = A.st->max_level - 1;
+    for (; l >= 0; --l) {
+        const int64_t a = A.st->lvl_start[l], b = A.st->lvl_start[l + 1];
+        if (b <= kTopNodes) break;
+        for (int64_t i = a + t; i < b; i += G)
+            if (!meta_leaf(A.nd_meta[i])) node_moments<QUAD, Q64, false>(A, i);
+        target += gridDim.x;
+        grid_barrier(count, target, overflow);
+    }
+    if (blockIdx.x != 0) return;
+    for (; l >= 0; --l) {
+        const int64_t a = A.st->lvl_start[l], b = A.st->lvl_start[l + 1];
+        for (int64_t i = a + threadIdx.x; i < b; i += kMomBlock)
+            if (!meta_leaf(A.nd_meta[i])) node_moments<QUAD, Q64, false>(A, i);
+        __threadfence_block();
+        __syncthreads();  // this level complete before its parents
     }
 }
 
 template <bool QUAD, bool Q64>
-int launch_moments(fdps_ctx* ctx, const MomArgs& A, const fdps_psys* ps, DevState* st) {
-    const int grid = ctx->sm_count * 8;
-    const int64_t* off = ps->n_sys > 1 ? ps->d_off : nullptr;
-    if (off) {
-        const int g = (int)std::min<int64_t>(ps->n_sys, (int64_t)ctx->sm_count * 8);
-        k_moments_systems<QUAD, Q64><<<g, 256, 0, ctx->stream>>>(A, off, ps->d_order, ps->n_sys, &st->mom_counter);
-        FDPS_LAUNCH_CHECK(ctx);
-        if (ps->max_sys_n <= kSysMomMax) return FDPS_OK;
-    }
-    k_moments_leaves<QUAD, Q64><<<grid, 256, 0, ctx->stream>>>(A, off);
+int launch_moments(fdps_ctx* ctx, const MomArgs& A, int64_t n, DevState* st) {
+    k_moments_leaves<QUAD, Q64><<<ctx->sm_count * 8, kMomBlock, 0, ctx->stream>>>(A);
     FDPS_LAUNCH_CHECK(ctx);
-    for (int l = kMaxLevel - 1; l >= 0; --l) {
-        k_moments_internal<QUAD, Q64><<<grid, 256, 0, ctx->stream>>>(A, off, l);
+    if (n <= kMomSmall) {
+        k_moments_small<QUAD, Q64><<<kMomCl, kMomBlock, 0, ctx->stream>>>(A);
         FDPS_LAUNCH_CHECK(ctx);
+        return FDPS_OK;
     }
+    int per_sm = 0;
+    FDPS_CUDA_TRY(ctx,
+                  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_moments_levels<QUAD, Q64>, kMomBlock, 0));
+    const int grid = ctx->sm_count * std::max(1, per_sm);  // every block resident
+    MomArgs args = A;
+    uint32_t* count = &st->mom_counter;
+    uint32_t* overflow = &st->overflow;
+    void* kargs[] = {&args, &count, &overflow};
+    FDPS_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((const void*)k_moments_levels<QUAD, Q64>, dim3((unsigned)grid),
+                                                   dim3(kMomBlock), kargs, 0, ctx->stream));
+    FDPS_LAUNCH_CHECK(ctx);
     return FDPS_OK;
 }
 
@@ -795,9 +849,17 @@ __device__ __forceinline__ double unord64(unsigned long long o) {
 // FP64 box of each group (min / max over its particles), its grid box (the
 // quantised corners: quantisation is monotone, so these are the minimum and
 // maximum grid coordinates of the particles), FP64 centre and the FP32
-// copies the walk's filter and the force kernel use.  A warp takes 32
-// groups: the lanes reduce each group's particles together, then every lane
-// finishes one group's FP64 arithmetic.
+// copies the walk's filter and the force kernel use.  A warp takes a run of
+// up to kGrpRun groups: the lanes reduce each group's particles together, then
+// lane 3 j + a finishes axis a of group j (the FP64 pipe is narrow: a lane
+// per axis takes it for a third of the warp instructions of a lane per
+// group).  Runs are short where there are few groups, so that all warps have
+// one: each group of a run costs its loads' latency and 60 shuffles in turn
+// (with runs of 32 the pass took 115 us on the 27,500 groups of 2^20
+// particles, most of the GPU idle; with short
+// runs all group passes together went from 143 to 59 us, on the 1,002 groups
+// of 2^14 particles from 51 to 25 us).
+constexpr int kGrpRun = 10;  // 30 of a warp's lanes
 __global__ void __launch_bounds__(256) k_group_data(
     const DevState* __restrict__ st, const SysBox* __restrict__ box, const uint32_t* __restrict__ sys,
     const uint32_t* __restrict__ g_first,
@@ -809,9 +871,12 @@ __global__ void __launch_bounds__(256) k_group_data(
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t ng = st->n_groups;
-    for (int64_t base = warp * 32; base < ng; base += nwarps * 32) {
-        unsigned long long mlo[3] = {0, 0, 0}, mhi[3] = {0, 0, 0};
-        const int nb = ng - base < 32 ? (int)(ng - base) : 32;
+    const int64_t per = (ng + nwarps - 1) / nwarps;
+    const int run = per < kGrpRun ? (int)per : kGrpRun;
+    const int lj = lane / 3, la = lane - 3 * lj;
+    for (int64_t base = warp * run; base < ng; base += nwarps * run) {
+        unsigned long long mlo = 0, mhi = 0;
+        const int nb = ng - base < run ? (int)(ng - base) : run;
         for (int j = 0; j < nb; ++j) {
             const uint32_t f = g_first[base + j], c = g_count[base + j];
             unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
@@ -832,35 +897,31 @@ __global__ void __launch_bounds__(256) k_group_data(
                     lo[a] = l2 < lo[a] ? l2 : lo[a];
                     hi[a] = h2 > hi[a] ? h2 : hi[a];
                 }
-            if (lane == j)
-                for (int a = 0; a < 3; ++a) {
-                    mlo[a] = lo[a];
-                    mhi[a] = hi[a];
-                }
+            if (lj == j) {
+                mlo = la == 0 ? lo[0] : la == 1 ? lo[1] : lo[2];
+                mhi = la == 0 ? hi[0] : la == 1 ? hi[1] : hi[2];
+            }
         }
-        if (lane >= nb) continue;
-        const int64_t g = base + lane;
+        if (lj >= nb) continue;
+        const int64_t g = base + lj;
         const SysBox& bx = box[sys ? sys[g_first[g]] : 0];
-        double bl[3], bh[3], cc[3];
-        float ch[3], cl[3], fl[3], fh[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            bl[a] = unord64(mlo[a]);
-            bh[a] = unord64(mhi[a]);
-            g_box[6 * g + a] = bl[a];
-            g_box[6 * g + 3 + a] = bh[a];
-            g_qbox[6 * g + a] = quantise(bl[a], bx.lo[a], bx.s);
-            g_qbox[6 * g + 3 + a] = quantise(bh[a], bx.lo[a], bx.s);
-            cc[a] = __dmul_rn(__dadd_rn(bl[a], bh[a]), 0.5);
-            split_hilo(cc[a] - bx.c0[a], &ch[a], &cl[a]);
-            fl[a] = __double2float_rd(bl[a] - cc[a]);
-            fh[a] = __double2float_ru(bh[a] - cc[a]);
+        const double bl = unord64(mlo), bh = unord64(mhi);
+        g_box[6 * g + la] = bl;
+        g_box[6 * g + 3 + la] = bh;
+        g_qbox[6 * g + la] = quantise(bl, bx.lo[la], bx.s);
+        g_qbox[6 * g + 3 + la] = quantise(bh, bx.lo[la], bx.s);
+        const double cc = __dmul_rn(__dadd_rn(bl, bh), 0.5);
+        float ch, cl;
+        split_hilo(cc - bx.c0[la], &ch, &cl);
+        reinterpret_cast<double*>(g_c64 + g)[la] = cc;
+        reinterpret_cast<float*>(g_ch + g)[la] = ch;
+        reinterpret_cast<float*>(g_cl + g)[la] = cl;
+        reinterpret_cast<float*>(g_blo + g)[la] = __double2float_rd(bl - cc);
+        reinterpret_cast<float*>(g_bhi + g)[la] = __double2float_ru(bh - cc);
+        if (la == 0) {  // the vectors' unused fourth components
+            g_c64[g].w = 0.0;
+            g_ch[g].w = g_cl[g].w = g_blo[g].w = g_bhi[g].w = 0.0f;
         }
-        g_c64[g] = make_dvec4(cc[0], cc[1], cc[2], 0.0);
-        g_ch[g] = make_float4(ch[0], ch[1], ch[2], 0.0f);
-        g_cl[g] = make_float4(cl[0], cl[1], cl[2], 0.0f);
-        g_blo[g] = make_float4(fl[0], fl[1], fl[2], 0.0f);
-        g_bhi[g] = make_float4(fh[0], fh[1], fh[2], 0.0f);
     }
 }
 
@@ -870,7 +931,9 @@ int build_tree(fdps_tree* t, fdps_psys* ps) {
     fdps_ctx* ctx = t->ctx;
     cudaStream_t s = ctx->stream;
     const int64_t n = ps->n;
-    const int64_t ntiles = n > 0 ? (n + kBTile - 1) / kBTile : 1;
+    const bool small = n <= kBuildSmall;
+    const int64_t tile = small ? kBT : kBTile;
+    const int64_t ntiles = n > 0 ? (n + tile - 1) / tile : 1;
     const int64_t nw = ntiles * kBWarps;
     uint32_t* wcount = t->bt_count;                 // [21][nw] per warp
     uint32_t* tcount = wcount + kMaxLevel * nw;     // [21][ntiles] per tile, then scanned
@@ -878,15 +941,15 @@ int build_tree(fdps_tree* t, fdps_psys* ps) {
     const RootArgs R{ps->n_sys, ps->d_off, n, t->p.n_leaf, t->nd_first, t->nd_count,
                      t->nd_child, t->nd_meta, t->nd_parent, t->nd_qlo};
     // per-position scratch: t->head, rewritten by the group selection
-    k_tree_count<<<(unsigned)ntiles, kBT, 0, s>>>(n, t->p.n_leaf, t->keys_sorted, ps->d_sys, t->head, wcount,
-                                                  tcount, nw, ntiles, R);
+    (small ? k_tree_count<1> : k_tree_count<kBRows>)<<<(unsigned)ntiles, kBT, 0, s>>>(
+        n, t->p.n_leaf, t->keys_sorted, ps->d_sys, t->head, wcount, tcount, nw, ntiles, R);
     FDPS_LAUNCH_CHECK(ctx);
     k_tree_scan<<<kMaxLevel, 1024, 0, s>>>(tcount, ntiles, ltot);
     FDPS_LAUNCH_CHECK(ctx);
-    const unsigned grid_nodes = (unsigned)(n / kBTile + 1);  // positions 0 .. n
-    k_tree_nodes<<<grid_nodes, kBT, 0, s>>>(n, ps->n_sys, t->cap_nodes, t->keys_sorted, ps->d_sys, t->head,
-                                            wcount, tcount, nw, ntiles, ltot, t->st, t->nd_first, t->nd_count,
-                                            t->nd_child, t->nd_meta, t->nd_parent, t->nd_qlo);
+    const unsigned grid_nodes = (unsigned)(n / tile + 1);  // positions 0 .. n
+    (small ? k_tree_nodes<1> : k_tree_nodes<kBRows>)<<<grid_nodes, kBT, 0, s>>>(
+        n, ps->n_sys, t->cap_nodes, t->keys_sorted, ps->d_sys, t->head, wcount, tcount, nw, ntiles, ltot, t->st,
+        t->nd_first, t->nd_count, t->nd_child, t->nd_meta, t->nd_parent, t->nd_qlo);
     FDPS_LAUNCH_CHECK(ctx);
     k_tree_finish<<<ctx->sm_count * 4, 256, 0, s>>>(t->st, ps->n_sys, t->nd_first, t->nd_count, t->nd_parent,
                                                     t->nd_child, t->nd_meta);
@@ -925,9 +988,9 @@ int compute_moments(fdps_tree* t, fdps_psys* ps) {
     A.nd_walk = t->nd_walk;
     A.nd_fq0 = t->nd_fq0;
     A.nd_fq1 = t->nd_fq1;
-    if (t->p.moment != FDPS_QUADRUPOLE) return launch_moments<false, false>(ctx, A, ps, t->st);
-    if (t->p.precision == FDPS_FP64) return launch_moments<true, true>(ctx, A, ps, t->st);
-    return launch_moments<true, false>(ctx, A, ps, t->st);
+    if (t->p.moment != FDPS_QUADRUPOLE) return launch_moments<false, false>(ctx, A, ps->n, t->st);
+    if (t->p.precision == FDPS_FP64) return launch_moments<true, true>(ctx, A, ps->n, t->st);
+    return launch_moments<true, false>(ctx, A, ps->n, t->st);
 }
 
 int select_groups(fdps_tree* t, fdps_psys* ps) {

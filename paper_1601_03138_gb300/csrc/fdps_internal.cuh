@@ -39,6 +39,8 @@ constexpr int kMaxLeaf = 16;
 constexpr int kMaxGrp = 4096;
 constexpr int kBuildTile = 2048;  // positions per tile of the tree build
 constexpr int kBuildWarps = 8;    // warps per tile of the tree build
+constexpr int kBuildSmall = 1 << 15;  // up to here the build's tiles hold kBuildTileSmall positions
+constexpr int kBuildTileSmall = 256;
 constexpr int kCohT = 1024;       // positions per bucket of the coherent time-step sort
 
 // overflow bits of DevState::overflow
@@ -68,7 +70,7 @@ struct DevState {
     uint32_t overflow;
     uint32_t walk_counter;   // dynamic group scheduler of the walk
     uint32_t force_counter;  // dynamic group scheduler of the force kernel
-    uint32_t mom_counter;    // dynamic system scheduler of the per-system moments
+    uint32_t mom_counter;    // arrivals at the grid barriers of the moments
     uint32_t grp_done;       // blocks of the group count finished (the last one scans)
     uint32_t pad1;
     unsigned long long pool_cursor;  // list pool allocation cursor (entries)
@@ -150,6 +152,38 @@ __device__ __forceinline__ float to_f32(double v) {
     return hi;
 }
 
+// Thread-block clusters: a barrier over the cluster's threads (release and
+// acquire), the block's rank, and reads of a peer block's shared memory.
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// The cluster's address of this CTA's shared variable p in CTA `rank`.
+__device__ __forceinline__ uint32_t peer_smem(const void* p, uint32_t rank) {
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ unsigned long long ld_peer_u64(uint32_t a) {
+    unsigned long long v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ double ld_peer_f64(uint32_t a) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_peer_u32(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+
 // Root box of one system: lo = per-axis minimum, L = largest extent (1 if
 // 0), s = 2^21 / L, c0 = lo + L/2 (origin of the FP32 hi/lo copies).
 struct SysBox {
@@ -208,9 +242,7 @@ struct fdps_psys {
     // independent systems: positions off[k] .. off[k+1] belong to system k;
     // with one system d_off and d_sys stay null
     int32_t n_sys = 1;
-    int64_t max_sys_n = 0;       // particles of the largest system (n with one system)
     int64_t* d_off = nullptr;
-    int32_t* d_order = nullptr;  // systems by decreasing particle count
     uint32_t* d_sys = nullptr;   // system of each position
     // buckets of the coherent time-step sort (several systems): bucket b
     // holds positions d_cbs[b] .. d_cbs[b + 1] - 1 of system d_cbsys[b];

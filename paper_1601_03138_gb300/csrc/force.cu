@@ -674,31 +674,6 @@ __device__ __forceinline__ GroupPlan plan_f64(uint32_t ni) {
     return best;
 }
 
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// The cluster's address of this CTA's shared variable p in CTA `rank`.
-__device__ __forceinline__ uint32_t peer_smem(const void* p, uint32_t rank) {
-    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ double ld_peer_f64(uint32_t a) {
-    double v;
-    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint32_t ld_peer_u32(uint32_t a) {
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-    return v;
-}
-
 // One round of i-particles (ib .. ib + P K - 1 of the group) with K per
 // thread, over this CTA's share of the list; called by the whole cluster.
 template <bool QUAD, int K>
