@@ -7,7 +7,8 @@
 //         and the product each rounded to nearest in FP64 (no FMA), then
 //         bits of q_x / q_y / q_z interleaved to key bits 3b+2 / 3b+1 / 3b
 //   sort  stable by key.  Up to kSmallMax particles of one system: box,
-//         keys and a merge sort of (key, position) pairs in one CTA.  Beyond,
+//         keys and a merge sort of (key, position) pairs in one cluster of
+//         CTAs.  Beyond,
 //         the force pipeline runs 8 LSD passes of 8-bit digits: the digit
 //         counts of all passes are taken while the keys are computed, then
 //         one kernel per pass (tile ranking, a bounded look-back over
@@ -151,10 +152,10 @@ __global__ void k_box_final(int nparts, const BoxPartial* __restrict__ part, Dev
     box->s = st->s;
 }
 
-// Root box of the particles whose mapped coordinates' minima and maxima the
-// threads of a block (WARPS warps) hold in lo and hi; valid in thread 0.
+// Minima and maxima over a block (WARPS warps) of the mapped coordinates
+// that its threads hold in lo and hi; valid in thread 0.
 template <int WARPS>
-__device__ __forceinline__ SysBox block_box(unsigned long long (&lo)[3], unsigned long long (&hi)[3]) {
+__device__ __forceinline__ void block_minmax(unsigned long long (&lo)[3], unsigned long long (&hi)[3]) {
     __shared__ unsigned long long s_lo[WARPS][3], s_hi[WARPS][3];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
@@ -172,24 +173,27 @@ __device__ __forceinline__ SysBox block_box(unsigned long long (&lo)[3], unsigne
             s_hi[w][a] = hi[a];
         }
     __syncthreads();
-    SysBox b;
-    if (threadIdx.x == 0) {
-        double L = 0.0;
-        for (int a = 0; a < 3; ++a) {
-            unsigned long long l = s_lo[0][a], h = s_hi[0][a];
-            for (int k = 1; k < WARPS; ++k) {
-                l = s_lo[k][a] < l ? s_lo[k][a] : l;
-                h = s_hi[k][a] > h ? s_hi[k][a] : h;
+    if (threadIdx.x == 0)
+        for (int k = 1; k < WARPS; ++k)
+            for (int a = 0; a < 3; ++a) {
+                lo[a] = s_lo[k][a] < lo[a] ? s_lo[k][a] : lo[a];
+                hi[a] = s_hi[k][a] > hi[a] ? s_hi[k][a] : hi[a];
             }
-            b.lo[a] = unord64(l);
-            const double e = __dsub_rn(unord64(h), b.lo[a]);
-            L = e > L ? e : L;
-        }
-        if (L == 0.0) L = 1.0;
-        b.L = L;
-        b.s = __ddiv_rn(2097152.0, L);
-        for (int a = 0; a < 3; ++a) b.c0[a] = __dadd_rn(b.lo[a], __dmul_rn(0.5, L));
+}
+
+// The root box of mapped minima and maxima.
+__device__ __forceinline__ SysBox box_of(const unsigned long long (&lo)[3], const unsigned long long (&hi)[3]) {
+    SysBox b;
+    double L = 0.0;
+    for (int a = 0; a < 3; ++a) {
+        b.lo[a] = unord64(lo[a]);
+        const double e = __dsub_rn(unord64(hi[a]), b.lo[a]);
+        L = e > L ? e : L;
     }
+    if (L == 0.0) L = 1.0;
+    b.L = L;
+    b.s = __ddiv_rn(2097152.0, L);
+    for (int a = 0; a < 3; ++a) b.c0[a] = __dadd_rn(b.lo[a], __dmul_rn(0.5, L));
     return b;
 }
 
@@ -211,8 +215,8 @@ __global__ void __launch_bounds__(256) k_box_seg(const int64_t* __restrict__ off
             hi[a] = v[a] > hi[a] ? v[a] : hi[a];
         }
     }
-    const SysBox b = block_box<8>(lo, hi);
-    if (threadIdx.x == 0) box[blockIdx.x] = b;
+    block_minmax<8>(lo, hi);
+    if (threadIdx.x == 0) box[blockIdx.x] = box_of(lo, hi);
 }
 
 // Spread the low 21 bits of v to every third bit (bit b -> bit 3b).
@@ -550,16 +554,14 @@ __global__ void __launch_bounds__(kCohBlock) k_coh_scatter(CohLayout L, const ui
     }
 }
 
-// Shared memory of a sort of up to CAP pairs: two key and two position
+// Shared memory of a sort of up to kCohCap pairs: two key and two position
 // buffers, element j at j + j / 16 (keys) and j + j / 32 (positions), so that
 // the threads of a warp reading or writing their EPT consecutive elements
 // fall in different banks.
-template <int CAP>
-struct PairShared {
-    unsigned long long k[2][CAP + CAP / 16];
-    uint32_t i[2][CAP + CAP / 32];
+struct CohShared {
+    unsigned long long k[2][kCohCap + kCohCap / 16];
+    uint32_t i[2][kCohCap + kCohCap / 32];
 };
-using CohShared = PairShared<kCohCap>;
 __device__ __forceinline__ int coh_kp(int j) { return j + (j >> 4); }
 __device__ __forceinline__ int coh_ip(int j) { return j + (j >> 5); }
 
@@ -569,14 +571,14 @@ __device__ __forceinline__ bool coh_less(unsigned long long ka, uint32_t ia, uns
     return ka < kb || (ka == kb && ia < ib);
 }
 
-// Merge sort of BLOCK * EPT pairs in buffer 0: each thread sorts its
+// Merge sort of kCohBlock * EPT pairs in buffer 0: each thread sorts its
 // EPT consecutive pairs in registers, then every round merges runs of
 // length L pairwise (L = EPT, 2 EPT, ...), each thread writing EPT
 // consecutive outputs from the split of its output diagonal found by
 // binary search (merge path).  Returns the buffer holding the result.
-template <int BLOCK, int EPT, class SM>
-__device__ __noinline__ int merge_sort_pairs(SM& sm) {
-    constexpr int np = BLOCK * EPT;
+template <int EPT>
+__device__ __noinline__ int merge_sort_pairs(CohShared& sm) {
+    constexpr int np = kCohBlock * EPT;
     const int o = threadIdx.x * EPT;
     {
         unsigned long long k[EPT];
@@ -651,17 +653,16 @@ __device__ __noinline__ int merge_sort_pairs(SM& sm) {
     return src;
 }
 
-template <int BLOCK, class SM>
-__device__ __forceinline__ int merge_sort_block(SM& sm, int ept) {
+__device__ __forceinline__ int merge_sort_block(CohShared& sm, int ept) {
     switch (ept) {
-        case 1: return merge_sort_pairs<BLOCK, 1>(sm);
-        case 2: return merge_sort_pairs<BLOCK, 2>(sm);
-        case 3: return merge_sort_pairs<BLOCK, 3>(sm);
-        case 4: return merge_sort_pairs<BLOCK, 4>(sm);
-        case 5: return merge_sort_pairs<BLOCK, 5>(sm);
-        case 6: return merge_sort_pairs<BLOCK, 6>(sm);
-        case 7: return merge_sort_pairs<BLOCK, 7>(sm);
-        default: return merge_sort_pairs<BLOCK, 8>(sm);
+        case 1: return merge_sort_pairs<1>(sm);
+        case 2: return merge_sort_pairs<2>(sm);
+        case 3: return merge_sort_pairs<3>(sm);
+        case 4: return merge_sort_pairs<4>(sm);
+        case 5: return merge_sort_pairs<5>(sm);
+        case 6: return merge_sort_pairs<6>(sm);
+        case 7: return merge_sort_pairs<7>(sm);
+        default: return merge_sort_pairs<8>(sm);
     }
 }
 
@@ -689,7 +690,7 @@ __global__ void __launch_bounds__(kCohBlock) k_coh_sort(const uint32_t* __restri
     }
     __syncthreads();
     static_assert(kCohCap == 8 * kCohBlock, "at most 8 pairs a thread");
-    const int src = merge_sort_block<kCohBlock>(sm, ept);
+    const int src = merge_sort_block(sm, ept);
     for (int j = threadIdx.x; j < m; j += kCohBlock) {
         keys_out[a0 + j] = sm.k[src][coh_kp(j)];
         perm_out[a0 + j] = sm.i[src][coh_ip(j)];
@@ -697,77 +698,6 @@ __global__ void __launch_bounds__(kCohBlock) k_coh_sort(const uint32_t* __restri
 }
 
 // ---------------------------------------------- small sets and sorted tiles
-
-// Root box, keys and stable sort of up to 8 BLOCK particles of one system in
-// one CTA: latency is all there is to it (13 launches of the box, histogram
-// and radix passes before; 35 of the allocation-free form), so one SM does
-// everything between two barriers' latency instead.  st (the box's copy in
-// the state word) and keys_in (keys in input order) may be null.
-// 4099 particles through the allocation-free entry point: 199 -> 53 us.
-constexpr int kSmallBlock = 1024;
-constexpr int64_t kSmallMax = 8 * kSmallBlock;
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK) k_sort_small(int n, const double* __restrict__ x,
-                                                      const double* __restrict__ y,
-                                                      const double* __restrict__ z, DevState* st, SysBox* box,
-                                                      uint64_t* __restrict__ keys_in,
-                                                      uint64_t* __restrict__ keys_out,
-                                                      uint32_t* __restrict__ perm_out) {
-    extern __shared__ __align__(16) unsigned char coh_dsm[];
-    PairShared<8 * BLOCK>& sm = *reinterpret_cast<PairShared<8 * BLOCK>*>(coh_dsm);
-    __shared__ SysBox s_box;
-    unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
-    for (int j = threadIdx.x; j < n; j += BLOCK) {
-        const unsigned long long v[3] = {ord64(x[j]), ord64(y[j]), ord64(z[j])};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = v[a] < lo[a] ? v[a] : lo[a];
-            hi[a] = v[a] > hi[a] ? v[a] : hi[a];
-        }
-    }
-    const SysBox b0 = block_box<BLOCK / 32>(lo, hi);
-    if (threadIdx.x == 0) {
-        s_box = b0;
-        if (box) *box = b0;
-        if (st) {
-            for (int a = 0; a < 3; ++a) {
-                st->lo[a] = b0.lo[a];
-                st->c0[a] = b0.c0[a];
-            }
-            st->L = b0.L;
-            st->s = b0.s;
-        }
-    }
-    __syncthreads();
-    const SysBox b = s_box;
-    const int ept = (n + BLOCK - 1) / BLOCK;
-    for (int j = threadIdx.x; j < ept * BLOCK; j += BLOCK) {
-        unsigned long long k = ~0ull;
-        if (j < n) {
-            k = morton_key(x[j], y[j], z[j], b);
-            if (keys_in) keys_in[j] = k;
-        }
-        sm.k[0][coh_kp(j)] = k;
-        sm.i[0][coh_ip(j)] = j < n ? (uint32_t)j : 0xFFFFFFFFu;
-    }
-    __syncthreads();
-    const int src = merge_sort_block<BLOCK>(sm, ept);
-    for (int j = threadIdx.x; j < n; j += BLOCK) {
-        keys_out[j] = sm.k[src][coh_kp(j)];
-        perm_out[j] = sm.i[src][coh_ip(j)];
-    }
-}
-
-int launch_sort_small(int64_t n, const double* x, const double* y, const double* z, DevState* st, SysBox* box,
-                      uint64_t* keys_in, uint64_t* keys_out, uint32_t* perm, cudaStream_t s) {
-    if (n <= 8 * kCohBlock)
-        k_sort_small<kCohBlock><<<1, kCohBlock, sizeof(PairShared<8 * kCohBlock>), s>>>((int)n, x, y, z, st, box,
-                                                                                        keys_in, keys_out, perm);
-    else
-        k_sort_small<kSmallBlock><<<1, kSmallBlock, sizeof(PairShared<8 * kSmallBlock>), s>>>(
-            (int)n, x, y, z, st, box, keys_in, keys_out, perm);
-    return cudaPeekAtLastError() == cudaSuccess ? FDPS_OK : FDPS_ECUDA;
-}
 
 // Keys of one tile of kSortTile particles per block, sorted.
 __global__ void __launch_bounds__(kCohBlock) k_tile_sort(int64_t n, const double* __restrict__ x,
@@ -788,7 +718,7 @@ __global__ void __launch_bounds__(kCohBlock) k_tile_sort(int64_t n, const double
         sm.i[0][coh_ip(j)] = j < m ? (uint32_t)(a0 + j) : 0xFFFFFFFFu;
     }
     __syncthreads();
-    const int src = merge_sort_block<kCohBlock>(sm, ept);
+    const int src = merge_sort_block(sm, ept);
     for (int j = threadIdx.x; j < m; j += kCohBlock) {
         keys_out[a0 + j] = sm.k[src][coh_kp(j)];
         perm_out[a0 + j] = sm.i[src][coh_ip(j)];
@@ -797,15 +727,14 @@ __global__ void __launch_bounds__(kCohBlock) k_tile_sort(int64_t n, const double
 
 // Merge path: of the first d outputs of sorted runs a [la] and b [lb] (equal
 // keys: a first), how many come from a.  A warp tests 32 splits at a time.
-__device__ __forceinline__ int merge_split(const uint64_t* __restrict__ a, int la, const uint64_t* __restrict__ b,
-                                           int lb, int d) {
+__device__ __forceinline__ int merge_split(const uint64_t* a, int la, const uint64_t* b, int lb, int d) {
     const int lane = threadIdx.x & 31;
     int lo = d > lb ? d - lb : 0, hi = d < la ? d : la;
     while (lo < hi) {
         const int step = (hi - lo + 31) / 32;
         const int i = lo + (lane + 1) * step - 1;
         // split i is too small iff a[i] precedes b[d - 1 - i]
-        const bool more = i < hi && a[i] <= b[d - 1 - i];
+        const bool more = i < hi && __ldcg(a + i) <= __ldcg(b + (d - 1 - i));
         const int c = __popc(__ballot_sync(0xFFFFFFFFu, more));  // a prefix of the lanes
         const int top = lo + (c + 1) * step - 1;
         lo += c * step;
@@ -814,22 +743,20 @@ __device__ __forceinline__ int merge_split(const uint64_t* __restrict__ a, int l
     return lo;
 }
 
-// One round of pairwise merges of sorted runs of L elements (a multiple of
-// kSortTile): a block writes kSortTile consecutive outputs, whose inputs it
-// stages in shared memory.  The runs hold consecutive positions, so taking
-// equal keys from the first run keeps the sort stable.
-__global__ void __launch_bounds__(kCohBlock) k_merge_runs(int64_t n, int L, const uint64_t* __restrict__ kin,
-                                                          const uint32_t* __restrict__ vin,
-                                                          uint64_t* __restrict__ kout, uint32_t* __restrict__ vout) {
-    extern __shared__ __align__(16) unsigned char coh_dsm[];
-    CohShared& sm = *reinterpret_cast<CohShared*>(coh_dsm);
+// Outputs o0 .. o0 + T - 1 (T <= kSortTile) of a round of pairwise merges of
+// sorted runs of L elements (a multiple of T), with the whole block: the
+// inputs are staged in shared memory, each thread merges EPT outputs.  The
+// runs hold consecutive positions, so taking equal keys from the first run
+// keeps the sort stable.
+__device__ __forceinline__ void merge_tile(CohShared& sm, int64_t n, int64_t L, int T, int64_t o0,
+                                           const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
+                                           uint32_t* vout) {
     __shared__ int s_split[2];
-    const int64_t o0 = (int64_t)blockIdx.x * kSortTile;
-    const int64_t a0 = o0 / (2 * (int64_t)L) * (2 * (int64_t)L);
-    const int la = n - a0 < L ? (int)(n - a0) : L;
-    const int lb = n - a0 - la < L ? (int)(n - a0 - la) : L;
+    const int64_t a0 = o0 / (2 * L) * (2 * L);
+    const int la = n - a0 < L ? (int)(n - a0) : (int)L;
+    const int lb = n - a0 - la < L ? (int)(n - a0 - la) : (int)L;
     const int d0 = (int)(o0 - a0);
-    const int d1 = d0 + kSortTile < la + lb ? d0 + kSortTile : la + lb;
+    const int d1 = d0 + T < la + lb ? d0 + T : la + lb;
     const int t = threadIdx.x, w = t >> 5;
     if (w < 2) {
         const int sp = merge_split(kin + a0, la, kin + a0 + la, lb, w == 0 ? d0 : d1);
@@ -839,11 +766,12 @@ __global__ void __launch_bounds__(kCohBlock) k_merge_runs(int64_t n, int L, cons
     const int ia0 = s_split[0], na = s_split[1] - ia0, ib0 = d0 - ia0, m = d1 - d0, nb = m - na;
     for (int j = t; j < m; j += kCohBlock) {
         const int64_t p = j < na ? a0 + ia0 + j : a0 + la + ib0 + (j - na);
-        sm.k[0][coh_kp(j)] = kin[p];
-        sm.i[0][coh_ip(j)] = vin[p];
+        sm.k[0][coh_kp(j)] = __ldcg(kin + p);
+        sm.i[0][coh_ip(j)] = __ldcg(vin + p);
     }
     __syncthreads();
-    const int d = t * 8;
+    const int ept = (m + kCohBlock - 1) / kCohBlock;
+    const int d = t * ept;
     if (d < m) {
         const unsigned long long* K = sm.k[0];
         int lo = d > nb ? d - nb : 0, hi = d < na ? d : na;
@@ -855,13 +783,12 @@ __global__ void __launch_bounds__(kCohBlock) k_merge_runs(int64_t n, int L, cons
                 hi = mid;
         }
         int ia = lo, ib = d - lo;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            if (d + r >= m) break;
+        const int e = d + ept < m ? d + ept : m;
+        for (int r = d; r < e; ++r) {
             const bool ta = ib >= nb || (ia < na && K[coh_kp(ia)] <= K[coh_kp(na + ib)]);
             const int j = ta ? ia : na + ib;
-            sm.k[1][coh_kp(d + r)] = K[coh_kp(j)];
-            sm.i[1][coh_ip(d + r)] = sm.i[0][coh_ip(j)];
+            sm.k[1][coh_kp(r)] = K[coh_kp(j)];
+            sm.i[1][coh_ip(r)] = sm.i[0][coh_ip(j)];
             ia += ta ? 1 : 0;
             ib += ta ? 0 : 1;
         }
@@ -873,6 +800,130 @@ __global__ void __launch_bounds__(kCohBlock) k_merge_runs(int64_t n, int L, cons
     }
 }
 
+// One round of pairwise merges, a tile of kSortTile outputs per block.
+__global__ void __launch_bounds__(kCohBlock) k_merge_runs(int64_t n, int64_t L, const uint64_t* __restrict__ kin,
+                                                          const uint32_t* __restrict__ vin,
+                                                          uint64_t* __restrict__ kout, uint32_t* __restrict__ vout) {
+    extern __shared__ __align__(16) unsigned char coh_dsm[];
+    merge_tile(*reinterpret_cast<CohShared*>(coh_dsm), n, L, kSortTile, blockIdx.x * (int64_t)kSortTile, kin, vin,
+               kout, vout);
+}
+
+// Root box, keys and stable sort of up to kSmallMax particles of one system
+// by one cluster of kSmallCl CTAs: latency is all there is to it (13 launches
+// of the box, histogram and radix passes before; 35 of the allocation-free
+// form).  Each CTA sorts an equal share in shared memory, then three rounds
+// merge the shares pairwise through L2, a share of the outputs per CTA, with
+// a cluster barrier between rounds (k1, v1: scratch of n pairs, the result
+// ends in k0, v0).  One CTA alone took 50 us for 4099 particles, its SM's two
+// FP64 lanes 6 us for the keys and its issue slots most of the rest.  st (the
+// box's copy in the state word), box and keys_in (keys in input order) may be
+// null.  4099 particles through the allocation-free entry point: 199 -> 26 us.
+constexpr int kSmallCl = 8;
+constexpr int64_t kSmallMax = kSmallCl * kSortTile;
+__global__ void __cluster_dims__(kSmallCl, 1, 1) __launch_bounds__(kCohBlock)
+    k_sort_small(int n, const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
+                 DevState* st, SysBox* box, uint64_t* __restrict__ keys_in, uint64_t* k0, uint32_t* v0, uint64_t* k1,
+                 uint32_t* v1) {
+    extern __shared__ __align__(16) unsigned char coh_dsm[];
+    CohShared& sm = *reinterpret_cast<CohShared*>(coh_dsm);
+    __shared__ unsigned long long s_mm[6];
+    __shared__ SysBox s_box;
+    const int t = threadIdx.x;
+    const uint32_t rank = cluster_rank();
+    const int T = (n + kSmallCl - 1) / kSmallCl;
+    const int a0 = (int)rank * T;
+    const int m = n - a0 < T ? (n > a0 ? n - a0 : 0) : T;
+    unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
+    for (int j = t; j < m; j += kCohBlock) {
+        const unsigned long long v[3] = {ord64(x[a0 + j]), ord64(y[a0 + j]), ord64(z[a0 + j])};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = v[a] < lo[a] ? v[a] : lo[a];
+            hi[a] = v[a] > hi[a] ? v[a] : hi[a];
+        }
+    }
+    block_minmax<kCohWarps>(lo, hi);
+    if (t == 0)
+        for (int a = 0; a < 3; ++a) {
+            s_mm[a] = lo[a];
+            s_mm[3 + a] = hi[a];
+        }
+    cluster_barrier();
+    if (t < 32) {
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = t < kSmallCl ? ld_peer_u64(peer_smem(&s_mm[a], (uint32_t)t)) : ~0ull;
+            hi[a] = t < kSmallCl ? ld_peer_u64(peer_smem(&s_mm[3 + a], (uint32_t)t)) : 0ull;
+        }
+#pragma unroll
+        for (int o = kSmallCl / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const unsigned long long l = __shfl_xor_sync(0xFFFFFFFFu, lo[a], o);
+                const unsigned long long h = __shfl_xor_sync(0xFFFFFFFFu, hi[a], o);
+                lo[a] = l < lo[a] ? l : lo[a];
+                hi[a] = h > hi[a] ? h : hi[a];
+            }
+        if (t == 0) {
+            const SysBox b0 = box_of(lo, hi);
+            s_box = b0;
+            if (rank == 0 && box) *box = b0;
+            if (rank == 0 && st) {
+                for (int a = 0; a < 3; ++a) {
+                    st->lo[a] = b0.lo[a];
+                    st->c0[a] = b0.c0[a];
+                }
+                st->L = b0.L;
+                st->s = b0.s;
+            }
+        }
+    }
+    __syncthreads();
+    const SysBox b = s_box;
+    const int ept = (m + kCohBlock - 1) / kCohBlock;
+    for (int j = t; j < ept * kCohBlock; j += kCohBlock) {
+        unsigned long long k = ~0ull;
+        if (j < m) {
+            k = morton_key(x[a0 + j], y[a0 + j], z[a0 + j], b);
+            if (keys_in) keys_in[a0 + j] = k;
+        }
+        sm.k[0][coh_kp(j)] = k;
+        sm.i[0][coh_ip(j)] = j < m ? (uint32_t)(a0 + j) : 0xFFFFFFFFu;
+    }
+    __syncthreads();
+    const int src = merge_sort_block(sm, ept > 0 ? ept : 1);
+    // three rounds: scratch, result, scratch, result
+    static_assert(kSmallCl == 8, "three merge rounds");
+    for (int j = t; j < m; j += kCohBlock) {
+        k1[a0 + j] = sm.k[src][coh_kp(j)];
+        v1[a0 + j] = sm.i[src][coh_ip(j)];
+    }
+    uint64_t* ki = k1;
+    uint32_t* vi = v1;
+    uint64_t* ko = k0;
+    uint32_t* vo = v0;
+    for (int r = 0; r < 3; ++r) {
+        __threadfence();
+        cluster_barrier();  // the runs are written
+        if (m > 0) merge_tile(sm, n, (int64_t)T << r, T, a0, ki, vi, ko, vo);
+        uint64_t* tk = ki;
+        ki = ko;
+        ko = tk;
+        uint32_t* tv = vi;
+        vi = vo;
+        vo = tv;
+        __syncthreads();  // the block's staging buffers are rewritten next round
+    }
+    // a block's shared memory was last read by its peers before the rounds'
+    // barriers: it may leave
+}
+
+int launch_sort_small(int64_t n, const double* x, const double* y, const double* z, DevState* st, SysBox* box,
+                      uint64_t* keys_in, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, cudaStream_t s) {
+    k_sort_small<<<kSmallCl, kCohBlock, sizeof(CohShared), s>>>((int)n, x, y, z, st, box, keys_in, k0, v0, k1, v1);
+    return cudaPeekAtLastError() == cudaSuccess ? FDPS_OK : FDPS_ECUDA;
+}
+
 // The dynamic shared memory of the kernels above, on the current device.
 bool pair_sort_setup() {
     return cudaFuncSetAttribute(k_coh_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CohShared)) ==
@@ -881,10 +932,8 @@ bool pair_sort_setup() {
                cudaSuccess &&
            cudaFuncSetAttribute(k_merge_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CohShared)) ==
                cudaSuccess &&
-           cudaFuncSetAttribute(k_sort_small<kCohBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sizeof(PairShared<8 * kCohBlock>)) == cudaSuccess &&
-           cudaFuncSetAttribute(k_sort_small<kSmallBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sizeof(PairShared<8 * kSmallBlock>)) == cudaSuccess;
+           cudaFuncSetAttribute(k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CohShared)) ==
+               cudaSuccess;
 }
 
 // Tile shape of the single-pass kernel and the look-back window: each
@@ -1151,7 +1200,7 @@ int keys_and_sort(fdps_tree* t, fdps_psys* ps) {
     const bool layout = ps->n_sys == 1 || ps->d_cbs;
     const int64_t nbl = ps->n_sys == 1 ? (n + kCohT - 1) / kCohT : ps->coh_nb;
     // one system of at most kSmallMax particles: box, keys and sort in one
-    // launch (a time step of 2001 particles: 332 -> 269 us)
+    // launch (Plummer 2^14: box, keys and sort 58 -> 43 us)
     const bool small = ps->n_sys == 1 && n <= kSmallMax;
     bool coherent = !small && layout && t->coh_ok && t->coh_ps == ps && t->coh_gen == ps->gen && t->coh_n == n &&
                     n >= 2 * (int64_t)kCohT;
@@ -1177,7 +1226,8 @@ int keys_and_sort(fdps_tree* t, fdps_psys* ps) {
     t->coh_n = n;
     t->sort_coherent = coherent;
     if (small) {
-        if (launch_sort_small(n, ps->x[c], ps->y[c], ps->z[c], t->st, t->sys_box, t->keys_in, t->keys_b, t->vals_b, s))
+        if (launch_sort_small(n, ps->x[c], ps->y[c], ps->z[c], t->st, t->sys_box, t->keys_in, t->keys_b, t->vals_b,
+                              t->keys_a, t->vals_a, s))
             return set_error(ctx, FDPS_ECUDA, "sort launch failed");
         FDPS_LAUNCH_CHECK(ctx);
         if (t->ev_ok && ctx->profiling && !ctx->capturing) cudaEventRecord(t->ev[1], s);
@@ -1388,7 +1438,7 @@ extern "C" int fdps_morton_sort_noalloc(const double* x, const double* y, const 
     uint32_t* vals_a = reinterpret_cast<uint32_t*>(base + kOffValsA);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (n <= kSmallMax) {
-        if (launch_sort_small(n, x, y, z, nullptr, nullptr, nullptr, keys_sorted, perm, s)) {
+        if (launch_sort_small(n, x, y, z, nullptr, nullptr, nullptr, keys_sorted, perm, keys_a, vals_a, s)) {
             cudaGetLastError();
             return FDPS_ECUDA;
         }
@@ -1409,7 +1459,7 @@ extern "C" int fdps_morton_sort_noalloc(const double* x, const double* y, const 
     int at = rounds & 1;
     k_tile_sort<<<ntiles, kCohBlock, sizeof(CohShared), s>>>(n, x, y, z, sbox, kb[at], vb[at]);
     for (int64_t L = kSortTile; L < n; L *= 2) {
-        k_merge_runs<<<ntiles, kCohBlock, sizeof(CohShared), s>>>(n, (int)L, kb[at], vb[at], kb[at ^ 1], vb[at ^ 1]);
+        k_merge_runs<<<ntiles, kCohBlock, sizeof(CohShared), s>>>(n, L, kb[at], vb[at], kb[at ^ 1], vb[at ^ 1]);
         at ^= 1;
     }
     if (cudaGetLastError() != cudaSuccess) return FDPS_ECUDA;

@@ -1,4 +1,4 @@
-"""The one-CTA sort of small sets and the tile-and-merge sort of the
+"""The one-cluster sort of small sets and the tile-and-merge sort of the
 allocation-free entry point, at the edges of a thread's, a tile's and a
 CTA's share, with many equal keys (ties keep the input order): keys and
 permutation bit for bit against the oracle's."""
@@ -28,7 +28,7 @@ def _set(n, ties):
 
 
 @pytest.mark.parametrize("ties", [False, True])
-@pytest.mark.parametrize("n", [1, 2, 255, 257, 2047, 2048, 2049, 4099, 8191, 8192, 8193, 10240, 12289, 65537, 262144])
+@pytest.mark.parametrize("n", [1, 2, 255, 257, 7, 9, 2041, 2048, 2049, 4099, 8192, 16383, 16384, 16385, 20481, 65537, 262144])
 def test_noalloc_sort(G, n, ties):
     torch = pytest.importorskip("torch")
     pos, mass, eps = _set(n, ties)
@@ -46,7 +46,7 @@ def test_noalloc_sort(G, n, ties):
         np.testing.assert_array_equal(keys.cpu().numpy().view(np.uint64), np.asarray(keys_ref)[np.asarray(perm_ref)])
 
 
-@pytest.mark.parametrize("n", [1, 3, 256, 2048, 2049, 8192, 8193])
+@pytest.mark.parametrize("n", [1, 3, 8, 9, 256, 2048, 2049, 16384, 16385])
 def test_pipeline_sort_over_steps(G, n):
     pos, mass, eps = _set(n, n % 2 == 0)
     vel = np.random.default_rng(n + 1).normal(size=(n, 3))
