@@ -65,8 +65,8 @@ struct __align__(16) Spj {
 
 namespace detail {
 
-constexpr int kThreads = 64;  // threads of a block, and list entries per step
-constexpr int kSlots = 4;     // blocks sharing a group's i-particles (grid y)
+constexpr int kThreads = 32;  // threads of a block, and list entries per step
+constexpr int kSlots = 8;     // blocks sharing a group's i-particles (grid y)
 constexpr int kSpjCall = 32;  // most superparticles per functor call
 constexpr int kEpjCall = 64;  // most leaf particles per functor call
 
@@ -78,14 +78,16 @@ __device__ __forceinline__ float4 ld4(const float* p, uint64_t i) {
 // kThreads: block (x, y) takes groups x, x + gridDim.x, ... and of each the
 // i-particles kThreads y .. + kThreads - 1 (and on by kThreads gridDim.y),
 // one per thread.  The block stages kThreads list entries at a time for all
-// its warps.  The law's own instructions bound it, so what counts is that
-// every SM has warps with i-particles until the end: one block per group and
-// 64 i-particles, started by the hardware as others finish, where a fixed
-// share of the groups for each warp of one resident wave, eight passes over
-// the list for a group of 256, left most of the SMs idle behind the warps
-// with the large groups (2^20 Hernquist particles, n_grp 256, gravity with
-// quadrupoles: 13.6 -> 10.1 ms for lists and law, 8.4 -> 8.1 ms a
-// call where the next call's lists overlap the law).
+// its warps.  The law's own instructions bound it (issue slots 74 % busy), so
+// what counts is that every SM has warps with i-particles until the end: one
+// block per group and 32 i-particles, started by the hardware as others
+// finish, where a fixed share of the groups for each warp of one resident
+// wave, eight passes over the list for a group of 256, left most of the SMs
+// idle behind the warps with the large groups.  One warp a block: with two or
+// four, groups of 30 particles leave warps that only wait at the barriers.
+// Gravity with quadrupoles, lists and law: 2^20 Hernquist particles, n_grp 256,
+// 13.9 ms before, 7.8 with 32 threads, 8.2 with 64, 8.0 with 128; 500,000 Plummer
+// particles with monopoles, n_grp 64: 5.6, 4.6, 6.5 and 5.0 ms.
 template <class Force, class FEpj, class FSpj>
 __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const FEpj& f_epj,
                                                 const FSpj& f_spj, Force* out) {
