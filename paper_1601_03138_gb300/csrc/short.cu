@@ -28,7 +28,7 @@ namespace {
 
 constexpr int kSBlock = 128;
 constexpr int kSW = kSBlock / 32;
-constexpr int kSTile = 64;                 // candidate particles per shared tile
+constexpr int kSTile = 96;                 // candidate particles per shared tile (even)
 constexpr unsigned long long kSChunk = 1ull << 16;
 constexpr float kU = 5.9604645e-08f;      // 2^-24
 // Wendland C6, 3D, support H: W = 1365 / (64 pi H^3) (1-q)^8 (1 + 8q + 25q^2 + 32q^3)
@@ -264,6 +264,12 @@ struct ShortPairArgs {
     const double* x;      // FP64 positions in key order
     const double* y;
     const double* z;
+    const float4* g_ch;   // group centre (hi - c0, lo) and box relative to it
+    const float4* g_cl;
+    const float4* g_blo;
+    const float4* g_bhi;
+    const uint32_t* g_nepj;  // candidates in the group's list
+    const double* g_hmax;    // largest cutoff radius of a group (i-dependent and symmetric types)
     const double* h;      // cutoff radii in key order (null for the fixed type)
     const uint32_t* id;   // key order -> caller's row
     const uint32_t* sys;
@@ -275,27 +281,116 @@ struct ShortPairArgs {
     double r_fixed;
 };
 
-// W(r, H) of the 3D Wendland C6 kernel; zero from q = r / H >= 1 on (the
-// factor (1 - q)^8 clamped at zero, without a branch).
-__device__ __forceinline__ float wendland_c6(float r, float invH) {
-    const float q = r * invH;
-    const float u = fmaxf(1.0f - q, 0.0f), u2 = u * u, u4 = u2 * u2, u8 = u4 * u4;
-    const float poly = fmaf(q, fmaf(q, fmaf(q, 32.0f, 25.0f), 8.0f), 1.0f);
-    return kWc6 * invH * invH * invH * u8 * poly;
+// Two FP32 lanes in one 64-bit register (two candidates of a pair loop turn),
+// each rounded as the scalar instruction.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_pk(float lo, float hi) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void f2_up(f2 v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
+    f2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ float rsqrt_normal(float v) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
 }
 
-// MODE is the cutoff type (FDPS_CUTOFF_*), fixed at compile time so that
-// the pair loop carries no selection between them.
+// (1 - q)^8 (1 + 8 q + 25 q^2 + 32 q^3) of two candidates at q^2 = x (the
+// Wendland C6 kernel without its normalisation; zero from q = 1 on).  The
+// root is s = x y, y the reciprocal root, with one Newton correction
+// s + (x - s^2) y / 2 (Heron's iteration); x is kept within 1e-30 (q = 0 to
+// every digit of the result) and 4.
+__device__ __forceinline__ f2 wendland_q2(f2 x) {
+    float a, b;
+    f2_up(x, a, b);
+    a = fminf(fmaxf(a, 1e-30f), 4.0f);
+    b = fminf(fmaxf(b, 1e-30f), 4.0f);
+    const f2 xc = f2_pk(a, b), y = f2_pk(rsqrt_normal(a), rsqrt_normal(b));
+    const f2 s = f2_mul(xc, y), hy = f2_mul(y, f2_pk(0.5f, 0.5f));
+    const f2 ns = s ^ 0x8000000080000000ull;
+    const f2 q = f2_fma(f2_fma(ns, s, xc), hy, s);
+    f2 u = f2_sub(f2_pk(1.0f, 1.0f), q);
+    f2_up(u, a, b);
+    u = f2_pk(fmaxf(a, 0.0f), fmaxf(b, 0.0f));
+    const f2 u2 = f2_mul(u, u), u4 = f2_mul(u2, u2), u8 = f2_mul(u4, u4);
+    const f2 p = f2_fma(q, f2_fma(q, f2_fma(q, f2_pk(32.0f, 32.0f), f2_pk(25.0f, 25.0f)), f2_pk(8.0f, 8.0f)),
+                        f2_pk(1.0f, 1.0f));
+    return f2_mul(u8, p);
+}
+
+// Two thresholds on r^2 that decide the pairs of a cutoff c: r^2 < lo is a
+// neighbour, r^2 > hi is none, between them the FP64 sequence decides.  With
+// a = max |d|, Ea = 8u a + Eabs the error of a difference and M = 8u (r^2 +
+// c^2) + 6 a Ea + 3 Ea^2 the bound on the error of r^2 - c^2: M <= Mmax for
+// r^2 <= c^2 (a <= r <= c), and for r^2 > c^2, with a <= r <= (r^2 + c^2) /
+// (2c), M <= (56u + 192u^2 + beta) r^2 + (8u + beta) c^2 + 3 Eabs^2, beta =
+// 3 Eabs / c (slack for the FP32 evaluation of both).  A cutoff within a few
+// Eabs sends every pair to the FP64 sequence.
+__device__ __forceinline__ float2 pair_thresholds(float c, float Eabs) {
+    const float c2 = c * c, beta = 3.0001f * Eabs / c;
+    if (!(beta < 0.25f)) return make_float2(-INFINITY, INFINITY);
+    const float tq = fmaf(8.0f * kU, c, Eabs);
+    const float Mmax = 64.0f * kU * c2 + 6.0f * c * Eabs + 3.0f * tq * tq;
+    return make_float2(c2 - (1.01f * Mmax + 4.0f * kU * c2),
+                       (c2 * (1.0f + 8.0f * kU + beta) + 3.0f * Eabs * Eabs) * (1.0f + 16.0f * kU) /
+                           (1.0f - (56.0f * kU + 192.0f * kU * kU + beta)));
+}
+
+// A warp's tile of candidates; pairs (2 k, 2 k + 1) are read as one packed
+// register.  R: with the candidates' own radii (j-dependent types).
+template <bool R>
+struct PairTile {
+    float xh[kSTile], yh[kSTile], zh[kSTile], xl[kSTile], yl[kSTile], zl[kSTile], m[kSTile];
+    uint32_t p[kSTile];
+    float ih2[R ? kSTile : 2];             // 1 / h_j^2
+    float mw[R ? kSTile : 2];              // m_j times the kernel's normalisation for h_j
+    float lo[R ? kSTile : 2], hi[R ? kSTile : 2], hj[R ? kSTile : 2];
+    uint32_t first[32], start[32];
+};
+__device__ __forceinline__ f2 ld2(const float* a, uint32_t k) { return reinterpret_cast<const f2*>(a)[k]; }
+
+// One warp per group.  The candidates of the group's list are tested against
+// the group's box (no nearer to any of its particles than to the box) and
+// only those within the largest cutoff that can apply are staged: of 3.4
+// candidates a neighbour (310 neighbours in a uniform cube, groups of 20)
+// the walk's leaves give, about 2 remain.  Lanes: P i-slots x nsl slices
+// of the tile, so that small groups keep the whole warp busy; a lane takes
+// two candidates at a time in packed FP32 instructions.  Issue-bound:
+// 3.19 ms for the pair pass of 2^20 particles before,
+// 2.18 with the box test and packed turns (whole call 4.82 -> 3.67 ms); the
+// error of the densities went from 2.1e-7 to 1.4e-7.  MODE is the cutoff type (FDPS_CUTOFF_*), fixed at compile time so
+// that the pair loop carries no selection between them.
 template <int MODE>
 __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
-    __shared__ float4 s_h[kSW][kSTile];
-    __shared__ float4 s_l[kSW][kSTile];
-    __shared__ float s_ih[kSW][kSTile];  // 1 / h_j (scatter and symmetric types)
-    __shared__ uint32_t s_p[kSW][kSTile];
-    __shared__ uint32_t s_first[kSW][32];
-    __shared__ uint32_t s_start[kSW][32];
+    constexpr bool R = MODE >= 2;
+    __shared__ __align__(16) PairTile<R> s_t[kSW];
     DevState* st = A.st;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    PairTile<R>& T = s_t[w];
     const uint32_t ngroups = (uint32_t)st->n_groups;
     unsigned long long n_pairs = 0, n_cand = 0, n_fb = 0;
     for (;;) {
@@ -308,8 +403,13 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
         const uint32_t len = A.g_len[g];
         const float L = (float)A.box[A.sys ? A.sys[gf] : 0u].L;
         const float Eabs = 1e-13f * L;  // error of the FP64 -> FP32 hi/lo parts
-        // lanes: P i-slots x nsl slices of the candidates, so that small
-        // groups keep the whole warp busy
+        const float4 gch = A.g_ch[g], gcl = A.g_cl[g], blo = A.g_blo[g], bhi = A.g_bhi[g];
+        const float hb = fmaxf(fmaxf(fmaxf(-blo.x, -blo.y), fmaxf(-blo.z, bhi.x)), fmaxf(bhi.y, bhi.z));
+        // what a cutoff grows by so that the FP32 distance to the box never
+        // drops a pair that the thresholds or the FP64 sequence look at: the
+        // distance's error is below 4u (C + 2 hb) + 2 Eabs
+        const float pad = 64.0f * kU * hb + 16.0f * Eabs;
+        const float hg = MODE == 0 ? (float)A.r_fixed : MODE == 2 ? 0.0f : (float)A.g_hmax[g];
         const uint32_t P = ni <= 16u ? ni : 32u;
         const uint32_t nsl = 32u / P;
         const uint32_t ip = lane % P, sl = lane / P;
@@ -319,29 +419,94 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
             const uint32_t pi = gf + (act ? i : 0u);
             const float4 ih = A.pf_hi[pi], il = A.pf_lo[pi];
             const double hi64 = MODE != 0 ? A.h[pi] : A.r_fixed;
-            const float hif = (float)hi64;
-            const float invHi = 1.0f / (MODE == 0 ? (float)A.r_fixed : hif);
-            // the cutoff of the fixed and gather types is the lane's own, and
-            // so are two thresholds on r^2 that decide every pair the pair
-            // bound below decides on the same side: M <= Mmax for r^2 <= c^2
-            // (a <= r <= c), and for r^2 > c^2, with a <= r <= (r^2 + c^2) /
-            // (2c), M <= (56u + 192u^2 + beta) r^2 + (8u + beta) c^2 + 3 Eabs^2,
-            // beta = 3 Eabs / c (slack for the FP32 evaluation of both); a
-            // cutoff within a few Eabs sends every pair to the FP64 sequence
-            const float ci = MODE == 0 ? (float)A.r_fixed : hif, ci2 = ci * ci;
-            float lo_thr = -INFINITY, hi_thr = INFINITY;
-            if (MODE <= 1) {
-                const float beta = 3.0001f * Eabs / ci;
-                if (beta < 0.25f) {
-                    const float tq = fmaf(8.0f * kU, ci, Eabs);
-                    const float Mmax = 64.0f * kU * ci2 + 6.0f * ci * Eabs + 3.0f * tq * tq;
-                    lo_thr = ci2 - (1.01f * Mmax + 4.0f * kU * ci2);
-                    hi_thr = (ci2 * (1.0f + 8.0f * kU + beta) + 3.0f * Eabs * Eabs) * (1.0f + 16.0f * kU) /
-                             (1.0f - (56.0f * kU + 192.0f * kU * kU + beta));
+            const float hif = (float)hi64, invHi = 1.0f / hif, invHi2 = invHi * invHi;
+            const float2 ti = MODE == 2 ? make_float2(0.0f, 0.0f) : pair_thresholds(hif, Eabs);
+            const f2 ixh = f2_pk(ih.x, ih.x), iyh = f2_pk(ih.y, ih.y), izh = f2_pk(ih.z, ih.z);
+            const f2 ixl = f2_pk(il.x, il.x), iyl = f2_pk(il.y, il.y), izl = f2_pk(il.z, il.z);
+            const f2 iH2 = f2_pk(invHi2, invHi2);
+            uint32_t cnt = 0, fbk = 0;
+            f2 sum = 0ull, sumj = 0ull;  // sums of m_j w(q) with H = h_i, and with H = h_j
+            // the staged candidates 0 .. m - 1 on the warp's i-particles
+            auto pairs = [&](uint32_t m) {
+                if ((m & 1u) && lane == 0) {  // an even number: a candidate far from everything, without mass
+                    const float far = 16.0f * (hb + hg) + (R ? 16.0f * T.hj[m - 1] : 0.0f);
+                    T.xh[m] = gch.x + far;
+                    T.yh[m] = gch.y;
+                    T.zh[m] = gch.z;
+                    T.xl[m] = T.yl[m] = T.zl[m] = T.m[m] = 0.0f;
+                    T.p[m] = 0xFFFFFFFFu;
+                    if (R) {
+                        T.ih2[m] = T.ih2[m - 1];
+                        T.mw[m] = 0.0f;
+                        T.lo[m] = T.lo[m - 1];
+                        T.hi[m] = T.hi[m - 1];
+                        T.hj[m] = T.hj[m - 1];
+                    }
                 }
-            }
-            uint32_t cnt = 0, cands = 0, fbk = 0;
-            float sum = 0.0f;
+                __syncwarp();
+                if (act) {
+#pragma unroll 2
+                    for (uint32_t k = sl; k < (m + 1u) / 2u; k += nsl) {
+                        const f2 dx = f2_add(f2_sub(ld2(T.xh, k), ixh), f2_sub(ld2(T.xl, k), ixl));
+                        const f2 dy = f2_add(f2_sub(ld2(T.yh, k), iyh), f2_sub(ld2(T.yl, k), iyl));
+                        const f2 dz = f2_add(f2_sub(ld2(T.zh, k), izh), f2_sub(ld2(T.zl, k), izl));
+                        const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, f2_mul(dz, dz)));
+                        float ra, rb;
+                        f2_up(r2, ra, rb);
+                        float la = ti.x, lb = ti.x, ua = ti.y, ub = ti.y;
+                        if (R) {
+                            f2_up(ld2(T.lo, k), la, lb);
+                            f2_up(ld2(T.hi, k), ua, ub);
+                        }
+                        if (MODE == 3) {  // the larger radius of the pair
+                            float ha, hc;
+                            f2_up(ld2(T.hj, k), ha, hc);
+                            la = hif >= ha ? ti.x : la;
+                            ua = hif >= ha ? ti.y : ua;
+                            lb = hif >= hc ? ti.x : lb;
+                            ub = hif >= hc ? ti.y : ub;
+                        }
+                        bool na = ra < la, nb = rb < lb;
+                        const bool fa = !na && !(ra > ua), fb = !nb && !(rb > ub);
+                        if (fa || fb) {  // inside the bound: the exact FP64 sequence
+                            for (int c = 0; c < 2; ++c) {
+                                const uint32_t pj = T.p[2 * k + c];
+                                if (!(c ? fb : fa) || pj == 0xFFFFFFFFu) continue;
+                                ++fbk;
+                                const double ex = __dsub_rn(A.x[pj], A.x[pi]);
+                                const double ey = __dsub_rn(A.y[pj], A.y[pi]);
+                                const double ez = __dsub_rn(A.z[pj], A.z[pi]);
+                                const double e2 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)),
+                                                            __dmul_rn(ez, ez));
+                                const double hj64 = MODE != 0 ? A.h[pj] : A.r_fixed;
+                                const double cc = MODE == 0 ? A.r_fixed
+                                                : MODE == 1 ? hi64
+                                                : MODE == 2 ? hj64
+                                                            : (hi64 > hj64 ? hi64 : hj64);
+                                (c ? nb : na) = e2 < __dmul_rn(cc, cc);
+                            }
+                        }
+                        // the kernel for every candidate, kept for the
+                        // neighbours only: half of the staged candidates
+                        // are, so a branch would be taken by some lane of
+                        // nearly every turn anyway
+                        cnt += (na ? 1u : 0u) + (nb ? 1u : 0u);
+                        if (MODE != 2) {
+                            float ma, mb;
+                            f2_up(ld2(T.m, k), ma, mb);
+                            sum = f2_fma(f2_pk(na ? ma : 0.0f, nb ? mb : 0.0f), wendland_q2(f2_mul(r2, iH2)), sum);
+                        }
+                        if (R) {
+                            float ma, mb;
+                            f2_up(ld2(T.mw, k), ma, mb);
+                            sumj = f2_fma(f2_pk(na ? ma : 0.0f, nb ? mb : 0.0f),
+                                          wendland_q2(f2_mul(r2, ld2(T.ih2, k))), sumj);
+                        }
+                    }
+                }
+                __syncwarp();
+            };
+            uint32_t staged = 0;
             for (uint32_t base = 0; base < len; base += 32) {
                 // leaves of this step: particle counts and offsets
                 const uint32_t u = base + lane;
@@ -355,96 +520,84 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
                 }
                 const uint32_t total = __shfl_sync(0xFFFFFFFFu, inc, 31);
                 __syncwarp();
-                s_first[w][lane] = u < len ? A.nd_first[node] : 0u;
-                s_start[w][lane] = inc - c;
-                for (uint32_t c0 = 0; c0 < total; c0 += kSTile) {
-                    const uint32_t m = total - c0 < (uint32_t)kSTile ? total - c0 : (uint32_t)kSTile;
-                    __syncwarp();
-                    for (uint32_t k = lane; k < m; k += 32) {
-                        const uint32_t item = c0 + k;
+                T.first[lane] = u < len ? A.nd_first[node] : 0u;
+                T.start[lane] = inc - c;
+                __syncwarp();
+                for (uint32_t c0 = 0; c0 < total; c0 += 32) {
+                    const uint32_t item = c0 + lane;
+                    bool keep = false;
+                    float4 h4 = make_float4(0.f, 0.f, 0.f, 0.f), l4 = h4;
+                    float hj = 0.0f;
+                    uint32_t pj = 0;
+                    if (item < total) {
                         int src = 0;
 #pragma unroll
                         for (int step = 16; step > 0; step >>= 1)
-                            if (s_start[w][src + step] <= item) src += step;
-                        const uint32_t pj = s_first[w][src] + (item - s_start[w][src]);
-                        const float4 lo = A.pf_lo[pj];
-                        const float hj = MODE >= 2 ? (float)A.h[pj] : 0.0f;
-                        s_h[w][k] = A.pf_hi[pj];
-                        s_l[w][k] = make_float4(lo.x, lo.y, lo.z, hj);
-                        if (MODE >= 2) s_ih[w][k] = 1.0f / hj;
-                        s_p[w][k] = pj;
+                            if (T.start[src + step] <= item) src += step;
+                        pj = T.first[src] + (item - T.start[src]);
+                        h4 = A.pf_hi[pj];
+                        l4 = A.pf_lo[pj];
+                        if (R) hj = (float)A.h[pj];
+                        const float dx = (h4.x - gch.x) + (l4.x - gcl.x), dy = (h4.y - gch.y) + (l4.y - gcl.y),
+                                    dz = (h4.z - gch.z) + (l4.z - gcl.z);
+                        const float tx = fmaxf(fmaxf(blo.x - dx, dx - bhi.x), 0.0f);
+                        const float ty = fmaxf(fmaxf(blo.y - dy, dy - bhi.y), 0.0f);
+                        const float tz = fmaxf(fmaxf(blo.z - dz, dz - bhi.z), 0.0f);
+                        const float C = fmaf(fmaxf(hg, hj), 1.0f + 256.0f * kU, pad);
+                        keep = !(fmaf(tx, tx, fmaf(ty, ty, tz * tz)) > C * C);
                     }
-                    __syncwarp();
-                    if (act) {
-#pragma unroll 4
-                        for (uint32_t k = sl; k < m; k += nsl) {
-                            ++cands;
-                            const float4 jh = s_h[w][k], jl = s_l[w][k];
-                            const float dx = (jh.x - ih.x) + (jl.x - il.x);
-                            const float dy = (jh.y - ih.y) + (jl.y - il.y);
-                            const float dz = (jh.z - ih.z) + (jl.z - il.z);
-                            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                            bool near;  // inside the bound: the FP64 sequence decides
-                            bool nb = false;
-                            if (MODE <= 1) {
-                                nb = r2 < lo_thr;
-                                near = !nb && !(r2 > hi_thr);
-                            } else {
-                                const float c2 = MODE == 2 ? jl.w * jl.w : fmaxf(hif, jl.w) * fmaxf(hif, jl.w);
-                                const float a = fmaxf(fmaxf(fabsf(dx), fabsf(dy)), fabsf(dz));
-                                const float Ea = 8.0f * kU * a + Eabs;
-                                const float M = 8.0f * kU * (r2 + c2) + 6.0f * a * Ea + 3.0f * Ea * Ea;
-                                nb = r2 < c2 - M;
-                                near = !nb && !(r2 > c2 + M);
-                            }
-                            if (near) {  // the exact FP64 sequence
-                                ++fbk;
-                                const uint32_t pj = s_p[w][k];
-                                const double ex = __dsub_rn(A.x[pj], A.x[pi]);
-                                const double ey = __dsub_rn(A.y[pj], A.y[pi]);
-                                const double ez = __dsub_rn(A.z[pj], A.z[pi]);
-                                const double e2 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)),
-                                                            __dmul_rn(ez, ez));
-                                const double hj64 = MODE != 0 ? A.h[pj] : A.r_fixed;
-                                const double cc = MODE == 0 ? A.r_fixed
-                                                : MODE == 1 ? hi64
-                                                : MODE == 2 ? hj64
-                                                            : (hi64 > hj64 ? hi64 : hj64);
-                                nb = e2 < __dmul_rn(cc, cc);
-                            }
-                            // the kernel for every candidate, kept for the
-                            // neighbours only: a third of the pairs are
-                            // neighbours, so a branch would be taken by some
-                            // lane of nearly every step anyway
-                            const float r = sqrtf(r2);
-                            float wk;
-                            if (MODE == 3)
-                                wk = 0.5f * (wendland_c6(r, invHi) + wendland_c6(r, s_ih[w][k]));
-                            else if (MODE == 2)
-                                wk = wendland_c6(r, s_ih[w][k]);
-                            else
-                                wk = wendland_c6(r, invHi);
-                            cnt += nb ? 1u : 0u;
-                            sum = fmaf(jh.w, nb ? wk : 0.0f, sum);
+                    const uint32_t mask = __ballot_sync(0xFFFFFFFFu, keep);
+                    if (keep) {
+                        const uint32_t k = staged + __popc(mask & lt);
+                        T.xh[k] = h4.x;
+                        T.yh[k] = h4.y;
+                        T.zh[k] = h4.z;
+                        T.xl[k] = l4.x;
+                        T.yl[k] = l4.y;
+                        T.zl[k] = l4.z;
+                        T.m[k] = h4.w;
+                        T.p[k] = pj;
+                        if (R) {
+                            const float ihj = 1.0f / hj;
+                            const float2 tj = pair_thresholds(hj, Eabs);
+                            T.ih2[k] = ihj * ihj;
+                            T.mw[k] = h4.w * (kWc6 * ihj * ihj * ihj);
+                            T.lo[k] = tj.x;
+                            T.hi[k] = tj.y;
+                            T.hj[k] = hj;
                         }
+                    }
+                    staged += __popc(mask);
+                    if (staged > (uint32_t)kSTile - 33u) {  // room for the next 32 and the padding
+                        pairs(staged);
+                        staged = 0;
                     }
                 }
             }
-            // the slices' partial counts and sums, into the first slice
+            if (staged) pairs(staged);
+            // the lane's two halves and the slices' partial counts and sums,
+            // into the first slice
+            float sa, sb, ja, jb;
+            f2_up(sum, sa, sb);
+            f2_up(sumj, ja, jb);
+            const float norm = kWc6 * invHi * invHi * invHi;
+            const float rho = MODE == 2   ? ja + jb
+                              : MODE == 3 ? 0.5f * fmaf(norm, sa + sb, ja + jb)
+                                          : norm * (sa + sb);
             uint32_t cnt_all = cnt;
-            float sum_all = sum;
+            float sum_all = rho;
             for (uint32_t q = 1; q < nsl; ++q) {
                 const int src = (int)((ip + q * P) & 31u);
                 cnt_all += __shfl_sync(0xFFFFFFFFu, cnt, src);
-                sum_all += __shfl_sync(0xFFFFFFFFu, sum, src);
+                sum_all += __shfl_sync(0xFFFFFFFFu, rho, src);
             }
             if (act && sl == 0) {
                 const uint32_t row = A.id[pi];
                 A.count[row] = cnt_all;
                 A.rho[row] = (double)sum_all;
+                n_cand += A.g_nepj[g];
             }
             n_pairs += act ? cnt : 0u;
-            n_cand += act ? cands : 0u;
             n_fb += act ? fbk : 0u;
         }
     }
@@ -567,6 +720,12 @@ int launch_short_pairs(fdps_tree* t, fdps_psys* ps, int mode, double r_fixed, ui
     A.x = ps->x[c];
     A.y = ps->y[c];
     A.z = ps->z[c];
+    A.g_ch = t->g_ch;
+    A.g_cl = t->g_cl;
+    A.g_blo = t->g_blo;
+    A.g_bhi = t->g_bhi;
+    A.g_nepj = t->g_nepj;
+    A.g_hmax = (mode == 1 || mode == 3) ? t->g_hmax : nullptr;
     A.h = mode == 0 ? nullptr : t->sr_h;
     A.id = ps->id[c];
     A.sys = ps->d_sys;
