@@ -1,4 +1,5 @@
-// walk.cu -- interaction lists: one warp walks the tree for one i-group.
+// walk.cu -- interaction lists: one warp walks the tree for one i-group (one
+// block in systems of few groups).
 //
 // The Barnes-Hut traversal with a fixed opening angle (Sect. 3.2), done
 // once per i-group as in the modified tree algorithm of Barnes (1990) that
@@ -106,29 +107,44 @@ __device__ __forceinline__ WalkState walk_state_init() {
 }
 
 
-// The list of group g, walked by the calling warp (all 32 lanes), with its
-// two frontier buffers fa and fb and the warp's per-level thresholds thr.
-__device__ __forceinline__ void walk_group(const WalkArgs& A, uint32_t g, uint32_t* fa, uint32_t* fb,
-                                           float2* thr, WalkState& S) {
-    DevState* st = A.st;
-    const int lane = threadIdx.x & 31;
-    const uint32_t lt = (1u << lane) - 1u;
-    const uint32_t F = A.cap_frontier;
-    // the group's system: its root node (node id = system index) and box
-    const uint32_t sysid = A.sys ? A.sys[A.g_first[g]] : 0u;
-    const double L = A.box[sysid].L;
-    const float Lf = __double2float_rn(L);
+// What the opening tests of one group read: its grid box, its centre and box
+// in FP32 relative to it, its FP64 box, its system's root box size.
+struct GroupGeom {
+    uint32_t sysid;  // the group's system: its root node (node id = system index) and box
+    double L;
+    const double* box64;
+    uint32_t qmin0, qmin1, qmin2, qmax0, qmax1, qmax2;
+    float4 gch, gcl, blo, bhi;
+};
+
+__device__ __forceinline__ GroupGeom group_geom(const WalkArgs& A, uint32_t g) {
+    GroupGeom G;
+    G.sysid = A.sys ? A.sys[A.g_first[g]] : 0u;
+    G.L = A.box[G.sysid].L;
+    G.box64 = A.g_box + 6 * (int64_t)g;
+    const uint32_t* qb = A.g_qbox + 6 * (int64_t)g;
+    G.qmin0 = qb[0];
+    G.qmin1 = qb[1];
+    G.qmin2 = qb[2];
+    G.qmax0 = qb[3];
+    G.qmax1 = qb[4];
+    G.qmax2 = qb[5];
+    G.gch = A.g_ch[g];
+    G.gcl = A.g_cl[g];
+    G.blo = A.g_blo[g];
+    G.bhi = A.g_bhi[g];
+    return G;
+}
+
+// The two thresholds on d^2 of the FP32 filter for cells of `level`: below
+// the first the cell opens, above the second it does not.
+__device__ __forceinline__ float2 level_thresholds(const WalkArgs& A, const GroupGeom& G, int level) {
+    const float Lf = __double2float_rn(G.L);
     // the FP32 filter's bound holds while the squares of cell sizes stay
     // normal FP32 numbers (with or without flushing of subnormals): outside
     // this range of root boxes every test takes the exact FP64 sequence
     const bool filt = Lf >= 0x1p-40f && Lf <= 0x1p60f;
-    const uint32_t* qb = A.g_qbox + 6 * (int64_t)g;
-    const uint32_t qmin0 = qb[0], qmin1 = qb[1], qmin2 = qb[2];
-    const uint32_t qmax0 = qb[3], qmax1 = qb[4], qmax2 = qb[5];
-    const float4 gch = A.g_ch[g], gcl = A.g_cl[g];
-    const float4 blo = A.g_blo[g], bhi = A.g_bhi[g];
-    const float hb = fmaxf(fmaxf(fmaxf(-blo.x, -blo.y), fmaxf(-blo.z, bhi.x)), fmaxf(bhi.y, bhi.z));
-    const double* box64 = A.g_box + 6 * (int64_t)g;
+    const float hb = fmaxf(fmaxf(fmaxf(-G.blo.x, -G.blo.y), fmaxf(-G.blo.z, G.bhi.x)), fmaxf(G.bhi.y, G.bhi.z));
     // Coefficients of the filter's error bound as a polynomial in M = max|d| +
     // hb (d the FP32 offset of a cell's centre of mass, hb the largest
     // |corner| of the group box): with E = 4uM + e0 the error of one
@@ -146,32 +162,65 @@ __device__ __forceinline__ void walk_group(const WalkArgs& A, uint32_t g, uint32
     // the margin is linear in d^2 and d^2 above hi rejects it.  Slack covers
     // the thresholds' own FP32 evaluation; outside the filter's range of L
     // (and at theta = 0, where every cell opens) no threshold decides.
-    __syncwarp();  // the previous group's walk has read thr
-    if (lane <= kMaxLevel) {
-        float lo = -INFINITY, hi = INFINITY;
-        if (!filt) {
-        } else if (A.theta2f == 0.0f) {
-            lo = INFINITY;
-        } else {
-            const float ell = __int_as_float(__float_as_int(Lf) - (lane << 23));
-            const float l2 = ell * ell;
-            const float D0 = sqrtf(l2 / A.theta2f);
-            const float Mb = D0 + 2.0f * hb;
-            const float Mo = fmaf(16.0f * kU32, l2, fmaf(fmaf(mc1, Mb, mc2), Mb, mc3));
-            lo = (l2 - Mo) / A.theta2f * (1.0f - 8.0f * kU32);
-            const float coef = A.theta2f - (8.0f * kU32 * A.theta2f + 2.0f * mc1 + mc2 / (2.0f * D0));
-            const float rhs = l2 * (1.0f + 8.0f * kU32) + 8.0f * mc1 * hb * hb + mc2 * (0.5f * D0 + 2.0f * hb) + mc3;
-            if (coef > 0.0f) hi = rhs * (1.0f + 16.0f * kU32) / coef;
-        }
-        thr[lane] = make_float2(lo, hi);
+    float lo = -INFINITY, hi = INFINITY;
+    if (!filt) {
+    } else if (A.theta2f == 0.0f) {
+        lo = INFINITY;
+    } else {
+        const float ell = __int_as_float(__float_as_int(Lf) - (level << 23));
+        const float l2 = ell * ell;
+        const float D0 = sqrtf(l2 / A.theta2f);
+        const float Mb = D0 + 2.0f * hb;
+        const float Mo = fmaf(16.0f * kU32, l2, fmaf(fmaf(mc1, Mb, mc2), Mb, mc3));
+        lo = (l2 - Mo) / A.theta2f * (1.0f - 8.0f * kU32);
+        const float coef = A.theta2f - (8.0f * kU32 * A.theta2f + 2.0f * mc1 + mc2 / (2.0f * D0));
+        const float rhs = l2 * (1.0f + 8.0f * kU32) + 8.0f * mc1 * hb * hb + mc2 * (0.5f * D0 + 2.0f * hb) + mc3;
+        if (coef > 0.0f) hi = rhs * (1.0f + 16.0f * kU32) / coef;
     }
+    return make_float2(lo, hi);
+}
+
+// The opening test of one cell (its walk record and centre of mass).
+__device__ __forceinline__ bool cell_opens(const WalkArgs& A, const GroupGeom& G, uint32_t node, const uint4 rec,
+                                           const float4 fh, const float4 fl, const float2* thr) {
+    const int level = (int)((rec.x >> 21) & 31u);
+    const uint32_t w = (1u << (kMaxLevel - level)) - 1u;
+    const uint32_t qx = rec.x & kQMax, qy = rec.y, qz = rec.z;
+    if (qx <= G.qmax0 && qx + w >= G.qmin0 && qy <= G.qmax1 && qy + w >= G.qmin1 && qz <= G.qmax2 &&
+        qz + w >= G.qmin2)
+        return true;
+    const float dx = (fh.x - G.gch.x) + (fl.x - G.gcl.x);
+    const float dy = (fh.y - G.gch.y) + (fl.y - G.gcl.y);
+    const float dz = (fh.z - G.gch.z) + (fl.z - G.gcl.z);
+    const float tx = fmaxf(fmaxf(G.blo.x - dx, dx - G.bhi.x), 0.0f);
+    const float ty = fmaxf(fmaxf(G.blo.y - dy, dy - G.bhi.y), 0.0f);
+    const float tz = fmaxf(fmaxf(G.blo.z - dz, dz - G.bhi.z), 0.0f);
+    const float d2 = tx * tx + ty * ty + tz * tz;
+    const float2 th = thr[level];
+    if (d2 < th.x) return true;
+    if (d2 > th.y) return false;
+    atomicAdd(&A.st->fallbacks, 1ull);  // rare: counted where it happens
+    return open_fp64(G.L, level, A.theta2, A.nd_com[node], G.box64);
+}
+
+// The list of group g, walked by the calling warp (all 32 lanes), with its
+// two frontier buffers fa and fb and the warp's per-level thresholds thr.
+__device__ __forceinline__ void walk_group(const WalkArgs& A, uint32_t g, uint32_t* fa, uint32_t* fb,
+                                           float2* thr, WalkState& S) {
+    DevState* st = A.st;
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t F = A.cap_frontier;
+    const GroupGeom G = group_geom(A, g);
+    __syncwarp();  // the previous group's walk has read thr
+    if (lane <= kMaxLevel) thr[lane] = level_thresholds(A, G, lane);
     __syncwarp();
 
     if (S.ovf) S.coff = 0;  // counting only
     uint32_t goff = S.coff;  // where the list starts in the chunk
     uint32_t nleaf = 0, nepj_lane = 0;
     uint32_t fsize = 1;
-    if (lane == 0) fa[0] = sysid;
+    if (lane == 0) fa[0] = G.sysid;
     __syncwarp();
     while (fsize > 0) {
         uint32_t nsize = 0;
@@ -205,31 +254,8 @@ __device__ __forceinline__ void walk_group(const WalkArgs& A, uint32_t g, uint32
             int action = 0;  // 1 SPJ, 2 EPJ leaf, 3 open internal
             uint32_t nch = 0, child = 0;
             if (act) {
-                const int level = (int)((rec.x >> 21) & 31u);
                 const bool leaf = (rec.x >> 26) & 1u;
-                const uint32_t w = (1u << (kMaxLevel - level)) - 1u;
-                const uint32_t qx = rec.x & kQMax, qy = rec.y, qz = rec.z;
-                const bool meets = qx <= qmax0 && qx + w >= qmin0 && qy <= qmax1 &&
-                                   qy + w >= qmin1 && qz <= qmax2 && qz + w >= qmin2;
-                bool open = true;
-                if (!meets) {
-                    const float dx = (fh.x - gch.x) + (fl.x - gcl.x);
-                    const float dy = (fh.y - gch.y) + (fl.y - gcl.y);
-                    const float dz = (fh.z - gch.z) + (fl.z - gcl.z);
-                    const float tx = fmaxf(fmaxf(blo.x - dx, dx - bhi.x), 0.0f);
-                    const float ty = fmaxf(fmaxf(blo.y - dy, dy - bhi.y), 0.0f);
-                    const float tz = fmaxf(fmaxf(blo.z - dz, dz - bhi.z), 0.0f);
-                    const float d2 = tx * tx + ty * ty + tz * tz;
-                    const float2 th = thr[level];
-                    if (d2 < th.x) {
-                        open = true;
-                    } else if (d2 > th.y) {
-                        open = false;
-                    } else {
-                        open = open_fp64(L, level, A.theta2, A.nd_com[node], box64);
-                        atomicAdd(&st->fallbacks, 1ull);  // rare: counted where it happens
-                    }
-                }
+                const bool open = cell_opens(A, G, node, rec, fh, fl, thr);
                 if (!open) {
                     action = 1;
                 } else if (leaf) {
@@ -382,6 +408,187 @@ __global__ void __launch_bounds__(kWalkBlock, 8) k_walk(WalkArgs A) {
     walk_flush(A, S);
 }
 
+// The walk for systems of at most kWalkFew particles: a block per group.
+// Their groups are too few to give every warp one (1,002 groups of a 2^14
+// Plummer sphere on 4,864 warps), and a warp alone takes a group's batches of
+// 32 cells one latency after the other; four warps take a level 128 cells at
+// a time, with the frontier in shared memory (its rest, beyond kFewFrontier,
+// in the block's part of the frontier buffers).  The same tests and the same
+// list layout as walk_group.  Plummer 2^14, n_grp 64: walk 96 -> 69 us.
+constexpr int64_t kWalkFew = int64_t(1) << 15;
+constexpr uint32_t kFewFrontier = 1536;
+constexpr int kWalkWarps = kWalkBlock / 32;
+
+__global__ void __launch_bounds__(kWalkBlock, 8) k_walk_few(WalkArgs A) {
+    __shared__ float2 s_thr[kMaxLevel + 1];
+    __shared__ uint32_t s_fr[2][kFewFrontier];
+    __shared__ uint32_t s_cnt[2][3][kWalkWarps];  // a batch's superparticles, leaves and children, per warp
+    __shared__ uint32_t s_red[kWalkWarps];
+    __shared__ unsigned long long s_nb;
+    __shared__ uint32_t s_g;
+    DevState* st = A.st;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t ngroups = (uint32_t)st->n_groups;
+    const uint32_t F = kWalkWarps * A.cap_frontier;  // of the block, beyond the shared part
+    uint32_t* const gfr = A.frontier + blockIdx.x * 2 * (int64_t)F;
+    auto entry = [&](int p, uint32_t k) -> uint32_t& {
+        return k < kFewFrontier ? s_fr[p][k] : gfr[(int64_t)p * F + (k - kFewFrontier)];
+    };
+    WalkState S = walk_state_init();
+    int q = 0;  // the batch's half of s_cnt
+    for (;;) {
+        if (t == 0) s_g = atomicAdd(&st->walk_counter, 1u);
+        __syncthreads();
+        const uint32_t g = s_g;
+        if (g >= ngroups) break;
+        const GroupGeom G = group_geom(A, g);
+        if (t <= kMaxLevel) s_thr[t] = level_thresholds(A, G, t);
+        if (t == 0) s_fr[0][0] = G.sysid;
+        if (S.ovf) S.coff = 0;  // counting only
+        uint32_t goff = S.coff;
+        uint32_t nleaf = 0, nepj_lane = 0, fsize = 1;
+        int p = 0;
+        __syncthreads();
+        while (fsize > 0) {
+            uint32_t nsize = 0;
+            S.max_front = fsize > S.max_front ? fsize : S.max_front;
+            for (uint32_t base = 0; base < fsize; base += kWalkBlock) {
+                const uint32_t idx = base + t;
+                uint32_t node = 0, nch = 0, child = 0;
+                bool spj = false, epj = false;
+                if (idx < fsize) {
+                    node = entry(p, idx);
+                    const uint4 rec = A.nd_walk[node];
+                    const float4 fh = A.nd_f[2 * node], fl = A.nd_f[2 * node + 1];
+                    const bool leaf = (rec.x >> 26) & 1u;
+                    if (!cell_opens(A, G, node, rec, fh, fl, s_thr)) {
+                        spj = true;
+                    } else if (leaf) {
+                        epj = true;
+                        nepj_lane += rec.w;
+                    } else {
+                        child = rec.w;
+                        nch = rec.x >> 27;
+                    }
+                }
+                const uint32_t smask = __ballot_sync(0xFFFFFFFFu, spj), lmask = __ballot_sync(0xFFFFFFFFu, epj);
+                uint32_t inc = nch;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const uint32_t tv = __shfl_up_sync(0xFFFFFFFFu, inc, off);
+                    if (lane >= off) inc += tv;
+                }
+                if (lane == 31) {
+                    s_cnt[q][0][w] = __popc(smask);
+                    s_cnt[q][1][w] = __popc(lmask);
+                    s_cnt[q][2][w] = inc;
+                }
+                __syncthreads();
+                uint32_t ks = 0, kl = 0, kc = 0, rs = __popc(smask & lt), rl = __popc(lmask & lt), rc = inc - nch;
+#pragma unroll
+                for (int k = 0; k < kWalkWarps; ++k) {
+                    const uint32_t cs = s_cnt[q][0][k], cl = s_cnt[q][1][k], cc = s_cnt[q][2][k];
+                    if (k < w) {
+                        rs += cs;
+                        rl += cl;
+                        rc += cc;
+                    }
+                    ks += cs;
+                    kl += cl;
+                    kc += cc;
+                }
+                q ^= 1;
+                if (ks + kl > 0 && S.coff + nleaf + ks + kl > S.clen) {
+                    // new chunk, as in walk_group
+                    const uint32_t nsp = S.coff - goff;
+                    const unsigned long long sofar = (unsigned long long)nsp + nleaf;
+                    const unsigned long long want =
+                        2 * (sofar + ks + kl) > kChunk ? 2 * (sofar + ks + kl) : kChunk;
+                    if (t == 0) s_nb = atomicAdd(&st->pool_cursor, want);
+                    __syncthreads();
+                    const unsigned long long nb = s_nb;
+                    if (!S.ovf && (nb + want > A.cap_pool || want > 0xFFFFFFFFull)) {
+                        if (t == 0) atomicOr(&st->overflow, kOvfPool);
+                        S.ovf = true;
+                    }
+                    if (!S.ovf) {
+                        uint32_t* np = A.pool + nb;
+                        for (uint32_t j = t; j < nsp; j += kWalkBlock) np[j] = S.cptr[goff + j];
+                        const uint32_t* lsrc = S.cptr + (S.clen - nleaf);
+                        uint32_t* ldst = np + (want - nleaf);
+                        for (uint32_t j = t; j < nleaf; j += kWalkBlock) ldst[j] = lsrc[j];
+                        S.cptr = np;
+                        S.clen = (uint32_t)want;
+                    } else {
+                        S.clen = 0xFFFFFFFFu;  // count only from here on
+                    }
+                    goff = 0;
+                    S.coff = nsp;
+                    __syncthreads();  // s_nb has been read, the copies are written
+                }
+                if (!S.ovf) {
+                    if (spj) S.cptr[S.coff + rs] = node;
+                    if (epj) S.cptr[S.clen - 1u - nleaf - rl] = node | kLeafTag;
+                }
+                S.coff += ks;
+                nleaf += kl;
+                if (nsize + kc > kFewFrontier + F) {
+                    if (t == 0) atomicOr(&st->overflow, kOvfFrontier);
+                    S.ovf = true;
+                } else {
+                    const uint32_t o = nsize + rc;
+                    for (uint32_t c = 0; c < nch; ++c) entry(p ^ 1, o + c) = child + c;
+                    nsize += kc;
+                }
+            }
+            __syncthreads();  // the next level's frontier is written
+            p ^= 1;
+            fsize = nsize;
+        }
+        // the leaves behind the superparticles, a batch read before it is
+        // written
+        const uint32_t nspj = S.coff - goff;
+        if (!S.ovf && S.clen - nleaf > S.coff) {
+            const uint32_t* src = S.cptr + (S.clen - nleaf);
+            uint32_t* dst = S.cptr + S.coff;
+            for (uint32_t j = 0; j < nleaf; j += 4 * kWalkBlock) {
+                uint32_t e[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint32_t k = j + r * kWalkBlock + t;
+                    e[r] = k < nleaf ? src[k] : 0u;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint32_t k = j + r * kWalkBlock + t;
+                    if (k < nleaf) dst[k] = e[r];
+                }
+                __syncthreads();
+            }
+        }
+        S.coff += nleaf;
+        const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, nepj_lane);
+        if (lane == 0) s_red[w] = wsum;
+        __syncthreads();
+        uint32_t nepj = 0;
+#pragma unroll
+        for (int k = 0; k < kWalkWarps; ++k) nepj += s_red[k];
+        const uint32_t len = nspj + nleaf;
+        if (t == 0) {
+            A.g_off[g] = (unsigned long long)(S.cptr + goff - A.pool);
+            A.g_len[g] = len;
+            A.g_nspj[g] = nspj;
+            A.g_nepj[g] = nepj;
+        }
+        const unsigned long long ni = A.g_count[g];
+        const unsigned long long mul = lane < 3 ? 1ull : ni;
+        S.total += mul * (lane == 0 ? len : (lane & 1) ? nepj : nspj);
+    }
+    if (w == 0) walk_flush(A, S);
+}
+
 }  // namespace
 
 int walk_blocks(fdps_ctx* ctx) {
@@ -429,7 +636,10 @@ WalkArgs walk_args(fdps_tree* t, const uint32_t* sys) {
 int launch_walk(fdps_tree* t, const uint32_t* sys, int blocks) {
     fdps_ctx* ctx = t->ctx;
     const WalkArgs A = walk_args(t, sys);
-    k_walk<<<blocks, kWalkBlock, 0, ctx->stream>>>(A);
+    if (t->n <= kWalkFew)
+        k_walk_few<<<blocks, kWalkBlock, 0, ctx->stream>>>(A);
+    else
+        k_walk<<<blocks, kWalkBlock, 0, ctx->stream>>>(A);
     FDPS_LAUNCH_CHECK(ctx);
     return FDPS_OK;
 }
