@@ -497,6 +497,7 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
     const SysBox& bx = A.box[A.sys ? A.sys[f] : 0];
     double M = 0.0, Sx = 0.0, Sy = 0.0, Sz = 0.0;
     if (leaf) {
+#pragma unroll 1
         for (uint32_t p = f; p < f + cnt; ++p) {
             M = __dadd_rn(M, A.pm[p]);
             Sx = __dadd_rn(Sx, A.pmx[p]);
@@ -591,6 +592,7 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
     } else {
         float q[6] = {0, 0, 0, 0, 0, 0};
         if (leaf) {
+#pragma unroll 1
             for (uint32_t p = f; p < f + cnt; ++p) {
                 const float4 ph = A.pf_hi[p], pl = A.pf_lo[p];
                 const float m = ph.w;
@@ -654,20 +656,57 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
 // at most kTopNodes nodes.  Systems of an ensemble go through the same passes (one CTA
 // per system before: 256 clusters of 256 to 65536 particles waited for the
 // largest).  The sums of a node keep their order, so results do not depend
-// on the split.  Moments of Plummer 2^14: 136 -> 57 us; of
-// Plummer 2^20 with quadrupoles 246 -> 205 us; of the 256 clusters 1.18 ->
-// 0.39 ms.
+// on the split.  Moments of Plummer 2^14: 136 -> 55 us; of
+// Plummer 2^20 with quadrupoles 246 -> 168 us; of the 256 clusters 1.18 ->
+// 0.27 ms.
 constexpr int kMomBlock = 256;
 constexpr int kMomCl = 8;
 constexpr int64_t kMomSmall = int64_t(1) << 16;
 constexpr int kTopNodes = 4 * kMomBlock;
 constexpr int kMaxGridSpin = 1 << 20;
 
+// The pass over the leaves is bound by the FP64 pipe, which a warp
+// instruction takes whatever its active lanes: a block collects the leaves of
+// kLeafTile nodes ordered by their particle counts (a counting sort; a leaf
+// holds more than kMaxLeaf particles only at the deepest level), so that a
+// warp's lanes sum leaves of like size.  With the internal nodes
+// collected likewise: moments of 2^24 particles (quadrupoles) 1.00 -> 0.92 ms, of
+// 3M clumpy particles (monopoles) 0.36 -> 0.24 ms.
+constexpr int kLeafTile = kMomBlock;
 template <bool QUAD, bool Q64>
 __global__ void __launch_bounds__(kMomBlock) k_moments_leaves(MomArgs A) {
+    __shared__ uint32_t s_id[kLeafTile];
+    __shared__ uint32_t s_bin[32], s_total;
+    const int t = threadIdx.x;
     const int64_t nn = A.st->n_nodes;
-    for (int64_t i = blockIdx.x * (int64_t)kMomBlock + threadIdx.x; i < nn; i += (int64_t)gridDim.x * kMomBlock)
-        if (meta_leaf(A.nd_meta[i])) node_moments<QUAD, Q64, false>(A, i);
+    for (int64_t base = (int64_t)blockIdx.x * kLeafTile; base < nn; base += (int64_t)gridDim.x * kLeafTile) {
+        const int64_t i = base + t;
+        uint32_t bin = 0, rank = 0;  // bin 0: no leaf
+        if (t < 32) s_bin[t] = 0;
+        __syncthreads();
+        if (i < nn && meta_leaf(A.nd_meta[i])) {
+            const uint32_t c = A.nd_count[i];
+            bin = c <= (uint32_t)kMaxLeaf ? c : (uint32_t)kMaxLeaf + 1u;
+            rank = atomicAdd(&s_bin[bin], 1u);
+        }
+        __syncthreads();
+        if (t < 32) {
+            const uint32_t v = s_bin[t];
+            uint32_t inc = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+                if (t >= o) inc += u;
+            }
+            s_bin[t] = inc - v;
+            if (t == 31) s_total = inc;
+        }
+        __syncthreads();
+        if (bin) s_id[s_bin[bin] + rank] = (uint32_t)i;
+        __syncthreads();
+        if (t < (int)s_total) node_moments<QUAD, Q64, false>(A, s_id[t]);
+        __syncthreads();  // the bins are rewritten
+    }
 }
 
 template <bool QUAD, bool Q64>
@@ -702,16 +741,37 @@ __device__ __forceinline__ void grid_barrier(uint32_t* count, uint32_t target, u
     __syncthreads();
 }
 
+// (A quarter or less of a level's nodes are internal: each warp collects 32
+// of them before it sums any, for the FP64 pipe's sake as above.)
 template <bool QUAD, bool Q64>
-__global__ void __launch_bounds__(kMomBlock) k_moments_levels(MomArgs A, uint32_t* count, uint32_t* overflow) {
-    const int64_t t = blockIdx.x * (int64_t)kMomBlock + threadIdx.x, G = (int64_t)gridDim.x * kMomBlock;
+__global__ void __launch_bounds__(kMomBlock, 2) k_moments_levels(MomArgs A, uint32_t* count, uint32_t* overflow) {
+    __shared__ uint32_t s_id[kMomBlock / 32][64];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)kMomBlock + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * kMomBlock) >> 5;
     uint32_t target = 0;
     int l = A.st->max_level - 1;
     for (; l >= 0; --l) {
         const int64_t a = A.st->lvl_start[l], b = A.st->lvl_start[l + 1];
         if (b <= kTopNodes) break;
-        for (int64_t i = a + t; i < b; i += G)
-            if (!meta_leaf(A.nd_meta[i])) node_moments<QUAD, Q64, false>(A, i);
+        uint32_t held = 0;
+        for (int64_t base = a + warp * 32; base < b; base += nwarps * 32) {
+            const int64_t i = base + lane;
+            const bool in = i < b && !meta_leaf(A.nd_meta[i]);
+            const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
+            if (in) s_id[w][held + __popc(m & ((1u << lane) - 1u))] = (uint32_t)i;
+            held += __popc(m);
+            __syncwarp();
+            if (held >= 32) {
+                node_moments<QUAD, Q64, true>(A, s_id[w][lane]);
+                held -= 32;
+                const uint32_t rest = s_id[w][32 + lane];
+                __syncwarp();
+                if (lane < held) s_id[w][lane] = rest;
+                __syncwarp();
+            }
+        }
+        if (lane < held) node_moments<QUAD, Q64, true>(A, s_id[w][lane]);
         target += gridDim.x;
         grid_barrier(count, target, overflow);
     }
@@ -719,7 +779,7 @@ __global__ void __launch_bounds__(kMomBlock) k_moments_levels(MomArgs A, uint32_
     for (; l >= 0; --l) {
         const int64_t a = A.st->lvl_start[l], b = A.st->lvl_start[l + 1];
         for (int64_t i = a + threadIdx.x; i < b; i += kMomBlock)
-            if (!meta_leaf(A.nd_meta[i])) node_moments<QUAD, Q64, false>(A, i);
+            if (!meta_leaf(A.nd_meta[i])) node_moments<QUAD, Q64, true>(A, i);
         __threadfence_block();
         __syncthreads();  // this level complete before its parents
     }
@@ -737,7 +797,8 @@ int launch_moments(fdps_ctx* ctx, const MomArgs& A, int64_t n, DevState* st) {
     int per_sm = 0;
     FDPS_CUDA_TRY(ctx,
                   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_moments_levels<QUAD, Q64>, kMomBlock, 0));
-    const int grid = ctx->sm_count * std::max(1, per_sm);  // every block resident
+    // every block resident, and no more than two per SM to meet at a barrier
+    const int grid = ctx->sm_count * std::max(1, std::min(2, per_sm));
     MomArgs args = A;
     uint32_t* count = &st->mom_counter;
     uint32_t* overflow = &st->overflow;
