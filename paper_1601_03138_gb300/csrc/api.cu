@@ -596,7 +596,7 @@ int fdps_psys_get(const fdps_psys* ps, double* pos3n, double* vel3n, double* acc
     const int64_t n = ps->n;
     fdps_psys* pm = const_cast<fdps_psys*>(ps);
     if (on_device) {
-        int rc = launch_gather_out(pm, pos3n, vel3n, acc3n, pot);
+        int rc = launch_gather_out(pm, pos3n, vel3n, acc3n, pot, true);
         if (rc) return rc;
         FDPS_CUDA_TRY(ctx, cudaStreamSynchronize(s));
         return FDPS_OK;
@@ -607,7 +607,7 @@ int fdps_psys_get(const fdps_psys* ps, double* pos3n, double* vel3n, double* acc
     double* va = const_cast<double*>(device_view(acc3n));
     double* vq = const_cast<double*>(device_view(pot));
     if ((!pos3n || vp) && (!vel3n || vv) && (!acc3n || va) && (!pot || vq)) {
-        int rc = launch_gather_out(pm, vp, vv, va, vq);
+        int rc = launch_gather_out(pm, vp, vv, va, vq, false);
         if (rc) return rc;
         FDPS_CUDA_TRY(ctx, cudaStreamSynchronize(s));
         return FDPS_OK;
@@ -619,7 +619,7 @@ int fdps_psys_get(const fdps_psys* ps, double* pos3n, double* vel3n, double* acc
     }
     double* stage = pm->stage;
     int rc = launch_gather_out(pm, pos3n ? stage : nullptr, vel3n ? stage + 3 * n : nullptr,
-                               acc3n ? stage + 6 * n : nullptr, pot ? stage + 9 * n : nullptr);
+                               acc3n ? stage + 6 * n : nullptr, pot ? stage + 9 * n : nullptr, true);
     cudaError_t e = cudaSuccess;
     if (!rc) {
         if (pos3n && !e) e = cudaMemcpyAsync(pos3n, stage, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s);

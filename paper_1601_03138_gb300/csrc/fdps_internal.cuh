@@ -441,8 +441,9 @@ int launch_energy(fdps_psys* ps, double* kin, double* pot);  // integrate.cu
 // at (id unchanged), else to position i (id = identity)
 int launch_scatter_in(fdps_psys* ps, const double* pos, const double* vel,
                       const double* mass, const double* eps, bool keep_order, uint32_t* bad);  // integrate.cu
-// current buffers and results out in the caller's order
+// current buffers and results out in the caller's order; device_out: the
+// outputs are device memory
 int launch_gather_out(fdps_psys* ps, double* pos, double* vel,
-                      double* acc, double* pot);       // integrate.cu
+                      double* acc, double* pot, bool device_out);  // integrate.cu
 
 }  // namespace fdps
