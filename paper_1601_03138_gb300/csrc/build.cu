@@ -508,7 +508,7 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
         double m8[8], x8[8], y8[8], z8[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            const uint32_t c = c0 + (k < (int)nc ? k : 0);
+            const uint32_t c = k < (int)nc ? c0 + k : (uint32_t)i;  // (a node cut off from its children has none)
             m8[k] = __ldcg(&A.nd_com[c].w);
             x8[k] = __ldcg(&A.nd_sx[c]);
             y8[k] = __ldcg(&A.nd_sy[c]);
@@ -624,7 +624,7 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
                 float2 q1[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    const uint32_t c = c0 + (k < (int)nc ? k : 0);
+                    const uint32_t c = k < (int)nc ? c0 + k : (uint32_t)i;
                     ch[k] = __ldcg(&A.nd_f[2 * c]);
                     cl[k] = __ldcg(&A.nd_f[2 * c + 1]);
                     q0[k] = __ldcg(&A.nd_fq0[c]);
