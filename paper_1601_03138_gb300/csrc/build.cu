@@ -472,7 +472,7 @@ struct MomArgs {
     dvec4* nd_com;
     double* nd_quad;
     float4* nd_f;
-    uint4* nd_walk;
+    WalkRec* nd_walk;
     float4* nd_fq0;
     float2* nd_fq1;
 };
@@ -548,12 +548,13 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
     split_hilo(cz - bx.c0[2], &hz, &lz);
     A.nd_f[2 * i] = make_float4(hx, hy, hz, to_f32(M));
     A.nd_f[2 * i + 1] = make_float4(lx, ly, lz, 0.0f);
-    // walk record: (q_x | level << 21 | leaf << 26 | children << 27, q_y, q_z,
-    // first child of an internal node or particle count of a leaf)
     const uint64_t qlo = A.nd_qlo[i];
-    const uint32_t lev = meta_level(meta), nch = nc;
-    A.nd_walk[i] = make_uint4((uint32_t)(qlo >> 42) | (lev << 21) | ((leaf ? 1u : 0u) << 26) | (nch << 27),
-                              (uint32_t)(qlo >> 21) & kQMax, (uint32_t)qlo & kQMax, leaf ? cnt : c0);
+    const uint32_t lev = meta_level(meta);
+    WalkRec rec;
+    rec.r = make_uint4((uint32_t)(qlo >> 42) | (lev << 21) | ((leaf ? 1u : 0u) << 26) | (nc << 27),
+                       (uint32_t)(qlo >> 21) & kQMax, (uint32_t)qlo & kQMax, leaf ? cnt : c0);
+    rec.c = make_float4(hx, hy, hz, 0.0f);
+    A.nd_walk[i] = rec;
     if (!QUAD) return;
     if (Q64) {
         double q[6] = {0, 0, 0, 0, 0, 0};

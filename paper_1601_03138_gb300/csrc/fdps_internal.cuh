@@ -85,6 +85,20 @@ struct DevState {
     int32_t max_level;
 };
 
+// What the walk's first test of a cell reads, in one 32-byte sector and one
+// 256-bit load: r = (q_x | level << 21 | leaf << 26 | children << 27, q_y, q_z,
+// first child of an internal node or particle count of a leaf), c = the
+// centre of mass relative to the root centre, rounded to FP32.
+struct __align__(32) WalkRec {
+    uint4 r;
+    float4 c;
+};
+__device__ __forceinline__ void ld_walk(const WalkRec* p, uint4& r, float4& c) {
+    asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w), "=f"(c.x), "=f"(c.y), "=f"(c.z), "=f"(c.w)
+        : "l"(p));
+}
+
 // FP64 -> FP32 conversions on the integer pipes (GB300's FP64 pipe is
 // narrow).  split_f32 gives hi = RN32(v) and lo = RN32(v - hi), the values
 // of __double2float_rn(v) and __double2float_rn(v - (double)hi): the 53-bit
@@ -310,8 +324,7 @@ struct fdps_tree {
     fdps::dvec4* nd_com = nullptr;      // FP64 (com_x, com_y, com_z, M)
     double* nd_quad = nullptr;      // FP64 [n][6]
     float4* nd_f = nullptr;         // FP32 pairs [2i] = (com_hi - c0, M), [2i+1] = (com_lo, 0)
-    uint4* nd_walk = nullptr;       // what one opening test reads: grid origin (2 words),
-                                    // first child, meta
+    fdps::WalkRec* nd_walk = nullptr;  // what one opening test reads
     float4* nd_fq0 = nullptr;       // FP32 (Qxx, Qyy, Qzz, Qxy)
     float2* nd_fq1 = nullptr;       // FP32 (Qxz, Qyz)
     // groups

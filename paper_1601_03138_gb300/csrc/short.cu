@@ -81,7 +81,7 @@ __global__ void k_group_hmax(int64_t ng, const uint32_t* __restrict__ first, con
 
 struct ShortWalkArgs {
     DevState* st;
-    const uint4* nd_walk;  // (q_x | level, leaf, children; q_y; q_z; first child | leaf count)
+    const WalkRec* nd_walk;
     const double* nd_hmax;
     const uint32_t* g_qbox;
     const uint32_t* g_first;
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kSBlock) k_short_walk(ShortWalkArgs A) {
             uint4 rec_nx = make_uint4(0, 0, 0, 0);
             float hc_nx = 0.f;
             if (lane < fsize) {
-                rec_nx = A.nd_walk[node_nx];
+                rec_nx = A.nd_walk[node_nx].r;
                 if (A.mode >= 2) hc_nx = (float)A.nd_hmax[node_nx];
             }
             for (uint32_t base = 0; base < fsize; base += 32) {
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kSBlock) k_short_walk(ShortWalkArgs A) {
                 const float hc = hc_nx;
                 if (idx + 32 < fsize) {
                     node_nx = node_nx2;
-                    rec_nx = A.nd_walk[node_nx];
+                    rec_nx = A.nd_walk[node_nx].r;
                     if (A.mode >= 2) hc_nx = (float)A.nd_hmax[node_nx];
                 }
                 if (idx + 64 < fsize) node_nx2 = fa[idx + 64];

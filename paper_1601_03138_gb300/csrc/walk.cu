@@ -34,7 +34,7 @@ namespace fdps {
 struct WalkArgs {
     DevState* st;
     const uint32_t* nd_count;
-    const uint4* nd_walk;  // (q_x | level, leaf, children; q_y; q_z; first child | leaf count)
+    const WalkRec* nd_walk;
     const float4* nd_f;    // COM hi/lo pairs per node
     const dvec4* nd_com;
     const uint32_t* g_count;
@@ -107,21 +107,25 @@ __device__ __forceinline__ WalkState walk_state_init() {
 }
 
 
-// What the opening tests of one group read: its grid box, its centre and box
-// in FP32 relative to it, its FP64 box, its system's root box size.
+// What the opening tests of one group read: its grid box, its centre and its
+// box about it in FP32, its system's root box size.  The box is kept as
+// half-widths h, the larger side of each axis; the two sides differ by the
+// roundings of the centre and of the corners, and the largest difference
+// (exact: the parts nearly cancel) joins the error of a coordinate.
 struct GroupGeom {
+    uint32_t g;
     uint32_t sysid;  // the group's system: its root node (node id = system index) and box
     double L;
-    const double* box64;
     uint32_t qmin0, qmin1, qmin2, qmax0, qmax1, qmax2;
-    float4 gch, gcl, blo, bhi;
+    float4 gch;
+    float hx, hy, hz, asym;
 };
 
 __device__ __forceinline__ GroupGeom group_geom(const WalkArgs& A, uint32_t g) {
     GroupGeom G;
+    G.g = g;
     G.sysid = A.sys ? A.sys[A.g_first[g]] : 0u;
     G.L = A.box[G.sysid].L;
-    G.box64 = A.g_box + 6 * (int64_t)g;
     const uint32_t* qb = A.g_qbox + 6 * (int64_t)g;
     G.qmin0 = qb[0];
     G.qmin1 = qb[1];
@@ -130,28 +134,34 @@ __device__ __forceinline__ GroupGeom group_geom(const WalkArgs& A, uint32_t g) {
     G.qmax1 = qb[4];
     G.qmax2 = qb[5];
     G.gch = A.g_ch[g];
-    G.gcl = A.g_cl[g];
-    G.blo = A.g_blo[g];
-    G.bhi = A.g_bhi[g];
+    const float4 lo = A.g_blo[g], hi = A.g_bhi[g];
+    G.hx = fmaxf(-lo.x, hi.x);
+    G.hy = fmaxf(-lo.y, hi.y);
+    G.hz = fmaxf(-lo.z, hi.z);
+    G.asym = fmaxf(fmaxf(fabsf(lo.x + hi.x), fabsf(lo.y + hi.y)), fabsf(lo.z + hi.z));
     return G;
 }
 
 // The two thresholds on d^2 of the FP32 filter for cells of `level`: below
-// the first the cell opens, above the second it does not.
-__device__ __forceinline__ float2 level_thresholds(const WalkArgs& A, const GroupGeom& G, int level) {
+// the first the cell opens, above the second it does not.  e0: the absolute
+// error of a coordinate of the cell's offset from the group.
+constexpr float kE0Hi = 6.2e-8f;   // times L: centre of mass and group centre rounded to FP32 (u L / 2 each)
+constexpr float kE0Pair = 1e-13f;  // times L: both as FP32 hi/lo pairs
+__device__ __forceinline__ float2 level_thresholds(const WalkArgs& A, const GroupGeom& G, int level,
+                                                   float e0rel) {
     const float Lf = __double2float_rn(G.L);
     // the FP32 filter's bound holds while the squares of cell sizes stay
     // normal FP32 numbers (with or without flushing of subnormals): outside
     // this range of root boxes every test takes the exact FP64 sequence
     const bool filt = Lf >= 0x1p-40f && Lf <= 0x1p60f;
-    const float hb = fmaxf(fmaxf(fmaxf(-G.blo.x, -G.blo.y), fmaxf(-G.blo.z, G.bhi.x)), fmaxf(G.bhi.y, G.bhi.z));
+    const float hb = fmaxf(fmaxf(G.hx, G.hy), G.hz);
     // Coefficients of the filter's error bound as a polynomial in M = max|d| +
     // hb (d the FP32 offset of a cell's centre of mass, hb the largest
     // |corner| of the group box): with E = 4uM + e0 the error of one
     // coordinate and S1 = t_x + t_y + t_z <= 3M, theta^2 (2 E S1 + 3 E^2) <=
     // theta^2 (25 u M^2 + 7 e0 M + 4 e0^2); 1 % on top covers the rounding of
     // the bound's own FP32 evaluation.
-    const float e0 = 1e-13f * Lf;
+    const float e0 = fmaf(e0rel, Lf, G.asym);
     const float mc1 = 1.01f * A.theta2f * 25.0f * kU32, mc2 = 1.01f * A.theta2f * 7.0f * e0,
                 mc3 = 1.01f * A.theta2f * 4.0f * e0 * e0;
     // The bound's largest value over the cells each side can decide, as two
@@ -180,40 +190,70 @@ __device__ __forceinline__ float2 level_thresholds(const WalkArgs& A, const Grou
     return make_float2(lo, hi);
 }
 
-// The opening test of one cell (its walk record and centre of mass).
+// Per-level thresholds of one group: for offsets from rounded centres, and
+// for offsets from hi/lo pairs.
+struct Thresholds {
+    float2 hi[kMaxLevel + 1], pair[kMaxLevel + 1];
+};
+
+__device__ __forceinline__ float box_dist2(float hx, float hy, float hz, float dx, float dy, float dz) {
+    const float tx = fmaxf(fabsf(dx) - hx, 0.0f);
+    const float ty = fmaxf(fabsf(dy) - hy, 0.0f);
+    const float tz = fmaxf(fabsf(dz) - hz, 0.0f);
+    return tx * tx + ty * ty + tz * tz;
+}
+
+// What the rounded centres leave undecided (1 test in 10^3 or less down to
+// levels where the cells are 10^-4 of the root box): the pairs' thresholds,
+// and between those the FP64 sequence.
+__device__ __noinline__ bool cell_opens_close(const WalkArgs& A, uint32_t g, uint32_t node, int level, double L,
+                                              const float2 th) {
+    const float4 fh = A.nd_f[2 * node], fl = A.nd_f[2 * node + 1];
+    const float4 ch = A.g_ch[g], cl = A.g_cl[g];
+    const float4 lo = A.g_blo[g], hi = A.g_bhi[g];
+    const float d2 = box_dist2(fmaxf(-lo.x, hi.x), fmaxf(-lo.y, hi.y), fmaxf(-lo.z, hi.z), (fh.x - ch.x) + (fl.x - cl.x), (fh.y - ch.y) + (fl.y - cl.y),
+                               (fh.z - ch.z) + (fl.z - cl.z));
+    if (d2 < th.x) return true;
+    if (d2 > th.y) return false;
+    atomicAdd(&A.st->fallbacks, 1ull);  // rare: counted where it happens
+    return open_fp64(L, level, A.theta2, A.nd_com[node], A.g_box + 6 * (int64_t)g);
+}
+
+// The opening test of one cell, from its walk record: the grid boxes, then
+// the FP32 filter on rounded centres (half of the loads of the hi/lo pairs,
+// which took the walk's L1 to 61 % of its rate beside 70 % of the issue
+// slots; with the box as half-widths and the children stored off
+// one address: 2^24 particles 5.95 -> 4.43 ms, 256 clusters 2.64 -> 1.88, 2^20
+// 0.63 -> 0.48).
 __device__ __forceinline__ bool cell_opens(const WalkArgs& A, const GroupGeom& G, uint32_t node, const uint4 rec,
-                                           const float4 fh, const float4 fl, const float2* thr) {
+                                           const float4 c, const Thresholds& thr) {
     const int level = (int)((rec.x >> 21) & 31u);
     const uint32_t w = (1u << (kMaxLevel - level)) - 1u;
     const uint32_t qx = rec.x & kQMax, qy = rec.y, qz = rec.z;
     if (qx <= G.qmax0 && qx + w >= G.qmin0 && qy <= G.qmax1 && qy + w >= G.qmin1 && qz <= G.qmax2 &&
         qz + w >= G.qmin2)
         return true;
-    const float dx = (fh.x - G.gch.x) + (fl.x - G.gcl.x);
-    const float dy = (fh.y - G.gch.y) + (fl.y - G.gcl.y);
-    const float dz = (fh.z - G.gch.z) + (fl.z - G.gcl.z);
-    const float tx = fmaxf(fmaxf(G.blo.x - dx, dx - G.bhi.x), 0.0f);
-    const float ty = fmaxf(fmaxf(G.blo.y - dy, dy - G.bhi.y), 0.0f);
-    const float tz = fmaxf(fmaxf(G.blo.z - dz, dz - G.bhi.z), 0.0f);
-    const float d2 = tx * tx + ty * ty + tz * tz;
-    const float2 th = thr[level];
+    const float d2 = box_dist2(G.hx, G.hy, G.hz, c.x - G.gch.x, c.y - G.gch.y, c.z - G.gch.z);
+    const float2 th = thr.hi[level];
     if (d2 < th.x) return true;
     if (d2 > th.y) return false;
-    atomicAdd(&A.st->fallbacks, 1ull);  // rare: counted where it happens
-    return open_fp64(G.L, level, A.theta2, A.nd_com[node], G.box64);
+    return cell_opens_close(A, G.g, node, level, G.L, thr.pair[level]);
 }
 
 // The list of group g, walked by the calling warp (all 32 lanes), with its
 // two frontier buffers fa and fb and the warp's per-level thresholds thr.
 __device__ __forceinline__ void walk_group(const WalkArgs& A, uint32_t g, uint32_t* fa, uint32_t* fb,
-                                           float2* thr, WalkState& S) {
+                                           Thresholds& thr, WalkState& S) {
     DevState* st = A.st;
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     const uint32_t F = A.cap_frontier;
     const GroupGeom G = group_geom(A, g);
     __syncwarp();  // the previous group's walk has read thr
-    if (lane <= kMaxLevel) thr[lane] = level_thresholds(A, G, lane);
+    if (lane <= kMaxLevel) {
+        thr.hi[lane] = level_thresholds(A, G, lane, kE0Hi);
+        thr.pair[lane] = level_thresholds(A, G, lane, kE0Pair);
+    }
     __syncwarp();
 
     if (S.ovf) S.coff = 0;  // counting only
@@ -225,37 +265,31 @@ __device__ __forceinline__ void walk_group(const WalkArgs& A, uint32_t g, uint32
     while (fsize > 0) {
         uint32_t nsize = 0;
         S.max_front = fsize > S.max_front ? fsize : S.max_front;
-        // the first batch's frontier entries, node records and COM pairs;
+        // the first batch's frontier entries and node records;
         // every batch then fetches the next one's before testing its own
         // (frontier ids two batches ahead, records one batch ahead, so
         // no batch waits on a load that depends on another load)
         uint32_t node_nx = lane < fsize ? fa[lane] : 0u;
         uint32_t node_nx2 = lane + 32 < fsize ? fa[lane + 32] : 0u;
         uint4 rec_nx = make_uint4(0, 0, 0, 0);
-        float4 fh_nx = make_float4(0.f, 0.f, 0.f, 0.f), fl_nx = fh_nx;
-        if (lane < fsize) {
-            rec_nx = A.nd_walk[node_nx];
-            fh_nx = A.nd_f[2 * node_nx];
-            fl_nx = A.nd_f[2 * node_nx + 1];
-        }
+        float4 c_nx = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (lane < fsize) ld_walk(A.nd_walk + node_nx, rec_nx, c_nx);
         for (uint32_t base = 0; base < fsize; base += 32) {
             const uint32_t idx = base + lane;
             const bool act = idx < fsize;
             const uint32_t node = node_nx;
             const uint4 rec = rec_nx;
-            const float4 fh = fh_nx, fl = fl_nx;
+            const float4 c = c_nx;
             if (idx + 32 < fsize) {
                 node_nx = node_nx2;
-                rec_nx = A.nd_walk[node_nx];
-                fh_nx = A.nd_f[2 * node_nx];
-                fl_nx = A.nd_f[2 * node_nx + 1];
+                ld_walk(A.nd_walk + node_nx, rec_nx, c_nx);
             }
             if (idx + 64 < fsize) node_nx2 = fa[idx + 64];
             int action = 0;  // 1 SPJ, 2 EPJ leaf, 3 open internal
             uint32_t nch = 0, child = 0;
             if (act) {
                 const bool leaf = (rec.x >> 26) & 1u;
-                const bool open = cell_opens(A, G, node, rec, fh, fl, thr);
+                const bool open = cell_opens(A, G, node, rec, c, thr);
                 if (!open) {
                     action = 1;
                 } else if (leaf) {
@@ -326,8 +360,11 @@ __device__ __forceinline__ void walk_group(const WalkArgs& A, uint32_t g, uint32
                     if (lane == 0) atomicOr(&st->overflow, kOvfFrontier);
                     S.ovf = true;
                 } else {
-                    const uint32_t o = nsize + inc - nch;
-                    for (uint32_t c = 0; c < nch; ++c) fb[o + c] = child + c;
+                    // at most 8 stores off one address
+                    uint32_t* f = fb + (nsize + inc - nch);
+#pragma unroll
+                    for (uint32_t c = 0; c < 8; ++c)
+                        if (c < nch) f[c] = child + c;
                     nsize += tot;
                 }
             }
@@ -396,7 +433,7 @@ __global__ void __launch_bounds__(kWalkBlock, 8) k_walk(WalkArgs A) {
     uint32_t* fa = A.frontier + wid * 2 * (int64_t)A.cap_frontier;
     uint32_t* fb = fa + A.cap_frontier;
     const uint32_t ngroups = (uint32_t)st->n_groups;
-    __shared__ float2 s_thr[kWalkBlock / 32][kMaxLevel + 1];
+    __shared__ Thresholds s_thr[kWalkBlock / 32];
     WalkState S = walk_state_init();
     for (;;) {
         uint32_t g = 0;
@@ -420,7 +457,7 @@ constexpr uint32_t kFewFrontier = 1536;
 constexpr int kWalkWarps = kWalkBlock / 32;
 
 __global__ void __launch_bounds__(kWalkBlock, 8) k_walk_few(WalkArgs A) {
-    __shared__ float2 s_thr[kMaxLevel + 1];
+    __shared__ Thresholds s_thr;
     __shared__ uint32_t s_fr[2][kFewFrontier];
     __shared__ uint32_t s_cnt[2][3][kWalkWarps];  // a batch's superparticles, leaves and children, per warp
     __shared__ uint32_t s_red[kWalkWarps];
@@ -443,7 +480,10 @@ __global__ void __launch_bounds__(kWalkBlock, 8) k_walk_few(WalkArgs A) {
         const uint32_t g = s_g;
         if (g >= ngroups) break;
         const GroupGeom G = group_geom(A, g);
-        if (t <= kMaxLevel) s_thr[t] = level_thresholds(A, G, t);
+        if (t <= kMaxLevel) {
+            s_thr.hi[t] = level_thresholds(A, G, t, kE0Hi);
+            s_thr.pair[t] = level_thresholds(A, G, t, kE0Pair);
+        }
         if (t == 0) s_fr[0][0] = G.sysid;
         if (S.ovf) S.coff = 0;  // counting only
         uint32_t goff = S.coff;
@@ -459,10 +499,11 @@ __global__ void __launch_bounds__(kWalkBlock, 8) k_walk_few(WalkArgs A) {
                 bool spj = false, epj = false;
                 if (idx < fsize) {
                     node = entry(p, idx);
-                    const uint4 rec = A.nd_walk[node];
-                    const float4 fh = A.nd_f[2 * node], fl = A.nd_f[2 * node + 1];
+                    uint4 rec;
+                    float4 c;
+                    ld_walk(A.nd_walk + node, rec, c);
                     const bool leaf = (rec.x >> 26) & 1u;
-                    if (!cell_opens(A, G, node, rec, fh, fl, s_thr)) {
+                    if (!cell_opens(A, G, node, rec, c, s_thr)) {
                         spj = true;
                     } else if (leaf) {
                         epj = true;
