@@ -199,23 +199,37 @@ __device__ __forceinline__ SysBox box_of(const unsigned long long (&lo)[3], cons
 
 // Root boxes of independent systems: one block per system (positions
 // off[k] .. off[k+1]), the same definitions as for a single system.
-__global__ void __launch_bounds__(256) k_box_seg(const int64_t* __restrict__ off,
-                                                 const double* __restrict__ x,
-                                                 const double* __restrict__ y,
-                                                 const double* __restrict__ z,
-                                                 SysBox* __restrict__ box) {
-    const int64_t a0 = off[blockIdx.x], a1 = off[blockIdx.x + 1];
+// A system's block is alone with its loads' latency: four positions a thread
+// in flight, 512 threads (256 clusters of 256 to 65536 particles:
+// 288 -> 130 us).
+constexpr int kSegBlock = 512;
+__global__ void __launch_bounds__(kSegBlock) k_box_seg(const int64_t* __restrict__ off,
+                                                       const double* __restrict__ x,
+                                                       const double* __restrict__ y,
+                                                       const double* __restrict__ z,
+                                                       SysBox* __restrict__ box) {
+    const int64_t a1 = off[blockIdx.x + 1];
     unsigned long long lo[3] = {~0ull, ~0ull, ~0ull};
     unsigned long long hi[3] = {0ull, 0ull, 0ull};
-    for (int64_t i = a0 + threadIdx.x; i < a1; i += blockDim.x) {
-        unsigned long long v[3] = {ord64(x[i]), ord64(y[i]), ord64(z[i])};
+    for (int64_t i = off[blockIdx.x] + threadIdx.x; i < a1; i += 4 * kSegBlock) {
+        double v[4][3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = v[a] < lo[a] ? v[a] : lo[a];
-            hi[a] = v[a] > hi[a] ? v[a] : hi[a];
+        for (int r = 0; r < 4; ++r) {
+            const int64_t k = i + r * kSegBlock < a1 ? i + r * kSegBlock : i;  // past the end: i again
+            v[r][0] = x[k];
+            v[r][1] = y[k];
+            v[r][2] = z[k];
         }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const unsigned long long o = ord64(v[r][a]);
+                lo[a] = o < lo[a] ? o : lo[a];
+                hi[a] = o > hi[a] ? o : hi[a];
+            }
     }
-    block_minmax<8>(lo, hi);
+    block_minmax<kSegBlock / 32>(lo, hi);
     if (threadIdx.x == 0) box[blockIdx.x] = box_of(lo, hi);
 }
 
@@ -1241,7 +1255,7 @@ int keys_and_sort(fdps_tree* t, fdps_psys* ps) {
         k_box_final<<<1, 32, 0, s>>>(t->box_blocks, t->box_part, t->st, t->sys_box);
         FDPS_LAUNCH_CHECK(ctx);
     } else {
-        k_box_seg<<<ps->n_sys, 256, 0, s>>>(ps->d_off, ps->x[c], ps->y[c], ps->z[c], t->sys_box);
+        k_box_seg<<<ps->n_sys, kSegBlock, 0, s>>>(ps->d_off, ps->x[c], ps->y[c], ps->z[c], t->sys_box);
         FDPS_LAUNCH_CHECK(ctx);
     }
     if (coherent) {
