@@ -298,7 +298,31 @@ __global__ void __launch_bounds__(kBT) k_tree_nodes(
     uint32_t* __restrict__ nd_meta, uint32_t* __restrict__ nd_parent, uint64_t* __restrict__ nd_qlo) {
     constexpr int kSpan = 32 * ROWS, kTile = kBT * ROWS;
     __shared__ int64_t s_lvl[kMaxLevel + 3];
+    __shared__ uint32_t s_tot[kMaxLevel], s_pre[kMaxLevel];  // a level's nodes: all, and in earlier tiles
     __shared__ int s_cut;
+    if (ROWS == 1) {  // few tiles: every block sums their counts itself (no scan pass)
+        for (int l = threadIdx.x >> 5; l < kMaxLevel; l += kBWarps) {
+            uint32_t tot = 0, pre = 0;
+            for (int64_t k = threadIdx.x & 31; k < ntiles; k += 32) {
+                const uint32_t v = tcount[(int64_t)l * ntiles + k];
+                tot += v;
+                pre += k < (int64_t)blockIdx.x ? v : 0u;
+            }
+            tot = __reduce_add_sync(0xFFFFFFFFu, tot);
+            pre = __reduce_add_sync(0xFFFFFFFFu, pre);
+            if ((threadIdx.x & 31) == 0) {
+                s_tot[l] = tot;
+                s_pre[l] = pre;
+            }
+        }
+    } else if (threadIdx.x < kMaxLevel) {
+        const int l = threadIdx.x;
+        s_tot[l] = ltot[l];
+        // a tile past the counted ones holds only position n: all of the
+        // level's nodes come before
+        s_pre[l] = (int64_t)blockIdx.x < ntiles ? tcount[(int64_t)l * ntiles + blockIdx.x] : ltot[l];
+    }
+    __syncthreads();
     __shared__ uint32_t s_wc[kMaxLevel][kBWarps];
     __shared__ uint32_t sP[1 + kTile];  // pk of positions t0 - 1 .. t0 + kTile - 1
     if (threadIdx.x == 0) {
@@ -310,10 +334,10 @@ __global__ void __launch_bounds__(kBT) k_tree_nodes(
         s_lvl[0] = 0;
         for (int l = 1; l <= kMaxLevel; ++l) {
             s_lvl[l] = s;
-            if (cut > kMaxLevel && s + ltot[l - 1] > cap_nodes) cut = l;
+            if (cut > kMaxLevel && s + s_tot[l - 1] > cap_nodes) cut = l;
             if (cut > kMaxLevel) {
-                s += ltot[l - 1];
-                if (ltot[l - 1]) top = l;
+                s += s_tot[l - 1];
+                if (s_tot[l - 1]) top = l;
             }
         }
         for (int l = cut; l <= kMaxLevel + 2; ++l) s_lvl[l] = s;
@@ -341,11 +365,10 @@ __global__ void __launch_bounds__(kBT) k_tree_nodes(
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     // next id of each level for this warp: level start + nodes of earlier
-    // tiles + nodes of earlier warps of this tile (a tile past the counted
-    // ones holds only position n: all of the level's nodes come before)
+    // tiles + nodes of earlier warps of this tile
     uint32_t nxt = 0u;
     if (lane >= 1 && lane <= kMaxLevel) {
-        nxt = (uint32_t)s_lvl[lane] + (tile < ntiles ? tcount[(int64_t)(lane - 1) * ntiles + tile] : ltot[lane - 1]);
+        nxt = (uint32_t)s_lvl[lane] + s_pre[lane - 1];
         for (int k = 0; k < w; ++k) nxt += s_wc[lane - 1][k];
     }
     uint32_t run[kMaxLevel];
@@ -712,9 +735,13 @@ __global__ void __launch_bounds__(kMomBlock) k_moments_leaves(MomArgs A) {
 
 template <bool QUAD, bool Q64>
 __global__ void __cluster_dims__(kMomCl, 1, 1) __launch_bounds__(kMomBlock) k_moments_small(MomArgs A) {
-    for (int l = A.st->max_level - 1; l >= 0; --l) {
-        const int64_t a = A.st->lvl_start[l], b = A.st->lvl_start[l + 1];
-        for (int64_t i = a + blockIdx.x * kMomBlock + threadIdx.x; i < b; i += kMomCl * kMomBlock)
+    __shared__ int32_t s_lvl[kMaxLevel + 3];
+    if (threadIdx.x < kMaxLevel + 3) s_lvl[threadIdx.x] = A.st->lvl_start[threadIdx.x];
+    const int top = A.st->max_level - 1;
+    __syncthreads();
+    const int t = blockIdx.x * kMomBlock + threadIdx.x;
+    for (int l = top; l >= 0; --l) {
+        for (int i = s_lvl[l] + t; i < s_lvl[l + 1]; i += kMomCl * kMomBlock)
             if (!meta_leaf(A.nd_meta[i])) node_moments<QUAD, Q64, true>(A, i);
         __threadfence();
         cluster_barrier();  // this level complete before its parents
@@ -899,6 +926,53 @@ __global__ void __launch_bounds__(kB) k_group_write(int64_t n, int64_t cap_group
     }
 }
 
+// The i-groups of at most kGroupSmall positions in one block: heads as bits
+// of a word per thread in shared memory, their ranks from one scan (a clear,
+// a mark, a count and a write pass over the positions before, 17 us of which
+// little was work; all group passes of 2^14
+// particles 25 -> 16 us, of 2001 25 -> 12 us).
+constexpr int kGroupSmallBlock = 1024;
+constexpr int64_t kGroupSmall = 32 * kGroupSmallBlock;
+__global__ void __launch_bounds__(kGroupSmallBlock) k_group_small(DevState* st, int n_grp, int n_roots,
+                                                                  int64_t cap_groups,
+                                                                  const uint32_t* __restrict__ nd_first,
+                                                                  const uint32_t* __restrict__ nd_count,
+                                                                  const uint32_t* __restrict__ nd_meta,
+                                                                  const uint32_t* __restrict__ nd_parent,
+                                                                  uint32_t* head, uint32_t* __restrict__ g_node,
+                                                                  uint32_t* __restrict__ g_first,
+                                                                  uint32_t* __restrict__ g_count) {
+    __shared__ uint32_t s_bits[kGroupSmallBlock];
+    const int t = threadIdx.x;
+    s_bits[t] = 0;
+    __syncthreads();
+    const int nn = st->n_nodes;
+    for (int i = t; i < nn; i += kGroupSmallBlock) {
+        const bool cand = nd_count[i] <= (uint32_t)n_grp || meta_leaf(nd_meta[i]);
+        if (cand && (i < n_roots || nd_count[nd_parent[i]] > (uint32_t)n_grp)) {
+            const uint32_t p = nd_first[i];
+            head[p] = (uint32_t)i;
+            atomicOr(&s_bits[p >> 5], 1u << (p & 31u));
+        }
+    }
+    __syncthreads();
+    uint32_t bits = s_bits[t], total;
+    int64_t g = block_excl(__popc(bits), &total);
+    for (; bits; bits &= bits - 1u, ++g) {
+        const uint32_t p = 32u * t + __ffs(bits) - 1u;
+        const uint32_t h = head[p];
+        if (g < cap_groups) {
+            g_node[g] = h;
+            g_first[g] = p;
+            g_count[g] = nd_count[h];
+        }
+    }
+    if (t == 0) {
+        if ((int64_t)total > cap_groups) st->overflow |= kOvfGroups;
+        st->n_groups = (int32_t)((int64_t)total > cap_groups ? cap_groups : total);
+    }
+}
+
 __device__ __forceinline__ unsigned long long ord64(double v) {
     unsigned long long u = (unsigned long long)__double_as_longlong(v);
     return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
@@ -1006,8 +1080,10 @@ int build_tree(fdps_tree* t, fdps_psys* ps) {
     (small ? k_tree_count<1> : k_tree_count<kBRows>)<<<(unsigned)ntiles, kBT, 0, s>>>(
         n, t->p.n_leaf, t->keys_sorted, ps->d_sys, t->head, wcount, tcount, nw, ntiles, R);
     FDPS_LAUNCH_CHECK(ctx);
-    k_tree_scan<<<kMaxLevel, 1024, 0, s>>>(tcount, ntiles, ltot);
-    FDPS_LAUNCH_CHECK(ctx);
+    if (!small) {
+        k_tree_scan<<<kMaxLevel, 1024, 0, s>>>(tcount, ntiles, ltot);
+        FDPS_LAUNCH_CHECK(ctx);
+    }
     const unsigned grid_nodes = (unsigned)(n / tile + 1);  // positions 0 .. n
     (small ? k_tree_nodes<1> : k_tree_nodes<kBRows>)<<<grid_nodes, kBT, 0, s>>>(
         n, ps->n_sys, t->cap_nodes, t->keys_sorted, ps->d_sys, t->head, wcount, tcount, nw, ntiles, ltot, t->st,
@@ -1061,15 +1137,22 @@ int select_groups(fdps_tree* t, fdps_psys* ps) {
     const int64_t n = ps->n;
     const int c = ps->cur;
     const int G = t->box_blocks;
-    FDPS_CUDA_TRY(ctx, cudaMemsetAsync(t->head, 0xFF, sizeof(uint32_t) * (size_t)n, s));
-    k_group_mark<<<ctx->sm_count * 8, 256, 0, s>>>(t->st, t->p.n_grp, ps->n_sys, t->nd_first, t->nd_count,
-                                                   t->nd_meta, t->nd_parent, t->head);
-    FDPS_LAUNCH_CHECK(ctx);
-    k_group_count<<<G, kB, 0, s>>>(n, t->head, t->grp_scan, t->st, t->cap_groups);
-    FDPS_LAUNCH_CHECK(ctx);
-    k_group_write<<<G, kB, 0, s>>>(n, t->cap_groups, t->head, t->grp_scan, t->nd_count, t->g_node,
-                                   t->g_first, t->g_count);
-    FDPS_LAUNCH_CHECK(ctx);
+    if (n <= kGroupSmall) {
+        k_group_small<<<1, kGroupSmallBlock, 0, s>>>(t->st, t->p.n_grp, ps->n_sys, t->cap_groups, t->nd_first,
+                                                     t->nd_count, t->nd_meta, t->nd_parent, t->head, t->g_node,
+                                                     t->g_first, t->g_count);
+        FDPS_LAUNCH_CHECK(ctx);
+    } else {
+        FDPS_CUDA_TRY(ctx, cudaMemsetAsync(t->head, 0xFF, sizeof(uint32_t) * (size_t)n, s));
+        k_group_mark<<<ctx->sm_count * 8, 256, 0, s>>>(t->st, t->p.n_grp, ps->n_sys, t->nd_first, t->nd_count,
+                                                       t->nd_meta, t->nd_parent, t->head);
+        FDPS_LAUNCH_CHECK(ctx);
+        k_group_count<<<G, kB, 0, s>>>(n, t->head, t->grp_scan, t->st, t->cap_groups);
+        FDPS_LAUNCH_CHECK(ctx);
+        k_group_write<<<G, kB, 0, s>>>(n, t->cap_groups, t->head, t->grp_scan, t->nd_count, t->g_node,
+                                       t->g_first, t->g_count);
+        FDPS_LAUNCH_CHECK(ctx);
+    }
     k_group_data<<<ctx->sm_count * 8, 256, 0, s>>>(t->st, t->sys_box, ps->d_sys, t->g_first, t->g_count, ps->x[c],
                                                    ps->y[c], ps->z[c], t->g_box, t->g_qbox,
                                                    t->g_c64, t->g_ch, t->g_cl, t->g_blo, t->g_bhi);

@@ -2,8 +2,14 @@
 particles far apart, each at the end of a chain of some fifteen cells.  The
 build cuts the tree at the level that does not fit (its last nodes then have
 no children), the kernels after it run on the cut tree, and the call is
-repeated with larger arrays: nodes and forces equal the oracle's (FP32 bound
-1e-5), for the moments of small systems, of large ones and of an ensemble."""
+repeated with larger arrays: nodes and forces equal the oracle's, for the
+moments of small systems, of large ones and of an ensemble.
+
+Force bound: the FP32 path's 1e-5.  It needs a softening well above the
+knots: coordinates relative to a group's centre are rounded to 2^-24 of its
+size (0.1), 6e-9 or 6e-4 of a separation inside a knot (1e-5), and with eps =
+1e-3 a knot's own force, m dx / eps^3 = 0.3 a particle, would carry that error
+into the sum.  With eps = 0.05 it is 2e-6 a particle, of forces of order 1."""
 import numpy as np
 import pytest
 
@@ -31,7 +37,7 @@ def test_node_arrays_grow(G, k, quad):
     rng = np.random.default_rng(k)
     pos = knots(k, rng)
     n = len(pos)
-    mass, eps = np.full(n, 1.0 / n), np.full(n, 1e-3)
+    mass, eps = np.full(n, 1.0 / n), np.full(n, 0.05)
     ref = oracle.Tree(pos, mass, eps, theta=0.7, n_leaf=16, n_grp=64, quad=quad)
     assert ref.n_nodes > n // 2 + 1024  # more than the first allocation
     with G.Context(0) as ctx:
@@ -62,7 +68,7 @@ def test_ensemble_node_arrays_grow(G):
     pos = np.concatenate([knots(1500, rng), rng.random((300, 3)), knots(2500, rng)])
     off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
     n = len(pos)
-    mass, eps = np.full(n, 1.0 / n), np.full(n, 1e-3)
+    mass, eps = np.full(n, 1.0 / n), np.full(n, 0.05)
     with G.Context(0) as ctx:
         ps = G.ParticleSystem(ctx, n)
         tree = G.Tree(ctx, theta=0.7, n_leaf=16, n_grp=64)
