@@ -177,10 +177,27 @@ int ensure_frontier(fdps_tree* t, int64_t per_warp) {
     return FDPS_OK;
 }
 
+int ensure_short_io(fdps_tree* t, int64_t n) {
+    if (n <= t->cap_sr_io) return FDPS_OK;
+    dev_free(t->sr_hin);
+    dev_free(t->sr_cnt);
+    dev_free(t->sr_rho);
+    t->cap_sr_io = 0;
+    if (dev_alloc(&t->sr_hin, n) != cudaSuccess || dev_alloc(&t->sr_cnt, n) != cudaSuccess ||
+        dev_alloc(&t->sr_rho, n) != cudaSuccess) {
+        cudaGetLastError();
+        return set_error(t->ctx, FDPS_ENOMEM, "neighbour buffer allocation for %lld particles failed", (long long)n);
+    }
+    t->cap_sr_io = n;
+    return FDPS_OK;
+}
+
+// The state word through the tree's page-locked copy.
 int read_state(fdps_tree* t) {
-    FDPS_CUDA_TRY(t->ctx, cudaMemcpyAsync(&t->h_st, t->st, sizeof(DevState), cudaMemcpyDeviceToHost,
+    FDPS_CUDA_TRY(t->ctx, cudaMemcpyAsync(t->h_pin, t->st, sizeof(DevState), cudaMemcpyDeviceToHost,
                                           t->ctx->stream));
     FDPS_CUDA_TRY(t->ctx, cudaStreamSynchronize(t->ctx->stream));
+    t->h_st = *t->h_pin;
     return FDPS_OK;
 }
 
@@ -243,12 +260,12 @@ int launch_force_pipeline(fdps_tree* t, fdps_psys* ps, int k_spj) {
     return compute_forces(t, ps, k_spj);
 }
 
-int run_tree_stages(fdps_tree* t, fdps_psys* ps) {
-    fdps_ctx* ctx = t->ctx;
+// Buffers of a force calculation of ps, at least as large as the estimates.
+int ensure_tree_buffers(fdps_tree* t, fdps_psys* ps) {
     const int64_t n = ps->n;
     int rc;
     if (n >= (int64_t(1) << 30))
-        return set_error(ctx, FDPS_EINVAL, "the tree handles fewer than 2^30 particles");
+        return set_error(t->ctx, FDPS_EINVAL, "the tree handles fewer than 2^30 particles");
     if ((rc = ensure_particles(t, n))) return rc;
     if ((rc = ensure_systems(t, ps->n_sys))) return rc;
     const int64_t nl = t->p.n_leaf, ng = t->p.n_grp;
@@ -258,72 +275,70 @@ int run_tree_stages(fdps_tree* t, fdps_psys* ps) {
     if ((rc = ensure_frontier(t, 4096))) return rc;
     t->n = n;
     t->valid = false;
-    cudaStream_t s = ctx->stream;
-    // a coherent sort whose bucket did not fit leaves the particles in
-    // their order (the kernels after it copy them as they are): the call
-    // starts over with the radix sort
-    for (int sort_try = 0;; ++sort_try) {
-    FDPS_CUDA_TRY(ctx, cudaMemsetAsync(t->st, 0, sizeof(DevState), s));
+    return FDPS_OK;
+}
+
+// S0-S3 (clears the state word, and with it every counter) and S4-S6.
+int launch_sorted(fdps_tree* t, fdps_psys* ps) {
+    int rc;
+    FDPS_CUDA_TRY(t->ctx, cudaMemsetAsync(t->st, 0, sizeof(DevState), t->ctx->stream));
     record(t, 0);
     if ((rc = keys_and_sort(t, ps))) return rc;
     record(t, 2);
     if ((rc = reorder_particles(t, ps))) return rc;
     record(t, 3);
-    bool redo = false;
-    for (int attempt = 0;; ++attempt) {
-        if ((rc = build_tree(t, ps))) return rc;
-        record(t, 4);
-        if ((rc = compute_moments(t, ps))) return rc;
-        record(t, 5);
-        if ((rc = select_groups(t, ps))) return rc;
-        record(t, 6);
-        if ((rc = read_state(t))) return rc;
-        const uint32_t ov = t->h_st.overflow;
-        if (ov & kSortStall) {
-            t->coh_ok = false;
-            return set_error(ctx, FDPS_ETIMEOUT, "a device-side wait (sort look-back or grid barrier) exceeded its bound");
-        }
-        if (ov & kSortRedo) {
-            if (sort_try > 0) return set_error(ctx, FDPS_ECUDA, "coherent sort asked for a second redo");
-            t->coh_ok = false;
-            ++t->retries;
-            redo = true;
-            break;
-        }
-        if (!(ov & (kOvfNodes | kOvfGroups))) break;
-        if (attempt > 8)
-            return set_error(ctx, FDPS_EOVERFLOW, "tree build did not fit after %d resizes", attempt);
-        ++t->retries;
-        if (ov & kOvfNodes)
-            if ((rc = ensure_nodes(t, 2 * t->cap_nodes))) return rc;
-        if (ov & kOvfGroups)
-            if ((rc = ensure_groups(t, std::min<int64_t>(n, 2 * t->cap_groups)))) return rc;
-        k_reset_counters<<<1, 32, 0, s>>>(t->st, 4);
-        FDPS_LAUNCH_CHECK(ctx);
-    }
-    if (!redo) break;
-    }
+    return FDPS_OK;
+}
+int launch_built(fdps_tree* t, fdps_psys* ps) {
+    int rc;
+    if ((rc = build_tree(t, ps))) return rc;
+    record(t, 4);
+    if ((rc = compute_moments(t, ps))) return rc;
+    record(t, 5);
+    if ((rc = select_groups(t, ps))) return rc;
+    record(t, 6);
     return FDPS_OK;
 }
 
-int run_force(fdps_tree* t, fdps_psys* ps, int k_spj, bool lists_only = false) {
+// How often the stages of one call were repeated, and from which on they are
+// to be launched (again).
+struct Redo {
+    enum Stage { kSort, kBuild, kWalk, kNone } from = kSort;
+    int sorts = 0, builds = 0, walks = 0;
+};
+
+// After the stages up to the i-groups (lists: up to the walk) ran with the
+// state word in t->h_st: what has to run again, with the buffers that were
+// too small grown and the counters of the stages cleared.  A coherent sort
+// whose bucket did not fit leaves the particles in their order (the kernels
+// after it copy them as they are): the call starts over with the radix sort.
+int plan_redo(fdps_tree* t, fdps_psys* ps, Redo& r, bool lists) {
     fdps_ctx* ctx = t->ctx;
-    int rc;
-    if ((rc = run_tree_stages(t, ps))) return rc;
-    cudaStream_t s = ctx->stream;
-    const int wblocks = (int)(t->n_walk_warps / walk_warps_per_block());
-    for (int attempt = 0;; ++attempt) {
-        k_reset_counters<<<1, 32, 0, s>>>(t->st, 1);
-        FDPS_LAUNCH_CHECK(ctx);
-        if ((rc = launch_walk(t, ps->d_sys, wblocks))) return rc;
-        record(t, 7);
-        if ((rc = read_state(t))) return rc;
-        const uint32_t ov = t->h_st.overflow;
-        if (!(ov & (kOvfPool | kOvfFrontier))) break;
-        if (attempt > 8)
-            return set_error(ctx, FDPS_EOVERFLOW, "interaction lists did not fit after %d resizes",
-                             attempt);
+    const uint32_t ov = t->h_st.overflow;
+    int rc, clear;
+    if (ov & kSortStall) {
+        t->coh_ok = false;
+        return set_error(ctx, FDPS_ETIMEOUT, "a device-side wait (sort look-back or grid barrier) exceeded its bound");
+    }
+    if (ov & kSortRedo) {
+        if (r.sorts++ > 0) return set_error(ctx, FDPS_ECUDA, "coherent sort asked for a second redo");
+        t->coh_ok = false;
         ++t->retries;
+        r.from = Redo::kSort;
+        return FDPS_OK;
+    }
+    if (ov & (kOvfNodes | kOvfGroups)) {
+        if (r.builds++ > 8)
+            return set_error(ctx, FDPS_EOVERFLOW, "tree build did not fit after %d resizes", r.builds);
+        if (ov & kOvfNodes)
+            if ((rc = ensure_nodes(t, 2 * t->cap_nodes))) return rc;
+        if (ov & kOvfGroups)
+            if ((rc = ensure_groups(t, std::min<int64_t>(ps->n, 2 * t->cap_groups)))) return rc;
+        r.from = Redo::kBuild;
+        clear = 7;
+    } else if (lists && (ov & (kOvfPool | kOvfFrontier))) {
+        if (r.walks++ > 8)
+            return set_error(ctx, FDPS_EOVERFLOW, "interaction lists did not fit after %d resizes", r.walks);
         if (ov & kOvfFrontier)
             if ((rc = ensure_frontier(t, 2 * t->cap_frontier))) return rc;
         if (ov & kOvfPool) {
@@ -331,21 +346,65 @@ int run_force(fdps_tree* t, fdps_psys* ps, int k_spj, bool lists_only = false) {
                                  2 * t->n_walk_warps * (int64_t)walk_chunk();
             if ((rc = ensure_pool(t, std::max<int64_t>(need, 2 * t->cap_pool)))) return rc;
         }
-    }
-    if (lists_only) {  // S0-S7 only: the lists stay for user interaction kernels
-        FDPS_CUDA_TRY(ctx, cudaGetLastError());
-        t->valid = true;
-        t->lists_of = ps;
+        r.from = Redo::kWalk;
+        clear = 3;
+    } else {
+        r.from = Redo::kNone;
         return FDPS_OK;
     }
-    k_reset_counters<<<1, 32, 0, s>>>(t->st, 2);
+    ++t->retries;
+    k_reset_counters<<<1, 32, 0, ctx->stream>>>(t->st, clear);
     FDPS_LAUNCH_CHECK(ctx);
-    if ((rc = compute_forces(t, ps, k_spj))) return rc;
-    record(t, 8);
+    return FDPS_OK;
+}
+
+int run_tree_stages(fdps_tree* t, fdps_psys* ps) {
+    int rc;
+    if ((rc = ensure_tree_buffers(t, ps))) return rc;
+    Redo r;
+    while (r.from != Redo::kNone) {
+        if (r.from == Redo::kSort && (rc = launch_sorted(t, ps))) return rc;
+        if ((rc = launch_built(t, ps))) return rc;
+        if ((rc = read_state(t))) return rc;
+        if ((rc = plan_redo(t, ps, r, false))) return rc;
+    }
+    return FDPS_OK;
+}
+
+// The whole calculation is queued before the host looks at the state word,
+// which it has copied between the walk and the force kernel: the GPU does not
+// wait for the host between stages, and the host returns once the lists are
+// known to fit, with the force kernel still running.  After an overflow the
+// later kernels have kept within their buffers (or returned at once) and the
+// stages from there on are queued again.  Plummer 2^14, a step and its read:
+// 313 -> 272 us with the group and build passes of small sets
+// above.
+int run_force(fdps_tree* t, fdps_psys* ps, int k_spj, bool lists_only = false) {
+    fdps_ctx* ctx = t->ctx;
+    cudaStream_t s = ctx->stream;
+    int rc;
+    if ((rc = ensure_tree_buffers(t, ps))) return rc;
+    const int wblocks = (int)(t->n_walk_warps / walk_warps_per_block());
+    Redo r;
+    while (r.from != Redo::kNone) {
+        if (r.from == Redo::kSort && (rc = launch_sorted(t, ps))) return rc;
+        if (r.from <= Redo::kBuild && (rc = launch_built(t, ps))) return rc;
+        if ((rc = launch_walk(t, ps->d_sys, wblocks))) return rc;
+        record(t, 7);
+        FDPS_CUDA_TRY(ctx, cudaMemcpyAsync(t->h_pin, t->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
+        FDPS_CUDA_TRY(ctx, cudaEventRecord(t->ev_state, s));
+        if (!lists_only) {  // else S0-S7 only: the lists stay for user interaction kernels
+            if ((rc = compute_forces(t, ps, k_spj))) return rc;
+            record(t, 8);
+        }
+        FDPS_CUDA_TRY(ctx, cudaEventSynchronize(t->ev_state));
+        t->h_st = *t->h_pin;
+        if ((rc = plan_redo(t, ps, r, true))) return rc;
+    }
     FDPS_CUDA_TRY(ctx, cudaGetLastError());
     t->valid = true;
     t->lists_of = ps;
-    ps->has_forces = true;
+    if (!lists_only) ps->has_forces = true;
     return FDPS_OK;
 }
 
@@ -361,11 +420,6 @@ bool valid_params(const fdps_tree_params* p) {
 }
 
 }  // namespace
-
-namespace fdps {
-int run_tree(fdps_tree* t, fdps_psys* ps) { return run_tree_stages(t, ps); }
-int read_device_state(fdps_tree* t) { return read_state(t); }
-}  // namespace fdps
 
 extern "C" {
 
@@ -652,7 +706,9 @@ int fdps_tree_create(fdps_ctx* ctx, const fdps_tree_params* params, fdps_tree** 
     t->n_walk_warps = (int64_t)walk_blocks(ctx) * walk_warps_per_block();
     bool ok = dev_alloc(&t->st, 1) == cudaSuccess && dev_alloc(&t->box_part, t->box_blocks) == cudaSuccess &&
               dev_alloc(&t->grp_scan, t->box_blocks) == cudaSuccess &&
-              dev_alloc(&t->sort_dtot, 4096) == cudaSuccess;
+              dev_alloc(&t->sort_dtot, 4096) == cudaSuccess &&
+              cudaMallocHost(reinterpret_cast<void**>(&t->h_pin), sizeof(DevState)) == cudaSuccess &&
+              cudaEventCreateWithFlags(&t->ev_state, cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         fdps_tree_destroy(t);
@@ -682,6 +738,12 @@ int fdps_tree_destroy(fdps_tree* t) {
     dev_free(t->sr_h);
     dev_free(t->nd_hmax);
     dev_free(t->g_hmax);
+    dev_free(t->sr_hin);
+    dev_free(t->sr_cnt);
+    dev_free(t->sr_rho);
+    dev_free(t->sr_info);
+    if (t->h_pin) cudaFreeHost(t->h_pin);
+    if (t->ev_state) cudaEventDestroy(t->ev_state);
     for (int k = 0; k < 10; ++k)
         if (t->ev[k]) cudaEventDestroy(t->ev[k]);
     delete t;
@@ -830,86 +892,48 @@ int fdps_tree_neighbors(fdps_tree* t, fdps_psys* ps, int32_t mode, double r_fixe
     int rc;
     if ((rc = run_tree_stages(t, ps))) return rc;
     t->lists_of = nullptr;  // the pool will hold neighbour lists, not gravity lists
-    double* d_h = nullptr;
-    uint32_t* d_cnt = nullptr;
-    double* d_rho = nullptr;
-    unsigned long long* d_info = nullptr;
-    auto cleanup = [&]() {
-        if (d_h && !h_on_device) cudaFree(d_h);
-        if (d_cnt && !out_on_device) cudaFree(d_cnt);
-        if (d_rho && !out_on_device) cudaFree(d_rho);
-        cudaFree(d_info);
-    };
+    // device copies of host arrays, kept with the tree (allocating and freeing
+    // them in each call cost 0.3 ms, most of it the frees' synchronisation)
+    if ((mode != FDPS_CUTOFF_FIXED && !h_on_device) || !out_on_device)
+        if ((rc = ensure_short_io(t, n))) return rc;
+    if (!t->sr_info && dev_alloc(&t->sr_info, 3) != cudaSuccess) {
+        cudaGetLastError();
+        return set_error(ctx, FDPS_ENOMEM, "neighbour output allocation failed");
+    }
+    const double* d_h = nullptr;
     if (mode != FDPS_CUTOFF_FIXED) {
-        if (h_on_device) {
-            d_h = const_cast<double*>(h);
-        } else if (cudaMalloc(&d_h, sizeof(double) * n) != cudaSuccess ||
-                   cudaMemcpyAsync(d_h, h, sizeof(double) * n, cudaMemcpyHostToDevice, s) != cudaSuccess) {
+        d_h = h_on_device ? h : t->sr_hin;
+        if (!h_on_device &&
+            cudaMemcpyAsync(t->sr_hin, h, sizeof(double) * n, cudaMemcpyHostToDevice, s) != cudaSuccess) {
             cudaGetLastError();
-            cleanup();
             return set_error(ctx, FDPS_ENOMEM, "radii transfer failed");
         }
     }
-    if ((rc = short_prepare(t, ps, mode, d_h))) {
-        cleanup();
-        return rc;
-    }
+    if ((rc = short_prepare(t, ps, mode, d_h))) return rc;
     const int wblocks = (int)(t->n_walk_warps / walk_warps_per_block());
-    for (int attempt = 0;; ++attempt) {
-        k_reset_counters<<<1, 32, 0, s>>>(t->st, 1);
-        FDPS_LAUNCH_CHECK(ctx);
-        if ((rc = launch_short_walk(t, ps, mode, r_fixed, wblocks)) || (rc = read_state(t))) {
-            cleanup();
-            return rc;
-        }
-        const uint32_t ov = t->h_st.overflow;
-        if (!(ov & (kOvfPool | kOvfFrontier))) break;
-        if (attempt > 8) {
-            cleanup();
-            return set_error(ctx, FDPS_EOVERFLOW, "neighbour lists did not fit after %d resizes", attempt);
-        }
-        ++t->retries;
-        if ((ov & kOvfFrontier) && (rc = ensure_frontier(t, 2 * t->cap_frontier))) {
-            cleanup();
-            return rc;
-        }
-        if (ov & kOvfPool) {
-            const int64_t need = (int64_t)(t->h_st.pool_needed * 3 / 2) +
-                                 2 * t->n_walk_warps * (int64_t)walk_chunk();
-            if ((rc = ensure_pool(t, std::max<int64_t>(need, 2 * t->cap_pool)))) {
-                cleanup();
-                return rc;
-            }
-        }
-    }
+    Redo r;
+    do {
+        if ((rc = launch_short_walk(t, ps, mode, r_fixed, wblocks)) || (rc = read_state(t))) return rc;
+        if ((rc = plan_redo(t, ps, r, true))) return rc;
+    } while (r.from != Redo::kNone);
     record(t, 7);  // stage times: ms_walk = radii preparation + walk, ms_force = pair pass
-    if (out_on_device) {
-        d_cnt = counts;
-        d_rho = rho;
-    }
-    if ((!d_cnt && cudaMalloc(&d_cnt, sizeof(uint32_t) * n) != cudaSuccess) ||
-        (!d_rho && cudaMalloc(&d_rho, sizeof(double) * n) != cudaSuccess) ||
-        cudaMalloc(&d_info, sizeof(unsigned long long) * 3) != cudaSuccess ||
-        cudaMemsetAsync(d_info, 0, sizeof(unsigned long long) * 3, s) != cudaSuccess) {
+    // outputs the caller does not want still go to the tree's buffers
+    if (out_on_device && (!counts || !rho) && (rc = ensure_short_io(t, n))) return rc;
+    uint32_t* d_cnt = out_on_device && counts ? counts : t->sr_cnt;
+    double* d_rho = out_on_device && rho ? rho : t->sr_rho;
+    if (cudaMemsetAsync(t->sr_info, 0, sizeof(unsigned long long) * 3, s) != cudaSuccess) {
         cudaGetLastError();
-        cleanup();
-        return set_error(ctx, FDPS_ENOMEM, "neighbour output allocation failed");
+        return set_error(ctx, FDPS_ECUDA, "neighbour counters could not be cleared");
     }
-    k_reset_counters<<<1, 32, 0, s>>>(t->st, 2);
-    FDPS_LAUNCH_CHECK(ctx);
-    if ((rc = launch_short_pairs(t, ps, mode, r_fixed, d_cnt, d_rho, d_info))) {
-        cleanup();
-        return rc;
-    }
+    if ((rc = launch_short_pairs(t, ps, mode, r_fixed, d_cnt, d_rho, t->sr_info))) return rc;
     record(t, 8);
     unsigned long long hinfo[3] = {0, 0, 0};
-    cudaError_t e = cudaMemcpyAsync(hinfo, d_info, sizeof(hinfo), cudaMemcpyDeviceToHost, s);
+    cudaError_t e = cudaMemcpyAsync(hinfo, t->sr_info, sizeof(hinfo), cudaMemcpyDeviceToHost, s);
     if (!out_on_device) {
         if (!e && counts) e = cudaMemcpyAsync(counts, d_cnt, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost, s);
         if (!e && rho) e = cudaMemcpyAsync(rho, d_rho, sizeof(double) * n, cudaMemcpyDeviceToHost, s);
     }
     const cudaError_t e2 = cudaStreamSynchronize(s);
-    cleanup();
     if (e || e2) return set_error(ctx, FDPS_ECUDA, "neighbour results copy failed");
     if (info3)
         for (int k = 0; k < 3; ++k) info3[k] = (int64_t)hinfo[k];

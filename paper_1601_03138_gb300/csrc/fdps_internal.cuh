@@ -290,6 +290,12 @@ struct fdps_tree {
     int64_t cap_nd_hmax = 0;
     double* g_hmax = nullptr;
     int64_t cap_g_hmax = 0;
+    // its host arrays' device copies (on first use) and pair counters
+    double* sr_hin = nullptr;
+    uint32_t* sr_cnt = nullptr;
+    double* sr_rho = nullptr;
+    int64_t cap_sr_io = 0;
+    unsigned long long* sr_info = nullptr;
     // coherent sort: the sorted keys of the last call (keys_b) belong to
     // psys coh_ps at generation coh_gen, whose particles are in that order
     bool coh_ok = false;
@@ -353,6 +359,8 @@ struct fdps_tree {
     // state
     fdps::DevState* st = nullptr;   // device
     fdps::DevState h_st{};          // host copy after a call
+    fdps::DevState* h_pin = nullptr;  // page-locked, where the copies arrive
+    cudaEvent_t ev_state = nullptr;   // the state copy of a force calculation has arrived
     fdps::BoxPartial* box_part = nullptr;
     int box_blocks = 0;
     fdps::SysBox* sys_box = nullptr;  // one per system
@@ -419,10 +427,6 @@ inline int grid_for(int64_t n, int block, int max_blocks) {
 // --------------------------------------------------------- stage entry points
 // (host functions, one per .cu file; all issue work on ctx->stream)
 
-// S0-S6 of a force calculation (root box to i-groups, resizing on
-// overflow) and a synchronous read of the device state word (api.cu)
-int run_tree(fdps_tree* t, fdps_psys* ps);
-int read_device_state(fdps_tree* t);
 int keys_and_sort(fdps_tree* t, fdps_psys* ps);        // keys_sort.cu
 int keys_sort_setup(fdps_ctx* ctx);                    // keys_sort.cu: once per context
 int launch_sys_index(fdps_psys* ps);                   // integrate.cu

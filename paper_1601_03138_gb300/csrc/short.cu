@@ -638,8 +638,7 @@ int short_prepare(fdps_tree* t, fdps_psys* ps, int mode, const double* h_user) {
     FDPS_CUDA_TRY(ctx, cudaMemcpyAsync(&bad, ps->d_flag, sizeof(bad), cudaMemcpyDeviceToHost, s));
     FDPS_CUDA_TRY(ctx, cudaStreamSynchronize(s));
     if (bad) return set_error(ctx, FDPS_EINVAL, "cutoff radii must be positive and finite");
-    int rc = read_device_state(t);
-    if (rc) return rc;
+    // (the state word was read after the tree stages)
     const int64_t nn = t->h_st.n_nodes, ng = t->h_st.n_groups;
     if (t->cap_nd_hmax < nn) {
         dev_free(t->nd_hmax);
