@@ -78,7 +78,7 @@ namespace {
 // mixed in the list, every chunk needed a scan and four smaller tiles with
 // two barriers each, about 70 barriers a group instead of 21: the pass over
 // 190,000 monopole groups of 16 particles (256 clusters, n_grp 64) took 7.51
-// ms and takes 6.03, 2^20 Plummer particles with quadrupoles at n_grp 128
+// ms and took 6.02 with 21, 2^20 Plummer particles with quadrupoles at n_grp 128
 // 3.94 and 3.72, 2^24 at n_grp 256 73.2 and 72.0 (FMA pipe 74 % busy: bound by
 // the FP32 pipe and its register-operand conflicts), for 4 % in the walk.
 
@@ -94,8 +94,9 @@ __device__ __forceinline__ GroupPlan plan_group(uint32_t ni) {
     float bu = -1.f;
     // an odd K is packed pairs plus one scalar lane: the scalar lane issues
     // as many instructions per list entry as a pair for half the work, so an
-    // odd K must fill the CTA 6 % better to be taken
-    constexpr float kOdd = 1.06f;
+    // odd K must fill the CTA 10 % better to be taken (2^24 particles: 73.4 ms
+    // with no handicap, 72.3 with 3 %, 72.0 with 6, 71.5 with 10, 71.6 with 15)
+    constexpr float kOdd = 1.1f;
     const int Ks[5] = {5, 4, 3, 2, 1};
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
@@ -267,18 +268,19 @@ __device__ __forceinline__ f2 f2_rsqrt(f2 v) {
 // i-particles are paired (2h, 2h+1) in the two lanes of a packed register;
 // each list entry is broadcast to both lanes.
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
+constexpr int cmin(int a, int b) { return a < b ? a : b; }
 template <bool QUAD, int EPT, int CB, int KMAX>
 struct F32Shared {
     static constexpr int kCE = CB * EPT;  // superparticles per chunk
     static constexpr int kCL = CB * EPT;  // leaves per batch
-    static constexpr int kCJ = 8 * CB < 1024 ? 8 * CB : 1024;  // leaf particles per tile
+    static constexpr int kCJ = cmin((QUAD ? 8 : 4) * CB, 1024);  // leaf particles per tile
     __align__(16) unsigned char u[cmax(kCE * (QUAD ? 40 : 16), kCJ * 16 + 2 * kCL * 4)];
     uint32_t w[2 * (CB / 32)];
     float k[KMAX * 8 * CB];  // Kahan sums and compensations
 };
 __device__ __forceinline__ f2 f2_bc(float v) { return f2_pk(v, v); }
 
-template <bool QUAD, int K, int EPT, int CB, int KMAX>
+template <bool QUAD, int K, int EPT, int CB, int KMAX, int WARPS>
 __device__ __forceinline__ void force_round_f32(const ForceArgs& A, uint32_t gf, uint32_t ni,
                                                 unsigned long long off, uint32_t nspj, uint32_t len, float4 gch,
                                                 float4 gcl, int P, int nsl, uint32_t ib,
@@ -292,11 +294,11 @@ __device__ __forceinline__ void force_round_f32(const ForceArgs& A, uint32_t gf,
     uint32_t* const s_ef = reinterpret_cast<uint32_t*>(sm.u + kCJ * 16);
     uint32_t* const s_es = s_ef + SM::kCL;
     float* const s_k = sm.k;
-    // list entries per loop turn, measured (2, 3, 5, 6 and 1 to 4): quadrupoles
-    // at 2^24 particles 73.5 ms with 2 and 2, 71.9 with 3 and 3; monopoles of
-    // 256 clusters 6.22 ms with 2 and 2, 6.03 with 6 and 2, 7.2 with 3 in the
-    // second loop (registers)
-    constexpr int kUnrollSpj = QUAD ? 5 : 6, kUnrollEpj = QUAD ? 3 : 2;
+    // list entries per loop turn, measured (cells 2 to 10, leaf particles 1 to
+    // 4): quadrupoles at 2^24 particles 73.5 ms with 2 and 2, 72.0 with 5 and 3;
+    // monopoles of 256 clusters 5.39 ms with 6 and 2 at six CTAs per SM, 5.15
+    // with 3 and 2 (3 in the second loop costs registers: 20 % more)
+    constexpr int kUnrollSpj = QUAD ? 5 : WARPS > 16 ? 3 : 6, kUnrollEpj = QUAD ? 3 : 2;
     constexpr int KP = K / 2;  // i-pairs; an odd K takes its last i-particle on the scalar path
     const int t = threadIdx.x;
     const int ip = t % P, sl = t / P;
@@ -544,39 +546,51 @@ __device__ __forceinline__ void force_round_f32(const ForceArgs& A, uint32_t gf,
         __syncthreads();  // chunk buffers are rewritten next
     }
     // ---- combine slices and write back.  A slice's Kahan pair (s, c) is the
-    // double-float s + (-c); the combining thread of a row reads the pairs
-    // of all its slices from the Kahan arrays, adds them with exact
-    // two-sums in FP32 and turns each component into FP64 once (FP64 is a
-    // narrow pipe on this part).  The potential's self term is removed with
-    // the value the list's own entry contributed, m_i rsqrt(eps_i^2) in
-    // FP32, so that the two cancel.
+    // double-float s + (-c); the pairs of a row's slices are added with exact
+    // two-sums in FP32 and each component turned into FP64 once (FP64 is a
+    // narrow pipe on this part).  A thread adds one component of one row, and
+    // where those are fewer than the threads, every parts-th slice of it, the
+    // parts meeting by shuffles (a thread per row, four components and up to
+    // 32 slices each, took a fifth of the time of groups of 16 particles; 256
+    // clusters at n_grp 64: 6.02 -> 5.76 ms).  The potential's self term is removed with the
+    // value the list's own entry contributed, m_i rsqrt(eps_i^2) in FP32, so
+    // that the two cancel.
     const int rows = P * K;  // i-slots of this round: row r = ip + q P
-    __syncthreads();         // every thread's Kahan sums are final
-    for (int r = t; r < rows; r += CB) {
+    const int items = 4 * rows;
+    int parts = 1;
+    while (parts < 32 && 2 * parts <= nsl && 2 * parts * items <= CB) parts *= 2;
+    __syncthreads();  // every thread's Kahan sums are final
+    for (int it0 = 0; it0 < items; it0 += CB / parts) {  // one turn if parts > 1
+        const int it = it0 + t / parts, pt = t & (parts - 1);
+        const int c = it / rows, r = it - c * rows;
         const uint32_t i = ib + (uint32_t)r;
-        if (i >= ni) continue;
-        const int q = r / P, ipr = r - q * P;
-        float hi[4] = {0.0f, 0.0f, 0.0f, 0.0f}, lo[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        for (int s2 = 0; s2 < nsl; ++s2) {
-            const int t2 = s2 * P + ipr;  // the thread of slice s2 holding row r
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                two_sum_acc(hi[c], lo[c], s_k[((q * 4 + c) * 2) * CB + t2]);
-                lo[c] -= s_k[((q * 4 + c) * 2 + 1) * CB + t2];
+        const bool valid = it < items && i < ni;
+        float hi = 0.0f, lo = 0.0f;
+        if (valid) {
+            const int q = r / P, ipr = r - q * P;
+            const float* sk = s_k + ((q * 4 + c) * 2) * CB + ipr;  // of slice s2: sk[s2 P], its compensation CB on
+            for (int s2 = pt; s2 < nsl; s2 += parts) {
+                two_sum_acc(hi, lo, sk[s2 * P]);
+                lo -= sk[s2 * P + CB];
             }
         }
-        const uint32_t p = gf + i;
-        two_sum_acc(hi[3], lo[3], A.pf_hi[p].w * rsqrtf(A.pf_lo[p].w));
-        A.ax[p] = (double)hi[0] + (double)lo[0];
-        A.ay[p] = (double)hi[1] + (double)lo[1];
-        A.az[p] = (double)hi[2] + (double)lo[2];
-        A.pot[p] = (double)hi[3] + (double)lo[3];
+        for (int o = parts >> 1; o > 0; o >>= 1) {
+            const float h2 = __shfl_xor_sync(0xFFFFFFFFu, hi, o), l2 = __shfl_xor_sync(0xFFFFFFFFu, lo, o);
+            two_sum_acc(hi, lo, h2);
+            lo += l2;
+        }
+        if (valid && pt == 0) {
+            const uint32_t p = gf + i;
+            if (c == 3) two_sum_acc(hi, lo, A.pf_hi[p].w * rsqrtf(A.pf_lo[p].w));
+            double* out = c == 0 ? A.ax : c == 1 ? A.ay : c == 2 ? A.az : A.pot;
+            out[p] = (double)hi + (double)lo;
+        }
     }
     __syncthreads();
 }
 
 // Forces on the particles of group g, with the whole CTA.
-template <bool QUAD, int EPT, int CB, int KMAX>
+template <bool QUAD, int EPT, int CB, int KMAX, int WARPS>
 __device__ __forceinline__ void force_group(const ForceArgs& A, uint32_t g, F32Shared<QUAD, EPT, CB, KMAX>& sm) {
     const uint32_t ni = A.g_count[g], gf = A.g_first[g];
     const unsigned long long off = A.g_off[g];
@@ -585,26 +599,33 @@ __device__ __forceinline__ void force_group(const ForceArgs& A, uint32_t g, F32S
     for (uint32_t ib = 0; ib < ni;) {
         const GroupPlan pl = plan_group<CB, KMAX>(ni - ib);
         if (pl.K == 1) {
-            force_round_f32<QUAD, 1, EPT, CB, KMAX>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
+            force_round_f32<QUAD, 1, EPT, CB, KMAX, WARPS>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
         } else if (KMAX >= 5 && pl.K == 5) {
             if constexpr (KMAX >= 5)
-                force_round_f32<QUAD, 5, EPT, CB, KMAX>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
+                force_round_f32<QUAD, 5, EPT, CB, KMAX, WARPS>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
         } else if (KMAX >= 4 && pl.K == 3) {
             if constexpr (KMAX >= 4)
-                force_round_f32<QUAD, 3, EPT, CB, KMAX>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
+                force_round_f32<QUAD, 3, EPT, CB, KMAX, WARPS>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
         } else if (KMAX == 2 || pl.K == 2) {
-            force_round_f32<QUAD, 2, EPT, CB, KMAX>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
+            force_round_f32<QUAD, 2, EPT, CB, KMAX, WARPS>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
         } else {
             if constexpr (KMAX >= 4)
-                force_round_f32<QUAD, 4, EPT, CB, KMAX>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
+                force_round_f32<QUAD, 4, EPT, CB, KMAX, WARPS>(A, gf, ni, off, nspj, len, gch, gcl, pl.P, pl.nsl, ib, sm);
         }
         ib += (uint32_t)(pl.P * pl.K);
     }
 }
 
-// Up to 16 warps per SM (four 128-thread CTAs: 128 registers a thread).
-template <bool QUAD, int EPT, int CB, int KMAX>
-__global__ void __launch_bounds__(CB, (QUAD ? 512 / CB : 1)) k_force_f32(ForceArgs A) {
+// WARPS per SM.  Quadrupoles: 16 (four 128-thread CTAs, 128 registers a
+// thread; with five they spill).  Monopoles: 24 (six CTAs, 80 registers): a
+// third of their time on small groups is the latency of staging, and more
+// CTAs hide it (256 clusters, n_grp 64: 5.76 ms with four CTAs, 5.27 with five,
+// 5.15 with six; 3M clumpy particles, n_grp 256: 2.50, 2.46 and 2.45); but 16
+// where the groups are too few to fill them, up to kFewParticles (16 steps of
+// 2001 particles: 2.41 ms with 16 warps, 2.52 with 24).
+constexpr int64_t kFewParticles = int64_t(1) << 15;
+template <bool QUAD, int EPT, int CB, int KMAX, int WARPS>
+__global__ void __launch_bounds__(CB, 32 * WARPS / CB) k_force_f32(ForceArgs A) {
     __shared__ F32Shared<QUAD, EPT, CB, KMAX> sm;
     __shared__ uint32_t s_g;
     DevState* st = A.st;
@@ -617,7 +638,7 @@ __global__ void __launch_bounds__(CB, (QUAD ? 512 / CB : 1)) k_force_f32(ForceAr
         __syncthreads();
         const uint32_t g = s_g;
         if (g >= ngroups) break;
-        force_group<QUAD, EPT, CB, KMAX>(A, g, sm);
+        force_group<QUAD, EPT, CB, KMAX, WARPS>(A, g, sm);
     }
 }
 
@@ -862,19 +883,19 @@ __global__ void __cluster_dims__(kCl64, 1, 1) __launch_bounds__(kF64Block, 4) k_
 
 // One resident wave of FP32 force CTAs of the given shape (chunk CE
 // entries, CB threads, at most KMAX i-particles a thread).
-template <bool QUAD, int CE, int CB, int KMAX>
+template <bool QUAD, int CE, int CB, int KMAX, int WARPS = QUAD ? 16 : 24>
 void launch_f32(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s) {
     constexpr int EPT = CE / CB;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_force_f32<QUAD, EPT, CB, KMAX>, CB, 0) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_force_f32<QUAD, EPT, CB, KMAX, WARPS>, CB, 0) !=
             cudaSuccess ||
         per_sm < 1)
         per_sm = 1;
-    k_force_f32<QUAD, EPT, CB, KMAX><<<per_sm * ctx->sm_count, CB, 0, s>>>(A);
+    k_force_f32<QUAD, EPT, CB, KMAX, WARPS><<<per_sm * ctx->sm_count, CB, 0, s>>>(A);
 }
 
 template <bool QUAD, int CE>
-void launch_f32_shape(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s, int cb, int kmax) {
+void launch_f32_shape(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s, int cb, int kmax, int64_t n) {
     if (cb == 64) {
         if (kmax == 2)
             launch_f32<QUAD, CE, 64, 2>(A, ctx, s);
@@ -889,6 +910,8 @@ void launch_f32_shape(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s, int cb,
             launch_f32<QUAD, CE, 128, 2>(A, ctx, s);
         else if (kmax == 4)
             launch_f32<QUAD, CE, 128, 4>(A, ctx, s);
+        else if (!QUAD && n <= kFewParticles)
+            launch_f32<QUAD, CE, 128, 5, 16>(A, ctx, s);
         else
             launch_f32<QUAD, CE, 128, 5>(A, ctx, s);
     }
@@ -958,14 +981,14 @@ int compute_forces(fdps_tree* t, fdps_psys* ps, int spj_kind) {
         const int kmax = t->p.i_per_thread ? t->p.i_per_thread : 5;
         if (quad) {
             if (shallow)
-                launch_f32_shape<true, 256>(A, ctx, s, cb, kmax);
+                launch_f32_shape<true, 256>(A, ctx, s, cb, kmax, t->n);
             else
-                launch_f32_shape<true, 512>(A, ctx, s, cb, kmax);
+                launch_f32_shape<true, 512>(A, ctx, s, cb, kmax, t->n);
         } else {
             if (shallow)
-                launch_f32_shape<false, 256>(A, ctx, s, cb, kmax);
+                launch_f32_shape<false, 256>(A, ctx, s, cb, kmax, t->n);
             else
-                launch_f32_shape<false, 512>(A, ctx, s, cb, kmax);
+                launch_f32_shape<false, 512>(A, ctx, s, cb, kmax, t->n);
         }
     }
     FDPS_LAUNCH_CHECK(ctx);
