@@ -221,8 +221,11 @@ __global__ void __launch_bounds__(kSBlock) k_short_walk(ShortWalkArgs A) {
                         if (lane == 0) atomicOr(&st->overflow, kOvfFrontier);
                         ovf = true;
                     } else {
-                        const uint32_t o = nsize + inc - nch;
-                        for (uint32_t c = 0; c < nch; ++c) fb[o + c] = child + c;
+                        // at most 8 stores off one address
+                        uint32_t* f = fb + (nsize + inc - nch);
+#pragma unroll
+                        for (uint32_t c = 0; c < 8; ++c)
+                            if (c < nch) f[c] = child + c;
                         nsize += tot;
                     }
                 }
@@ -368,7 +371,6 @@ struct PairTile {
     float ih2[R ? kSTile : 2];             // 1 / h_j^2
     float mw[R ? kSTile : 2];              // m_j times the kernel's normalisation for h_j
     float lo[R ? kSTile : 2], hi[R ? kSTile : 2], hj[R ? kSTile : 2];
-    uint32_t first[32], start[32];
 };
 __device__ __forceinline__ f2 ld2(const float* a, uint32_t k) { return reinterpret_cast<const f2*>(a)[k]; }
 
@@ -519,22 +521,22 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
                     if (lane >= o) inc += tv;
                 }
                 const uint32_t total = __shfl_sync(0xFFFFFFFFu, inc, 31);
-                __syncwarp();
-                T.first[lane] = u < len ? A.nd_first[node] : 0u;
-                T.start[lane] = inc - c;
-                __syncwarp();
+                const uint32_t first = u < len ? A.nd_first[node] : 0u;
+                const uint32_t start = inc - c;
                 for (uint32_t c0 = 0; c0 < total; c0 += 32) {
                     const uint32_t item = c0 + lane;
+                    // the leaf of each item (none is empty): the leaves that
+                    // start before these 32 items, and among them as bits
+                    const uint32_t before = __popc(__ballot_sync(0xFFFFFFFFu, c > 0u && start < c0));
+                    const uint32_t bits = __reduce_or_sync(
+                        0xFFFFFFFFu, c > 0u && start >= c0 && start < c0 + 32u ? 1u << (start - c0) : 0u);
+                    const int src = (int)(before + __popc(bits & (lt | (1u << lane)))) - 1;
+                    const uint32_t pj = __shfl_sync(0xFFFFFFFFu, first, src) +
+                                        (item - __shfl_sync(0xFFFFFFFFu, start, src));
                     bool keep = false;
                     float4 h4 = make_float4(0.f, 0.f, 0.f, 0.f), l4 = h4;
                     float hj = 0.0f;
-                    uint32_t pj = 0;
                     if (item < total) {
-                        int src = 0;
-#pragma unroll
-                        for (int step = 16; step > 0; step >>= 1)
-                            if (T.start[src + step] <= item) src += step;
-                        pj = T.first[src] + (item - T.start[src]);
                         h4 = A.pf_hi[pj];
                         l4 = A.pf_lo[pj];
                         if (R) hj = (float)A.h[pj];
