@@ -131,10 +131,13 @@ __device__ __forceinline__ void direct_tile(const float4* s_h, const float4* s_l
             const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, f2_fma(dz, dz, e2[q])));
             float ra, rb;
             f2_up(r2, ra, rb);
-            const f2 ri = NORMAL ? f2_pk(rsqrt_normal(ra), rsqrt_normal(rb)) : f2_pk(rsqrtf(ra), rsqrtf(rb));
-            const f2 mj = SELF ? f2_pk((uint32_t)k == rel[2 * q] ? 0.0f : jh.w, (uint32_t)k == rel[2 * q + 1] ? 0.0f : jh.w) : jm;
+            const bool oa = SELF && (uint32_t)k == rel[2 * q], ob = SELF && (uint32_t)k == rel[2 * q + 1];
+            // (the own term of a vanishing eps^2 has an infinite 1/r)
+            const f2 ri = NORMAL ? f2_pk(rsqrt_normal(ra), rsqrt_normal(rb))
+                                 : f2_pk(oa ? 0.0f : rsqrtf(ra), ob ? 0.0f : rsqrtf(rb));
+            const f2 mj = SELF ? f2_pk(oa ? 0.0f : jh.w, ob ? 0.0f : jh.w) : jm;
             const f2 mri = f2_mul(mj, ri);
-            const f2 mri3 = f2_mul(mri, f2_mul(ri, ri));
+            const f2 mri3 = f2_mul(f2_mul(mri, ri), ri);
             ax[q] = f2_fma(mri3, dx, ax[q]);
             ay[q] = f2_fma(mri3, dy, ay[q]);
             az[q] = f2_fma(mri3, dz, az[q]);
