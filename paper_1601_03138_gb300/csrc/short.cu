@@ -121,9 +121,9 @@ __global__ void __launch_bounds__(kSBlock) k_short_walk(ShortWalkArgs A) {
         g = __shfl_sync(0xFFFFFFFFu, g, 0);
         if (g >= ngroups) break;
         const uint32_t sysid = A.sys ? A.sys[A.g_first[g]] : 0u;
-        // grid spacing of the system, squared, in FP32
-        const float dq = (float)(A.box[sysid].L * (1.0 / 2097152.0));
-        const float dq2 = dq * dq;
+        // cutoffs are compared in units of the grid spacing (its square need
+        // not be a normal FP32 number)
+        const float idq = 1.0f / (float)(A.box[sysid].L * (1.0 / 2097152.0));
         const uint32_t* qb = A.g_qbox + 6 * (int64_t)g;
         const uint32_t qmin0 = qb[0], qmin1 = qb[1], qmin2 = qb[2];
         const uint32_t qmax0 = qb[3], qmax1 = qb[4], qmax2 = qb[5];
@@ -169,8 +169,8 @@ __global__ void __launch_bounds__(kSBlock) k_short_walk(ShortWalkArgs A) {
                     const float gx = (float)max(0, max((int)qx - (int)(qmax0 + 1), (int)qmin0 - (int)(qx + w + 1)));
                     const float gy = (float)max(0, max((int)qy - (int)(qmax1 + 1), (int)qmin1 - (int)(qy + w + 1)));
                     const float gz = (float)max(0, max((int)qz - (int)(qmax2 + 1), (int)qmin2 - (int)(qz + w + 1)));
-                    const float d2 = (gx * gx + gy * gy + gz * gz) * dq2;
-                    const float R = short_bound(A.mode, A.r_fixed, hc, hg);
+                    const float d2 = gx * gx + gy * gy + gz * gz;
+                    const float R = short_bound(A.mode, A.r_fixed, hc, hg) * idq;
                     // margin: FP32 rounding of the bound and of the gaps
                     const bool near = d2 <= R * R * (1.0f + 64.0f * kU);
                     if (near) {
