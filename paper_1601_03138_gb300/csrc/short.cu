@@ -21,6 +21,8 @@
 // each candidate pair exactly: an FP32 evaluation on hi/lo parts with a
 // bound on its error settles all but the pairs within the bound of the
 // cutoff, which are decided by the FP64 operation sequence above.
+#include <type_traits>
+
 #include "fdps_internal.cuh"
 
 namespace fdps {
@@ -28,7 +30,7 @@ namespace {
 
 constexpr int kSBlock = 128;
 constexpr int kSW = kSBlock / 32;
-constexpr int kSTile = 96;                 // candidate particles per shared tile (even)
+constexpr int kSTile = 128;                 // candidate particles per shared tile (even)
 constexpr unsigned long long kSChunk = 1ull << 16;
 constexpr float kU = 5.9604645e-08f;      // 2^-24
 // Wendland C6, 3D, support H: W = 1365 / (64 pi H^3) (1-q)^8 (1 + 8q + 25q^2 + 32q^3)
@@ -321,25 +323,34 @@ __device__ __forceinline__ float rsqrt_normal(float v) {
     return r;
 }
 
-// (1 - q)^8 (1 + 8 q + 25 q^2 + 32 q^3) of two candidates at q^2 = x (the
-// Wendland C6 kernel without its normalisation; zero from q = 1 on).  The
+// (1 - q)^8 (1 + 8 q + 25 q^2 + 32 q^3) of two candidates at q^2 = x = r2 / H^2
+// (the Wendland C6 kernel without its normalisation).  nih2 = -1 / H^2.  The
 // root is s = x y, y the reciprocal root, with one Newton correction
-// s + (x - s^2) y / 2 (Heron's iteration); x is kept within 1e-30 (q = 0 to
-// every digit of the result) and 4.
-__device__ __forceinline__ f2 wendland_q2(f2 x) {
+// s + (x - s^2) y / 2 (Heron's iteration), evaluated as -q from -x so that
+// nothing needs a change of sign; x is kept from 0 by 1e-30 (q = 0 to every
+// digit of the result).  CLAMP: x may be anything, and the result is 0 from
+// q = 1 on; otherwise x is at most 2e4 (the result then stays finite, and is
+// read for q <= 1 + 1e-5 only, where (1 - q)^8 vanishes from q = 1 on).
+template <bool CLAMP>
+__device__ __forceinline__ f2 wendland_q2(f2 r2, f2 nih2) {
+    f2 nx = f2_fma(r2, nih2, f2_pk(-1e-30f, -1e-30f));
     float a, b;
-    f2_up(x, a, b);
-    a = fminf(fmaxf(a, 1e-30f), 4.0f);
-    b = fminf(fmaxf(b, 1e-30f), 4.0f);
-    const f2 xc = f2_pk(a, b), y = f2_pk(rsqrt_normal(a), rsqrt_normal(b));
-    const f2 s = f2_mul(xc, y), hy = f2_mul(y, f2_pk(0.5f, 0.5f));
-    const f2 ns = s ^ 0x8000000080000000ull;
-    const f2 q = f2_fma(f2_fma(ns, s, xc), hy, s);
-    f2 u = f2_sub(f2_pk(1.0f, 1.0f), q);
-    f2_up(u, a, b);
-    u = f2_pk(fmaxf(a, 0.0f), fmaxf(b, 0.0f));
+    f2_up(nx, a, b);
+    if (CLAMP) {
+        a = fmaxf(a, -4.0f);
+        b = fmaxf(b, -4.0f);
+        nx = f2_pk(a, b);
+    }
+    const f2 y = f2_pk(rsqrt_normal(-a), rsqrt_normal(-b));
+    const f2 ns = f2_mul(nx, y), hy = f2_mul(y, f2_pk(0.5f, 0.5f));
+    const f2 nq = f2_fma(f2_fma(ns, ns, nx), hy, ns);
+    f2 u = f2_add(f2_pk(1.0f, 1.0f), nq);
+    if (CLAMP) {
+        f2_up(u, a, b);
+        u = f2_pk(fmaxf(a, 0.0f), fmaxf(b, 0.0f));
+    }
     const f2 u2 = f2_mul(u, u), u4 = f2_mul(u2, u2), u8 = f2_mul(u4, u4);
-    const f2 p = f2_fma(q, f2_fma(q, f2_fma(q, f2_pk(32.0f, 32.0f), f2_pk(25.0f, 25.0f)), f2_pk(8.0f, 8.0f)),
+    const f2 p = f2_fma(nq, f2_fma(nq, f2_fma(nq, f2_pk(-32.0f, -32.0f), f2_pk(25.0f, 25.0f)), f2_pk(-8.0f, -8.0f)),
                         f2_pk(1.0f, 1.0f));
     return f2_mul(u8, p);
 }
@@ -368,7 +379,7 @@ template <bool R>
 struct PairTile {
     float xh[kSTile], yh[kSTile], zh[kSTile], xl[kSTile], yl[kSTile], zl[kSTile], m[kSTile];
     uint32_t p[kSTile];
-    float ih2[R ? kSTile : 2];             // 1 / h_j^2
+    float nih2[R ? kSTile : 2];            // -1 / h_j^2
     float mw[R ? kSTile : 2];              // m_j times the kernel's normalisation for h_j
     float lo[R ? kSTile : 2], hi[R ? kSTile : 2], hj[R ? kSTile : 2];
 };
@@ -377,14 +388,20 @@ __device__ __forceinline__ f2 ld2(const float* a, uint32_t k) { return reinterpr
 // One warp per group.  The candidates of the group's list are tested against
 // the group's box (no nearer to any of its particles than to the box) and
 // only those within the largest cutoff that can apply are staged: of 3.4
-// candidates a neighbour (310 neighbours in a uniform cube, groups of 20)
+// candidates a neighbour (310 neighbours in a uniform cube, groups of 8)
 // the walk's leaves give, about 2 remain.  Lanes: P i-slots x nsl slices
 // of the tile, so that small groups keep the whole warp busy; a lane takes
-// two candidates at a time in packed FP32 instructions.  Issue-bound:
-// 3.19 ms for the pair pass of 2^20 particles before,
-// 2.18 with the box test and packed turns (whole call 4.82 -> 3.67 ms); the
-// error of the densities went from 2.1e-7 to 1.4e-7.  MODE is the cutoff type (FDPS_CUTOFF_*), fixed at compile time so
-// that the pair loop carries no selection between them.
+// two candidates at a time in packed FP32 instructions.  Where the cutoff is
+// the i-particle's own and the group's box is at most half of it (nearly
+// always: the groups of a uniform cube are a quarter of it), candidates and
+// i-particles are FP32 coordinates relative to the group's centre, exact to 2u
+// of a separation at the cutoff, instead of hi/lo pairs: a third of the loads
+// and differences; there the kernel's argument is bounded too and needs no
+// clamps.  MODE is the cutoff type (FDPS_CUTOFF_*), fixed at compile time so
+// that the pair loop carries no selection between them.  Issue-bound (78 % of
+// the slots, ALU 61 %): pair pass of 2^20 particles 3.19 ms with one candidate a
+// turn and no box test, 2.18 with them, 1.97 with a candidate's leaf from
+// ballots, 1.64 with the relative coordinates and tiles of 128 (96 before).
 template <int MODE>
 __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
     constexpr bool R = MODE >= 2;
@@ -406,7 +423,9 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
         const float L = (float)A.box[A.sys ? A.sys[gf] : 0u].L;
         const float Eabs = 1e-13f * L;  // error of the FP64 -> FP32 hi/lo parts
         const float4 gch = A.g_ch[g], gcl = A.g_cl[g], blo = A.g_blo[g], bhi = A.g_bhi[g];
-        const float hb = fmaxf(fmaxf(fmaxf(-blo.x, -blo.y), fmaxf(-blo.z, bhi.x)), fmaxf(bhi.y, bhi.z));
+        // the box as half-widths about its centre (as in the gravity walk)
+        const float hx = fmaxf(-blo.x, bhi.x), hy = fmaxf(-blo.y, bhi.y), hz = fmaxf(-blo.z, bhi.z);
+        const float hb = fmaxf(hx, fmaxf(hy, hz));
         // what a cutoff grows by so that the FP32 distance to the box never
         // drops a pair that the thresholds or the FP64 sequence look at: the
         // distance's error is below 4u (C + 2 hb) + 2 Eabs
@@ -419,26 +438,35 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
             const uint32_t i = ib + ip;
             const bool act = sl < nsl && i < ni;
             const uint32_t pi = gf + (act ? i : 0u);
-            const float4 ih = A.pf_hi[pi], il = A.pf_lo[pi];
+            float4 ih = A.pf_hi[pi];
+            const float4 il = A.pf_lo[pi];
             const double hi64 = MODE != 0 ? A.h[pi] : A.r_fixed;
-            const float hif = (float)hi64, invHi = 1.0f / hif, invHi2 = invHi * invHi;
-            const float2 ti = MODE == 2 ? make_float2(0.0f, 0.0f) : pair_thresholds(hif, Eabs);
+            const float hif = (float)hi64, invHi = 1.0f / hif, invHi2 = fminf(invHi * invHi, 3e38f);
+            // FP32 coordinates relative to the group's centre: their rounding, 2u
+            // of |x_i| <= hb and of |x_j| <= hb + a each beside 3u a of the
+            // difference, is within Ea with Eabs + 5u hb in Eabs' place
+            const bool rel = !R && __all_sync(0xFFFFFFFFu, !act || (hb <= 0.5f * hif && hg <= 8.0f * hif && hif > 1e-17f && hif < 1e17f));
+            const float2 ti = MODE == 2 ? make_float2(0.0f, 0.0f)
+                                        : pair_thresholds(hif, rel ? fmaf(5.0f * kU, hb, 2.0f * Eabs) : Eabs);
+            if (rel) ih.x = (ih.x - gch.x) + (il.x - gcl.x), ih.y = (ih.y - gch.y) + (il.y - gcl.y),
+                     ih.z = (ih.z - gch.z) + (il.z - gcl.z);
             const f2 ixh = f2_pk(ih.x, ih.x), iyh = f2_pk(ih.y, ih.y), izh = f2_pk(ih.z, ih.z);
             const f2 ixl = f2_pk(il.x, il.x), iyl = f2_pk(il.y, il.y), izl = f2_pk(il.z, il.z);
-            const f2 iH2 = f2_pk(invHi2, invHi2);
+            const f2 niH2 = f2_pk(-invHi2, -invHi2);
             uint32_t cnt = 0, fbk = 0;
             f2 sum = 0ull, sumj = 0ull;  // sums of m_j w(q) with H = h_i, and with H = h_j
             // the staged candidates 0 .. m - 1 on the warp's i-particles
-            auto pairs = [&](uint32_t m) {
+            auto pairs = [&](auto relc, uint32_t m) {
+                constexpr bool REL = decltype(relc)::value;
                 if ((m & 1u) && lane == 0) {  // an even number: a candidate far from everything, without mass
                     const float far = 16.0f * (hb + hg) + (R ? 16.0f * T.hj[m - 1] : 0.0f);
-                    T.xh[m] = gch.x + far;
-                    T.yh[m] = gch.y;
-                    T.zh[m] = gch.z;
+                    T.xh[m] = REL ? far : gch.x + far;
+                    T.yh[m] = REL ? 0.0f : gch.y;
+                    T.zh[m] = REL ? 0.0f : gch.z;
                     T.xl[m] = T.yl[m] = T.zl[m] = T.m[m] = 0.0f;
                     T.p[m] = 0xFFFFFFFFu;
                     if (R) {
-                        T.ih2[m] = T.ih2[m - 1];
+                        T.nih2[m] = T.nih2[m - 1];
                         T.mw[m] = 0.0f;
                         T.lo[m] = T.lo[m - 1];
                         T.hi[m] = T.hi[m - 1];
@@ -447,11 +475,14 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
                 }
                 __syncwarp();
                 if (act) {
-#pragma unroll 2
+#pragma unroll 1
                     for (uint32_t k = sl; k < (m + 1u) / 2u; k += nsl) {
-                        const f2 dx = f2_add(f2_sub(ld2(T.xh, k), ixh), f2_sub(ld2(T.xl, k), ixl));
-                        const f2 dy = f2_add(f2_sub(ld2(T.yh, k), iyh), f2_sub(ld2(T.yl, k), iyl));
-                        const f2 dz = f2_add(f2_sub(ld2(T.zh, k), izh), f2_sub(ld2(T.zl, k), izl));
+                        f2 dx = f2_sub(ld2(T.xh, k), ixh);
+                        if (!REL) dx = f2_add(dx, f2_sub(ld2(T.xl, k), ixl));
+                        f2 dy = f2_sub(ld2(T.yh, k), iyh);
+                        if (!REL) dy = f2_add(dy, f2_sub(ld2(T.yl, k), iyl));
+                        f2 dz = f2_sub(ld2(T.zh, k), izh);
+                        if (!REL) dz = f2_add(dz, f2_sub(ld2(T.zl, k), izl));
                         const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, f2_mul(dz, dz)));
                         float ra, rb;
                         f2_up(r2, ra, rb);
@@ -496,17 +527,23 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
                         if (MODE != 2) {
                             float ma, mb;
                             f2_up(ld2(T.m, k), ma, mb);
-                            sum = f2_fma(f2_pk(na ? ma : 0.0f, nb ? mb : 0.0f), wendland_q2(f2_mul(r2, iH2)), sum);
+                            sum = f2_fma(f2_pk(na ? ma : 0.0f, nb ? mb : 0.0f), wendland_q2<!REL>(r2, niH2), sum);
                         }
                         if (R) {
                             float ma, mb;
                             f2_up(ld2(T.mw, k), ma, mb);
                             sumj = f2_fma(f2_pk(na ? ma : 0.0f, nb ? mb : 0.0f),
-                                          wendland_q2(f2_mul(r2, ld2(T.ih2, k))), sumj);
+                                          wendland_q2<true>(r2, ld2(T.nih2, k)), sumj);
                         }
                     }
                 }
                 __syncwarp();
+            };
+            auto run = [&](uint32_t m) {
+                if constexpr (!R) {
+                    if (rel) return pairs(std::true_type{}, m);
+                }
+                pairs(std::false_type{}, m);
             };
             uint32_t staged = 0;
             for (uint32_t base = 0; base < len; base += 32) {
@@ -535,34 +572,37 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
                                         (item - __shfl_sync(0xFFFFFFFFu, start, src));
                     bool keep = false;
                     float4 h4 = make_float4(0.f, 0.f, 0.f, 0.f), l4 = h4;
+                    float dx = 0.0f, dy = 0.0f, dz = 0.0f;
                     float hj = 0.0f;
                     if (item < total) {
                         h4 = A.pf_hi[pj];
                         l4 = A.pf_lo[pj];
                         if (R) hj = (float)A.h[pj];
-                        const float dx = (h4.x - gch.x) + (l4.x - gcl.x), dy = (h4.y - gch.y) + (l4.y - gcl.y),
-                                    dz = (h4.z - gch.z) + (l4.z - gcl.z);
-                        const float tx = fmaxf(fmaxf(blo.x - dx, dx - bhi.x), 0.0f);
-                        const float ty = fmaxf(fmaxf(blo.y - dy, dy - bhi.y), 0.0f);
-                        const float tz = fmaxf(fmaxf(blo.z - dz, dz - bhi.z), 0.0f);
+                        dx = (h4.x - gch.x) + (l4.x - gcl.x);
+                        dy = (h4.y - gch.y) + (l4.y - gcl.y);
+                        dz = (h4.z - gch.z) + (l4.z - gcl.z);
+                        const float tx = fmaxf(fabsf(dx) - hx, 0.0f), ty = fmaxf(fabsf(dy) - hy, 0.0f),
+                                    tz = fmaxf(fabsf(dz) - hz, 0.0f);
                         const float C = fmaf(fmaxf(hg, hj), 1.0f + 256.0f * kU, pad);
                         keep = !(fmaf(tx, tx, fmaf(ty, ty, tz * tz)) > C * C);
                     }
                     const uint32_t mask = __ballot_sync(0xFFFFFFFFu, keep);
                     if (keep) {
                         const uint32_t k = staged + __popc(mask & lt);
-                        T.xh[k] = h4.x;
-                        T.yh[k] = h4.y;
-                        T.zh[k] = h4.z;
-                        T.xl[k] = l4.x;
-                        T.yl[k] = l4.y;
-                        T.zl[k] = l4.z;
+                        T.xh[k] = rel ? dx : h4.x;
+                        T.yh[k] = rel ? dy : h4.y;
+                        T.zh[k] = rel ? dz : h4.z;
+                        if (!rel) {
+                            T.xl[k] = l4.x;
+                            T.yl[k] = l4.y;
+                            T.zl[k] = l4.z;
+                        }
                         T.m[k] = h4.w;
                         T.p[k] = pj;
                         if (R) {
                             const float ihj = 1.0f / hj;
                             const float2 tj = pair_thresholds(hj, Eabs);
-                            T.ih2[k] = ihj * ihj;
+                            T.nih2[k] = -fminf(ihj * ihj, 3e38f);
                             T.mw[k] = h4.w * (kWc6 * ihj * ihj * ihj);
                             T.lo[k] = tj.x;
                             T.hi[k] = tj.y;
@@ -571,12 +611,12 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
                     }
                     staged += __popc(mask);
                     if (staged > (uint32_t)kSTile - 33u) {  // room for the next 32 and the padding
-                        pairs(staged);
+                        run(staged);
                         staged = 0;
                     }
                 }
             }
-            if (staged) pairs(staged);
+            if (staged) run(staged);
             // the lane's two halves and the slices' partial counts and sums,
             // into the first slice
             float sa, sb, ja, jb;
