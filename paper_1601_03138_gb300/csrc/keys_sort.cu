@@ -585,14 +585,15 @@ __device__ __forceinline__ bool coh_less(unsigned long long ka, uint32_t ia, uns
     return ka < kb || (ka == kb && ia < ib);
 }
 
-// Merge sort of kCohBlock * EPT pairs in buffer 0: each thread sorts its
+// Merge sort of BLOCK * EPT pairs in buffer 0: each thread sorts its
 // EPT consecutive pairs in registers, then every round merges runs of
 // length L pairwise (L = EPT, 2 EPT, ...), each thread writing EPT
 // consecutive outputs from the split of its output diagonal found by
 // binary search (merge path).  Returns the buffer holding the result.
-template <int EPT>
+template <int BLOCK, int EPT>
 __device__ __noinline__ int merge_sort_pairs(CohShared& sm) {
-    constexpr int np = kCohBlock * EPT;
+    constexpr int np = BLOCK * EPT;
+    static_assert(np <= kCohCap, "fits the buffers");
     const int o = threadIdx.x * EPT;
     {
         unsigned long long k[EPT];
@@ -667,16 +668,21 @@ __device__ __noinline__ int merge_sort_pairs(CohShared& sm) {
     return src;
 }
 
+template <int BLOCK>
 __device__ __forceinline__ int merge_sort_block(CohShared& sm, int ept) {
+    if constexpr (8 * BLOCK <= kCohCap) {
+        switch (ept) {
+            case 5: return merge_sort_pairs<BLOCK, 5>(sm);
+            case 6: return merge_sort_pairs<BLOCK, 6>(sm);
+            case 7: return merge_sort_pairs<BLOCK, 7>(sm);
+            case 8: return merge_sort_pairs<BLOCK, 8>(sm);
+        }
+    }
     switch (ept) {
-        case 1: return merge_sort_pairs<1>(sm);
-        case 2: return merge_sort_pairs<2>(sm);
-        case 3: return merge_sort_pairs<3>(sm);
-        case 4: return merge_sort_pairs<4>(sm);
-        case 5: return merge_sort_pairs<5>(sm);
-        case 6: return merge_sort_pairs<6>(sm);
-        case 7: return merge_sort_pairs<7>(sm);
-        default: return merge_sort_pairs<8>(sm);
+        case 1: return merge_sort_pairs<BLOCK, 1>(sm);
+        case 2: return merge_sort_pairs<BLOCK, 2>(sm);
+        case 3: return merge_sort_pairs<BLOCK, 3>(sm);
+        default: return merge_sort_pairs<BLOCK, 4>(sm);
     }
 }
 
@@ -704,7 +710,7 @@ __global__ void __launch_bounds__(kCohBlock) k_coh_sort(const uint32_t* __restri
     }
     __syncthreads();
     static_assert(kCohCap == 8 * kCohBlock, "at most 8 pairs a thread");
-    const int src = merge_sort_block(sm, ept);
+    const int src = merge_sort_block<kCohBlock>(sm, ept);
     for (int j = threadIdx.x; j < m; j += kCohBlock) {
         keys_out[a0 + j] = sm.k[src][coh_kp(j)];
         perm_out[a0 + j] = sm.i[src][coh_ip(j)];
@@ -732,7 +738,7 @@ __global__ void __launch_bounds__(kCohBlock) k_tile_sort(int64_t n, const double
         sm.i[0][coh_ip(j)] = j < m ? (uint32_t)(a0 + j) : 0xFFFFFFFFu;
     }
     __syncthreads();
-    const int src = merge_sort_block(sm, ept);
+    const int src = merge_sort_block<kCohBlock>(sm, ept);
     for (int j = threadIdx.x; j < m; j += kCohBlock) {
         keys_out[a0 + j] = sm.k[src][coh_kp(j)];
         perm_out[a0 + j] = sm.i[src][coh_ip(j)];
@@ -762,6 +768,7 @@ __device__ __forceinline__ int merge_split(const uint64_t* a, int la, const uint
 // inputs are staged in shared memory, each thread merges EPT outputs.  The
 // runs hold consecutive positions, so taking equal keys from the first run
 // keeps the sort stable.
+template <int BLOCK>
 __device__ __forceinline__ void merge_tile(CohShared& sm, int64_t n, int64_t L, int T, int64_t o0,
                                            const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
                                            uint32_t* vout) {
@@ -778,13 +785,13 @@ __device__ __forceinline__ void merge_tile(CohShared& sm, int64_t n, int64_t L, 
     }
     __syncthreads();
     const int ia0 = s_split[0], na = s_split[1] - ia0, ib0 = d0 - ia0, m = d1 - d0, nb = m - na;
-    for (int j = t; j < m; j += kCohBlock) {
+    for (int j = t; j < m; j += BLOCK) {
         const int64_t p = j < na ? a0 + ia0 + j : a0 + la + ib0 + (j - na);
         sm.k[0][coh_kp(j)] = __ldcg(kin + p);
         sm.i[0][coh_ip(j)] = __ldcg(vin + p);
     }
     __syncthreads();
-    const int ept = (m + kCohBlock - 1) / kCohBlock;
+    const int ept = (m + BLOCK - 1) / BLOCK;
     const int d = t * ept;
     if (d < m) {
         const unsigned long long* K = sm.k[0];
@@ -808,7 +815,7 @@ __device__ __forceinline__ void merge_tile(CohShared& sm, int64_t n, int64_t L, 
         }
     }
     __syncthreads();
-    for (int j = t; j < m; j += kCohBlock) {
+    for (int j = t; j < m; j += BLOCK) {
         kout[o0 + j] = sm.k[1][coh_kp(j)];
         vout[o0 + j] = sm.i[1][coh_ip(j)];
     }
@@ -819,7 +826,7 @@ __global__ void __launch_bounds__(kCohBlock) k_merge_runs(int64_t n, int64_t L, 
                                                           const uint32_t* __restrict__ vin,
                                                           uint64_t* __restrict__ kout, uint32_t* __restrict__ vout) {
     extern __shared__ __align__(16) unsigned char coh_dsm[];
-    merge_tile(*reinterpret_cast<CohShared*>(coh_dsm), n, L, kSortTile, blockIdx.x * (int64_t)kSortTile, kin, vin,
+    merge_tile<kCohBlock>(*reinterpret_cast<CohShared*>(coh_dsm), n, L, kSortTile, blockIdx.x * (int64_t)kSortTile, kin, vin,
                kout, vout);
 }
 
@@ -835,7 +842,12 @@ __global__ void __launch_bounds__(kCohBlock) k_merge_runs(int64_t n, int64_t L, 
 // null.  4099 particles through the allocation-free entry point: 199 -> 26 us.
 constexpr int kSmallCl = 8;
 constexpr int64_t kSmallMax = kSmallCl * kSortTile;
-__global__ void __cluster_dims__(kSmallCl, 1, 1) __launch_bounds__(kCohBlock)
+// 256 threads a CTA up to here, 512 (fewer pairs a thread, dearer barriers)
+// beyond: 18.5 against 20.6 us for 2001 particles, 26.7 / 28.6 for 6000, 27.7 /
+// 26.7 for 8192, 40.5 / 36.9 for 16384.
+constexpr int64_t kSmallHalf = 8192;
+template <int BLOCK>
+__global__ void __cluster_dims__(kSmallCl, 1, 1) __launch_bounds__(BLOCK)
     k_sort_small(int n, const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
                  DevState* st, SysBox* box, uint64_t* __restrict__ keys_in, uint64_t* k0, uint32_t* v0, uint64_t* k1,
                  uint32_t* v1) {
@@ -849,7 +861,7 @@ __global__ void __cluster_dims__(kSmallCl, 1, 1) __launch_bounds__(kCohBlock)
     const int a0 = (int)rank * T;
     const int m = n - a0 < T ? (n > a0 ? n - a0 : 0) : T;
     unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
-    for (int j = t; j < m; j += kCohBlock) {
+    for (int j = t; j < m; j += BLOCK) {
         const unsigned long long v[3] = {ord64(x[a0 + j]), ord64(y[a0 + j]), ord64(z[a0 + j])};
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -857,7 +869,7 @@ __global__ void __cluster_dims__(kSmallCl, 1, 1) __launch_bounds__(kCohBlock)
             hi[a] = v[a] > hi[a] ? v[a] : hi[a];
         }
     }
-    block_minmax<kCohWarps>(lo, hi);
+    block_minmax<BLOCK / 32>(lo, hi);
     if (t == 0)
         for (int a = 0; a < 3; ++a) {
             s_mm[a] = lo[a];
@@ -894,8 +906,8 @@ __global__ void __cluster_dims__(kSmallCl, 1, 1) __launch_bounds__(kCohBlock)
     }
     __syncthreads();
     const SysBox b = s_box;
-    const int ept = (m + kCohBlock - 1) / kCohBlock;
-    for (int j = t; j < ept * kCohBlock; j += kCohBlock) {
+    const int ept = (m + BLOCK - 1) / BLOCK;
+    for (int j = t; j < ept * BLOCK; j += BLOCK) {
         unsigned long long k = ~0ull;
         if (j < m) {
             k = morton_key(x[a0 + j], y[a0 + j], z[a0 + j], b);
@@ -905,10 +917,10 @@ __global__ void __cluster_dims__(kSmallCl, 1, 1) __launch_bounds__(kCohBlock)
         sm.i[0][coh_ip(j)] = j < m ? (uint32_t)(a0 + j) : 0xFFFFFFFFu;
     }
     __syncthreads();
-    const int src = merge_sort_block(sm, ept > 0 ? ept : 1);
+    const int src = merge_sort_block<BLOCK>(sm, ept > 0 ? ept : 1);
     // three rounds: scratch, result, scratch, result
     static_assert(kSmallCl == 8, "three merge rounds");
-    for (int j = t; j < m; j += kCohBlock) {
+    for (int j = t; j < m; j += BLOCK) {
         k1[a0 + j] = sm.k[src][coh_kp(j)];
         v1[a0 + j] = sm.i[src][coh_ip(j)];
     }
@@ -919,7 +931,7 @@ __global__ void __cluster_dims__(kSmallCl, 1, 1) __launch_bounds__(kCohBlock)
     for (int r = 0; r < 3; ++r) {
         __threadfence();
         cluster_barrier();  // the runs are written
-        if (m > 0) merge_tile(sm, n, (int64_t)T << r, T, a0, ki, vi, ko, vo);
+        if (m > 0) merge_tile<BLOCK>(sm, n, (int64_t)T << r, T, a0, ki, vi, ko, vo);
         uint64_t* tk = ki;
         ki = ko;
         ko = tk;
@@ -934,7 +946,10 @@ __global__ void __cluster_dims__(kSmallCl, 1, 1) __launch_bounds__(kCohBlock)
 
 int launch_sort_small(int64_t n, const double* x, const double* y, const double* z, DevState* st, SysBox* box,
                       uint64_t* keys_in, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, cudaStream_t s) {
-    k_sort_small<<<kSmallCl, kCohBlock, sizeof(CohShared), s>>>((int)n, x, y, z, st, box, keys_in, k0, v0, k1, v1);
+    if (n <= kSmallHalf)
+        k_sort_small<256><<<kSmallCl, 256, sizeof(CohShared), s>>>((int)n, x, y, z, st, box, keys_in, k0, v0, k1, v1);
+    else
+        k_sort_small<512><<<kSmallCl, 512, sizeof(CohShared), s>>>((int)n, x, y, z, st, box, keys_in, k0, v0, k1, v1);
     return cudaPeekAtLastError() == cudaSuccess ? FDPS_OK : FDPS_ECUDA;
 }
 
@@ -946,7 +961,9 @@ bool pair_sort_setup() {
                cudaSuccess &&
            cudaFuncSetAttribute(k_merge_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CohShared)) ==
                cudaSuccess &&
-           cudaFuncSetAttribute(k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CohShared)) ==
+           cudaFuncSetAttribute(k_sort_small<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CohShared)) ==
+               cudaSuccess &&
+           cudaFuncSetAttribute(k_sort_small<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CohShared)) ==
                cudaSuccess;
 }
 
