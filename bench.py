@@ -102,7 +102,7 @@ def parse():
 # bench reports null once that source has changed
 FORCE_TRAFFIC = {
     "hernquist N=16777216 theta=0.5 quad n_leaf=16 n_grp=256 eps=0.005 dt=0.00195312":
-        ("fd36d91a7f88cc47", 4.3238e9 + 532.26e6),
+        ("9b162e165d74a8a3", 4.3133e9 + 532.50e6),
 }
 
 

@@ -798,7 +798,7 @@ __device__ __forceinline__ void force_round_f64(const ForceArgs& A, uint32_t gf,
                     const double r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, e2[q])));
                     const double ri = rsqrt(r2);
                     const double mri = j.w * ri;
-                    const double mri3 = mri * (ri * ri);
+                    const double mri3 = mri * ri * ri;
                     ax[q] = fma(mri3, dx, ax[q]);
                     ay[q] = fma(mri3, dy, ay[q]);
                     az[q] = fma(mri3, dz, az[q]);
