@@ -22,7 +22,8 @@
  *
  * Each thread owns one i-particle; it calls the functors with tiles of up
  * to 64 particles of opened leaves (EPJ) and up to 32 superparticles (SPJ),
- * which together make the i-particle's group's whole list, in list order.
+ * which together make the i-particle's group's whole list, from its end (the
+ * opened leaves) to its start (the coarsest cells) in steps of 32 entries.
  * The particle itself is among its EPJ (zero separation): the law decides
  * what that term contributes.  Positions are FP32 relative to the group's
  * centre, formed from hi/lo parts as in the built-in kernel.  out[row] gets
@@ -118,8 +119,11 @@ __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const F
             }
             Force f;
             f.clear();
-            for (uint32_t base = 0; base < len; base += kThreads) {
-                const uint32_t u = base + t;
+            // from the list's end, the opened leaves, to its start, the coarsest
+            // cells: a law's running sums are short while the many particles
+            // of the leaves are added
+            for (uint32_t left = (len + kThreads - 1) / kThreads; left-- > 0;) {
+                const uint32_t u = left * kThreads + t;
                 const bool valid = u < len;
                 const uint32_t e = valid ? v.pool[off + u] : 0u;
                 const bool leaf = valid && (e & v.leaf_tag);
