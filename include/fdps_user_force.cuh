@@ -22,8 +22,8 @@
  *
  * Each thread owns one i-particle; it calls the functors with tiles of up
  * to 64 particles of opened leaves (EPJ) and up to 32 superparticles (SPJ),
- * which together make the i-particle's group's whole list, from its end (the
- * opened leaves) to its start (the coarsest cells) in steps of 32 entries.
+ * which together make the i-particle's group's whole list, the superparticles
+ * and the opened leaves each in list order, in turn.
  * The particle itself is among its EPJ (zero separation): the law decides
  * what that term contributes.  Positions are FP32 relative to the group's
  * centre, formed from hi/lo parts as in the built-in kernel.  out[row] gets
@@ -105,6 +105,20 @@ __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const F
         const unsigned long long off = v.g_off[g];
         const uint32_t len = v.g_len[g];
         const float4 ch = ld4(v.g_ch, (uint64_t)g), cl = ld4(v.g_cl, (uint64_t)g);
+        // steps of kThreads entries, the first nsp of them with superparticles
+        // (a list holds its superparticles before its leaves): every lane
+        // probes one of 32 steps until none is left between two of them
+        const uint32_t steps = (len + kThreads - 1) / kThreads;
+        uint32_t nsp = 0;
+        for (uint32_t n = steps; n > 0;) {
+            const uint32_t stride = (n + 31) / 32, at = lane * stride;
+            const bool sp = at < n && !(v.pool[off + (uint64_t)(nsp + at) * kThreads] & v.leaf_tag);
+            const uint32_t c = __popc(__ballot_sync(0xFFFFFFFFu, sp));
+            if (c == 0) break;
+            const uint32_t past = (c - 1) * stride + 1, end = c * stride < n ? c * stride : n;
+            nsp += past;
+            n = end - past;
+        }
         for (uint32_t ib = blockIdx.y * kThreads; ib < ni; ib += kThreads * gridDim.y) {
             const uint32_t i = ib + t;
             const bool act = i < ni;
@@ -119,11 +133,14 @@ __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const F
             }
             Force f;
             f.clear();
-            // from the list's end, the opened leaves, to its start, the coarsest
-            // cells: a law's running sums are short while the many particles
-            // of the leaves are added
-            for (uint32_t left = (len + kThreads - 1) / kThreads; left-- > 0;) {
-                const uint32_t u = left * kThreads + t;
+            // steps with superparticles and steps with leaves in turn, in
+            // proportion: a law's plain sums round with every entry, by more
+            // the larger they are, and either kind last costs up to half as
+            // much error again
+            uint32_t ks = 0, kl = 0;
+            while (ks + kl < steps) {
+                const bool cells = kl == steps - nsp || (ks < nsp && (uint64_t)ks * (steps - nsp) <= (uint64_t)kl * nsp);
+                const uint32_t u = (cells ? ks++ : nsp + kl++) * kThreads + t;
                 const bool valid = u < len;
                 const uint32_t e = valid ? v.pool[off + u] : 0u;
                 const bool leaf = valid && (e & v.leaf_tag);
