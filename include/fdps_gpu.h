@@ -117,7 +117,8 @@ typedef struct {
     int64_t fp64_fallbacks;    /* opening tests decided in FP64 */
     int64_t retries;           /* buffer resize-and-retry count */
     int64_t sort_coherent;     /* 1: the last sort was the coherent time-step
-                                  sort, 0: the radix sort */
+                                  sort, 0: the radix sort, or the one-launch
+                                  merge sort of up to 16384 particles */
     double ms_box_keys;        /* root box + Morton keys */
     double ms_sort;            /* sort (after the keys) */
     double ms_permute;         /* reorder into key order */
@@ -148,8 +149,8 @@ int fdps_set_stream(fdps_ctx* ctx, void* stream);
 /* Number of CUDA kernels this library has launched on the context so far
    (-1 for NULL). */
 int64_t fdps_kernel_launches(const fdps_ctx* ctx);
-/* Diagnostic of the failure path of the library's one kind of device-side
-   wait (the radix sort's look-back on earlier tiles, bounded to about 2^20
+/* Diagnostic of the failure path of the library's device-side waits, on
+   the radix sort's (its look-back on earlier tiles, bounded to about 2^20
    polls): runs a single look-back whose predecessor never publishes.
    Returns FDPS_ETIMEOUT when the wait gave up and reported it, as designed;
    the context stays usable.  Any other result is a fault of the library. */
@@ -203,7 +204,7 @@ int fdps_tree_create(fdps_ctx* ctx, const fdps_tree_params* params,
 int fdps_tree_destroy(fdps_tree* tree);
 
 /* calcForceAllAndWriteBack (Sect. 2.2; steps of Sect. 3.2 on one GPU):
-   root box -> Morton keys -> radix sort -> reorder -> octree -> moments ->
+   root box -> Morton keys -> sort -> reorder -> octree -> moments ->
    i-groups -> interaction lists -> forces, written back into ps
    (acceleration and potential of every particle, overwriting old values).
    k_epj must be FDPS_GRAV_EPJ; k_spj FDPS_GRAV_SPJ_MONO, or
@@ -453,7 +454,7 @@ int fdps_user_law_destroy(fdps_user_law* law);
    real-time loops that may not take the implicit synchronisation and
    unbounded latency of a cudaMalloc / cudaFree.  It computes what
    fdps_tree_calc_force_all_and_write_back
-   computes first (root box, 63-bit Morton keys, stable radix sort) for one
+   computes first (root box, 63-bit Morton keys, stable merge sort) for one
    particle set and allocates nothing: its scratch (about 3.2 MB) is a
    file-scope device array that every GPU which loads the library holds
    until the process exits.

@@ -694,7 +694,7 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
 // at most kTopNodes nodes.  Systems of an ensemble go through the same passes (one CTA
 // per system before: 256 clusters of 256 to 65536 particles waited for the
 // largest).  The sums of a node keep their order, so results do not depend
-// on the split.  Moments of Plummer 2^14: 136 -> 55 us; of
+// on the split.  Moments of Plummer 2^14: 136 -> 49 us; of
 // Plummer 2^20 with quadrupoles 246 -> 168 us; of the 256 clusters 1.18 ->
 // 0.27 ms.
 constexpr int kMomBlock = 256;
