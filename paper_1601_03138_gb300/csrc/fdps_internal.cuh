@@ -166,8 +166,9 @@ __device__ __forceinline__ float to_f32(double v) {
     return hi;
 }
 
-// Thread-block clusters: a barrier over the cluster's threads (release and
-// acquire), the block's rank, and reads of a peer block's shared memory.
+// Thread-block clusters: a barrier over the cluster's threads (its arrive
+// releases and its wait acquires at cluster scope, global memory included, so
+// no fence stands beside it), the block's rank, and reads of a peer block's shared memory.
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
 }

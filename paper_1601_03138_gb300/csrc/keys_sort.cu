@@ -839,12 +839,12 @@ __global__ void __launch_bounds__(kCohBlock) k_merge_runs(int64_t n, int64_t L, 
 // ends in k0, v0).  One CTA alone took 50 us for 4099 particles, its SM's two
 // FP64 lanes 6 us for the keys and its issue slots most of the rest.  st (the
 // box's copy in the state word), box and keys_in (keys in input order) may be
-// null.  4099 particles through the allocation-free entry point: 199 -> 26 us.
+// null.  4099 particles through the allocation-free entry point: 199 -> 25 us.
 constexpr int kSmallCl = 8;
 constexpr int64_t kSmallMax = kSmallCl * kSortTile;
 // 256 threads a CTA up to here, 512 (fewer pairs a thread, dearer barriers)
 // beyond: 18.5 against 20.6 us for 2001 particles, 26.7 / 28.6 for 6000, 27.7 /
-// 26.7 for 8192, 40.5 / 36.9 for 16384.
+// 26.7 for 8192, 40.5 / 36.9 for 16384 (both with a fence before each merge round).
 constexpr int64_t kSmallHalf = 8192;
 template <int BLOCK>
 __global__ void __cluster_dims__(kSmallCl, 1, 1) __launch_bounds__(BLOCK)
@@ -929,7 +929,6 @@ __global__ void __cluster_dims__(kSmallCl, 1, 1) __launch_bounds__(BLOCK)
     uint64_t* ko = k0;
     uint32_t* vo = v0;
     for (int r = 0; r < 3; ++r) {
-        __threadfence();
         cluster_barrier();  // the runs are written
         if (m > 0) merge_tile<BLOCK>(sm, n, (int64_t)T << r, T, a0, ki, vi, ko, vo);
         uint64_t* tk = ki;
