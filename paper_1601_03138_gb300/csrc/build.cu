@@ -510,10 +510,9 @@ struct MomArgs {
 // positions relative to the node's COM formed from FP32 hi/lo pairs, and the
 // parallel-axis shift for internal nodes.
 // AHEAD: a node's children are all loaded before the first is summed (where
-// latency counts and registers are free).  PART: everything, only the sums M
-// and S (all that a parent needs of a monopole tree), or only what follows
-// from them.
-enum MomPart { kMomAll, kMomSums, kMomFinish };
+// latency counts and registers are free).  PART: everything, or only what
+// follows from the sums M and S (kept in the node by k_moments_small).
+enum MomPart { kMomAll, kMomFinish };
 template <bool QUAD, bool Q64, bool AHEAD, MomPart PART = kMomAll>
 __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
     const uint32_t meta = A.nd_meta[i];
@@ -565,10 +564,6 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
         A.nd_sx[i] = Sx;
         A.nd_sy[i] = Sy;
         A.nd_sz[i] = Sz;
-    }
-    if (PART == kMomSums) {
-        A.nd_com[i].w = M;
-        return;
     }
     double cx = 0.0, cy = 0.0, cz = 0.0;
     if (M > 0.0) {
@@ -694,7 +689,7 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
 // at most kTopNodes nodes.  Systems of an ensemble go through the same passes (one CTA
 // per system before: 256 clusters of 256 to 65536 particles waited for the
 // largest).  The sums of a node keep their order, so results do not depend
-// on the split.  Moments of Plummer 2^14: 136 -> 49 us; of
+// on the split.  Moments of Plummer 2^14: 136 -> 39 us; of
 // Plummer 2^20 with quadrupoles 246 -> 168 us; of the 256 clusters 1.18 ->
 // 0.27 ms.
 constexpr int kMomBlock = 256;
@@ -749,8 +744,12 @@ __global__ void __launch_bounds__(kMomBlock) k_moments_leaves(MomArgs A) {
 
 // (A monopole tree's levels pass on the sums alone: the division and the FP32
 // copies, two thirds of a node's chain of FP64 operations, follow for all
-// internal nodes at once: moments of 2^14 Plummer particles 55 -> 49 us, of 2001
-// 39 -> 35.  A quadrupole needs its children's centres.)
+// internal nodes at once.  Four lanes share a node, one for each of M, Sx, Sy
+// and Sz: a level's few nodes are a chain of loads and FP64 additions whose
+// length counts, not their number; and a lane reads its node of the next level
+// and that node's children's ids before it waits for this level.  Moments of
+// 2^14 Plummer particles 55 -> 39 us, of 2001 39 -> 27 (49 and 35 with one lane a
+// node and nothing read ahead).  A quadrupole needs its children's centres.)
 template <bool QUAD, bool Q64>
 __global__ void __cluster_dims__(kMomCl, 1, 1) __launch_bounds__(kMomBlock) k_moments_small(MomArgs A) {
     __shared__ int32_t s_lvl[kMaxLevel + 3];
@@ -758,14 +757,47 @@ __global__ void __cluster_dims__(kMomCl, 1, 1) __launch_bounds__(kMomBlock) k_mo
     const int top = A.st->max_level - 1;
     __syncthreads();
     const int t = blockIdx.x * kMomBlock + threadIdx.x;
+    if (top < 0) return;  // (the whole cluster)
+    // monopoles: four lanes a node, one for each of M, Sx, Sy, Sz
+    constexpr int kLanes = QUAD ? 1 : 4, kNodes = kMomCl * kMomBlock / kLanes;
+    const int comp = t % 4;
+    double* const sum = comp == 0 ? &A.nd_com[0].w : comp == 1 ? A.nd_sx : comp == 2 ? A.nd_sy : A.nd_sz;
+    const int64_t stride = comp == 0 ? 4 : 1;
+    int next = s_lvl[top] + t / kLanes;
+    uint32_t next_meta = next < s_lvl[top + 1] ? A.nd_meta[next] : 0u;
+    uint32_t next_child = next < s_lvl[top + 1] ? A.nd_child[next] : 0u;
     for (int l = top; l >= 0; --l) {
-        for (int i = s_lvl[l] + t; i < s_lvl[l + 1]; i += kMomCl * kMomBlock)
-            if (!meta_leaf(A.nd_meta[i])) node_moments<QUAD, Q64, true, QUAD ? kMomAll : kMomSums>(A, i);
-        __threadfence();
+        int i = next;
+        uint32_t meta = next_meta, child = next_child;
+        if (l > 0) {
+            next = s_lvl[l - 1] + t / kLanes;
+            next_meta = next < s_lvl[l] ? A.nd_meta[next] : 0u;
+            next_child = next < s_lvl[l] ? A.nd_child[next] : 0u;
+        }
+        while (i < s_lvl[l + 1]) {
+            if (meta_leaf(meta)) {
+            } else if (QUAD) {
+                node_moments<QUAD, Q64, true>(A, i);
+            } else {
+                const int nc = (int)meta_nchild(meta);
+                double v[8], S = 0.0;
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    v[k] = __ldcg(sum + (int64_t)(k < nc ? child + k : (uint32_t)i) * stride);
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (k < nc) S = __dadd_rn(S, v[k]);
+                sum[i * stride] = S;
+            }
+            i += kNodes;
+            if (i >= s_lvl[l + 1]) break;
+            meta = A.nd_meta[i];
+            child = A.nd_child[i];
+        }
         cluster_barrier();  // this level complete before its parents
     }
     if (!QUAD)
-        for (int i = t; i < (top < 0 ? 0 : s_lvl[top + 1]); i += kMomCl * kMomBlock)
+        for (int i = t; i < s_lvl[top + 1]; i += kMomCl * kMomBlock)
             if (!meta_leaf(A.nd_meta[i])) node_moments<QUAD, Q64, true, kMomFinish>(A, i);
 }
 
