@@ -108,17 +108,16 @@ __device__ __forceinline__ float rsqrt_normal(float v) {
     return r;
 }
 
-// One tile of m j-particles, entries kbeg, kbeg + kstep, ... of it, on the
-// 2 KP i-particles of a thread.  SELF: an i-particle of the warp is in the
+// One tile of m j-particles on the 2 KP i-particles of a thread.  SELF: an i-particle of the warp is in the
 // tile (at rel), and its own term gets no mass.  NORMAL: every eps^2
 // of the warp is a normal FP32 number, so every r^2 is.
 template <int KP, bool SELF, bool NORMAL>
-__device__ __forceinline__ void direct_tile(const float4* s_h, const float4* s_l, int m, int kbeg, int kstep,
+__device__ __forceinline__ void direct_tile(const float4* s_h, const float4* s_l, int m,
                                             const uint32_t* rel, const f2* hx, const f2* hy, const f2* hz,
                                             const f2* lx, const f2* ly, const f2* lz, const f2* e2, f2* ax, f2* ay,
                                             f2* az, f2* pp) {
 #pragma unroll 2
-    for (int k = kbeg; k < m; k += kstep) {
+    for (int k = 0; k < m; ++k) {
         const float4 jh = s_h[k], jl = s_l[k];
         const f2 jx = f2_pk(jh.x, jh.x), jy = f2_pk(jh.y, jh.y), jz = f2_pk(jh.z, jh.z);
         const f2 kx = f2_pk(jl.x, jl.x), ky = f2_pk(jl.y, jl.y), kz = f2_pk(jl.z, jl.z);
@@ -146,24 +145,37 @@ __device__ __forceinline__ void direct_tile(const float4* s_h, const float4* s_l
     }
 }
 
+// The j range in tiles of up to kDT: slices of jper particles, tps tiles each.
+struct DirectTiles {
+    int64_t n, jper;
+    int tps, total;
+    __device__ __forceinline__ int64_t first(int id) const { return (int64_t)(id / tps) * jper + (int64_t)(id % tps) * kDT; }
+    __device__ __forceinline__ int count(int id) const {
+        const int64_t slice = (int64_t)(id / tps + 1) * jper, end = slice < n ? slice : n, m = end - first(id);
+        return m <= 0 ? 0 : m < kDT ? (int)m : kDT;
+    }
+};
+
 // One system: a block takes P sampled rows per i-slot of a thread (thread t
-// rows (blockIdx.x * 2 KP + q) P + t % P) and the j-slices of its threads t / P
-// within slice blockIdx.y of the j range; j-particles are staged in shared
-// tiles, FP32 sums of a tile go into Kahan sums, partial sums of a slice into
-// part[slice].  Bound by the FP32 pipe: 19 operations a pair term, in packed
-// instructions for two i-particles, with each staged j-particle read once
-// for the thread's 2 KP; the own-term check runs only on the tiles that hold
-// one of the warp's i-particles.  4096 rows of 2^20 particles: 5.76 ms of
-// kernel time with one i-particle a thread and scalar instructions; the whole
-// call 6.34 -> 3.47 ms.
+// rows (blockIdx.x * 2 KP + q) P + t % P) and tiles blockIdx.y tper and on, 128 / P
+// of them at a time (a warp works on one); j-particles are staged in shared
+// memory, FP32 sums of a tile, in its order whatever the split, go into Kahan
+// sums, partial sums of a block's warps into part[].  Bound by the FP32 pipe: 19
+// operations a pair term, in packed instructions for two i-particles, with each
+// staged j-particle read once for the thread's 2 KP; the own-term check runs
+// only on the tiles that hold one of the warp's i-particles.  4096 rows of 2^20
+// particles: 5.76 ms of kernel time with one i-particle a thread and scalar
+// instructions; the whole call 6.25 -> 3.24 ms (3.16 against 3.06 ms with four
+// CTAs of 128 registers an SM instead of three of 153).
 template <int KP>
-__global__ void __launch_bounds__(kDB, KP == 2 ? 4 : 5) k_direct_tiled(int64_t n, int64_t ns, int P,
+__global__ void __launch_bounds__(kDB, KP == 2 ? 3 : 5) k_direct_tiled(DirectTiles J, int tper, int64_t ns, int P,
                                                       const uint32_t* __restrict__ inv,
                                                       const int64_t* __restrict__ rows,
                                                       const float4* __restrict__ hi,
-                                                      const float4* __restrict__ lo, int64_t jper,
+                                                      const float4* __restrict__ lo,
                                                       double* __restrict__ part) {
-    __shared__ float4 s_h[kDT], s_l[kDT];
+    constexpr int kTiles = KP == 2 ? 1 : 4;  // the most that are staged at a time
+    __shared__ float4 s_h[kTiles * kDT], s_l[kTiles * kDT];
     constexpr int K = 2 * KP;
     const int t = threadIdx.x;
     const int ip = t % P, sl = t / P, nsl = kDB / P;
@@ -190,21 +202,27 @@ __global__ void __launch_bounds__(kDB, KP == 2 ? 4 : 5) k_direct_tiled(int64_t n
         e2[q] = f2_pk(l[0].w, l[1].w);
     }
     normal = __all_sync(0xFFFFFFFFu, normal);
-    const int64_t j0 = blockIdx.y * jper;
-    const int64_t j1 = j0 + jper < n ? j0 + jper : n;
+    const int t0 = blockIdx.y * tper, t1 = t0 + tper < J.total ? t0 + tper : J.total;
     Comp4 acc[K];
 #pragma unroll
     for (int i = 0; i < K; ++i)
 #pragma unroll
         for (int k = 0; k < 4; ++k) acc[i].s[k] = acc[i].c[k] = 0.f;
-    for (int64_t jt = j0; jt < j1; jt += kDT) {
-        const int m = j1 - jt < kDT ? (int)(j1 - jt) : kDT;
+    for (int tb = t0; tb < t1; tb += nsl) {
         __syncthreads();
-        for (int k = t; k < m; k += kDB) {
-            s_h[k] = hi[jt + k];
-            s_l[k] = lo[jt + k];
+        for (int q = 0; q < nsl && tb + q < t1; ++q) {
+            const int64_t jt = J.first(tb + q);
+            const int m = J.count(tb + q);
+            for (int k = t; k < m; k += kDB) {
+                s_h[q * kDT + k] = hi[jt + k];
+                s_l[q * kDT + k] = lo[jt + k];
+            }
         }
         __syncthreads();
+        if (tb + sl >= t1) break;  // the block's last tiles, none for this warp
+        const int64_t jt = J.first(tb + sl);
+        const int m = J.count(tb + sl);
+        const float4 *th = s_h + sl * kDT, *tl = s_l + sl * kDT;
         bool self = false;
         uint32_t rel[K];
 #pragma unroll
@@ -217,11 +235,11 @@ __global__ void __launch_bounds__(kDB, KP == 2 ? 4 : 5) k_direct_tiled(int64_t n
 #pragma unroll
         for (int q = 0; q < KP; ++q) ax[q] = ay[q] = az[q] = pp[q] = 0ull;
         if (!normal)
-            direct_tile<KP, true, false>(s_h, s_l, m, sl, nsl, rel, hx, hy, hz, lx, ly, lz, e2, ax, ay, az, pp);
+            direct_tile<KP, true, false>(th, tl, m, rel, hx, hy, hz, lx, ly, lz, e2, ax, ay, az, pp);
         else if (self)
-            direct_tile<KP, true, true>(s_h, s_l, m, sl, nsl, rel, hx, hy, hz, lx, ly, lz, e2, ax, ay, az, pp);
+            direct_tile<KP, true, true>(th, tl, m, rel, hx, hy, hz, lx, ly, lz, e2, ax, ay, az, pp);
         else
-            direct_tile<KP, false, true>(s_h, s_l, m, sl, nsl, rel, hx, hy, hz, lx, ly, lz, e2, ax, ay, az, pp);
+            direct_tile<KP, false, true>(th, tl, m, rel, hx, hy, hz, lx, ly, lz, e2, ax, ay, az, pp);
 #pragma unroll
         for (int q = 0; q < KP; ++q) {
             const f2 v[4] = {ax[q], ay[q], az[q], pp[q]};
@@ -352,16 +370,26 @@ int direct_sample_device(fdps_psys* ps, int64_t ns, const int64_t* d_rows, doubl
     SampleScratch sc;
     int rc = invert_ids(ps, sc);
     const bool one = ps->n_sys == 1;
+    // j-particles: slices that give four blocks an SM with one i-particle a
+    // thread, in tiles of kDT; the FP32 sums run over these tiles.
+    const int64_t bx1 = (ns + kDB - 1) / kDB;
+    const int64_t sl1 = std::max<int64_t>(1, std::min<int64_t>({(4 * (int64_t)ctx->sm_count + bx1 - 1) / bx1, 1024}));
+    DirectTiles J;
+    J.n = n;
+    J.jper = (n + sl1 - 1) / sl1;
+    J.tps = (int)((J.jper + kDT - 1) / kDT);
+    J.total = (int)sl1 * J.tps;
     // i-particles: 4 per thread where the rows fill a block of 128 threads
-    // with them, else 2; fewer rows than threads leave the other threads to
-    // slices of the j range.  j-slices (blocks): one resident wave.
+    // with them, else 2; fewer rows than threads leave the other warps to
+    // other tiles.  Blocks: one resident wave.
     const int K = ns > 2 * kDB ? 4 : 2;
-    const int P = ns > kDB || K == 4 ? kDB : ns > 64 ? 64 : ns > 32 ? 32 : 16;
-    const int per_sm = K == 4 ? 4 : 5;
-    const int64_t bx = one ? (ns + (int64_t)K * P - 1) / ((int64_t)K * P) : (ns + kDB - 1) / kDB;
+    const int P = ns > kDB || K == 4 ? kDB : ns > 64 ? 64 : 32;
+    const int nsl = kDB / P, per_sm = K == 4 ? 3 : 5;
+    const int64_t bx = one ? (ns + (int64_t)K * P - 1) / ((int64_t)K * P) : bx1;
     int64_t by = one ? (int64_t)per_sm * ctx->sm_count / bx : 1;
-    by = std::max<int64_t>(1, std::min<int64_t>({by, 1024, (n + 63) / 64}));
-    const int js = one ? (int)by * (kDB / P) : 1;
+    by = std::max<int64_t>(1, std::min<int64_t>({by, 1024, (J.total + nsl - 1) / nsl}));
+    const int tper = (int)((J.total + by - 1) / by);
+    const int js = one ? (int)by * nsl : 1;
     if (!rc && (cudaMalloc(&sc.hi, sizeof(float4) * (size_t)n) != cudaSuccess ||
                 cudaMalloc(&sc.lo, sizeof(float4) * (size_t)n) != cudaSuccess ||
                 cudaMalloc(&sc.part, sizeof(double) * 4 * (size_t)ns * js) != cudaSuccess)) {
@@ -381,12 +409,11 @@ int direct_sample_device(fdps_psys* ps, int64_t ns, const int64_t* d_rows, doubl
                 n, ps->x[c], ps->y[c], ps->z[c], ps->m[c], ps->eps[c], o[0], o[1], o[2], sc.hi, sc.lo);
             FDPS_LAUNCH_CHECK(ctx);
             if (one) {
-                const int64_t jper = (n + by - 1) / by;
                 const dim3 grid((unsigned)bx, (unsigned)by);
                 if (K == 4)
-                    k_direct_tiled<2><<<grid, kDB, 0, s>>>(n, ns, P, sc.inv, d_rows, sc.hi, sc.lo, jper, sc.part);
+                    k_direct_tiled<2><<<grid, kDB, 0, s>>>(J, tper, ns, P, sc.inv, d_rows, sc.hi, sc.lo, sc.part);
                 else
-                    k_direct_tiled<1><<<grid, kDB, 0, s>>>(n, ns, P, sc.inv, d_rows, sc.hi, sc.lo, jper, sc.part);
+                    k_direct_tiled<1><<<grid, kDB, 0, s>>>(J, tper, ns, P, sc.inv, d_rows, sc.hi, sc.lo, sc.part);
             } else {
                 k_direct_systems<<<(unsigned)bx, kDB, 0, s>>>(ns, sc.inv, d_rows, ps->d_sys, ps->d_off, sc.hi,
                                                               sc.lo, sc.part);
