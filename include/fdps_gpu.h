@@ -387,6 +387,7 @@ int fdps_tree_choose_theta(fdps_tree* tree, fdps_psys* ps, double target,
                        system's root centre c0 as FP32 hi and lo parts
      pool              list entries: a node id; (id | leaf_tag) marks an
                        opened leaf, whose particles are EPJ; else an SPJ
+                       (a list holds its SPJ before its opened leaves)
      nd_first, nd_count  [nodes] first sorted position and size of a node
      nd_f              [2 nodes] float4: (COM hi - c0, M), (COM lo, 0)
      nd_fq0, nd_fq1    [nodes] float4 (Qxx, Qyy, Qzz, Qxy) and float2
