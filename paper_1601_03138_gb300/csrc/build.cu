@@ -694,6 +694,8 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
 // 0.27 ms.
 constexpr int kMomBlock = 256;
 constexpr int kMomCl = 8;
+// (65,536 Plummer / Hernquist particles, monopoles: 76 / 88 us by the cluster, 80 / 111 by
+// the grid; 90,000: 92 / 108 and 80 / 107)
 constexpr int64_t kMomSmall = int64_t(1) << 16;
 constexpr int kTopNodes = 4 * kMomBlock;
 constexpr int kMaxGridSpin = 1 << 20;
