@@ -538,7 +538,7 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
         double m8[8], x8[8], y8[8], z8[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            const uint32_t c = k < (int)nc ? c0 + k : (uint32_t)i;  // (a node cut off from its children has none)
+            const uint32_t c = k < (int)nc ? c0 + k : (uint32_t)i;  // past its children: the node itself
             m8[k] = __ldcg(&A.nd_com[c].w);
             x8[k] = __ldcg(&A.nd_sx[c]);
             y8[k] = __ldcg(&A.nd_sy[c]);
@@ -678,7 +678,7 @@ __device__ __forceinline__ void node_moments(const MomArgs& A, int64_t i) {
 }
 
 // Leaves of every level in one launch, then the internal nodes level by
-// level from the deepest up in one more: a barrier between levels, so that
+// level from the deepest but one up in one more: a barrier between levels, so that
 // each internal node finds its children complete.  With a launch per level
 // (21, most of them for levels with few or no nodes) the internal nodes were
 // all latency below about 10^6 particles.  Up to kMomSmall particles one
@@ -707,6 +707,11 @@ constexpr int kMaxGridSpin = 1 << 20;
 // warp's lanes sum leaves of like size.  With the internal nodes
 // collected likewise: moments of 2^24 particles (quadrupoles) 1.00 -> 0.92 ms, of
 // 3M clumpy particles (monopoles) 0.36 -> 0.24 ms.
+// The pass takes every node without children: beside the leaves the last kept
+// level's internal nodes of a cut tree (node arrays too small, or roots only
+// after a sort that gave up), whose records the passes over the levels do not
+// reach.  Such a node gets no mass and a record without children, so that
+// whatever follows a record stays within the tree.
 constexpr int kLeafTile = kMomBlock;
 template <bool QUAD, bool Q64>
 __global__ void __launch_bounds__(kMomBlock) k_moments_leaves(MomArgs A) {
@@ -719,7 +724,7 @@ __global__ void __launch_bounds__(kMomBlock) k_moments_leaves(MomArgs A) {
         uint32_t bin = 0, rank = 0;  // bin 0: no leaf
         if (t < 32) s_bin[t] = 0;
         __syncthreads();
-        if (i < nn && meta_leaf(A.nd_meta[i])) {
+        if (i < nn && meta_nchild(A.nd_meta[i]) == 0u) {
             const uint32_t c = A.nd_count[i];
             bin = c <= (uint32_t)kMaxLeaf ? c : (uint32_t)kMaxLeaf + 1u;
             rank = atomicAdd(&s_bin[bin], 1u);

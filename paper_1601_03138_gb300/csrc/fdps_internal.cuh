@@ -53,10 +53,13 @@ constexpr uint32_t kOvfChunk = 32u;
 constexpr uint32_t kSortStall = 64u;  // a radix-sort look-back wait gave up
 constexpr uint32_t kSortRedo = 256u;  // a bucket of the coherent sort overflowed: redo with the radix sort
 constexpr uint32_t kSortInvalid = kSortStall | kSortRedo;  // this call's order is not sorted
+// Any of these leaves the tree or its groups incomplete: the walk has nothing
+// to walk (the host redoes the build).
+constexpr uint32_t kTreeInvalid = kOvfNodes | kOvfGroups | kSortStall | kSortRedo;
 // Any of these leaves the step's lists or particle order invalid: the
 // kernels downstream skip their work (the host redoes the step).
 constexpr uint32_t kStepInvalid =
-    kOvfNodes | kOvfPool | kOvfFrontier | kOvfGroups | kOvfChunk | kSortStall | kSortRedo;
+    kTreeInvalid | kOvfPool | kOvfFrontier | kOvfChunk;
 
 // Per-tree device-resident state written by the kernels of one force call.
 struct DevState {

@@ -428,6 +428,7 @@ constexpr int kWalkBlock = 128;
 
 __global__ void __launch_bounds__(kWalkBlock, 8) k_walk(WalkArgs A) {
     DevState* st = A.st;
+    if (st->overflow & kTreeInvalid) return;  // the host redoes the build
     const int lane = threadIdx.x & 31;
     const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     uint32_t* fa = A.frontier + wid * 2 * (int64_t)A.cap_frontier;
@@ -464,6 +465,7 @@ __global__ void __launch_bounds__(kWalkBlock, 8) k_walk_few(WalkArgs A) {
     __shared__ unsigned long long s_nb;
     __shared__ uint32_t s_g;
     DevState* st = A.st;
+    if (st->overflow & kTreeInvalid) return;  // as in k_walk
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const uint32_t ngroups = (uint32_t)st->n_groups;
