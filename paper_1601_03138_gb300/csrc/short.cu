@@ -460,10 +460,13 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
                 constexpr bool REL = decltype(relc)::value;
                 if ((m & 1u) && lane == 0) {  // an even number: a candidate far from everything, without mass
                     const float far = 16.0f * (hb + hg) + (R ? 16.0f * T.hj[m - 1] : 0.0f);
-                    T.xh[m] = REL ? far : gch.x + far;
+                    // (beside hi parts the displacement is a low part: a few cutoffs
+                    // may be lost in a sum with the centre's coordinate)
+                    T.xh[m] = REL ? far : gch.x;
                     T.yh[m] = REL ? 0.0f : gch.y;
                     T.zh[m] = REL ? 0.0f : gch.z;
-                    T.xl[m] = T.yl[m] = T.zl[m] = T.m[m] = 0.0f;
+                    T.xl[m] = far;
+                    T.yl[m] = T.zl[m] = T.m[m] = 0.0f;
                     T.p[m] = 0xFFFFFFFFu;
                     if (R) {
                         T.nih2[m] = T.nih2[m - 1];
