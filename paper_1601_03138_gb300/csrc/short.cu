@@ -393,15 +393,15 @@ __device__ __forceinline__ f2 ld2(const float* a, uint32_t k) { return reinterpr
 // of the tile, so that small groups keep the whole warp busy; a lane takes
 // two candidates at a time in packed FP32 instructions.  Where the cutoff is
 // the i-particle's own and the group's box is at most half of it (nearly
-// always: the groups of a uniform cube are a quarter of it), candidates and
-// i-particles are FP32 coordinates relative to the group's centre, exact to 2u
-// of a separation at the cutoff, instead of hi/lo pairs: a third of the loads
-// and differences; there the kernel's argument is bounded too and needs no
-// clamps.  MODE is the cutoff type (FDPS_CUTOFF_*), fixed at compile time so
+// always: the groups of a uniform cube are a quarter of it), the kernel's
+// argument is bounded and needs no clamps.  MODE is the cutoff type (FDPS_CUTOFF_*), fixed at compile time so
 // that the pair loop carries no selection between them.  Issue-bound (78 % of
 // the slots, ALU 61 %): pair pass of 2^20 particles 3.19 ms with one candidate a
 // turn and no box test, 2.18 with them, 1.97 with a candidate's leaf from
-// ballots, 1.64 with the relative coordinates and tiles of 128 (96 before).
+// ballots, 1.78 without the clamps and with tiles of 128 (96 before).  FP32
+// coordinates relative to the group's centre instead of the hi/lo pairs took
+// 1.64, but a separation was then off by up to 10u of the cutoff instead of a
+// few u of itself, and the density errors grew by up to 1 %: not taken.
 template <int MODE>
 __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
     constexpr bool R = MODE >= 2;
@@ -438,33 +438,28 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
             const uint32_t i = ib + ip;
             const bool act = sl < nsl && i < ni;
             const uint32_t pi = gf + (act ? i : 0u);
-            float4 ih = A.pf_hi[pi];
-            const float4 il = A.pf_lo[pi];
+            const float4 ih = A.pf_hi[pi], il = A.pf_lo[pi];
             const double hi64 = MODE != 0 ? A.h[pi] : A.r_fixed;
             const float hif = (float)hi64, invHi = 1.0f / hif, invHi2 = fminf(invHi * invHi, 3e38f);
-            // FP32 coordinates relative to the group's centre: their rounding, 2u
-            // of |x_i| <= hb and of |x_j| <= hb + a each beside 3u a of the
-            // difference, is within Ea with Eabs + 5u hb in Eabs' place
-            const bool rel = !R && __all_sync(0xFFFFFFFFu, !act || (hb <= 0.5f * hif && hg <= 8.0f * hif && hif > 1e-17f && hif < 1e17f));
+            // no staged candidate is further than 137 of the lane's cutoffs
+            const bool bounded = !R && __all_sync(0xFFFFFFFFu, !act || (hb <= 0.5f * hif && hg <= 8.0f * hif && hif > 1e-17f && hif < 1e17f));
             const float2 ti = MODE == 2 ? make_float2(0.0f, 0.0f)
-                                        : pair_thresholds(hif, rel ? fmaf(5.0f * kU, hb, 2.0f * Eabs) : Eabs);
-            if (rel) ih.x = (ih.x - gch.x) + (il.x - gcl.x), ih.y = (ih.y - gch.y) + (il.y - gcl.y),
-                     ih.z = (ih.z - gch.z) + (il.z - gcl.z);
+                                        : pair_thresholds(hif, Eabs);
             const f2 ixh = f2_pk(ih.x, ih.x), iyh = f2_pk(ih.y, ih.y), izh = f2_pk(ih.z, ih.z);
             const f2 ixl = f2_pk(il.x, il.x), iyl = f2_pk(il.y, il.y), izl = f2_pk(il.z, il.z);
             const f2 niH2 = f2_pk(-invHi2, -invHi2);
             uint32_t cnt = 0, fbk = 0;
             f2 sum = 0ull, sumj = 0ull;  // sums of m_j w(q) with H = h_i, and with H = h_j
             // the staged candidates 0 .. m - 1 on the warp's i-particles
-            auto pairs = [&](auto relc, uint32_t m) {
-                constexpr bool REL = decltype(relc)::value;
+            auto pairs = [&](auto clamp, uint32_t m) {
+                constexpr bool CLAMP = decltype(clamp)::value;
                 if ((m & 1u) && lane == 0) {  // an even number: a candidate far from everything, without mass
                     const float far = 16.0f * (hb + hg) + (R ? 16.0f * T.hj[m - 1] : 0.0f);
-                    // (beside hi parts the displacement is a low part: a few cutoffs
-                    // may be lost in a sum with the centre's coordinate)
-                    T.xh[m] = REL ? far : gch.x;
-                    T.yh[m] = REL ? 0.0f : gch.y;
-                    T.zh[m] = REL ? 0.0f : gch.z;
+                    // (as a low part: a few cutoffs may be lost in a sum with the
+                    // centre's coordinate)
+                    T.xh[m] = gch.x;
+                    T.yh[m] = gch.y;
+                    T.zh[m] = gch.z;
                     T.xl[m] = far;
                     T.yl[m] = T.zl[m] = T.m[m] = 0.0f;
                     T.p[m] = 0xFFFFFFFFu;
@@ -480,12 +475,9 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
                 if (act) {
 #pragma unroll 1
                     for (uint32_t k = sl; k < (m + 1u) / 2u; k += nsl) {
-                        f2 dx = f2_sub(ld2(T.xh, k), ixh);
-                        if (!REL) dx = f2_add(dx, f2_sub(ld2(T.xl, k), ixl));
-                        f2 dy = f2_sub(ld2(T.yh, k), iyh);
-                        if (!REL) dy = f2_add(dy, f2_sub(ld2(T.yl, k), iyl));
-                        f2 dz = f2_sub(ld2(T.zh, k), izh);
-                        if (!REL) dz = f2_add(dz, f2_sub(ld2(T.zl, k), izl));
+                        const f2 dx = f2_add(f2_sub(ld2(T.xh, k), ixh), f2_sub(ld2(T.xl, k), ixl));
+                        const f2 dy = f2_add(f2_sub(ld2(T.yh, k), iyh), f2_sub(ld2(T.yl, k), iyl));
+                        const f2 dz = f2_add(f2_sub(ld2(T.zh, k), izh), f2_sub(ld2(T.zl, k), izl));
                         const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, f2_mul(dz, dz)));
                         float ra, rb;
                         f2_up(r2, ra, rb);
@@ -530,7 +522,7 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
                         if (MODE != 2) {
                             float ma, mb;
                             f2_up(ld2(T.m, k), ma, mb);
-                            sum = f2_fma(f2_pk(na ? ma : 0.0f, nb ? mb : 0.0f), wendland_q2<!REL>(r2, niH2), sum);
+                            sum = f2_fma(f2_pk(na ? ma : 0.0f, nb ? mb : 0.0f), wendland_q2<CLAMP>(r2, niH2), sum);
                         }
                         if (R) {
                             float ma, mb;
@@ -544,9 +536,9 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
             };
             auto run = [&](uint32_t m) {
                 if constexpr (!R) {
-                    if (rel) return pairs(std::true_type{}, m);
+                    if (bounded) return pairs(std::false_type{}, m);
                 }
-                pairs(std::false_type{}, m);
+                pairs(std::true_type{}, m);
             };
             uint32_t staged = 0;
             for (uint32_t base = 0; base < len; base += 32) {
@@ -592,14 +584,12 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
                     const uint32_t mask = __ballot_sync(0xFFFFFFFFu, keep);
                     if (keep) {
                         const uint32_t k = staged + __popc(mask & lt);
-                        T.xh[k] = rel ? dx : h4.x;
-                        T.yh[k] = rel ? dy : h4.y;
-                        T.zh[k] = rel ? dz : h4.z;
-                        if (!rel) {
-                            T.xl[k] = l4.x;
-                            T.yl[k] = l4.y;
-                            T.zl[k] = l4.z;
-                        }
+                        T.xh[k] = h4.x;
+                        T.yh[k] = h4.y;
+                        T.zh[k] = h4.z;
+                        T.xl[k] = l4.x;
+                        T.yl[k] = l4.y;
+                        T.zl[k] = l4.z;
                         T.m[k] = h4.w;
                         T.p[k] = pj;
                         if (R) {

@@ -1,9 +1,6 @@
-"""Neighbours on both sides of the rule that takes coordinates relative to the
-group's centre (group box at most half the cutoff, the group's radii within a
-factor 8): counts bit for bit, densities against the oracle.  Density bound:
-a separation is off by at most 10.5 u of the cutoff an axis, 1e-6 of q, and W
-changes by at most 3.5 W(0) a unit of q, independently from neighbour to
-neighbour beside W(0) of the particle itself: 1e-5."""
+"""Neighbours on both sides of the rule that evaluates the kernel without clamps
+(group box at most half the cutoff, the group's radii within a factor 8): counts
+bit for bit, densities against the oracle.  Density bound: the FP32 path's 1e-5."""
 import numpy as np
 import pytest
 
