@@ -656,7 +656,7 @@ __global__ void __launch_bounds__(CB, 32 * WARPS / CB) k_force_f32(ForceArgs A) 
 // warp or CTA per group the last groups of a 10^5-particle system left most
 // of the SMs idle.  Entries are staged in shared memory by chunk.  Slices
 // and CTAs are summed in a fixed order, through distributed shared memory.
-// Plummer N = 100,003, quadrupoles, n_grp 128: 56.4 -> 19.3 ms for the
+// Plummer N = 100,003, quadrupoles, n_grp 128: 56.4 -> 19.4 ms for the
 // whole force calculation (one warp per group before).
 constexpr int kF64Block = 128;
 constexpr int kCl64 = 8;     // CTAs per cluster
@@ -756,19 +756,22 @@ __device__ __forceinline__ void force_round_f64(const ForceArgs& A, uint32_t gf,
                 const double R2 = fma(rx, rx, fma(ry, ry, fma(rz, rz, e2[q])));
                 const double Ri = rsqrt(R2);
                 const double Ri2 = Ri * Ri;
-                if (QUAD) {  // regrouped as in the FP32 kernel: 32 operations and the root
-                    const double Ri4 = Ri2 * Ri2;
-                    const double Ri5 = Ri4 * Ri;
-                    const double Qrx = fma(qxx, rx, fma(qxy, ry, qxz * rz));
-                    const double Qry = fma(qxy, rx, fma(qyy, ry, qyz * rz));
-                    const double Qrz = fma(qxz, rx, fma(qyz, ry, qzz * rz));
-                    const double rQr = fma(rx, Qrx, fma(ry, Qry, rz * Qrz));
-                    const double w = rQr * Ri4;
+                if (QUAD) {
+                    // v = r / R^2 stands for r in the quadrupole, so that no power
+                    // beyond R^-3 appears: like the monopole's m / R^3 the term
+                    // holds from R = 1e-102 to 1e102 (regrouped around R^-5 as in
+                    // the FP32 kernel, one operation less, it vanished from 1e65 on)
+                    const double vx = rx * Ri2, vy = ry * Ri2, vz = rz * Ri2;
+                    const double Qvx = fma(qxx, vx, fma(qxy, vy, qxz * vz));
+                    const double Qvy = fma(qxy, vx, fma(qyy, vy, qyz * vz));
+                    const double Qvz = fma(qxz, vx, fma(qyz, vy, qzz * vz));
+                    const double rQv = fma(rx, Qvx, fma(ry, Qvy, rz * Qvz));
+                    const double w = rQv * Ri2;
                     const double hh = fma(-2.5, w, c.w);
-                    const double hR2 = hh * R2;
-                    ax[q] = fma(Ri5, fma(hR2, rx, Qrx), ax[q]);
-                    ay[q] = fma(Ri5, fma(hR2, ry, Qry), ay[q]);
-                    az[q] = fma(Ri5, fma(hR2, rz, Qrz), az[q]);
+                    const double Ri3 = Ri2 * Ri;
+                    ax[q] = fma(Ri3, fma(hh, rx, Qvx), ax[q]);
+                    ay[q] = fma(Ri3, fma(hh, ry, Qvy), ay[q]);
+                    az[q] = fma(Ri3, fma(hh, rz, Qvz), az[q]);
                     pp[q] = fma(Ri, fma(2.0, w, hh), pp[q]);
                 } else {
                     const double nMRi = c.w * Ri;
