@@ -22,7 +22,13 @@
  *   - Every function returning int returns FDPS_OK (0) or a negative
  *     FDPS_E* code; fdps_last_error(ctx) then holds a one-line message.
  *     No call exits the process or traps the GPU.
- *   - Handles own all their device memory; *_destroy frees it.
+ *   - Handles own all their device memory; *_destroy frees it.  Some of it is
+ *     scratch kept for the next call: 64 bytes a particle after data was set
+ *     again or 2^21 particles or more were read to device or pageable host
+ *     memory (32 if only accelerations and potentials were), 20 after a
+ *     neighbour search on host arrays.  An allocation that finds no room gives
+ *     this scratch of all the context's handles back and tries again before
+ *     it fails.
  *   - All work is issued on the context's CUDA stream (fdps_get_stream);
  *     calls that return data to host memory synchronise that stream.
  *   - Positions, velocities and accelerations are row-major [n][3] FP64

@@ -54,15 +54,15 @@ int ensure_particles(fdps_tree* t, int64_t n) {
     const int64_t tiles = (n + kSortTile - 1) / kSortTile;
     // a smaller set on this tree has its build tiles of kBuildTileSmall
     const int64_t small_tiles = (std::min<int64_t>(n, kBuildSmall) + kBuildTileSmall - 1) / kBuildTileSmall;
-    bool ok = dev_alloc(&t->keys_in, n) == cudaSuccess && dev_alloc(&t->keys_a, n) == cudaSuccess &&
-              dev_alloc(&t->keys_b, n) == cudaSuccess && dev_alloc(&t->vals_a, n) == cudaSuccess &&
-              dev_alloc(&t->vals_b, n) == cudaSuccess && dev_alloc(&t->pf_hi, n) == cudaSuccess &&
-              dev_alloc(&t->pf_lo, n) == cudaSuccess && dev_alloc(&t->head, n) == cudaSuccess &&
-              dev_alloc(&t->pmx, n) == cudaSuccess && dev_alloc(&t->pmy, n) == cudaSuccess &&
-              dev_alloc(&t->pmz, n) == cudaSuccess &&
-              dev_alloc(&t->sort_hist, 2 * 256 * tiles) == cudaSuccess &&
-              dev_alloc(&t->bt_count, kMaxLevel * (kBuildWarps + 1) * (std::max(tiles, small_tiles) + 1) + 32) == cudaSuccess &&
-              dev_alloc(&t->coh_bkt, n) == cudaSuccess && dev_alloc(&t->coh_cnt, 3 * ((n + kCohT - 1) / kCohT + 1) + 8) == cudaSuccess;
+    bool ok = dev_alloc(t->ctx, &t->keys_in, n) == cudaSuccess && dev_alloc(t->ctx, &t->keys_a, n) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->keys_b, n) == cudaSuccess && dev_alloc(t->ctx, &t->vals_a, n) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->vals_b, n) == cudaSuccess && dev_alloc(t->ctx, &t->pf_hi, n) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->pf_lo, n) == cudaSuccess && dev_alloc(t->ctx, &t->head, n) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->pmx, n) == cudaSuccess && dev_alloc(t->ctx, &t->pmy, n) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->pmz, n) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->sort_hist, 2 * 256 * tiles) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->bt_count, kMaxLevel * (kBuildWarps + 1) * (std::max(tiles, small_tiles) + 1) + 32) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->coh_bkt, n) == cudaSuccess && dev_alloc(t->ctx, &t->coh_cnt, 3 * ((n + kCohT - 1) / kCohT + 1) + 8) == cudaSuccess;
     t->cap_coh = ok ? 3 * ((n + kCohT - 1) / kCohT + 1) + 8 : 0;
     if (!ok) {
         cudaGetLastError();
@@ -97,15 +97,15 @@ void free_nodes(fdps_tree* t) {
 int ensure_nodes(fdps_tree* t, int64_t cap) {
     if (cap <= t->cap_nodes) return FDPS_OK;
     free_nodes(t);
-    bool ok = dev_alloc(&t->nd_first, cap) == cudaSuccess && dev_alloc(&t->nd_count, cap) == cudaSuccess &&
-              dev_alloc(&t->nd_child, cap) == cudaSuccess && dev_alloc(&t->nd_meta, cap) == cudaSuccess &&
-              dev_alloc(&t->nd_parent, cap) == cudaSuccess &&
-              dev_alloc(&t->nd_qlo, cap) == cudaSuccess &&
-              dev_alloc(&t->nd_sx, cap) == cudaSuccess &&
-              dev_alloc(&t->nd_sy, cap) == cudaSuccess && dev_alloc(&t->nd_sz, cap) == cudaSuccess &&
-              dev_alloc(&t->nd_com, cap) == cudaSuccess && dev_alloc(&t->nd_quad, 6 * cap) == cudaSuccess &&
-              dev_alloc(&t->nd_f, 2 * cap) == cudaSuccess && dev_alloc(&t->nd_walk, cap) == cudaSuccess &&
-              dev_alloc(&t->nd_fq0, cap) == cudaSuccess && dev_alloc(&t->nd_fq1, cap) == cudaSuccess;
+    bool ok = dev_alloc(t->ctx, &t->nd_first, cap) == cudaSuccess && dev_alloc(t->ctx, &t->nd_count, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->nd_child, cap) == cudaSuccess && dev_alloc(t->ctx, &t->nd_meta, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->nd_parent, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->nd_qlo, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->nd_sx, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->nd_sy, cap) == cudaSuccess && dev_alloc(t->ctx, &t->nd_sz, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->nd_com, cap) == cudaSuccess && dev_alloc(t->ctx, &t->nd_quad, 6 * cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->nd_f, 2 * cap) == cudaSuccess && dev_alloc(t->ctx, &t->nd_walk, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->nd_fq0, cap) == cudaSuccess && dev_alloc(t->ctx, &t->nd_fq1, cap) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         free_nodes(t);
@@ -136,13 +136,13 @@ void free_groups(fdps_tree* t) {
 int ensure_groups(fdps_tree* t, int64_t cap) {
     if (cap <= t->cap_groups) return FDPS_OK;
     free_groups(t);
-    bool ok = dev_alloc(&t->g_first, cap) == cudaSuccess && dev_alloc(&t->g_count, cap) == cudaSuccess &&
-              dev_alloc(&t->g_node, cap) == cudaSuccess && dev_alloc(&t->g_box, 6 * cap) == cudaSuccess &&
-              dev_alloc(&t->g_qbox, 6 * cap) == cudaSuccess && dev_alloc(&t->g_ch, cap) == cudaSuccess &&
-              dev_alloc(&t->g_cl, cap) == cudaSuccess && dev_alloc(&t->g_blo, cap) == cudaSuccess &&
-              dev_alloc(&t->g_bhi, cap) == cudaSuccess && dev_alloc(&t->g_c64, cap) == cudaSuccess &&
-              dev_alloc(&t->g_off, cap) == cudaSuccess && dev_alloc(&t->g_len, cap) == cudaSuccess &&
-              dev_alloc(&t->g_nspj, cap) == cudaSuccess && dev_alloc(&t->g_nepj, cap) == cudaSuccess;
+    bool ok = dev_alloc(t->ctx, &t->g_first, cap) == cudaSuccess && dev_alloc(t->ctx, &t->g_count, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->g_node, cap) == cudaSuccess && dev_alloc(t->ctx, &t->g_box, 6 * cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->g_qbox, 6 * cap) == cudaSuccess && dev_alloc(t->ctx, &t->g_ch, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->g_cl, cap) == cudaSuccess && dev_alloc(t->ctx, &t->g_blo, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->g_bhi, cap) == cudaSuccess && dev_alloc(t->ctx, &t->g_c64, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->g_off, cap) == cudaSuccess && dev_alloc(t->ctx, &t->g_len, cap) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->g_nspj, cap) == cudaSuccess && dev_alloc(t->ctx, &t->g_nepj, cap) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         free_groups(t);
@@ -156,7 +156,7 @@ int ensure_pool(fdps_tree* t, int64_t cap) {
     if (cap <= t->cap_pool) return FDPS_OK;
     dev_free(t->pool);
     t->cap_pool = 0;
-    if (dev_alloc(&t->pool, cap) != cudaSuccess) {
+    if (dev_alloc(t->ctx, &t->pool, cap) != cudaSuccess) {
         cudaGetLastError();
         return set_error(t->ctx, FDPS_ENOMEM, "device allocation of a %lld-entry list pool failed",
                          (long long)cap);
@@ -169,7 +169,7 @@ int ensure_frontier(fdps_tree* t, int64_t per_warp) {
     if (per_warp <= t->cap_frontier) return FDPS_OK;
     dev_free(t->frontier);
     t->cap_frontier = 0;
-    if (dev_alloc(&t->frontier, 2 * per_warp * t->n_walk_warps) != cudaSuccess) {
+    if (dev_alloc(t->ctx, &t->frontier, 2 * per_warp * t->n_walk_warps) != cudaSuccess) {
         cudaGetLastError();
         return set_error(t->ctx, FDPS_ENOMEM, "device allocation of walk frontiers failed");
     }
@@ -177,18 +177,24 @@ int ensure_frontier(fdps_tree* t, int64_t per_warp) {
     return FDPS_OK;
 }
 
-int ensure_short_io(fdps_tree* t, int64_t n) {
-    if (n <= t->cap_sr_io) return FDPS_OK;
+int ensure_short_radii(fdps_tree* t, int64_t n) {
+    if (n <= t->cap_sr_hin) return FDPS_OK;
     dev_free(t->sr_hin);
+    t->cap_sr_hin = 0;
+    if (dev_alloc(t->ctx, &t->sr_hin, n) != cudaSuccess)
+        return set_error(t->ctx, FDPS_ENOMEM, "neighbour buffer allocation for %lld particles failed", (long long)n);
+    t->cap_sr_hin = n;
+    return FDPS_OK;
+}
+
+int ensure_short_out(fdps_tree* t, int64_t n) {
+    if (n <= t->cap_sr_out) return FDPS_OK;
     dev_free(t->sr_cnt);
     dev_free(t->sr_rho);
-    t->cap_sr_io = 0;
-    if (dev_alloc(&t->sr_hin, n) != cudaSuccess || dev_alloc(&t->sr_cnt, n) != cudaSuccess ||
-        dev_alloc(&t->sr_rho, n) != cudaSuccess) {
-        cudaGetLastError();
+    t->cap_sr_out = 0;
+    if (dev_alloc(t->ctx, &t->sr_cnt, n) != cudaSuccess || dev_alloc(t->ctx, &t->sr_rho, n) != cudaSuccess)
         return set_error(t->ctx, FDPS_ENOMEM, "neighbour buffer allocation for %lld particles failed", (long long)n);
-    }
-    t->cap_sr_io = n;
+    t->cap_sr_out = n;
     return FDPS_OK;
 }
 
@@ -232,7 +238,7 @@ int ensure_systems(fdps_tree* t, int64_t n_sys) {
     if (n_sys <= t->cap_sys) return FDPS_OK;
     dev_free(t->sys_box);
     t->cap_sys = 0;
-    if (dev_alloc(&t->sys_box, n_sys) != cudaSuccess) {
+    if (dev_alloc(t->ctx, &t->sys_box, n_sys) != cudaSuccess) {
         cudaGetLastError();
         return set_error(t->ctx, FDPS_ENOMEM, "device allocation for %lld system boxes failed",
                          (long long)n_sys);
@@ -421,6 +427,34 @@ bool valid_params(const fdps_tree_params* p) {
 
 }  // namespace
 
+namespace fdps {
+
+bool give_back_scratch(fdps_ctx* ctx) {
+    bool any = false;
+    if (ctx->capturing) return any;
+    for (fdps_psys* ps = ctx->systems.head; ps; ps = ps->next) {
+        any = any || ps->rec;
+        dev_free(ps->rec);
+        ps->cap_rec = 0;
+    }
+    for (fdps_tree* t = ctx->trees.head; t; t = t->next) {
+        if (!(t->sr_busy & 1)) {
+            any = any || t->sr_hin;
+            dev_free(t->sr_hin);
+            t->cap_sr_hin = 0;
+        }
+        if (!(t->sr_busy & 2)) {
+            any = any || t->sr_cnt || t->sr_rho;
+            dev_free(t->sr_cnt);
+            dev_free(t->sr_rho);
+            t->cap_sr_out = 0;
+        }
+    }
+    return any;
+}
+
+}  // namespace fdps
+
 extern "C" {
 
 int fdps_init(int device, fdps_ctx** out) {
@@ -457,6 +491,8 @@ int fdps_finalize(fdps_ctx* ctx) {
     if (!ctx) return FDPS_EINVAL;
     cudaSetDevice(ctx->device);
     if (ctx->own_stream) cudaStreamDestroy(ctx->own_stream);
+    ctx->systems.clear();
+    ctx->trees.clear();
     delete ctx;
     return FDPS_OK;
 }
@@ -500,26 +536,28 @@ int fdps_psys_create(fdps_ctx* ctx, int64_t n, fdps_psys** out) {
     ps->n = n;
     bool ok = true;
     for (int b = 0; b < 2; ++b)
-        ok = ok && dev_alloc(&ps->x[b], n) == cudaSuccess && dev_alloc(&ps->y[b], n) == cudaSuccess &&
-             dev_alloc(&ps->z[b], n) == cudaSuccess && dev_alloc(&ps->vx[b], n) == cudaSuccess &&
-             dev_alloc(&ps->vy[b], n) == cudaSuccess && dev_alloc(&ps->vz[b], n) == cudaSuccess &&
-             dev_alloc(&ps->m[b], n) == cudaSuccess && dev_alloc(&ps->eps[b], n) == cudaSuccess &&
-             dev_alloc(&ps->id[b], n) == cudaSuccess;
-    ok = ok && dev_alloc(&ps->ax, n) == cudaSuccess && dev_alloc(&ps->ay, n) == cudaSuccess &&
-         dev_alloc(&ps->az, n) == cudaSuccess && dev_alloc(&ps->pot, n) == cudaSuccess &&
-         dev_alloc(&ps->d_flag, 1) == cudaSuccess &&
-         dev_alloc(&ps->d_red, energy_scratch_doubles()) == cudaSuccess;
+        ok = ok && dev_alloc(ctx, &ps->x[b], n) == cudaSuccess && dev_alloc(ctx, &ps->y[b], n) == cudaSuccess &&
+             dev_alloc(ctx, &ps->z[b], n) == cudaSuccess && dev_alloc(ctx, &ps->vx[b], n) == cudaSuccess &&
+             dev_alloc(ctx, &ps->vy[b], n) == cudaSuccess && dev_alloc(ctx, &ps->vz[b], n) == cudaSuccess &&
+             dev_alloc(ctx, &ps->m[b], n) == cudaSuccess && dev_alloc(ctx, &ps->eps[b], n) == cudaSuccess &&
+             dev_alloc(ctx, &ps->id[b], n) == cudaSuccess;
+    ok = ok && dev_alloc(ctx, &ps->ax, n) == cudaSuccess && dev_alloc(ctx, &ps->ay, n) == cudaSuccess &&
+         dev_alloc(ctx, &ps->az, n) == cudaSuccess && dev_alloc(ctx, &ps->pot, n) == cudaSuccess &&
+         dev_alloc(ctx, &ps->d_flag, 1) == cudaSuccess &&
+         dev_alloc(ctx, &ps->d_red, energy_scratch_doubles()) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         fdps_psys_destroy(ps);
         return set_error(ctx, FDPS_ENOMEM, "device allocation for %lld particles failed", (long long)n);
     }
+    ctx->systems.add(ps);
     *out = ps;
     return FDPS_OK;
 }
 
 int fdps_psys_destroy(fdps_psys* ps) {
     if (!ps) return FDPS_EINVAL;
+    Chain<fdps_psys>::remove(ps);
     cudaSetDevice(ps->ctx->device);
     for (int b = 0; b < 2; ++b) {
         dev_free(ps->x[b]);
@@ -606,7 +644,7 @@ int fdps_psys_set(fdps_psys* ps, const double* pos3n, const double* vel3n, const
         if (rc) return rc;
     } else {
         // host data is staged in the psys's transfer buffer
-        if (!ps->stage && dev_alloc(&ps->stage, 10 * n) != cudaSuccess) {
+        if (!ps->stage && dev_alloc(ctx, &ps->stage, 10 * n) != cudaSuccess) {
             cudaGetLastError();
             ps->stage = nullptr;
             return set_error(ctx, FDPS_ENOMEM, "staging allocation failed");
@@ -666,7 +704,7 @@ int fdps_psys_get(const fdps_psys* ps, double* pos3n, double* vel3n, double* acc
         FDPS_CUDA_TRY(ctx, cudaStreamSynchronize(s));
         return FDPS_OK;
     }
-    if (!pm->stage && dev_alloc(&pm->stage, 10 * n) != cudaSuccess) {
+    if (!pm->stage && dev_alloc(ctx, &pm->stage, 10 * n) != cudaSuccess) {
         cudaGetLastError();
         pm->stage = nullptr;
         return set_error(ctx, FDPS_ENOMEM, "staging allocation failed");
@@ -704,9 +742,9 @@ int fdps_tree_create(fdps_ctx* ctx, const fdps_tree_params* params, fdps_tree** 
     t->p = *params;
     t->box_blocks = std::min(1024, ctx->sm_count * 4);
     t->n_walk_warps = (int64_t)walk_blocks(ctx) * walk_warps_per_block();
-    bool ok = dev_alloc(&t->st, 1) == cudaSuccess && dev_alloc(&t->box_part, t->box_blocks) == cudaSuccess &&
-              dev_alloc(&t->grp_scan, t->box_blocks) == cudaSuccess &&
-              dev_alloc(&t->sort_dtot, 4096) == cudaSuccess &&
+    bool ok = dev_alloc(t->ctx, &t->st, 1) == cudaSuccess && dev_alloc(t->ctx, &t->box_part, t->box_blocks) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->grp_scan, t->box_blocks) == cudaSuccess &&
+              dev_alloc(t->ctx, &t->sort_dtot, 4096) == cudaSuccess &&
               cudaMallocHost(reinterpret_cast<void**>(&t->h_pin), sizeof(DevState)) == cudaSuccess &&
               cudaEventCreateWithFlags(&t->ev_state, cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
@@ -718,12 +756,14 @@ int fdps_tree_create(fdps_ctx* ctx, const fdps_tree_params* params, fdps_tree** 
     for (int k = 0; k < 10; ++k)
         if (cudaEventCreate(&t->ev[k]) != cudaSuccess) t->ev_ok = false;
     cudaGetLastError();
+    ctx->trees.add(t);
     *out = t;
     return FDPS_OK;
 }
 
 int fdps_tree_destroy(fdps_tree* t) {
     if (!t) return FDPS_EINVAL;
+    Chain<fdps_tree>::remove(t);
     cudaSetDevice(t->ctx->device);
     free_particles(t);
     free_nodes(t);
@@ -774,8 +814,7 @@ int fdps_direct_sample(fdps_psys* ps, int64_t n_sample, const int64_t* rows, dou
     cudaStream_t s = ctx->stream;
     int64_t* d_rows = nullptr;
     double* d_out = nullptr;
-    if (cudaMalloc(&d_rows, sizeof(int64_t) * n_sample) != cudaSuccess ||
-        cudaMalloc(&d_out, sizeof(double) * 4 * n_sample) != cudaSuccess) {
+    if (dev_alloc(ctx, &d_rows, n_sample) != cudaSuccess || dev_alloc(ctx, &d_out, 4 * n_sample) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(d_rows);
         return set_error(ctx, FDPS_ENOMEM, "sample allocation failed");
@@ -819,9 +858,8 @@ int fdps_tree_choose_theta(fdps_tree* t, fdps_psys* ps, double target, int64_t n
     for (int64_t k = 0; k < ns; ++k) rows[k] = (int64_t)(((__int128)k * ps->n) / ns);  // evenly spaced rows
     int64_t* d_rows = nullptr;
     double *d_ref = nullptr, *d_tree = nullptr;
-    if (cudaMalloc(&d_rows, sizeof(int64_t) * ns) != cudaSuccess ||
-        cudaMalloc(&d_ref, sizeof(double) * 4 * ns) != cudaSuccess ||
-        cudaMalloc(&d_tree, sizeof(double) * 4 * ns) != cudaSuccess) {
+    if (dev_alloc(ctx, &d_rows, ns) != cudaSuccess || dev_alloc(ctx, &d_ref, 4 * ns) != cudaSuccess ||
+        dev_alloc(ctx, &d_tree, 4 * ns) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(d_rows);
         cudaFree(d_ref);
@@ -894,14 +932,20 @@ int fdps_tree_neighbors(fdps_tree* t, fdps_psys* ps, int32_t mode, double r_fixe
     t->lists_of = nullptr;  // the pool will hold neighbour lists, not gravity lists
     // device copies of host arrays, kept with the tree (allocating and freeing
     // them in each call cost 0.3 ms, most of it the frees' synchronisation)
-    if ((mode != FDPS_CUTOFF_FIXED && !h_on_device) || !out_on_device)
-        if ((rc = ensure_short_io(t, n))) return rc;
-    if (!t->sr_info && dev_alloc(&t->sr_info, 3) != cudaSuccess) {
+    struct Busy {  // what this call still needs is not given back
+        fdps_tree* t;
+        ~Busy() { t->sr_busy = 0; }
+    } busy{t};
+    if (!t->sr_info && dev_alloc(t->ctx, &t->sr_info, 3) != cudaSuccess) {
         cudaGetLastError();
         return set_error(ctx, FDPS_ENOMEM, "neighbour output allocation failed");
     }
     const double* d_h = nullptr;
     if (mode != FDPS_CUTOFF_FIXED) {
+        if (!h_on_device) {
+            t->sr_busy = 1;
+            if ((rc = ensure_short_radii(t, n))) return rc;
+        }
         d_h = h_on_device ? h : t->sr_hin;
         if (!h_on_device &&
             cudaMemcpyAsync(t->sr_hin, h, sizeof(double) * n, cudaMemcpyHostToDevice, s) != cudaSuccess) {
@@ -910,6 +954,7 @@ int fdps_tree_neighbors(fdps_tree* t, fdps_psys* ps, int32_t mode, double r_fixe
         }
     }
     if ((rc = short_prepare(t, ps, mode, d_h))) return rc;
+    t->sr_busy = 0;
     const int wblocks = (int)(t->n_walk_warps / walk_warps_per_block());
     Redo r;
     do {
@@ -918,7 +963,8 @@ int fdps_tree_neighbors(fdps_tree* t, fdps_psys* ps, int32_t mode, double r_fixe
     } while (r.from != Redo::kNone);
     record(t, 7);  // stage times: ms_walk = radii preparation + walk, ms_force = pair pass
     // outputs the caller does not want still go to the tree's buffers
-    if (out_on_device && (!counts || !rho) && (rc = ensure_short_io(t, n))) return rc;
+    t->sr_busy = 2;
+    if ((!out_on_device || !counts || !rho) && (rc = ensure_short_out(t, n))) return rc;
     uint32_t* d_cnt = out_on_device && counts ? counts : t->sr_cnt;
     double* d_rho = out_on_device && rho ? rho : t->sr_rho;
     if (cudaMemsetAsync(t->sr_info, 0, sizeof(unsigned long long) * 3, s) != cudaSuccess) {
@@ -1330,8 +1376,8 @@ int fdps_psys_set_systems(fdps_psys* ps, int32_t n_sys, const int64_t* offsets) 
     ps->has_data = false;
     ps->has_forces = false;
     if (n_sys == 1) return FDPS_OK;
-    if (dev_alloc(&ps->d_off, n_sys + 1) != cudaSuccess || dev_alloc(&ps->d_sys, ps->n) != cudaSuccess ||
-        dev_alloc(&ps->d_sys_red, 2 * (int64_t)n_sys) != cudaSuccess) {
+    if (dev_alloc(ctx, &ps->d_off, n_sys + 1) != cudaSuccess || dev_alloc(ctx, &ps->d_sys, ps->n) != cudaSuccess ||
+        dev_alloc(ctx, &ps->d_sys_red, 2 * (int64_t)n_sys) != cudaSuccess) {
         cudaGetLastError();
         dev_free(ps->d_off);
         dev_free(ps->d_sys);
@@ -1356,8 +1402,8 @@ int fdps_psys_set_systems(fdps_psys* ps, int32_t n_sys, const int64_t* offsets) 
     csfb[n_sys] = (uint32_t)cbs.size();
     const int64_t nbk = (int64_t)cbsys.size();
     cbs.push_back((uint32_t)ps->n);
-    if (dev_alloc(&ps->d_cbs, nbk + 1) == cudaSuccess && dev_alloc(&ps->d_cbsys, nbk) == cudaSuccess &&
-        dev_alloc(&ps->d_csfb, (int64_t)n_sys + 1) == cudaSuccess) {
+    if (dev_alloc(ctx, &ps->d_cbs, nbk + 1) == cudaSuccess && dev_alloc(ctx, &ps->d_cbsys, nbk) == cudaSuccess &&
+        dev_alloc(ctx, &ps->d_csfb, (int64_t)n_sys + 1) == cudaSuccess) {
         FDPS_CUDA_TRY(ctx, cudaMemcpyAsync(ps->d_cbs, cbs.data(), sizeof(uint32_t) * (nbk + 1),
                                            cudaMemcpyHostToDevice, ctx->stream));
         FDPS_CUDA_TRY(ctx, cudaMemcpyAsync(ps->d_cbsys, cbsys.data(), sizeof(uint32_t) * nbk,

@@ -353,7 +353,7 @@ static void free_sample_scratch(SampleScratch& sc) {
 
 static int invert_ids(fdps_psys* ps, SampleScratch& sc) {
     fdps_ctx* ctx = ps->ctx;
-    if (!sc.inv && cudaMalloc(&sc.inv, sizeof(uint32_t) * (size_t)ps->n) != cudaSuccess) {
+    if (!sc.inv && dev_alloc(ctx, &sc.inv, ps->n) != cudaSuccess) {
         cudaGetLastError();
         return set_error(ctx, FDPS_ENOMEM, "sample scratch allocation failed");
     }
@@ -390,9 +390,8 @@ int direct_sample_device(fdps_psys* ps, int64_t ns, const int64_t* d_rows, doubl
     by = std::max<int64_t>(1, std::min<int64_t>({by, 1024, (J.total + nsl - 1) / nsl}));
     const int tper = (int)((J.total + by - 1) / by);
     const int js = one ? (int)by * nsl : 1;
-    if (!rc && (cudaMalloc(&sc.hi, sizeof(float4) * (size_t)n) != cudaSuccess ||
-                cudaMalloc(&sc.lo, sizeof(float4) * (size_t)n) != cudaSuccess ||
-                cudaMalloc(&sc.part, sizeof(double) * 4 * (size_t)ns * js) != cudaSuccess)) {
+    if (!rc && (dev_alloc(ctx, &sc.hi, n) != cudaSuccess || dev_alloc(ctx, &sc.lo, n) != cudaSuccess ||
+                dev_alloc(ctx, &sc.part, 4 * ns * js) != cudaSuccess)) {
         cudaGetLastError();
         rc = set_error(ctx, FDPS_ENOMEM, "sample scratch allocation failed");
     }

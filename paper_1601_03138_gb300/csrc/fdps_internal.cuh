@@ -217,9 +217,34 @@ struct BoxPartial {
     double hi[3];
 };
 
+// A context's handles of one kind (linked through the handles themselves).
+template <class T>
+struct Chain {
+    T* head = nullptr;
+    void add(T* p) {
+        p->chain = this;
+        p->prev = nullptr;
+        p->next = head;
+        if (head) head->prev = p;
+        head = p;
+    }
+    static void remove(T* p) {
+        if (!p->chain) return;
+        if (p->prev) p->prev->next = p->next;
+        if (p->next) p->next->prev = p->prev;
+        if (p->chain->head == p) p->chain->head = p->next;
+        p->chain = nullptr;
+    }
+    void clear() {
+        while (head) remove(head);
+    }
+};
+
 }  // namespace fdps
 
 struct fdps_ctx {
+    fdps::Chain<fdps_psys> systems;
+    fdps::Chain<fdps_tree> trees;
     int device = 0;
     int sm_count = 0;
     cudaStream_t own_stream = nullptr;
@@ -231,6 +256,8 @@ struct fdps_ctx {
 };
 
 struct fdps_psys {
+    fdps::Chain<fdps_psys>* chain = nullptr;  // the context's systems
+    fdps_psys *prev = nullptr, *next = nullptr;
     fdps_ctx* ctx = nullptr;
     int64_t n = 0;
     // current particle order (double-buffered for reordering)
@@ -256,7 +283,10 @@ struct fdps_psys {
     double* d_red = nullptr;     // reduction scratch (energy)
     double* stage = nullptr;     // host-transfer staging (10 n doubles, on first use)
     uint32_t* inv = nullptr;     // inverse of the current order (on first use)
-    double* rec = nullptr;       // [n][8] records of new data in the current order (on first use)
+    // records of data on its way in or out, 8 doubles a particle or 4 (on
+    // first use; given back when another allocation needs the room)
+    double* rec = nullptr;
+    int64_t cap_rec = 0;         // doubles
     // independent systems: positions off[k] .. off[k+1] belong to system k;
     // with one system d_off and d_sys stay null
     int32_t n_sys = 1;
@@ -273,6 +303,8 @@ struct fdps_psys {
 };
 
 struct fdps_tree {
+    fdps::Chain<fdps_tree>* chain = nullptr;  // the context's trees
+    fdps_tree *prev = nullptr, *next = nullptr;
     fdps_ctx* ctx = nullptr;
     fdps_tree_params p{};
     // per-particle scratch
@@ -294,11 +326,14 @@ struct fdps_tree {
     int64_t cap_nd_hmax = 0;
     double* g_hmax = nullptr;
     int64_t cap_g_hmax = 0;
-    // its host arrays' device copies (on first use) and pair counters
+    // its host arrays' device copies (on first use; given back when another
+    // allocation needs the room, unless sr_busy holds them) and pair counters
     double* sr_hin = nullptr;
+    int64_t cap_sr_hin = 0;
     uint32_t* sr_cnt = nullptr;
     double* sr_rho = nullptr;
-    int64_t cap_sr_io = 0;
+    int64_t cap_sr_out = 0;
+    int sr_busy = 0;  // 1: sr_hin, 2: sr_cnt and sr_rho
     unsigned long long* sr_info = nullptr;
     // coherent sort: the sorted keys of the last call (keys_b) belong to
     // psys coh_ps at generation coh_gen, whose particles are in that order
@@ -408,11 +443,26 @@ inline int set_error(fdps_ctx* ctx, int code, const char* fmt, ...) {
         FDPS_CUDA_TRY(ctx, cudaGetLastError());  \
     } while (0)
 
+// Frees the buffers that the context's handles only keep for their next call;
+// false if there were none (api.cu).
+bool give_back_scratch(fdps_ctx* ctx);
+
+// An allocation that may fail without harm takes dev_try.
 template <class T>
-inline cudaError_t dev_alloc(T** p, int64_t count) {
+inline cudaError_t dev_try(T** p, int64_t count) {
     *p = nullptr;
     if (count <= 0) count = 1;
-    return cudaMalloc(reinterpret_cast<void**>(p), sizeof(T) * (size_t)count);
+    const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), sizeof(T) * (size_t)count);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        *p = nullptr;
+    }
+    return e;
+}
+template <class T>
+inline cudaError_t dev_alloc(fdps_ctx* ctx, T** p, int64_t count) {
+    const cudaError_t e = dev_try(p, count);
+    return e == cudaErrorMemoryAllocation && give_back_scratch(ctx) ? dev_try(p, count) : e;
 }
 
 template <class T>

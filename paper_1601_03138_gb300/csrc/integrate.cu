@@ -410,27 +410,33 @@ int launch_energy_systems(fdps_psys* ps, double* kin, double* pot) {
 
 int energy_scratch_doubles() { return 2 * kEnergyBlocks + 2; }
 
+// The record buffer for `per` doubles a particle, null without room for it.
+static double2* ensure_rec(fdps_psys* ps, int per) {
+    const int64_t need = per * ps->n;
+    if (ps->cap_rec < need) {
+        dev_free(ps->rec);
+        ps->cap_rec = dev_try(&ps->rec, need) == cudaSuccess ? need : 0;
+    }
+    return reinterpret_cast<double2*>(ps->rec);
+}
+
 int launch_scatter_in(fdps_psys* ps, const double* pos, const double* vel, const double* mass,
                       const double* eps, bool keep_order, uint32_t* bad) {
     fdps_ctx* ctx = ps->ctx;
     if (!keep_order) ps->cur = 0;
     const int c = ps->cur;
     if (keep_order) {
-        if (!ps->inv && dev_alloc(&ps->inv, ps->n) != cudaSuccess) {
+        if (!ps->inv && dev_alloc(ctx, &ps->inv, ps->n) != cudaSuccess) {
             cudaGetLastError();
             ps->inv = nullptr;
             return set_error(ctx, FDPS_ENOMEM, "inverse-order allocation failed");
         }
         k_invert<<<grid_for(ps->n, 256, ctx->sm_count * 16), 256, 0, ctx->stream>>>(ps->n, ps->id[c], ps->inv);
         FDPS_LAUNCH_CHECK(ctx);
-        // without the record buffer the values are written straight into
-        // the arrays (scattered 8-byte writes, slower)
-        if (!ps->rec && dev_alloc(&ps->rec, 8 * ps->n) != cudaSuccess) {
-            cudaGetLastError();
-            ps->rec = nullptr;
-        }
     }
-    double2* rec = keep_order ? reinterpret_cast<double2*>(ps->rec) : nullptr;
+    // without the record buffer the values are written straight into the
+    // arrays (scattered 8-byte writes, slower)
+    double2* rec = keep_order ? ensure_rec(ps, 8) : nullptr;
     FDPS_CUDA_TRY(ctx, cudaMemsetAsync(ps->d_flag, 0, sizeof(uint32_t), ctx->stream));
     k_scatter_in<<<grid_for(ps->n, kIoTile, ctx->sm_count * 8), kIoTile, 0, ctx->stream>>>(
         ps->n, pos, vel, mass, eps, ps->x[c], ps->y[c], ps->z[c], ps->vx[c], ps->vy[c], ps->vz[c],
@@ -457,7 +463,7 @@ constexpr int64_t kGatherRec = int64_t(1) << 21;
 int launch_gather_out(fdps_psys* ps, double* pos, double* vel, double* acc, double* pot, bool device_out) {
     fdps_ctx* ctx = ps->ctx;
     const int c = ps->cur;
-    if (!ps->inv && dev_alloc(&ps->inv, ps->n) != cudaSuccess) {
+    if (!ps->inv && dev_alloc(ctx, &ps->inv, ps->n) != cudaSuccess) {
         cudaGetLastError();
         ps->inv = nullptr;
         return set_error(ctx, FDPS_ENOMEM, "inverse-order allocation failed");
@@ -466,14 +472,8 @@ int launch_gather_out(fdps_psys* ps, double* pos, double* vel, double* acc, doub
     k_invert<<<grid, 256, 0, ctx->stream>>>(ps->n, ps->id[c], ps->inv);
     FDPS_LAUNCH_CHECK(ctx);
     const bool state = pos && vel, force = acc && pot;
-    bool by_rec = device_out && ps->n >= kGatherRec && (state || force);
-    if (by_rec && !ps->rec && dev_alloc(&ps->rec, 8 * ps->n) != cudaSuccess) {
-        cudaGetLastError();  // no room for the records: the plain gather
-        ps->rec = nullptr;
-        by_rec = false;
-    }
-    if (by_rec) {
-        double2* rec = reinterpret_cast<double2*>(ps->rec);
+    // (no room for the records: the plain gather)
+    if (double2* rec = device_out && ps->n >= kGatherRec && (state || force) ? ensure_rec(ps, state ? 8 : 4) : nullptr) {
         const int tiles = grid_for(ps->n, kIoTile, ctx->sm_count * 8);
         if (state) {
             k_pack_state<<<grid, 256, 0, ctx->stream>>>(ps->n, ps->x[c], ps->y[c], ps->z[c], ps->vx[c], ps->vy[c],

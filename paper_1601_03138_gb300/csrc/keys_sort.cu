@@ -1242,7 +1242,7 @@ int keys_and_sort(fdps_tree* t, fdps_psys* ps) {
         } else {
             dev_free(t->coh_cnt);
             t->cap_coh = 0;
-            if (dev_alloc(&t->coh_cnt, 3 * nbl + 8) != cudaSuccess) {
+            if (dev_alloc(ctx, &t->coh_cnt, 3 * nbl + 8) != cudaSuccess) {
                 cudaGetLastError();
                 t->coh_cnt = nullptr;
                 return set_error(ctx, FDPS_ENOMEM, "coherent-sort counters allocation failed");

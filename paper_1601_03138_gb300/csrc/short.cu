@@ -660,7 +660,7 @@ int short_prepare(fdps_tree* t, fdps_psys* ps, int mode, const double* h_user) {
     if (t->cap_sr_h < n) {
         dev_free(t->sr_h);
         t->cap_sr_h = 0;
-        if (dev_alloc(&t->sr_h, n) != cudaSuccess) {
+        if (dev_alloc(ctx, &t->sr_h, n) != cudaSuccess) {
             cudaGetLastError();
             return set_error(ctx, FDPS_ENOMEM, "cutoff radii allocation failed");
         }
@@ -678,7 +678,7 @@ int short_prepare(fdps_tree* t, fdps_psys* ps, int mode, const double* h_user) {
     if (t->cap_nd_hmax < nn) {
         dev_free(t->nd_hmax);
         t->cap_nd_hmax = 0;
-        if (dev_alloc(&t->nd_hmax, t->cap_nodes) != cudaSuccess) {
+        if (dev_alloc(ctx, &t->nd_hmax, t->cap_nodes) != cudaSuccess) {
             cudaGetLastError();
             return set_error(ctx, FDPS_ENOMEM, "node radii allocation failed");
         }
@@ -687,7 +687,7 @@ int short_prepare(fdps_tree* t, fdps_psys* ps, int mode, const double* h_user) {
     if (t->cap_g_hmax < ng) {
         dev_free(t->g_hmax);
         t->cap_g_hmax = 0;
-        if (dev_alloc(&t->g_hmax, t->cap_groups) != cudaSuccess) {
+        if (dev_alloc(ctx, &t->g_hmax, t->cap_groups) != cudaSuccess) {
             cudaGetLastError();
             return set_error(ctx, FDPS_ENOMEM, "group radii allocation failed");
         }
