@@ -173,8 +173,10 @@ __global__ void __launch_bounds__(kSBlock) k_short_walk(ShortWalkArgs A) {
                     const float gz = (float)max(0, max((int)qz - (int)(qmax2 + 1), (int)qmin2 - (int)(qz + w + 1)));
                     const float d2 = gx * gx + gy * gy + gz * gz;
                     const float R = short_bound(A.mode, A.r_fixed, hc, hg) * idq;
-                    // margin: FP32 rounding of the bound and of the gaps
-                    const bool near = d2 <= R * R * (1.0f + 64.0f * kU);
+                    // margin: FP32 rounding of the bound and of the gaps (a NaN,
+                    // where a radius or the spacing is 0 or infinite in FP32,
+                    // keeps the cell: the pairs are decided one by one)
+                    const bool near = !(d2 > R * R * (1.0f + 64.0f * kU));
                     if (near) {
                         if (leaf) {
                             emit = true;
