@@ -364,10 +364,12 @@ __device__ __forceinline__ f2 wendland_q2(f2 r2, f2 nih2) {
 // r^2 <= c^2 (a <= r <= c), and for r^2 > c^2, with a <= r <= (r^2 + c^2) /
 // (2c), M <= (56u + 192u^2 + beta) r^2 + (8u + beta) c^2 + 3 Eabs^2, beta =
 // 3 Eabs / c (slack for the FP32 evaluation of both).  A cutoff within a few
-// Eabs sends every pair to the FP64 sequence.
+// Eabs sends every pair to the FP64 sequence, and so does one whose square's
+// roundings come near the spacing of subnormal numbers (1.4e-45 against M >= 64u
+// c^2 = 4e-40 from 1e-17 on).
 __device__ __forceinline__ float2 pair_thresholds(float c, float Eabs) {
     const float c2 = c * c, beta = 3.0001f * Eabs / c;
-    if (!(beta < 0.25f)) return make_float2(-INFINITY, INFINITY);
+    if (!(beta < 0.25f) || c < 1e-17f) return make_float2(-INFINITY, INFINITY);
     const float tq = fmaf(8.0f * kU, c, Eabs);
     const float Mmax = 64.0f * kU * c2 + 6.0f * c * Eabs + 3.0f * tq * tq;
     return make_float2(c2 - (1.01f * Mmax + 4.0f * kU * c2),
@@ -430,7 +432,8 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
         const float hb = fmaxf(hx, fmaxf(hy, hz));
         // what a cutoff grows by so that the FP32 distance to the box never
         // drops a pair that the thresholds or the FP64 sequence look at: the
-        // distance's error is below 4u (C + 2 hb) + 2 Eabs
+        // distance's error is below 4u (C + 2 hb) + 2 Eabs; squares are compared
+        // from 1e-34 on, far above the subnormal numbers
         const float pad = 64.0f * kU * hb + 16.0f * Eabs;
         const float hg = MODE == 0 ? (float)A.r_fixed : MODE == 2 ? 0.0f : (float)A.g_hmax[g];
         const uint32_t P = ni <= 16u ? ni : 32u;
@@ -581,7 +584,7 @@ __global__ void __launch_bounds__(kSBlock, 8) k_short_pairs(ShortPairArgs A) {
                         const float tx = fmaxf(fabsf(dx) - hx, 0.0f), ty = fmaxf(fabsf(dy) - hy, 0.0f),
                                     tz = fmaxf(fabsf(dz) - hz, 0.0f);
                         const float C = fmaf(fmaxf(hg, hj), 1.0f + 256.0f * kU, pad);
-                        keep = !(fmaf(tx, tx, fmaf(ty, ty, tz * tz)) > C * C);
+                        keep = !(fmaf(tx, tx, fmaf(ty, ty, tz * tz)) > fmaxf(C * C, 1e-34f));
                     }
                     const uint32_t mask = __ballot_sync(0xFFFFFFFFu, keep);
                     if (keep) {
