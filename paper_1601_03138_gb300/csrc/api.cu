@@ -414,6 +414,42 @@ int run_force(fdps_tree* t, fdps_psys* ps, int k_spj, bool lists_only = false) {
     return FDPS_OK;
 }
 
+// A small force calculation, and its walk and force kernels once more with the
+// bit of a wait that gave up in the state word: they must not take any group.
+int selftest_stalled_step(fdps_ctx* ctx, int64_t n, bool fp64) {
+    fdps_tree_params p{};
+    p.theta = 0.5;
+    p.n_leaf = 8;
+    p.n_grp = 64;
+    p.moment = FDPS_MONOPOLE;
+    p.precision = fp64 ? FDPS_FP64 : FDPS_FP32REL;
+    std::vector<double> pos(3 * (size_t)n), vel(3 * (size_t)n, 0.0), one((size_t)n, 1.0);
+    for (size_t i = 0; i < pos.size(); ++i) pos[i] = std::fmod(0.6180339887498949 * (double)(i + 1) * (double)(i % 3 + 1), 1.0);
+    fdps_psys* ps = nullptr;
+    fdps_tree* t = nullptr;
+    int rc = fdps_psys_create(ctx, n, &ps);
+    if (!rc) rc = fdps_psys_set(ps, pos.data(), vel.data(), one.data(), one.data(), 0);
+    if (!rc) rc = fdps_tree_create(ctx, &p, &t);
+    if (!rc) rc = run_force(t, ps, FDPS_GRAV_SPJ_MONO);
+    if (!rc) rc = read_state(t);
+    if (!rc) {
+        DevState h = t->h_st;
+        const bool ran = h.walk_counter > 0 && h.force_counter > 0;
+        h.walk_counter = h.force_counter = 0;
+        h.overflow = kSortStall;
+        if (cudaMemcpyAsync(t->st, &h, sizeof(h), cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess)
+            rc = set_error(ctx, FDPS_ECUDA, "self-test set-up failed");
+        if (!rc) rc = launch_walk(t, ps->d_sys, (int)(t->n_walk_warps / walk_warps_per_block()));
+        if (!rc) rc = compute_forces(t, ps, FDPS_GRAV_SPJ_MONO);
+        if (!rc) rc = read_state(t);
+        if (!rc && (!ran || t->h_st.walk_counter || t->h_st.force_counter || t->h_st.overflow != kSortStall))
+            rc = set_error(ctx, FDPS_ECUDA, "a kernel ran on after a wait that gave up");
+    }
+    if (t) fdps_tree_destroy(t);
+    if (ps) fdps_psys_destroy(ps);
+    return rc;
+}
+
 bool valid_params(const fdps_tree_params* p) {
     return p && p->theta >= 0.0 && p->theta < 1e6 && p->theta == p->theta && p->n_leaf >= 1 &&
            p->n_leaf <= kMaxLeaf && p->n_grp >= p->n_leaf && p->n_grp <= kMaxGrp &&
@@ -512,11 +548,14 @@ int64_t fdps_kernel_launches(const fdps_ctx* ctx) { return ctx ? ctx->launches :
 int fdps_selftest_bounded_wait(fdps_ctx* ctx) {
     if (!ctx) return FDPS_EINVAL;
     cudaSetDevice(ctx->device);
-    uint32_t flags = 0;
-    int rc = selftest_lookback_timeout(ctx, &flags);
+    uint32_t lookback = 0, barrier = 0;
+    int rc = selftest_lookback_timeout(ctx, &lookback);
+    if (!rc) rc = selftest_barrier_timeout(ctx, &barrier);
     if (rc) return rc;
-    if (flags & kSortStall) return set_error(ctx, FDPS_ETIMEOUT, "bounded wait gave up as designed");
-    return FDPS_OK;
+    if (!(lookback & barrier & kSortStall)) return FDPS_OK;
+    for (int k = 0; k < 3; ++k)
+        if ((rc = selftest_stalled_step(ctx, k == 1 ? 40000 : 300, k == 2))) return rc;
+    return set_error(ctx, FDPS_ETIMEOUT, "bounded wait gave up as designed");
 }
 
 int fdps_set_profiling(fdps_ctx* ctx, int on) {

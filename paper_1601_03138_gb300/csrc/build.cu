@@ -813,14 +813,15 @@ __global__ void __cluster_dims__(kMomCl, 1, 1) __launch_bounds__(kMomBlock) k_mo
 // each barrier.  The wait is bounded: beyond it the error bit of a device
 // wait is set and the block goes on (its sums are then invalid, every access
 // stays within the node arrays).
-__device__ __forceinline__ void grid_barrier(uint32_t* count, uint32_t target, uint32_t* overflow) {
+__device__ __forceinline__ void grid_barrier(uint32_t* count, uint32_t target, uint32_t* overflow,
+                                             int max_spin = kMaxGridSpin) {
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(count, 1u);
         int spin = 0;
         while (*(volatile uint32_t*)count < target)
-            if (++spin > kMaxGridSpin) {
+            if (++spin > max_spin) {
                 atomicOr(overflow, kSortStall);
                 break;
             }
@@ -871,6 +872,11 @@ __global__ void __launch_bounds__(kMomBlock, 2) k_moments_levels(MomArgs A, uint
         __threadfence_block();
         __syncthreads();  // this level complete before its parents
     }
+}
+
+// A barrier of one block that waits for an arrival that never comes.
+__global__ void k_barrier_selftest(uint32_t* count, uint32_t* flags, int max_spin) {
+    grid_barrier(count, 2u, flags, max_spin);
 }
 
 template <bool QUAD, bool Q64>
@@ -1152,6 +1158,25 @@ int build_tree(fdps_tree* t, fdps_psys* ps) {
     k_tree_finish<<<ctx->sm_count * 4, 256, 0, s>>>(t->st, ps->n_sys, t->nd_first, t->nd_count, t->nd_parent,
                                                     t->nd_child, t->nd_meta);
     FDPS_LAUNCH_CHECK(ctx);
+    return FDPS_OK;
+}
+
+int selftest_barrier_timeout(fdps_ctx* ctx, uint32_t* flags_out) {
+    uint32_t* w = nullptr;  // count, flags
+    uint32_t h[2] = {0, 0};
+    if (dev_alloc(ctx, &w, 2) != cudaSuccess) return set_error(ctx, FDPS_ENOMEM, "self-test allocation failed");
+    cudaStream_t s = ctx->stream;
+    cudaError_t e = cudaMemsetAsync(w, 0, sizeof(h), s);
+    if (!e) {
+        k_barrier_selftest<<<1, kMomBlock, 0, s>>>(w, w + 1, 1 << 12);
+        ++ctx->launches;
+        e = cudaGetLastError();
+    }
+    if (!e) e = cudaMemcpyAsync(h, w, sizeof(h), cudaMemcpyDeviceToHost, s);
+    if (!e) e = cudaStreamSynchronize(s);
+    cudaFree(w);
+    if (e) return set_error(ctx, FDPS_ECUDA, "self-test failed: %s", cudaGetErrorString(e));
+    *flags_out = h[1];
     return FDPS_OK;
 }
 

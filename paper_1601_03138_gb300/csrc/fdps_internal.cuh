@@ -50,7 +50,7 @@ constexpr uint32_t kOvfFrontier = 4u;
 constexpr uint32_t kOvfGroups = 8u;
 constexpr uint32_t kBadInput = 16u;
 constexpr uint32_t kOvfChunk = 32u;
-constexpr uint32_t kSortStall = 64u;  // a radix-sort look-back wait gave up
+constexpr uint32_t kSortStall = 64u;  // a device-side wait gave up (a radix-sort look-back or the moments' grid barrier)
 constexpr uint32_t kSortRedo = 256u;  // a bucket of the coherent sort overflowed: redo with the radix sort
 constexpr uint32_t kSortInvalid = kSortStall | kSortRedo;  // this call's order is not sorted
 // Any of these leaves the tree or its groups incomplete: the walk has nothing
@@ -487,6 +487,7 @@ int launch_sys_index(fdps_psys* ps);                   // integrate.cu
 int launch_energy_systems(fdps_psys* ps, double* kin, double* pot);  // integrate.cu
 int reorder_particles(fdps_tree* t, fdps_psys* ps);    // keys_sort.cu
 int selftest_lookback_timeout(fdps_ctx* ctx, uint32_t* flags_out);  // keys_sort.cu
+int selftest_barrier_timeout(fdps_ctx* ctx, uint32_t* flags_out);   // build.cu
 int build_tree(fdps_tree* t, fdps_psys* ps);           // build.cu
 int compute_moments(fdps_tree* t, fdps_psys* ps);      // build.cu
 int select_groups(fdps_tree* t, fdps_psys* ps);        // build.cu

@@ -1,9 +1,11 @@
 """Failure detection on the GPU without a GPU fault.
 
-The only device-side waits are the radix sort's look-backs on earlier tiles;
-each is bounded.  The self-test runs a look-back whose predecessor never
-publishes: the wait must give up, report FDPS_ETIMEOUT, and leave the
-context usable for a normal force calculation right after.
+The device-side waits are the radix sort's look-backs on earlier tiles and the
+grid barriers of the moments of large sets; each is bounded.  The self-test runs
+one of each whose counterpart never comes, and the walk and force kernels on a
+state word that reports such a wait: the waits must give up, the kernels take no
+group, the call report FDPS_ETIMEOUT, and the context must stay usable for normal
+force calculations right after.
 """
 import numpy as np
 import pytest
@@ -14,7 +16,8 @@ import oracle
 pytestmark = pytest.mark.gpu
 
 
-def test_bounded_wait_gives_up_and_context_survives():
+@pytest.mark.parametrize("n", [4000, 100003])
+def test_bounded_wait_gives_up_and_context_survives(n):
     from paper_1601_03138_gb300 import build as B
     B.build()
     import paper_1601_03138_gb300 as G
@@ -23,7 +26,6 @@ def test_bounded_wait_gives_up_and_context_survives():
         rc = G.fdps_selftest_bounded_wait(ctx.h)
         assert rc == G.FDPS_ETIMEOUT
         assert "gave up" in G.fdps_last_error(ctx.h)
-        n = 4000
         pos, vel, mass, eps = ics.make("plummer", n, 3, 0.02)
         ps = G.ParticleSystem(ctx, n)
         tree = G.Tree(ctx, theta=0.5, n_leaf=8, n_grp=64)
