@@ -23,7 +23,11 @@
  * Each thread owns one i-particle; it calls the functors with tiles of up
  * to 64 particles of opened leaves (EPJ) and up to 32 superparticles (SPJ),
  * which together make the i-particle's group's whole list, the superparticles
- * and the opened leaves each in list order, in turn.
+ * and the opened leaves each in list order, in turn: in which order calls
+ * with cells and calls with particles follow one another, and how many
+ * entries a call gets, is the library's choice and may change.  Arrays of Epj
+ * and Spj are to be indexed as such (they are 16 and 48 bytes, 16-byte
+ * aligned, the last 8 bytes of an Spj without meaning).
  * The particle itself is among its EPJ (zero separation): the law decides
  * what that term contributes.  Positions are FP32 relative to the group's
  * centre, formed from hi/lo parts as in the built-in kernel.  out[row] gets
@@ -66,9 +70,8 @@ struct __align__(16) Spj {
 
 namespace detail {
 
-constexpr int kThreads = 32;  // threads of a block, and list entries per step
+constexpr int kThreads = 32;  // threads of a block (one warp), and list entries per step
 constexpr int kSlots = 8;     // blocks sharing a group's i-particles (grid y)
-constexpr int kSpjCall = 32;  // most superparticles per functor call
 constexpr int kEpjCall = 64;  // most leaf particles per functor call
 
 __device__ __forceinline__ float4 ld4(const float* p, uint64_t i) {
@@ -78,28 +81,27 @@ __device__ __forceinline__ float4 ld4(const float* p, uint64_t i) {
 // The walk of the view's groups by a grid (any x, any y) of blocks of
 // kThreads: block (x, y) takes groups x, x + gridDim.x, ... and of each the
 // i-particles kThreads y .. + kThreads - 1 (and on by kThreads gridDim.y),
-// one per thread.  The block stages kThreads list entries at a time for all
-// its warps.  The law's own instructions bound it (issue slots 74 % busy), so
+// one per thread.  The block stages kThreads list entries at a time.  The law's own instructions bound it (issue slots 74 % busy), so
 // what counts is that every SM has warps with i-particles until the end: one
 // block per group and 32 i-particles, started by the hardware as others
 // finish, where a fixed share of the groups for each warp of one resident
 // wave, eight passes over the list for a group of 256, left most of the SMs
 // idle behind the warps with the large groups.  One warp a block: with two or
 // four, groups of 30 particles leave warps that only wait at the barriers.
-// Gravity with quadrupoles, lists and law: 2^20 Hernquist particles, n_grp 256,
-// 13.9 ms before, 7.8 with 32 threads, 8.2 with 64, 8.0 with 128; 500,000 Plummer
-// particles with monopoles, n_grp 64: 5.6, 4.6, 6.5 and 5.0 ms.
+// Gravity with quadrupoles, lists and law on one stream: 2^20 Hernquist
+// particles, n_grp 256, 13.9 ms before, 7.8 with 32 threads, 8.2 with 64, 8.0 with
+// 128; 500,000 Plummer particles with monopoles, n_grp 64: 5.6, 4.5, 6.5 and 5.0
+// ms.  (Calls of several contexts that overlap had filled the idle SMs with one
+// another's work: 8.4 ms a call before, 7.7 now.)
 template <class Force, class FEpj, class FSpj>
 __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const FEpj& f_epj,
                                                 const FSpj& f_spj, Force* out) {
-    constexpr int kW = kThreads / 32;
     __shared__ Spj s_spj[kThreads];
     __shared__ Epj s_epj[kEpjCall];
     __shared__ uint32_t s_first[kThreads];
     __shared__ uint32_t s_start[kThreads];
-    __shared__ uint32_t s_sum[2 * kW];
-    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    const uint32_t lt = (1u << lane) - 1u;
+    const int t = threadIdx.x;
+    const uint32_t lt = (1u << t) - 1u;
     for (int64_t g = blockIdx.x; g < v.n_groups; g += gridDim.x) {
         const uint32_t gf = v.g_first[g], ni = v.g_count[g];
         const unsigned long long off = v.g_off[g];
@@ -111,7 +113,7 @@ __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const F
         const uint32_t steps = (len + kThreads - 1) / kThreads;
         uint32_t nsp = 0;
         for (uint32_t n = steps; n > 0;) {
-            const uint32_t stride = (n + 31) / 32, at = lane * stride;
+            const uint32_t stride = (n + 31) / 32, at = t * stride;
             const bool sp = at < n && !(v.pool[off + (uint64_t)(nsp + at) * kThreads] & v.leaf_tag);
             const uint32_t c = __popc(__ballot_sync(0xFFFFFFFFu, sp));
             if (c == 0) break;
@@ -154,23 +156,10 @@ __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const F
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-                    if (lane >= o) inc += x;
+                    if (t >= o) inc += x;
                 }
-                if (lane == 31) {
-                    s_sum[w] = __popc(smask);
-                    s_sum[kW + w] = inc;
-                }
-                __syncthreads();  // also: the previous step's tiles are consumed
-                uint32_t rank = __popc(smask & lt), start = inc - cnt, nspj = 0, total = 0;
-#pragma unroll
-                for (int k = 0; k < kW; ++k) {
-                    if (k < w) {
-                        rank += s_sum[k];
-                        start += s_sum[kW + k];
-                    }
-                    nspj += s_sum[k];
-                    total += s_sum[kW + k];
-                }
+                const uint32_t nspj = __popc(smask), total = __shfl_sync(0xFFFFFFFFu, inc, 31);
+                __syncwarp();  // the previous step's tiles are consumed
                 if (spj) {
                     const float4 fh = ld4(v.nd_f, 2ull * node), fl = ld4(v.nd_f, 2ull * node + 1);
                     Spj s;
@@ -189,17 +178,15 @@ __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const F
                         s.qxz = q1.x;
                         s.qyz = q1.y;
                     }
-                    s_spj[rank] = s;
+                    s_spj[__popc(smask & lt)] = s;
                 }
                 s_first[t] = leaf ? v.nd_first[node] : 0u;
-                s_start[t] = start;
-                __syncthreads();
-                if (act)
-                    for (uint32_t k = 0; k < nspj; k += kSpjCall)
-                        f_spj(epi, &s_spj[k], (int)(nspj - k < (uint32_t)kSpjCall ? nspj - k : (uint32_t)kSpjCall), f);
+                s_start[t] = inc - cnt;
+                __syncwarp();
+                if (act && nspj > 0) f_spj(epi, &s_spj[0], (int)nspj, f);
                 for (uint32_t c0 = 0; c0 < total; c0 += kEpjCall) {
                     const uint32_t m = total - c0 < (uint32_t)kEpjCall ? total - c0 : (uint32_t)kEpjCall;
-                    if (c0 > 0) __syncthreads();
+                    if (c0 > 0) __syncwarp();
                     for (uint32_t k = t; k < m; k += kThreads) {
                         // the owning entry: the last one whose start <= item
                         // (entries with no particles share the next one's start)
@@ -213,12 +200,12 @@ __device__ __forceinline__ void calc_force_body(const fdps_tree_view& v, const F
                         s_epj[k] = Epj{(h.x - ch.x) + (l.x - cl.x), (h.y - ch.y) + (l.y - cl.y),
                                        (h.z - ch.z) + (l.z - cl.z), h.w};
                     }
-                    __syncthreads();
+                    __syncwarp();
                     if (act) f_epj(epi, &s_epj[0], (int)m, f);
                 }
             }
             if (act) out[epi.row] = f;
-            __syncthreads();  // the tiles are rewritten for the next i-particles
+            __syncwarp();  // the tiles are rewritten for the next i-particles
         }
     }
 }
