@@ -485,7 +485,6 @@ struct MomArgs {
     const uint32_t* nd_count;
     const uint32_t* nd_child;
     const uint32_t* nd_meta;
-    const uint32_t* nd_parent;
     const uint64_t* nd_qlo;
     // written here and read back for the parent in a later launch (read
     // through L2 with __ldcg)
@@ -1200,7 +1199,6 @@ int compute_moments(fdps_tree* t, fdps_psys* ps) {
     A.nd_count = t->nd_count;
     A.nd_child = t->nd_child;
     A.nd_meta = t->nd_meta;
-    A.nd_parent = t->nd_parent;
     A.nd_qlo = t->nd_qlo;
     A.nd_sx = t->nd_sx;
     A.nd_sy = t->nd_sy;

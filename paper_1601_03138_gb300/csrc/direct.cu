@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "fdps_internal.cuh"
+#include "packed.cuh"
 
 namespace fdps {
 namespace {
@@ -67,45 +68,6 @@ __device__ __forceinline__ void pair(const float4 ih, const float4 il, const flo
     ay = fmaf(mri3, dy, ay);
     az = fmaf(mri3, dz, az);
     pp -= mri;
-}
-
-// Two FP32 lanes in one 64-bit register: one packed instruction evaluates
-// an operation of the pair law for two i-particles, each lane rounded as the
-// scalar instruction.
-typedef unsigned long long f2;
-__device__ __forceinline__ f2 f2_pk(float lo, float hi) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void f2_up(f2 v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
-    f2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
-    f2 d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
-    f2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-// rsqrtf for arguments that are no subnormals: the bare MUFU operation
-__device__ __forceinline__ float rsqrt_normal(float v) {
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-    return r;
 }
 
 // One tile of m j-particles on the 2 KP i-particles of a thread.  SELF: an i-particle of the warp is in the

@@ -30,6 +30,7 @@
 // (a cluster of CTAs per group) evaluates the same terms on FP64 absolute
 // coordinates with FP64 sums.
 #include "fdps_internal.cuh"
+#include "packed.cuh"
 
 namespace fdps {
 
@@ -162,10 +163,6 @@ __device__ __forceinline__ uint32_t block_scan1(uint32_t a, uint32_t* total, uin
         const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, ia, o);
         if (lane >= o) ia += v;
     }
-    if (CB == 32) {
-        *total = __shfl_sync(0xFFFFFFFFu, ia, 31);
-        return ia - a;
-    }
     if (lane == 31) s_w[w] = ia;
     __syncthreads();
     uint32_t o = 0, sum = 0;
@@ -226,34 +223,7 @@ __device__ __forceinline__ void kahan_smem_add(float* s_k, int q, int c, float v
     *s = t;
 }
 
-// Two FP32 lanes in one 64-bit register (low = i-particle 2h, high =
-// 2h+1): each packed instruction evaluates one operation of the pair law
-// for two interactions, halving the FP32 instructions the scheduler issues.
-// Each lane is rounded exactly as the scalar instruction.
-typedef unsigned long long f2;
-__device__ __forceinline__ f2 f2_pk(float lo, float hi) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void f2_up(f2 v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
-    f2 d;
-    asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
-    f2 d;
-    asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
-    f2 d;
-    asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
+// (the packed operations flush subnormals, as the whole file is compiled to)
 __device__ __forceinline__ f2 f2_rsqrt(f2 v) {
     float a, b;
     f2_up(v, a, b);
@@ -438,31 +408,31 @@ __device__ __forceinline__ void force_round_f32(const ForceArgs& A, uint32_t gf,
                 }
 #pragma unroll
                 for (int h = 0; h < KP; ++h) {
-                    const f2 rx = f2_sub(xp[h], jx), ry = f2_sub(yp[h], jy), rz = f2_sub(zp[h], jz);
-                    const f2 R2 = f2_fma(rx, rx, f2_fma(ry, ry, f2_fma(rz, rz, ep[h])));
+                    const f2 rx = f2_sub<true>(xp[h], jx), ry = f2_sub<true>(yp[h], jy), rz = f2_sub<true>(zp[h], jz);
+                    const f2 R2 = f2_fma<true>(rx, rx, f2_fma<true>(ry, ry, f2_fma<true>(rz, rz, ep[h])));
                     const f2 Ri = f2_rsqrt(R2);
-                    const f2 Ri2 = f2_mul(Ri, Ri);
+                    const f2 Ri2 = f2_mul<true>(Ri, Ri);
                     if (QUAD) {
-                        const f2 Ri4 = f2_mul(Ri2, Ri2);
-                        const f2 Ri5 = f2_mul(Ri4, Ri);
-                        const f2 Qrx = f2_fma(qxx, rx, f2_fma(qxy, ry, f2_mul(qxz, rz)));
-                        const f2 Qry = f2_fma(qxy, rx, f2_fma(qyy, ry, f2_mul(qyz, rz)));
-                        const f2 Qrz = f2_fma(qxz, rx, f2_fma(qyz, ry, f2_mul(qzz, rz)));
-                        const f2 rQr = f2_fma(rx, Qrx, f2_fma(ry, Qry, f2_mul(rz, Qrz)));
-                        const f2 w = f2_mul(rQr, Ri4);         // r.Q.r / R^4
-                        const f2 hh = f2_fma(cm25, w, nM);     // -M - 5/2 w
-                        const f2 hR2 = f2_mul(hh, R2);
-                        pax[h] = f2_fma(Ri5, f2_fma(hR2, rx, Qrx), pax[h]);
-                        pay[h] = f2_fma(Ri5, f2_fma(hR2, ry, Qry), pay[h]);
-                        paz[h] = f2_fma(Ri5, f2_fma(hR2, rz, Qrz), paz[h]);
-                        pp[h] = f2_fma(Ri, f2_fma(c2, w, hh), pp[h]);  // (-M - w/2) / R
+                        const f2 Ri4 = f2_mul<true>(Ri2, Ri2);
+                        const f2 Ri5 = f2_mul<true>(Ri4, Ri);
+                        const f2 Qrx = f2_fma<true>(qxx, rx, f2_fma<true>(qxy, ry, f2_mul<true>(qxz, rz)));
+                        const f2 Qry = f2_fma<true>(qxy, rx, f2_fma<true>(qyy, ry, f2_mul<true>(qyz, rz)));
+                        const f2 Qrz = f2_fma<true>(qxz, rx, f2_fma<true>(qyz, ry, f2_mul<true>(qzz, rz)));
+                        const f2 rQr = f2_fma<true>(rx, Qrx, f2_fma<true>(ry, Qry, f2_mul<true>(rz, Qrz)));
+                        const f2 w = f2_mul<true>(rQr, Ri4);         // r.Q.r / R^4
+                        const f2 hh = f2_fma<true>(cm25, w, nM);     // -M - 5/2 w
+                        const f2 hR2 = f2_mul<true>(hh, R2);
+                        pax[h] = f2_fma<true>(Ri5, f2_fma<true>(hR2, rx, Qrx), pax[h]);
+                        pay[h] = f2_fma<true>(Ri5, f2_fma<true>(hR2, ry, Qry), pay[h]);
+                        paz[h] = f2_fma<true>(Ri5, f2_fma<true>(hR2, rz, Qrz), paz[h]);
+                        pp[h] = f2_fma<true>(Ri, f2_fma<true>(c2, w, hh), pp[h]);  // (-M - w/2) / R
                     } else {
-                        const f2 Ri3 = f2_mul(Ri, Ri2);
-                        const f2 nMRi3 = f2_mul(nM, Ri3);  // -M/R^3
-                        pax[h] = f2_fma(nMRi3, rx, pax[h]);
-                        pay[h] = f2_fma(nMRi3, ry, pay[h]);
-                        paz[h] = f2_fma(nMRi3, rz, paz[h]);
-                        pp[h] = f2_fma(nM, Ri, pp[h]);
+                        const f2 Ri3 = f2_mul<true>(Ri, Ri2);
+                        const f2 nMRi3 = f2_mul<true>(nM, Ri3);  // -M/R^3
+                        pax[h] = f2_fma<true>(nMRi3, rx, pax[h]);
+                        pay[h] = f2_fma<true>(nMRi3, ry, pay[h]);
+                        paz[h] = f2_fma<true>(nMRi3, rz, paz[h]);
+                        pp[h] = f2_fma<true>(nM, Ri, pp[h]);
                     }
                 }
             }
@@ -529,15 +499,15 @@ __device__ __forceinline__ void force_round_f32(const ForceArgs& A, uint32_t gf,
                     const f2 jx = f2_bc(j.x), jy = f2_bc(j.y), jz = f2_bc(j.z), jm = f2_bc(j.w);
 #pragma unroll
                     for (int h = 0; h < KP; ++h) {
-                        const f2 dx = f2_sub(jx, xp[h]), dy = f2_sub(jy, yp[h]), dz = f2_sub(jz, zp[h]);
-                        const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, f2_fma(dz, dz, ep[h])));
+                        const f2 dx = f2_sub<true>(jx, xp[h]), dy = f2_sub<true>(jy, yp[h]), dz = f2_sub<true>(jz, zp[h]);
+                        const f2 r2 = f2_fma<true>(dx, dx, f2_fma<true>(dy, dy, f2_fma<true>(dz, dz, ep[h])));
                         const f2 ri = f2_rsqrt(r2);
-                        const f2 mri = f2_mul(jm, ri);
-                        const f2 mri3 = f2_mul(mri, f2_mul(ri, ri));
-                        pax[h] = f2_fma(mri3, dx, pax[h]);
-                        pay[h] = f2_fma(mri3, dy, pay[h]);
-                        paz[h] = f2_fma(mri3, dz, paz[h]);
-                        pp[h] = f2_sub(pp[h], mri);
+                        const f2 mri = f2_mul<true>(jm, ri);
+                        const f2 mri3 = f2_mul<true>(mri, f2_mul<true>(ri, ri));
+                        pax[h] = f2_fma<true>(mri3, dx, pax[h]);
+                        pay[h] = f2_fma<true>(mri3, dy, pay[h]);
+                        paz[h] = f2_fma<true>(mri3, dz, paz[h]);
+                        pp[h] = f2_sub<true>(pp[h], mri);
                     }
                 }
             }

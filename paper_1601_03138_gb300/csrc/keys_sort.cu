@@ -297,7 +297,7 @@ constexpr uint32_t kValMask = kFlagAgg - 1u;
 constexpr int kMaxSpin = 1 << 20;
 constexpr int kHistBlocks = 608;
 
-// Morton keys (as k_keys) plus the histograms of all digit passes: hist
+// Morton keys plus the histograms of all digit passes: hist
 // [pass][256] with passes 0..7 the key bytes and, for several systems,
 // passes 8, 9 the two low bytes of the system id.  The last block to finish
 // (counted in *done, zero on entry) turns every pass's counts into the
@@ -414,8 +414,8 @@ __device__ __forceinline__ uint32_t coh_bucket(uint64_t k, uint32_t t, uint32_t 
     return a;
 }
 
-// Pass 1 (one block per bucket's positions, at most kCohT): Morton keys as
-// k_keys, the bucket of every key, bucket counts; the last block turns the
+// Pass 1 (one block per bucket's positions, at most kCohT): Morton keys,
+// the bucket of every key, bucket counts; the last block turns the
 // counts into offsets and cursors and flags a bucket above kCohCap.
 __global__ void __launch_bounds__(kCohBlock) k_coh_keys(CohLayout L, const double* __restrict__ x,
                                                         const double* __restrict__ y,

@@ -24,6 +24,7 @@
 #include <type_traits>
 
 #include "fdps_internal.cuh"
+#include "packed.cuh"
 
 namespace fdps {
 namespace {
@@ -284,46 +285,8 @@ struct ShortPairArgs {
     uint32_t* count;      // caller order
     double* rho;
     unsigned long long* info;  // neighbour pairs, candidate pairs, FP64 decisions
-    int mode;
     double r_fixed;
 };
-
-// Two FP32 lanes in one 64-bit register (two candidates of a pair loop turn),
-// each rounded as the scalar instruction.
-typedef unsigned long long f2;
-__device__ __forceinline__ f2 f2_pk(float lo, float hi) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void f2_up(f2 v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
-    f2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
-    f2 d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
-    f2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ float rsqrt_normal(float v) {
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-    return r;
-}
 
 // (1 - q)^8 (1 + 8 q + 25 q^2 + 32 q^3) of two candidates at q^2 = x = r2 / H^2
 // (the Wendland C6 kernel without its normalisation).  nih2 = -1 / H^2.  The
@@ -772,7 +735,6 @@ int launch_short_pairs(fdps_tree* t, fdps_psys* ps, int mode, double r_fixed, ui
     A.count = count;
     A.rho = rho;
     A.info = info3;
-    A.mode = mode;
     A.r_fixed = r_fixed;
     void (*kern)(ShortPairArgs) = mode == 0 ? k_short_pairs<0> : mode == 1 ? k_short_pairs<1>
                                 : mode == 2 ? k_short_pairs<2> : k_short_pairs<3>;

@@ -33,7 +33,6 @@ namespace fdps {
 
 struct WalkArgs {
     DevState* st;
-    const uint32_t* nd_count;
     const WalkRec* nd_walk;
     const float4* nd_f;    // COM hi/lo pairs per node
     const dvec4* nd_com;
@@ -649,7 +648,6 @@ unsigned long long walk_chunk() { return kChunk; }
 WalkArgs walk_args(fdps_tree* t, const uint32_t* sys) {
     WalkArgs A;
     A.st = t->st;
-    A.nd_count = t->nd_count;
     A.nd_walk = t->nd_walk;
     A.nd_f = t->nd_f;
     A.nd_com = t->nd_com;
