@@ -23,10 +23,12 @@
 // A thread's i-particles are paired: the pair loop evaluates one list entry
 // against two i-particles with packed two-lane FP32 instructions plus two
 // MUFU rsqrt (one i-particle per thread: plain FP32); each thread
-// accumulates one chunk of
-// the list in plain FP32 and adds the chunk's sum to its running total with
-// Kahan compensation.  Small groups split their list over several threads
-// per i-particle ("slices"), reduced in FP64 at the end.  The FP64 kernel
+// accumulates one chunk of the list in plain FP32 and adds the chunk's sum to
+// its running total with Kahan compensation.  A chunk is up to 512
+// superparticles, or 1024 particles of up to 512 leaves (before the lists held
+// the two apart: 512 entries, with all particles of the leaves among them).
+// Small groups split their list over several threads per i-particle
+// ("slices"), added with exact two-sums at the end.  The FP64 kernel
 // (a cluster of CTAs per group) evaluates the same terms on FP64 absolute
 // coordinates with FP64 sums.
 #include "fdps_internal.cuh"
