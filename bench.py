@@ -102,7 +102,7 @@ def parse():
 # bench reports null once that source has changed
 FORCE_TRAFFIC = {
     "hernquist N=16777216 theta=0.5 quad n_leaf=16 n_grp=256 eps=0.005 dt=0.00195312":
-        ("c50778b0668c3ef8", 4.3110e9 + 532.40e6),
+        ("47fb5f1929888319", 4.3138e9 + 532.58e6),
 }
 
 

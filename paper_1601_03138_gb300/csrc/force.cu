@@ -31,6 +31,8 @@
 // ("slices"), added with exact two-sums at the end.  The FP64 kernel
 // (a cluster of CTAs per group) evaluates the same terms on FP64 absolute
 // coordinates with FP64 sums.
+#include <algorithm>
+
 #include "fdps_internal.cuh"
 #include "packed.cuh"
 
@@ -615,14 +617,15 @@ __global__ void __launch_bounds__(CB, 32 * WARPS / CB) k_force_f32(ForceArgs A) 
 }
 
 // ---------------------------------------------------------------- FP64
-// One cluster of kCl64 CTAs (128 threads each) per i-group.  Bound by the
+// One cluster of CL = 8 CTAs (B = 128 threads each) per i-group, or one CTA of 64
+// threads where groups hold few particles (compute_forces).  Bound by the
 // FP64 pipe (two lanes per SM and clock: a warp instruction takes it for 16
 // clocks whatever its active lanes), so the split is the one that costs the
 // pipe least: thread t of a CTA owns K <= 4 i-particles (i = t % P + k P) and
 // slice t / P of the CTA's list entries, (K, P, slices) minimising the warps
 // times K per entry (plan_f64: 9 in 10 lanes busy on groups of 30 to 128
 // particles, where one warp per group kept 6 in 10 busy).  The entries of a
-// list go to the cluster's CTAs in turn (entry u to CTA u % kCl64), so every
+// list go to the cluster's CTAs in turn (entry u to CTA u % CL), so every
 // CTA has the same mix of cells and opened leaves, and a group of a few
 // thousand entries takes a twelfth of the time one CTA would need: with one
 // warp or CTA per group the last groups of a 10^5-particle system left most
@@ -630,34 +633,42 @@ __global__ void __launch_bounds__(CB, 32 * WARPS / CB) k_force_f32(ForceArgs A) 
 // and CTAs are summed in a fixed order, through distributed shared memory.
 // Plummer N = 100,003, quadrupoles, n_grp 128: 56.4 -> 19.4 ms for the
 // whole force calculation (one warp per group before).
-constexpr int kF64Block = 128;
-constexpr int kCl64 = 8;     // CTAs per cluster
-constexpr int kCE64 = 128;   // list entries of a CTA staged per chunk (one per thread)
-constexpr int kCJ64 = 128;   // leaf particles per shared tile
-constexpr int kK64 = 4;      // most i-particles per thread
+// (CL CTAs per cluster of B threads; a CTA stages B list entries per chunk, one
+// per thread, and B leaf particles per tile)
+constexpr int kK64 = 4;  // most i-particles per thread
 
+template <int B>
 struct F64Shared {
-    dvec4 spj[kCE64];            // centre of mass and -M
-    double q[kCE64][6];          // quadrupole (xx yy zz xy xz yz)
-    dvec4 j[kCJ64];
-    uint32_t ef[kCE64];
-    uint32_t es[kCE64];
-    uint32_t w[2 * (kF64Block / 32)];
-    double part[kK64 * 4][kF64Block];  // a thread's sums: row q * 4 + component
-    double row[4][kK64 * kF64Block];   // the CTA's sums of its i-rows
+    dvec4 spj[B];            // centre of mass and -M
+    double q[B][6];          // quadrupole (xx yy zz xy xz yz)
+    dvec4 j[B];
+    uint32_t ef[B];
+    uint32_t es[B];
+    uint32_t w[2 * (B / 32)];
+    double part[kK64 * 4][B];  // a thread's sums: row q * 4 + component
+    double row[4][kK64 * B];   // the CTA's sums of its i-rows
     uint32_t g;
 };
 
+template <int CL>
+__device__ __forceinline__ void group_barrier() {
+    if (CL > 1)
+        cluster_barrier();
+    else
+        __syncthreads();
+}
+
 // (K, P, slices) of ni i-particles: least FP64 pipe time K * warps / slices
 // per list entry; more slices on ties.
+template <int B>
 __device__ __forceinline__ GroupPlan plan_f64(uint32_t ni) {
-    GroupPlan best{kK64, kF64Block, 1};  // more than a CTA holds: rounds
+    GroupPlan best{kK64, B, 1};  // more than a CTA holds: rounds
     float bc = 3.0e38f;
 #pragma unroll
     for (int K = 1; K <= kK64; ++K) {
         const int P = (int)((ni + K - 1) / K);
-        if (P > kF64Block) continue;
-        const int nsl = kF64Block / P;
+        if (P > B) continue;
+        const int nsl = B / P;
         const float c = (float)(K * ((P * nsl + 31) / 32)) / (float)nsl;
         if (c < bc - 1e-6f) {
             bc = c;
@@ -669,10 +680,10 @@ __device__ __forceinline__ GroupPlan plan_f64(uint32_t ni) {
 
 // One round of i-particles (ib .. ib + P K - 1 of the group) with K per
 // thread, over this CTA's share of the list; called by the whole cluster.
-template <bool QUAD, int K>
+template <bool QUAD, int CL, int B, int K>
 __device__ __forceinline__ void force_round_f64(const ForceArgs& A, uint32_t gf, uint32_t ni,
                                                 unsigned long long off, uint32_t len, int P, int nsl,
-                                                uint32_t ib, uint32_t rank, F64Shared& sm) {
+                                                uint32_t ib, uint32_t rank, F64Shared<B>& sm) {
     const int t = threadIdx.x;
     const int ip = t % P, sl = t / P;
     const bool on = sl < nsl;
@@ -690,17 +701,17 @@ __device__ __forceinline__ void force_round_f64(const ForceArgs& A, uint32_t gf,
         ax[q] = ay[q] = az[q] = pp[q] = 0.0;
     }
     const int kbeg = on ? sl : 0x3FFFFFFF;
-    // entries rank, rank + kCl64, ... of the list are this CTA's
-    const uint32_t mine = len > rank ? (len - rank + kCl64 - 1) / kCl64 : 0u;
-    for (uint32_t base = 0; base < mine; base += kCE64) {
+    // entries rank, rank + CL, ... of the list are this CTA's
+    const uint32_t mine = len > rank ? (len - rank + CL - 1) / CL : 0u;
+    for (uint32_t base = 0; base < mine; base += B) {
         const uint32_t u = base + t;
-        const uint32_t ent = u < mine ? A.pool[off + rank + (unsigned long long)u * kCl64] : 0xFFFFFFFFu;
+        const uint32_t ent = u < mine ? A.pool[off + rank + (unsigned long long)u * CL] : 0xFFFFFFFFu;
         const bool leaf = ent != 0xFFFFFFFFu && (ent & kLeafTag);
         const bool spj = ent != 0xFFFFFFFFu && !(ent & kLeafTag);
         const uint32_t node = ent & ~kLeafTag;
         const uint32_t cnt = leaf ? A.nd_count[node] : 0u;
         uint32_t rs, es, ns, total;
-        block_scan2<kF64Block>(spj ? 1u : 0u, cnt, &rs, &es, &ns, &total, sm.w);
+        block_scan2<B>(spj ? 1u : 0u, cnt, &rs, &es, &ns, &total, sm.w);
         if (spj) {
             const dvec4 c = A.nd_com[node];
             sm.spj[rs] = make_dvec4(c.x, c.y, c.z, -c.w);
@@ -755,12 +766,12 @@ __device__ __forceinline__ void force_round_f64(const ForceArgs& A, uint32_t gf,
                 }
             }
         }
-        for (uint32_t c0 = 0; c0 < total; c0 += kCJ64) {
-            const uint32_t m = total - c0 < (uint32_t)kCJ64 ? total - c0 : (uint32_t)kCJ64;
+        for (uint32_t c0 = 0; c0 < total; c0 += B) {
+            const uint32_t m = total - c0 < (uint32_t)B ? total - c0 : (uint32_t)B;
             if (c0 > 0) __syncthreads();  // previous tile fully consumed
-            for (uint32_t k = t; k < m; k += kF64Block) {
+            for (uint32_t k = t; k < m; k += B) {
                 const uint32_t item = c0 + k;
-                const int src = owner_chunk<kCE64>(sm.es, item);
+                const int src = owner_chunk<B>(sm.es, item);
                 const uint32_t p = sm.ef[src] + (item - sm.es[src]);
                 sm.j[k] = make_dvec4(A.px[p], A.py[p], A.pz[p], A.pm[p]);
             }
@@ -793,22 +804,22 @@ __device__ __forceinline__ void force_round_f64(const ForceArgs& A, uint32_t gf,
     }
     __syncthreads();
     const int rows = P * K;
-    for (int k = t; k < 4 * rows; k += kF64Block) {
+    for (int k = t; k < 4 * rows; k += B) {
         const int c = k / rows, r = k - c * rows;
         const int q = r / P, ipr = r - q * P;
         double v = 0.0;
         for (int s2 = 0; s2 < nsl; ++s2) v += sm.part[q * 4 + c][s2 * P + ipr];
         sm.row[c][r] = v;
     }
-    cluster_barrier();  // every CTA's rows are written
-    // each CTA finishes every kCl64-th value
-    for (int k = t * kCl64 + (int)rank; k < 4 * rows; k += kF64Block * kCl64) {
+    group_barrier<CL>();  // every CTA's rows are written
+    // each CTA finishes every CL-th value
+    for (int k = t * CL + (int)rank; k < 4 * rows; k += B * CL) {
         const int r = k >> 2, c = k & 3;
         const uint32_t i = ib + (uint32_t)r;
         if (i >= ni) continue;
         double v = 0.0;
 #pragma unroll
-        for (int b = 0; b < kCl64; ++b) v += ld_peer_f64(peer_smem(&sm.row[c][r], (uint32_t)b));
+        for (int b = 0; b < CL; ++b) v += CL > 1 ? ld_peer_f64(peer_smem(&sm.row[c][r], (uint32_t)b)) : sm.row[c][r];
         const uint32_t p = gf + i;
         if (c == 0)
             A.ax[p] = v;
@@ -819,36 +830,36 @@ __device__ __forceinline__ void force_round_f64(const ForceArgs& A, uint32_t gf,
         else
             A.pot[p] = v + A.pm[p] / A.peps[p];  // without the particle's own entry
     }
-    cluster_barrier();  // the rows have been read: they may be rewritten
+    group_barrier<CL>();  // the rows have been read: they may be rewritten
 }
 
-template <bool QUAD>
-__global__ void __cluster_dims__(kCl64, 1, 1) __launch_bounds__(kF64Block, 4) k_force_f64(ForceArgs A) {
+template <bool QUAD, int CL, int B>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(B, 512 / B) k_force_f64(ForceArgs A) {
     extern __shared__ __align__(32) unsigned char f64_smem[];
-    F64Shared& sm = *reinterpret_cast<F64Shared*>(f64_smem);
+    F64Shared<B>& sm = *reinterpret_cast<F64Shared<B>*>(f64_smem);
     DevState* st = A.st;
     if (st->overflow & kStepInvalid) return;  // as in the FP32 kernel
     const uint32_t ngroups = (uint32_t)st->n_groups;
-    const uint32_t rank = cluster_rank();
+    const uint32_t rank = CL > 1 ? cluster_rank() : 0u;
     for (;;) {
         if (rank == 0 && threadIdx.x == 0) sm.g = atomicAdd(&st->force_counter, 1u);
-        cluster_barrier();
-        const uint32_t g = ld_peer_u32(peer_smem(&sm.g, 0));
-        cluster_barrier();  // read by all before it is rewritten or its CTA ends
+        group_barrier<CL>();
+        const uint32_t g = CL > 1 ? ld_peer_u32(peer_smem(&sm.g, 0)) : sm.g;
+        group_barrier<CL>();  // read by all before it is rewritten or its CTA ends
         if (g >= ngroups) break;
         const uint32_t ni = A.g_count[g], gf = A.g_first[g];
         const unsigned long long off = A.g_off[g];
         const uint32_t len = A.g_len[g];
         for (uint32_t ib = 0; ib < ni;) {
-            const GroupPlan pl = plan_f64(ni - ib);
+            const GroupPlan pl = plan_f64<B>(ni - ib);
             if (pl.K == 1)
-                force_round_f64<QUAD, 1>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
+                force_round_f64<QUAD, CL, B, 1>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
             else if (pl.K == 2)
-                force_round_f64<QUAD, 2>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
+                force_round_f64<QUAD, CL, B, 2>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
             else if (pl.K == 3)
-                force_round_f64<QUAD, 3>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
+                force_round_f64<QUAD, CL, B, 3>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
             else
-                force_round_f64<QUAD, 4>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
+                force_round_f64<QUAD, CL, B, 4>(A, gf, ni, off, len, pl.P, pl.nsl, ib, rank, sm);
             ib += (uint32_t)(pl.P * pl.K);
         }
     }
@@ -892,18 +903,17 @@ void launch_f32_shape(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s, int cb,
     }
 }
 
-// One resident wave of clusters of FP64 force CTAs.
-template <bool QUAD>
+// One resident wave of clusters of CL FP64 force CTAs of B threads.
+template <bool QUAD, int CL, int B>
 int launch_f64(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s) {
-    FDPS_CUDA_TRY(ctx, cudaFuncSetAttribute(k_force_f64<QUAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)sizeof(F64Shared)));
+    const int bytes = (int)sizeof(F64Shared<B>);
+    FDPS_CUDA_TRY(ctx, cudaFuncSetAttribute(k_force_f64<QUAD, CL, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_force_f64<QUAD>, kF64Block, sizeof(F64Shared)) !=
-            cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_force_f64<QUAD, CL, B>, B, bytes) != cudaSuccess ||
         per_sm < 1)
         per_sm = 1;
-    const int clusters = per_sm * ctx->sm_count / kCl64;
-    k_force_f64<QUAD><<<(clusters > 0 ? clusters : 1) * kCl64, kF64Block, sizeof(F64Shared), s>>>(A);
+    const int clusters = per_sm * ctx->sm_count / CL;
+    k_force_f64<QUAD, CL, B><<<(clusters > 0 ? clusters : 1) * CL, B, bytes, s>>>(A);
     return FDPS_OK;
 }
 
@@ -946,7 +956,20 @@ int compute_forces(fdps_tree* t, fdps_psys* ps, int spj_kind) {
     const bool quad = spj_kind == FDPS_GRAV_SPJ_QUAD;
     cudaStream_t s = ctx->stream;
     if (t->p.precision == FDPS_FP64) {
-        const int rc = quad ? launch_f64<true>(A, ctx, s) : launch_f64<false>(A, ctx, s);
+        // Groups of few particles (n_grp, or whole systems of an ensemble) take
+        // one CTA of 64 threads each: a cluster's barriers and its sums over 8 x
+        // 128 slices outlast their lists.  Up to 8 particles always; up to 16 and
+        // 32 where there are enough groups to keep the SMs busy to the end.
+        // Plummer, monopoles, cluster / CTA: n_grp 8: 0.080 / 0.074 ms at 1000
+        // particles, 9.00 / 4.79 at 10^5; n_grp 16: 0.27 / 0.32 at 5000, 1.25 /
+        // 1.00 at 20000; n_grp 32: 1.10 / 1.40 at 20000, 28.4 / 26.0 at 400000; n_grp
+        // 64: 29.5 / 29.6.  (One warp per group, before both: 5.9 ms at 10^5 and
+        // n_grp 8, 40.6 at 400000 and n_grp 64.)
+        const int64_t w = std::min<int64_t>(t->p.n_grp, ps->n / ps->n_sys);
+        const bool cta = w <= 8 || (w <= 16 && ps->n >= (1 << 14)) || (w <= 32 && ps->n >= (1 << 17));
+        const int rc = cta    ? (quad ? launch_f64<true, 1, 64>(A, ctx, s) : launch_f64<false, 1, 64>(A, ctx, s))
+                       : quad ? launch_f64<true, 8, 128>(A, ctx, s)
+                              : launch_f64<false, 8, 128>(A, ctx, s);
         if (rc) return rc;
     } else {
         // tile depth: list entries staged per chunk (0 = default 512); block
