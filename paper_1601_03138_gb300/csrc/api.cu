@@ -280,6 +280,8 @@ int ensure_tree_buffers(fdps_tree* t, fdps_psys* ps) {
     if ((rc = ensure_pool(t, 32 * n + t->n_walk_warps * (int64_t)walk_chunk()))) return rc;
     if ((rc = ensure_frontier(t, 4096))) return rc;
     t->n = n;
+    // (n_grp 16 to 256 of Plummer and Hernquist spheres: 3.2 to 3.8 n / n_grp)
+    t->est_groups = std::min<int64_t>(n, std::max<int64_t>(ps->n_sys, 4 * n / ng));
     t->valid = false;
     return FDPS_OK;
 }

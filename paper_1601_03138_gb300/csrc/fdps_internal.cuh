@@ -310,6 +310,7 @@ struct fdps_tree {
     // per-particle scratch
     int64_t cap_n = 0;
     int64_t n = 0;  // particles of the last call
+    int64_t est_groups = 0;  // and about how many i-groups they make (rules of the launches)
     uint64_t* keys_in = nullptr;   // keys in the call's starting order
     uint64_t* keys_a = nullptr;    // sort ping-pong
     uint64_t* keys_b = nullptr;

@@ -445,14 +445,17 @@ __global__ void __launch_bounds__(kWalkBlock, 8) k_walk(WalkArgs A) {
     walk_flush(A, S);
 }
 
-// The walk for systems of at most kWalkFew particles: a block per group.
-// Their groups are too few to give every warp one (1,002 groups of a 2^14
+// The walk for systems of at most kWalkFew particles and about kWalkFewGroups
+// groups: a block per group.  Their groups are too few to give every warp one (1,002 groups of a 2^14
 // Plummer sphere on 4,864 warps), and a warp alone takes a group's batches of
 // 32 cells one latency after the other; four warps take a level 128 cells at
 // a time, with the frontier in shared memory (its rest, beyond kFewFrontier,
 // in the block's part of the frontier buffers).  The same tests and the same
-// list layout as walk_group.  Plummer 2^14, n_grp 64: walk 96 -> 69 us.
+// list layout as walk_group.  Plummer 2^14, n_grp 64: walk 96 -> 69 us.  A warp per
+// group against a block, by groups: 645 49 / 41 us, 1106 51 / 41, 1835 68 / 66, 2141
+// 53 / 59, 3522 64 / 88, 11956 143 / 303.
 constexpr int64_t kWalkFew = int64_t(1) << 15;
+constexpr int64_t kWalkFewGroups = 2048;
 constexpr uint32_t kFewFrontier = 1536;
 constexpr int kWalkWarps = kWalkBlock / 32;
 
@@ -677,7 +680,7 @@ WalkArgs walk_args(fdps_tree* t, const uint32_t* sys) {
 int launch_walk(fdps_tree* t, const uint32_t* sys, int blocks) {
     fdps_ctx* ctx = t->ctx;
     const WalkArgs A = walk_args(t, sys);
-    if (t->n <= kWalkFew)
+    if (t->n <= kWalkFew && t->est_groups <= kWalkFewGroups)
         k_walk_few<<<blocks, kWalkBlock, 0, ctx->stream>>>(A);
     else
         k_walk<<<blocks, kWalkBlock, 0, ctx->stream>>>(A);

@@ -1,0 +1,35 @@
+"""Group sizes and leaf sizes on both sides of the lines where the walk, the i-group
+pass, the moments and the monopole force change their kernel by the estimated
+number of groups or nodes: structure bit for bit and forces within 1e-5 RMS of the
+oracle's."""
+import numpy as np
+import pytest
+
+import ics
+import oracle
+from test_gpu_parity import G, check_structure, ctx, rms_rel, run_gpu  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(G, ctx, n, n_grp, n_leaf, quad=False):
+    pos, vel, mass, eps = ics.make("plummer", n, 29, 0.02)
+    ps, tree = run_gpu(G, ctx, pos, vel, mass, eps, 0.7, n_leaf, n_grp, quad)
+    try:
+        ref = oracle.Tree(pos, mass, eps, theta=0.7, n_leaf=n_leaf, n_grp=n_grp, quad=quad)
+        sample = np.random.default_rng(n).choice(ref.n_groups, min(40, ref.n_groups), replace=False)
+        check_structure(G, tree, ref, n, sample)
+        _, _, acc, pot = ps.get()
+        acc_r, pot_r, tot = ref.force()
+        assert rms_rel(acc, acc_r) <= 1e-5 and rms_rel(pot, pot_r) <= 1e-5
+        st = tree.stats()
+        assert st["interactions_epj"] + st["interactions_spj"] == tot[2] and st["interactions_spj"] == tot[3]
+    finally:
+        tree.close()
+        ps.close()
+
+
+@pytest.mark.parametrize("n,n_grp,n_leaf", [(2048, 1, 1), (2049, 1, 1), (16384, 32, 8), (16385, 32, 8), (32768, 64, 8),
+                                            (32768, 8, 8), (32768, 1, 1)])
+def test_walk_lines(G, ctx, n, n_grp, n_leaf):
+    _check(G, ctx, n, n_grp, n_leaf)
