@@ -998,6 +998,9 @@ __global__ void __launch_bounds__(kB) k_group_write(int64_t n, int64_t cap_group
 // particles 25 -> 16 us, of 2001 25 -> 12 us).
 constexpr int kGroupSmallBlock = 1024;
 constexpr int64_t kGroupSmall = 32 * kGroupSmallBlock;
+// (the passes over the positions against the block, by groups: 1106 27 / 16 us,
+// 2659 27 / 25, 3522 27 / 25, 5871 29 / 31, 11956 31 / 51)
+constexpr int64_t kGroupSmallGroups = 4096;
 __global__ void __launch_bounds__(kGroupSmallBlock) k_group_small(DevState* st, int n_grp, int n_roots,
                                                                   int64_t cap_groups,
                                                                   const uint32_t* __restrict__ nd_first,
@@ -1220,7 +1223,7 @@ int select_groups(fdps_tree* t, fdps_psys* ps) {
     const int64_t n = ps->n;
     const int c = ps->cur;
     const int G = t->box_blocks;
-    if (n <= kGroupSmall) {
+    if (n <= kGroupSmall && t->est_groups <= kGroupSmallGroups) {
         k_group_small<<<1, kGroupSmallBlock, 0, s>>>(t->st, t->p.n_grp, ps->n_sys, t->cap_groups, t->nd_first,
                                                      t->nd_count, t->nd_meta, t->nd_parent, t->head, t->g_node,
                                                      t->g_first, t->g_count);

@@ -33,3 +33,8 @@ def _check(G, ctx, n, n_grp, n_leaf, quad=False):
                                             (32768, 8, 8), (32768, 1, 1)])
 def test_walk_lines(G, ctx, n, n_grp, n_leaf):
     _check(G, ctx, n, n_grp, n_leaf)
+
+
+@pytest.mark.parametrize("n,n_grp,n_leaf", [(4096, 1, 1), (4097, 1, 1), (16384, 16, 8), (16385, 16, 8)])
+def test_group_pass_lines(G, ctx, n, n_grp, n_leaf):
+    _check(G, ctx, n, n_grp, n_leaf)
