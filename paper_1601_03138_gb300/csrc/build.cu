@@ -696,6 +696,10 @@ constexpr int kMomCl = 8;
 // (65,536 Plummer / Hernquist particles, monopoles: 76 / 88 us by the cluster, 80 / 111 by
 // the grid; 90,000: 92 / 108 and 80 / 107)
 constexpr int64_t kMomSmall = int64_t(1) << 16;
+// and up to about this many nodes (grid / cluster by nodes, n_leaf 1 or 8: 14,000
+// 76 / 57 us, 24,319 117 / 111, 27,700 86 / 82, 35,600 113 / 147, 97,000 135 / 336).
+// Leaves of up to n_leaf >= 8 make about 3.5 n / n_leaf nodes, single particles 1.5 n.
+constexpr int64_t kMomSmallNodes = 28672;
 constexpr int kTopNodes = 4 * kMomBlock;
 constexpr int kMaxGridSpin = 1 << 20;
 
@@ -879,10 +883,10 @@ __global__ void k_barrier_selftest(uint32_t* count, uint32_t* flags, int max_spi
 }
 
 template <bool QUAD, bool Q64>
-int launch_moments(fdps_ctx* ctx, const MomArgs& A, int64_t n, DevState* st) {
+int launch_moments(fdps_ctx* ctx, const MomArgs& A, int64_t n, int n_leaf, DevState* st) {
     k_moments_leaves<QUAD, Q64><<<ctx->sm_count * 8, kMomBlock, 0, ctx->stream>>>(A);
     FDPS_LAUNCH_CHECK(ctx);
-    if (n <= kMomSmall) {
+    if (n <= kMomSmall && std::min(3 * n / 2, 7 * n / (2 * n_leaf)) <= kMomSmallNodes) {
         k_moments_small<QUAD, Q64><<<kMomCl, kMomBlock, 0, ctx->stream>>>(A);
         FDPS_LAUNCH_CHECK(ctx);
         return FDPS_OK;
@@ -1212,9 +1216,9 @@ int compute_moments(fdps_tree* t, fdps_psys* ps) {
     A.nd_walk = t->nd_walk;
     A.nd_fq0 = t->nd_fq0;
     A.nd_fq1 = t->nd_fq1;
-    if (t->p.moment != FDPS_QUADRUPOLE) return launch_moments<false, false>(ctx, A, ps->n, t->st);
-    if (t->p.precision == FDPS_FP64) return launch_moments<true, true>(ctx, A, ps->n, t->st);
-    return launch_moments<true, false>(ctx, A, ps->n, t->st);
+    if (t->p.moment != FDPS_QUADRUPOLE) return launch_moments<false, false>(ctx, A, ps->n, t->p.n_leaf, t->st);
+    if (t->p.precision == FDPS_FP64) return launch_moments<true, true>(ctx, A, ps->n, t->p.n_leaf, t->st);
+    return launch_moments<true, false>(ctx, A, ps->n, t->p.n_leaf, t->st);
 }
 
 int select_groups(fdps_tree* t, fdps_psys* ps) {

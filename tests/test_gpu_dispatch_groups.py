@@ -38,3 +38,9 @@ def test_walk_lines(G, ctx, n, n_grp, n_leaf):
 @pytest.mark.parametrize("n,n_grp,n_leaf", [(4096, 1, 1), (4097, 1, 1), (16384, 16, 8), (16385, 16, 8)])
 def test_group_pass_lines(G, ctx, n, n_grp, n_leaf):
     _check(G, ctx, n, n_grp, n_leaf)
+
+
+@pytest.mark.parametrize("quad", [False, True])
+@pytest.mark.parametrize("n,n_leaf", [(19115, 1), (19116, 1), (32768, 4), (32769, 4), (65536, 8), (65536, 16)])
+def test_moments_lines(G, ctx, n, n_leaf, quad):
+    _check(G, ctx, n, 64, n_leaf, quad)
