@@ -102,7 +102,7 @@ def parse():
 # bench reports null once that source has changed
 FORCE_TRAFFIC = {
     "hernquist N=16777216 theta=0.5 quad n_leaf=16 n_grp=256 eps=0.005 dt=0.00195312":
-        ("47fb5f1929888319", 4.3138e9 + 532.58e6),
+        ("5cf18aa19492317e", 4.3152e9 + 532.33e6),
 }
 
 

@@ -595,9 +595,16 @@ __device__ __forceinline__ void force_group(const ForceArgs& A, uint32_t g, F32S
 // third of their time on small groups is the latency of staging, and more
 // CTAs hide it (256 clusters, n_grp 64: 5.76 ms with four CTAs, 5.27 with five,
 // 5.15 with six; 3M clumpy particles, n_grp 256: 2.50, 2.46 and 2.45); but 16
-// where the groups are too few to fill them, up to kFewParticles (16 steps of
-// 2001 particles: 2.41 ms with 16 warps, 2.52 with 24).
-constexpr int64_t kFewParticles = int64_t(1) << 15;
+// where the groups are few for their size, so that the last ones' own time
+// counts (24 / 16 warps: 16 steps of 2001 particles, n_grp 64, 2.52 / 2.41 ms;
+// Plummer, n_grp 16 1117 groups 29 / 31 us; n_grp 64 1835 groups 88 / 84, 6754 283 /
+// 291; n_grp 128 6936 groups 574 / 557; n_grp 512 6668 groups 2.72 / 2.56 ms; n_grp
+// 1024 278 groups 1.25 / 0.99 ms).
+constexpr int64_t kFewGroups = 8192;
+static bool few_groups(const fdps_tree* t, const fdps_psys* ps) {
+    const int64_t w = std::min<int64_t>(t->p.n_grp, ps->n / ps->n_sys);
+    return ps->n <= 13 * w * w && t->est_groups <= kFewGroups;
+}
 template <bool QUAD, int EPT, int CB, int KMAX, int WARPS>
 __global__ void __launch_bounds__(CB, 32 * WARPS / CB) k_force_f32(ForceArgs A) {
     __shared__ F32Shared<QUAD, EPT, CB, KMAX> sm;
@@ -881,7 +888,7 @@ void launch_f32(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s) {
 }
 
 template <bool QUAD, int CE>
-void launch_f32_shape(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s, int cb, int kmax, int64_t n) {
+void launch_f32_shape(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s, int cb, int kmax, bool few) {
     if (cb == 64) {
         if (kmax == 2)
             launch_f32<QUAD, CE, 64, 2>(A, ctx, s);
@@ -896,7 +903,7 @@ void launch_f32_shape(const ForceArgs& A, fdps_ctx* ctx, cudaStream_t s, int cb,
             launch_f32<QUAD, CE, 128, 2>(A, ctx, s);
         else if (kmax == 4)
             launch_f32<QUAD, CE, 128, 4>(A, ctx, s);
-        else if (!QUAD && n <= kFewParticles)
+        else if (!QUAD && few)
             launch_f32<QUAD, CE, 128, 5, 16>(A, ctx, s);
         else
             launch_f32<QUAD, CE, 128, 5>(A, ctx, s);
@@ -977,16 +984,17 @@ int compute_forces(fdps_tree* t, fdps_psys* ps, int spj_kind) {
         const bool shallow = t->p.tile_depth == 256;
         const int cb = t->p.block ? t->p.block : 128;
         const int kmax = t->p.i_per_thread ? t->p.i_per_thread : 5;
+        const bool few = few_groups(t, ps);
         if (quad) {
             if (shallow)
-                launch_f32_shape<true, 256>(A, ctx, s, cb, kmax, t->n);
+                launch_f32_shape<true, 256>(A, ctx, s, cb, kmax, few);
             else
-                launch_f32_shape<true, 512>(A, ctx, s, cb, kmax, t->n);
+                launch_f32_shape<true, 512>(A, ctx, s, cb, kmax, few);
         } else {
             if (shallow)
-                launch_f32_shape<false, 256>(A, ctx, s, cb, kmax, t->n);
+                launch_f32_shape<false, 256>(A, ctx, s, cb, kmax, few);
             else
-                launch_f32_shape<false, 512>(A, ctx, s, cb, kmax, t->n);
+                launch_f32_shape<false, 512>(A, ctx, s, cb, kmax, few);
         }
     }
     FDPS_LAUNCH_CHECK(ctx);

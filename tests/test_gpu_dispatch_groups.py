@@ -44,3 +44,9 @@ def test_group_pass_lines(G, ctx, n, n_grp, n_leaf):
 @pytest.mark.parametrize("n,n_leaf", [(19115, 1), (19116, 1), (32768, 4), (32769, 4), (65536, 8), (65536, 16)])
 def test_moments_lines(G, ctx, n, n_leaf, quad):
     _check(G, ctx, n, 64, n_leaf, quad)
+
+
+@pytest.mark.parametrize("n,n_grp", [(3328, 16), (3329, 16), (53248, 64), (53249, 64), (100000, 1024), (212992, 128),
+                                     (212993, 128)])
+def test_monopole_force_lines(G, ctx, n, n_grp):
+    _check(G, ctx, n, n_grp, 8)
